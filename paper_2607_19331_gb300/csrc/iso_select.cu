@@ -23,6 +23,8 @@
 // tensor and unit change rarely and are tracked incrementally.
 #include "iso_kernels.cuh"
 
+#include <type_traits>
+
 namespace iso {
 
 // ---------------------------------------------------------------------------
@@ -282,6 +284,8 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
     uint32_t lo, hi;
     uint32_t that = 0;                       // fused pass: the estimate of the threshold
     const bool fused_t = P.fused && P.scope == ISO_SCOPE_TENSOR;
+    const bool want_t = fused_t || !P.ccv;   // the counting pass sets a run of ties apart as well
+    bool run_t = false;                      // ... when the sample shows one
     __shared__ long long s_rk[SEL_R];
     __shared__ uint32_t s_kv[SEL_R];
     __shared__ int s_edge[2];
@@ -291,6 +295,7 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
         __syncthreads();
         block_select_ranks(s_keys, S, 1, s_rk, s_hist, s_kv);
         hi = lo = that = s_kv[0];
+        run_t = true;
     } else {
         // the band's sample ranks, by one thread (binary64 is slow on this
         // GPU), then every rank in one selection: the band edges and, for
@@ -304,17 +309,19 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
             auto clampr = [&](long long x) { return x < 1 ? 1LL : (x > S ? (long long)S : x); };
             s_rk[0] = clampr(ra);
             s_rk[1] = clampr(rb);
-            s_rk[2] = clampr(rk - h);
-            s_rk[3] = clampr(rk);
+            s_rk[2] = clampr(rk);
+            s_rk[3] = clampr(rk - h);
             s_rk[4] = clampr(rk + h);
             s_edge[0] = ra >= 1;
             s_edge[1] = rb <= S;
         }
         __syncthreads();
-        block_select_ranks(s_keys, S, fused_t ? 5 : 2, s_rk, s_hist, s_kv);
+        block_select_ranks(s_keys, S, want_t ? 5 : 2, s_rk, s_hist, s_kv);
+        // no two of the five ranks share a key: no run of ties worth setting apart
+        const bool distinct = s_kv[0] != s_kv[3] && s_kv[3] != s_kv[2] && s_kv[2] != s_kv[4] && s_kv[4] != s_kv[1];
         hi = s_edge[0] ? s_kv[0] : KEY_MAX;
         lo = s_edge[1] ? s_kv[1] : 0u;
-        if (fused_t) {
+        if (fused_t || (want_t && !distinct)) {
             // t^: of the sampled keys at five ranks across the band (the band
             // edges, the rank of k and halfway between), the one that occurs
             // most often in the sample -- a run of ties wider than a fifth
@@ -322,8 +329,8 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
             // small whichever side of that run rank k falls on.
             uint32_t pv[5];
             pv[0] = s_kv[0];
-            pv[1] = s_kv[2];
-            pv[2] = s_kv[3];
+            pv[1] = s_kv[3];
+            pv[2] = s_kv[2];
             pv[3] = s_kv[4];
             pv[4] = s_kv[1];
             unsigned cnt[5] = {0, 0, 0, 0, 0};
@@ -352,7 +359,9 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
             // threshold is t^ but for a small chance, which the counts catch
             // (then the unit is resolved exactly and re-applied): the band
             // collapses to t^ and the fused pass needs no band test
-            if (pv[1] == that && pv[3] == that) { lo = that; hi = that; }
+            // (the counting pass keeps its band: a miss there costs full reads)
+            if (fused_t && pv[1] == that && pv[3] == that) { lo = that; hi = that; }
+            run_t = true;
         }
     }
     // Fused K = 1 pass: the estimate t^ of the threshold (the sample's key at
@@ -389,6 +398,7 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
         U.lo = lo;
         U.hi = hi;
         if (chat >= 0) { U.mode_t = 1; U.that = that; U.chat = chat; }
+        else if (want_t && run_t) { U.mode_t = 1; U.that = that; }
         U.state = ST_BAND;
     }
 }
@@ -614,6 +624,8 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
     uint32_t ch_pos = 0, ch_left = 0, cap = 0;
     bool ovf = false;
     uint32_t lo = 0, hi = 0, span = 0;
+    uint32_t that = 0;                            // the unit's run of ties (run mode)
+    bool run = false;
     bool want_gamma = false;
     // compact candidates (P.ccv): the warp's chunk of the unit's value
     // segment; a tile needs at most TILE slots, taken before the tile
@@ -628,8 +640,8 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
         if (lane == 0) {
             if (a_gt) atomicAdd(&au->c_gt, (unsigned long long)a_gt);
             if (a_int) atomicAdd(&au->n_int, (unsigned long long)a_int);
-            if (a_hi) atomicAdd(&au->c_hi, (unsigned long long)a_hi);
-            if (a_lo) atomicAdd(&au->c_lo, (unsigned long long)a_lo);
+            if (a_hi) atomicAdd(run ? &au->c_abv : &au->c_hi, (unsigned long long)a_hi);
+            if (a_lo) atomicAdd(run ? &au->c_eq : &au->c_lo, (unsigned long long)a_lo);
             if (want_gamma) {
                 if (gg != 0.0) atomicAdd(&au->gamma_acc, gg);
                 if (gb != 0.0) atomicAdd(&au->gamma_band, gb);
@@ -661,6 +673,8 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
             lo = au->lo;
             hi = au->hi;
             span = hi - lo;
+            run = !EMIT && au->mode_t;
+            that = au->that;
             want_gamma = au->want_gamma != 0;
             cap = (uint32_t)au->cand_cap;
             cseg = P.cand + au->cand_off;
@@ -700,47 +714,58 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
             for (int j = 0; j < VEC; ++j) d[j] = tau[j];
         };
 
-        // pass 1: every entry
-        uint32_t n_gt = 0;
+        // pass 1: every entry.  In run mode (RUN: the sample's ranks around k
+        // share a key t^) the keys equal to t^ are counted apart and never
+        // staged.  Task vectors of bf16 checkpoints hold several per cent of
+        // their entries at t^: as candidates they cost more in the select
+        // (K = 3, 1.54G entries: histogram 2.92 -> 0.59 ms, ties 0.51 -> 0.25
+        // ms) than the extra compare here (4.14 -> 4.56 ms).  Task vectors
+        // without such a run keep the plain form.
+        uint32_t n_gt = 0, n_eq = 0;
         float f_gg = 0.0f;                         // tau^2 above hi (also the non-finite detector)
         uint32_t* sp = sbl;
-        if (rem >= TILE) {
-#pragma unroll
-            for (int v = 0; v < WVEC; ++v) {
-                float tau[VEC];
-                rt.tau(v, tau);
-                if (more) rt.load_step(v, r2.xp, r2.bp, ne0, nrem, lane);
-#pragma unroll
-                for (int j = 0; j < VEC; ++j) {
-                    const uint32_t kk = key_of(tau[j]);
-                    const bool gt = kk > hi;
-                    n_gt += gt;
-                    f_gg = gt ? __fmaf_rn(tau[j], tau[j], f_gg) : f_gg;
-                    *sp = kk;
-                    sp += (kk - lo <= span) ? 32 : 0;
-                }
-                if constexpr (EMIT) stash(v, tau);
+        auto entry = [&](float tau, auto run_c) {
+            constexpr bool RUN = decltype(run_c)::value;
+            const uint32_t kk = key_of(tau);
+            const bool gt = kk > hi;
+            n_gt += gt;
+            f_gg = gt ? __fmaf_rn(tau, tau, f_gg) : f_gg;
+            *sp = kk;
+            if constexpr (RUN) {
+                const bool eq = kk == that;
+                n_eq += eq;
+                sp += (kk - lo <= span && !eq) ? 32 : 0;
+            } else {
+                sp += (kk - lo <= span) ? 32 : 0;
             }
-        } else {
+        };
+        auto pass1 = [&](auto run_c) {
+            if (rem >= TILE) {
 #pragma unroll
-            for (int v = 0; v < WVEC; ++v) {
-                float tau[VEC];
-                rt.tau(v, tau);
-                if (more) rt.load_step(v, r2.xp, r2.bp, ne0, nrem, lane);
-                const uint32_t o = (uint32_t)(v * (32 * VEC) + lane * VEC);
+                for (int v = 0; v < WVEC; ++v) {
+                    float tau[VEC];
+                    rt.tau(v, tau);
+                    if (more) rt.load_step(v, r2.xp, r2.bp, ne0, nrem, lane);
 #pragma unroll
-                for (int j = 0; j < VEC; ++j) {
-                    if (o + j >= rem) continue;
-                    const uint32_t kk = key_of(tau[j]);
-                    const bool gt = kk > hi;
-                    n_gt += gt;
-                    f_gg = gt ? __fmaf_rn(tau[j], tau[j], f_gg) : f_gg;
-                    *sp = kk;
-                    sp += ((kk >= lo) & !gt) ? 32 : 0;
+                    for (int j = 0; j < VEC; ++j) entry(tau[j], run_c);
+                    if constexpr (EMIT) stash(v, tau);
                 }
-                if constexpr (EMIT) stash(v, tau);
+            } else {
+#pragma unroll
+                for (int v = 0; v < WVEC; ++v) {
+                    float tau[VEC];
+                    rt.tau(v, tau);
+                    if (more) rt.load_step(v, r2.xp, r2.bp, ne0, nrem, lane);
+                    const uint32_t o = (uint32_t)(v * (32 * VEC) + lane * VEC);
+#pragma unroll
+                    for (int j = 0; j < VEC; ++j)
+                        if (o + j < rem) entry(tau[j], run_c);
+                    if constexpr (EMIT) stash(v, tau);
+                }
             }
-        }
+        };
+        if (!EMIT && run) pass1(std::integral_constant<bool, true>{});
+        else pass1(std::integral_constant<bool, false>{});
         const uint32_t nb = (uint32_t)(sp - sbl) >> 5;
         if (__any_sync(FULL, !(fabsf(f_gg) <= 3.402823466e38f))) {
             // a non-finite (or overflowing) sum: read the tile's keys again
@@ -786,11 +811,15 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
             for (uint32_t q = 0; q < nb; ++q) {
                 const uint32_t kk = sbl[q * 32];
                 if (store) dst[q] = kk;
-                n_hi += (kk == hi);
-                n_lo += (kk == lo) && (kk != hi);
+                n_hi += run ? (kk > that) : (kk == hi);
+                n_lo += !run && (kk == lo) && (kk != hi);
                 kbad |= (kk >= KEY_INF);
-                if (want_gamma && kk != lo) { const float f = __uint_as_float(kk); f_band = __fmaf_rn(f, f, f_band); }
+                if (want_gamma && (run ? kk > that : kk != lo)) { const float f = __uint_as_float(kk); f_band = __fmaf_rn(f, f, f_band); }
             }
+        }
+        if (run) {
+            n_lo = n_eq;
+            kbad |= n_eq && that >= KEY_INF;
         }
         if (__any_sync(FULL, kbad) && lane == 0) set_status(P.hdr, ISO_ERR_NONFINITE);
         if (want_gamma) two_sum_add(s_gb, e_gb, f_band);
@@ -800,7 +829,7 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
         if (lane == 0) {
             P.tcand[rec] = make_uint2(store ? ch_pos : 0u, store ? t_int : 0u);
             P.teq_lo[rec] = t_lo;
-            P.teq_hi[rec] = t_hi;
+            P.teq_hi[rec] = run ? t_lo : t_hi;    // the ties of t^, or of hi
             if (EMIT) P.tval[rec] = v_ovf ? KEY_NONE : (uint32_t)v_pos;
         }
         if constexpr (EMIT) {
@@ -872,8 +901,9 @@ __global__ void k_decide(Plan P) {
     const long long r = U.k - c_gt;
     U.r_src = SRC_CAND;
     if (U.mode_t) {
-        // fused pass: the band holds A candidates above t^, the E keys equal
-        // to t^ (not candidates), and the candidates below t^
+        // fused pass, or a run of ties set apart: the band holds A candidates
+        // above t^, the E keys equal to t^ (not candidates), and the
+        // candidates below t^
         const long long A = (long long)U.c_abv, E = (long long)U.c_eq;
         const long long tot = nband + E;
         if (r >= 1 && r <= tot && !U.overflow) {
@@ -934,33 +964,21 @@ __global__ void k_decide(Plan P) {
 }
 
 // ---------------------------------------------------------------------------
-// radix levels: one block per contiguous item range, one warp per tile, a
-// shared-memory histogram per (unit, run) flushed to the unit's global one.
-// Equal bins inside a warp are merged with __match_any_sync (the band keys
-// hold long runs of exact ties).  Each bin also keeps its smallest and
-// largest key (the smallest as the maximum of complements, so zero-filled
-// memory is the identity), which lets the pick stop at a single-key bin.
+// radix levels: one block per contiguous item range, a shared-memory histogram
+// per (unit, run) flushed to the unit's global one.  The keys are counted one
+// by one (equal bins of a warp's lanes are merged by the shared-memory unit;
+// merging them first with __match_any_sync measured slower).  Each bin also
+// keeps its first key and whether another was seen, which lets the pick stop
+// at a single-key bin.  A warp reads 32 tiles' lists as the few slot ranges
+// they form; one list per thread (uncoalesced, one load at a time) took 892 us
+// for the three levels of a 58.7M-entry binary32 mask at 20 % and 575 us for
+// eight binary32 experts of 0.7G entries at 10 %, this form with the runs of
+// ties set apart 62 and 365 us.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void hist_add(uint32_t* h, uint32_t* mxc, uint32_t* mx, int bin, uint32_t key,
-                                         bool valid) {
-    const unsigned active = __ballot_sync(0xFFFFFFFFu, valid);
-    if (!valid) return;
-    // lanes with equal bins form disjoint groups; each reduces over its own mask
-    const unsigned grp = __match_any_sync(active, bin);
-    const int leader = __ffs(grp) - 1;
-    const uint32_t kmin = __reduce_min_sync(grp, key);
-    const uint32_t kmax = __reduce_max_sync(grp, key);
-    if ((int)(threadIdx.x & 31) == leader) {
-        atomicAdd(&h[bin], (uint32_t)__popc(grp));
-        atomicMax(&mxc[bin], ~kmin);
-        atomicMax(&mx[bin], kmax);
-    }
-}
-
 // A unit in radix select over a pool filled by k_count (not the fused pass,
 // whose pool is not sealed) and large enough to scan as one flat array.
 __device__ __forceinline__ bool radix_flat(const Plan& P, const Unit& U) {
-    return P.scope == ISO_SCOPE_GLOBAL && U.state == ST_RADIX && U.r_src == SRC_CAND && !U.mode_t && !U.overflow &&
+    return P.scope == ISO_SCOPE_GLOBAL && U.state == ST_RADIX && U.r_src == SRC_CAND && !P.fused && !U.overflow &&
            U.n_alloc >= RADIX_FLAT_MIN;
 }
 
@@ -1048,12 +1066,12 @@ __global__ void __launch_bounds__(TPB) k_radix_flat(Plan P) {
 }
 
 template <typename XT, typename BT, bool CK>
-__global__ void __launch_bounds__(TPB) k_radix_hist(Plan P) {
+__global__ void __launch_bounds__(TPB, 4) k_radix_hist(Plan P) {
     __shared__ uint32_t s_hist[RADIX_BINS];
-    __shared__ uint32_t s_mxc[RADIX_BINS];
-    __shared__ uint32_t s_mx[RADIX_BINS];
+    __shared__ uint32_t s_key[RADIX_BINS];     // the bin's first key
+    __shared__ uint32_t s_mixed[RADIX_BINS];   // another key was seen
     if (*(volatile int32_t*)&P.hdr->n_radix == 0) return;
-    for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) { s_hist[b] = 0; s_mxc[b] = 0; s_mx[b] = 0; }
+    for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) { s_hist[b] = 0; s_key[b] = KEY_NONE; s_mixed[b] = 0; }
     __syncthreads();
     const long long items = (long long)P.K * P.n_tiles;
     const long long per = (items + gridDim.x - 1) / gridDim.x;
@@ -1074,59 +1092,76 @@ __global__ void __launch_bounds__(TPB) k_radix_hist(Plan P) {
         const int nb = 1 << (pshift - shift);
         const uint32_t base = U->r_base, prefix = U->r_prefix;
         const long long ntile = run_end - it;
+        auto add = [&](uint32_t kk, uint32_t v) {
+            const int bin = (int)((v >> shift) & (uint32_t)(nb - 1));
+            atomicAdd(&s_hist[bin], 1u);
+            uint32_t bk = s_key[bin];
+            if (bk == KEY_NONE) {
+                const uint32_t old = atomicCAS(&s_key[bin], KEY_NONE, kk);
+                bk = old == KEY_NONE ? kk : old;
+            }
+            if (kk != bk) s_mixed[bin] = 1u;
+        };
         if (U->r_src == SRC_CAND) {
-            // one tile's candidate list per thread; runs of one bin (ties)
-            // become one update
+            // 32 tiles per warp step.  A counting warp's consecutive tiles hold
+            // consecutive candidate slots until its chunk ends, so the lists
+            // of the 32 tiles form a few slot ranges, read consecutively with
+            // eight loads in flight per lane
             const uint32_t* cs = P.cand + U->cand_off;
-            for (long long q = threadIdx.x; q < ntile; q += blockDim.x) {
-                const uint2 r = P.tcand[(long long)c.i * P.n_tiles + c.g + q];
-                int cb = -1;
-                uint32_t cn = 0, cmin = 0, cmax = 0;
-                for (uint32_t j = 0; j < r.y; ++j) {
-                    const uint32_t kk = cs[r.x + j];
-                    const uint32_t v = kk - base;
-                    if ((v >> pshift) != prefix) continue;
-                    const int bin = (v >> shift) & (nb - 1);
-                    if (bin != cb) {
-                        if (cb >= 0) { atomicAdd(&s_hist[cb], cn); atomicMax(&s_mxc[cb], ~cmin); atomicMax(&s_mx[cb], cmax); }
-                        cb = bin; cn = 0; cmin = kk; cmax = kk;
+            const uint2* tc = P.tcand + (long long)c.i * P.n_tiles + c.g;
+            for (long long q0 = warp * 32; q0 < ntile; q0 += WPB * 32) {
+                const uint2 r = q0 + lane < ntile ? tc[q0 + lane] : make_uint2(0, 0);
+                const unsigned nz = __ballot_sync(0xFFFFFFFFu, r.y != 0);
+                const unsigned below = nz & ((1u << lane) - 1u);
+                const uint32_t pend = __shfl_sync(0xFFFFFFFFu, r.x + r.y, below ? 31 - __clz(below) : 0);
+                unsigned starts = __ballot_sync(0xFFFFFFFFu, r.y != 0 && (!below || pend != r.x));
+                while (starts) {
+                    const int a = __ffs(starts) - 1;
+                    starts &= starts - 1;
+                    const unsigned in = starts ? nz & ((1u << (__ffs(starts) - 1)) - 1u) : nz;
+                    const uint32_t s0 = __shfl_sync(0xFFFFFFFFu, r.x, a);
+                    const uint32_t s1 = __shfl_sync(0xFFFFFFFFu, r.x + r.y, 31 - __clz(in));
+                    for (uint32_t j = s0 + lane; j < s1; j += 256) {
+                        uint32_t kk[8];
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) kk[q] = j + 32 * q < s1 ? cs[j + 32 * q] : KEY_NONE;
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            const uint32_t v = kk[q] - base;
+                            if (kk[q] != KEY_NONE && (v >> pshift) == prefix) add(kk[q], v);
+                        }
                     }
-                    cn++;
-                    cmin = min(cmin, kk);
-                    cmax = max(cmax, kk);
                 }
-                if (cb >= 0) { atomicAdd(&s_hist[cb], cn); atomicMax(&s_mxc[cb], ~cmin); atomicMax(&s_mx[cb], cmax); }
             }
         } else {
             // full data, one tile per warp
             const void* x = P.xptr[c.i * P.n_tensors + c.t];
             for (long long q = warp; q < ntile; q += WPB) {
-                RawTile<XT, BT, CK> rt;
                 const long long e0 = (c.g + q - d.tile_base) * TILE;
-                rt.load(x, d.base, e0, d.numel, lane);
-#pragma unroll
                 for (int v = 0; v < WVEC; ++v) {
-                    float tau[VEC];
-                    rt.tau(v, tau);
                     const long long e = e0 + v * (32 * VEC) + lane * VEC;
+                    float tau[VEC];
+                    TauSrc<XT, BT, CK>::load8(x, d.base, e, d.numel, tau);
 #pragma unroll
                     for (int j = 0; j < VEC; ++j) {
                         const uint32_t kk = key_of(tau[j]);
-                        const bool ok = (e + j < d.numel) && (kk >> pshift) == prefix;
-                        hist_add(s_hist, s_mxc, s_mx, (kk >> shift) & (nb - 1), kk, ok);
+                        if ((e + j < d.numel) && (kk >> pshift) == prefix) add(kk, kk);
                     }
                 }
             }
         }
         __syncthreads();
+        // a single key k: (max, max of complements) = (k, ~k); several: both
+        // all ones, so the pick's minimum (the complement) and maximum differ
         for (int b = threadIdx.x; b < nb; b += blockDim.x) {
             if (s_hist[b]) {
+                const bool mx = s_mixed[b] != 0;
                 atomicAdd(&P.hist[ui * RADIX_BINS + b], s_hist[b]);
-                atomicMax(&P.hmxc[ui * RADIX_BINS + b], s_mxc[b]);
-                atomicMax(&P.hmx[ui * RADIX_BINS + b], s_mx[b]);
+                atomicMax(&P.hmxc[ui * RADIX_BINS + b], mx ? 0xFFFFFFFFu : ~s_key[b]);
+                atomicMax(&P.hmx[ui * RADIX_BINS + b], mx ? 0xFFFFFFFFu : s_key[b]);
                 s_hist[b] = 0;
-                s_mxc[b] = 0;
-                s_mx[b] = 0;
+                s_key[b] = KEY_NONE;
+                s_mixed[b] = 0;
             }
         }
         __syncthreads();
@@ -1200,7 +1235,8 @@ __global__ void __launch_bounds__(TPB) k_tie(Plan P) {
         uint32_t* tc = P.tcnt + (long long)c.i * P.n_tiles + c.g;
         double g_warp = 0.0;
         if (U->r_src == SRC_CAND) {
-            // one tile's candidate list per thread
+            // one tile's candidate list per thread, 16-byte loads (segments
+            // start at and are padded to multiples of four slots)
             const uint32_t* cs = P.cand + U->cand_off;
             for (long long q0 = 0; q0 < ntile; q0 += blockDim.x) {
                 const long long q = q0 + threadIdx.x;
@@ -1208,10 +1244,15 @@ __global__ void __launch_bounds__(TPB) k_tie(Plan P) {
                 float fg = 0.0f;
                 if (q < ntile) {
                     const uint2 r = P.tcand[(long long)c.i * P.n_tiles + c.g + q];
-                    for (uint32_t j = 0; j < r.y; ++j) {
-                        const uint32_t kk = cs[r.x + j];
+                    const uint32_t r1 = r.x + r.y;
+                    auto one = [&](uint32_t j, uint32_t kk) {
+                        if (j < r.x || j >= r1) return;
                         cnt += (kk == tk);
                         if (want_g && kk > tk) { const float f = __uint_as_float(kk); fg = __fmaf_rn(f, f, fg); }
+                    };
+                    for (uint32_t j = r.x & ~3u; j < r1; j += 4) {
+                        const uint4 w = *reinterpret_cast<const uint4*>(cs + j);
+                        one(j, w.x); one(j + 1, w.y); one(j + 2, w.z); one(j + 3, w.w);
                     }
                     if (want_cnt) tc[q] = cnt;
                 }
@@ -1259,7 +1300,7 @@ __device__ __forceinline__ void write_unit_stats(const Plan& P, int idx, const U
     const int i = idx / P.n_units, u = idx % P.n_units;
     iso_unit_stats s;
     s.thresh_key = (U.state == ST_OFF) ? KEY_NONE : U.t;
-    s.flags = (U.fallback ? 1u : 0u) | (U.mode_t ? 2u : 0u) | (U.overflow ? 8u : 0u) | (U.v_ok ? 32u : 0u);
+    s.flags = (U.fallback ? 1u : 0u) | (P.fused && U.mode_t ? 2u : 0u) | (U.overflow ? 8u : 0u) | (U.v_ok ? 32u : 0u);
     s.k = U.k;
     s.count_above = (U.state == ST_DONE) ? U.count_above : 0;
     s.ties_at_thresh = (U.state == ST_DONE) ? U.ties : 0;
@@ -1436,7 +1477,7 @@ __global__ void __launch_bounds__(CUT_TPB) k_cut(Plan P) {
             double above;
             if (U.r_src == SRC_DATA) above = U.gamma_rad;              // every entry above t
             else if (U.mode_t) {
-                // fused pass: gamma_band holds the candidates above t^
+                // gamma_band holds the candidates above t^
                 if (U.tie_src == TIE_EQ_HI) above = U.gamma_acc + U.gamma_band;   // t == t^
                 else above = U.gamma_acc + U.gamma_rad + (U.t < U.that ? (double)U.c_eq * sq(U.that) : 0.0);
             }
