@@ -44,6 +44,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 #include <vector>
 
 namespace iso {
@@ -297,113 +298,116 @@ __global__ void __launch_bounds__(256) k_fr_split_r(SplitR a) {
     }
 }
 
-// A_i = F_0^T dF_i in binary64 on the CUDA cores (dF_i = s_i F_i - F_0 formed
-// on the fly).  The Gram is a small difference of large terms whenever
-// frames rotate inside near-degenerate singular subspaces while the proxies
-// stay small, so this contraction (and only this one) is carried at the
-// paper's binary64 precision.  64 x 64 output tile per block, 16 rows of the
-// contraction per step, a 4 x 4 register tile per thread.
-__global__ void __launch_bounds__(256) k_fr_ftdf(Frames f, const double* dots, int i, double* A) {
-    __shared__ double sa[16][64], sb[16][64];
-    __shared__ double sg[64];
-    const long long q = f.q, d = f.d;
-    const long long k0 = (long long)blockIdx.y * 64, l0 = (long long)blockIdx.x * 64;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    if (threadIdx.x < 64) sg[threadIdx.x] = (l0 + threadIdx.x < q) ? sign_of(dots, q, i, l0 + threadIdx.x) : 0.0;
-    double acc[4][4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-    const double* F0 = f.F0;
-    const double* Fi = f.F[i];
-    __syncthreads();
-    for (long long r0 = 0; r0 < d; r0 += 16) {
-        for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-            const int rr = e >> 6, cc = e & 63;
-            const long long r = r0 + rr;
-            const long long ka = k0 + cc, lb = l0 + cc;
-            sa[rr][cc] = (r < d && ka < q) ? F0[r * q + ka] : 0.0;
-            sb[rr][cc] = (r < d && lb < q) ? fma(sg[cc], Fi[r * q + lb], -F0[r * q + lb]) : 0.0;
-        }
-        __syncthreads();
-#pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = sa[kk][ty * 4 + a];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = sb[kk][tx * 4 + b];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
-        }
-        __syncthreads();
-    }
-#pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const long long k = k0 + ty * 4 + a, l = l0 + tx * 4 + b;
-            if (k < q && l < q) A[((long long)i * q + k) * q + l] = acc[a][b];
-        }
+// ---------------------------------------------------------------------------
+// Exact-slice operands (iso_gemm.cuh) of binary64 columns.  Source z of a
+// call: 0 the first operand's columns (F_0, or F_0 + X), 1 + i the columns of
+// dF_i = s_i F_i - F_0.
+// ---------------------------------------------------------------------------
+struct OzSrc {
+    Frames f;
+    const double* dots;
+    const double* X;                 // optional: operand 0 is F_0 + X
+    unsigned long long* mx;          // [1 + K][q] largest |bits| of each column (zeroed by the caller)
+    int32_t* ex;                     // [1 + K][Qp] column exponents
+    long long Qp;
+};
+__device__ __forceinline__ double oz_value(const OzSrc& a, int z, long long e, long long k) {
+    if (z == 0) return a.X ? a.f.F0[e] + a.X[e] : a.f.F0[e];
+    return fma(sign_of(a.dots, a.f.q, z - 1, k), a.f.F[z - 1][e], -a.f.F0[e]);
 }
 
-// N = (F + dF)^T (F + dF) - I in binary64, the polar retraction's argument
-// (any departure of F^T F from I included, so the retraction also restores
-// orthonormality lost to rounding).  N is symmetric: one block per 64 x 64
-// tile on or above the diagonal (nt (nt + 1) / 2 blocks for nt tiles a side),
-// written to both halves.  Entry (k, l) and entry (l, k) are the same sum of
-// the same products in the same order, so the two halves agree bit for bit
-// also inside a diagonal tile.  Tiling as in k_fr_ftdf.
-__global__ void __launch_bounds__(256) k_op_gram64(const double* F, const double* dF, long long d, long long q,
-                                                   double* N) {
-    __shared__ double sa[16][64], sb[16][64];
-    const long long nt = (q + 63) / 64;
-    long long rest = blockIdx.x, tr = 0;
-    while (rest >= nt - tr) { rest -= nt - tr; ++tr; }      // at most nt steps
-    const long long k0 = tr * 64, l0 = (tr + rest) * 64;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    double acc[4][4];
+// every column's largest magnitude, all sources in one pass (reads each
+// array once: bound by HBM)
+__global__ void __launch_bounds__(256) k_oz_colmax(OzSrc a, int sources, int row_chunks) {
+    const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
+    const long long per = (a.f.d + row_chunks - 1) / row_chunks;
+    const long long r0 = (long long)blockIdx.y * per, r1 = min(a.f.d, r0 + per);
+    if (k >= a.f.q) return;
+    unsigned long long m[MAXK + 1];
+    double sg[MAXK];
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int z = 0; z <= MAXK; ++z) m[z] = 0;
 #pragma unroll
-        for (int b = 0; b < 4; ++b) acc[a][b] = 0.0;
-    for (long long r0 = 0; r0 < d; r0 += 16) {
-        for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-            const int rr = e >> 6, cc = e & 63;
-            const long long r = r0 + rr;
-            const long long ka = k0 + cc, lb = l0 + cc;
-            sa[rr][cc] = (r < d && ka < q) ? F[r * q + ka] + dF[r * q + ka] : 0.0;
-            sb[rr][cc] = (r < d && lb < q) ? F[r * q + lb] + dF[r * q + lb] : 0.0;
-        }
-        __syncthreads();
+    for (int i = 0; i < MAXK; ++i) sg[i] = i + 1 < sources ? sign_of(a.dots, a.f.q, i, k) : 0.0;
+    auto up = [](unsigned long long& x, double v) {
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+        x = b > x ? b : x;
+    };
+    for (long long r = r0 + threadIdx.y; r < r1; r += 8) {
+        const long long e = r * a.f.q + k;
+        const double f0 = a.f.F0[e];
+        up(m[0], a.X ? f0 + a.X[e] : f0);
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            double av[4], bv[4];
-#pragma unroll
-            for (int a = 0; a < 4; ++a) av[a] = sa[kk][ty * 4 + a];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) bv[b] = sb[kk][tx * 4 + b];
-#pragma unroll
-            for (int a = 0; a < 4; ++a)
-#pragma unroll
-                for (int b = 0; b < 4; ++b) acc[a][b] = fma(av[a], bv[b], acc[a][b]);
-        }
-        __syncthreads();
+        for (int i = 0; i < MAXK; ++i)
+            if (i + 1 < sources) up(m[i + 1], fma(sg[i], a.f.F[i][e], -f0));
     }
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
+    for (int z = 0; z <= MAXK; ++z)
+        if (z < sources) atomicMax(&a.mx[(long long)z * a.f.q + k], m[z]);
+}
+
+// |x| < 2^e for a column whose largest magnitude has these bits; columns
+// below 2^-900 share the exponent -900, OZ_NONFINITE marks NaN / infinity
+__device__ __forceinline__ int oz_exponent(unsigned long long bits) {
+    const int be = (int)(bits >> 52);
+    if (be >= 0x7FF) return OZ_NONFINITE;
+    return max(be - 1022, -900);
+}
+
+// The slabs of source z0 + blockIdx.z (slot blockIdx.z of `out`): thread =
+// (column, 8-row half) of one 16-row chunk.  x 2^(55 - e) as a 64-bit integer,
+// its signed base-256 digits from the bottom, one 16-byte store per slice
+// (consecutive columns consecutive).
+__global__ void __launch_bounds__(256) k_oz_split(OzSrc a, int z0, unsigned char* out, unsigned long long slot_bytes) {
+    const int z = z0 + blockIdx.z;
+    const int kl = threadIdx.x & 127, half = threadIdx.x >> 7;
+    const long long k = (long long)blockIdx.y * OZ_BM + kl;
+    const long long chunk = blockIdx.x, r0 = chunk * OZ_BK + 8 * half;
+    const long long q = a.f.q, d = a.f.d;
+    int e = 0;
+    if (k < q) e = oz_exponent(a.mx[(long long)z * q + k]);
+    if (chunk == 0 && half == 0) a.ex[(long long)z * a.Qp + k] = e;
+    const bool live = k < q && e < OZ_NONFINITE;
+    const double scale = __longlong_as_double((long long)(1023 + 55 - (live ? e : 0)) << 52);
+    long long v[8];
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-            const long long k = k0 + ty * 4 + a, l = l0 + tx * 4 + b;
-            if (k < q && l < q) {
-                const double v = acc[a][b] - (k == l ? 1.0 : 0.0);
-                N[k * q + l] = v;
-                if (k0 != l0) N[l * q + k] = v;
-            }
+    for (int j = 0; j < 8; ++j)
+        v[j] = (live && r0 + j < d) ? __double2ll_rn(oz_value(a, z, (r0 + j) * q + k, k) * scale) : 0;
+    unsigned char* dst = out + blockIdx.z * slot_bytes +
+                         ((unsigned long long)blockIdx.y * gridDim.x + chunk) * OZ_SLAB_BYTES +
+                         (kl >> 3) * 256 + half * 128 + (kl & 7) * 16;
+#pragma unroll
+    for (int t = OZ_SLICES - 1; t >= 0; --t) {
+        float g[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int dg = t ? (int)(signed char)v[j] : (int)v[j];
+            v[j] = (v[j] - dg) >> 8;
+            g[j] = (float)dg;
         }
+        uint32_t w[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const __nv_bfloat162 h = __floats2bfloat162_rn(g[2 * j], g[2 * j + 1]);
+            w[j] = *reinterpret_cast<const uint32_t*>(&h);
+        }
+        *reinterpret_cast<uint4*>(dst + t * OZ_SLICE_BYTES) = make_uint4(w[0], w[1], w[2], w[3]);
+    }
+}
+
+// C (qq entries per z) = the sum of the splits' partial sums, in split order
+__global__ void __launch_bounds__(256) k_oz_reduce(const double* part, int splits, int nz, long long q, double* C,
+                                                   int minus_identity) {
+    const long long total = (long long)nz * q * q;
+    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
+        double s = part[e];
+        for (int p = 1; p < splits; ++p) s += part[(long long)p * total + e];
+        if (minus_identity) {
+            const long long x = e % (q * q);
+            if (x / q == x % q) s -= 1.0;
+        }
+        C[e] = s;
+    }
 }
 
 // Split operands of an m x n bf16 / fp32 matrix G (row stride n): row-major
@@ -723,7 +727,8 @@ size_t al256(size_t v) { return (v + 255) & ~(size_t)255; }
 
 struct FrameLayout {
     long long m, n, q, Mp, Np, Qp, K;
-    size_t hdr, gram, coef, dots, vcopy;
+    size_t hdr, gram, coef, dots, mx[2], zero_end, ex, vcopy;
+    size_t tail;      // from here on: unused until A_i is formed (its operands' slabs)
     size_t cd[2], ft4[2], aq[2], sym[2], kw[2], fr4[2], y4[2], e[2], xi[2], nq[2];
     size_t ns_y, ns_z, ns_m, ns_y4, ns_z4, ns_m4, ns_t1, ns_t2, ns_t3;
     size_t a6, b6, total;
@@ -742,13 +747,19 @@ FrameLayout frame_layout(long long m, long long n, int K) {
     L.coef = take(sizeof(double) * K);
     L.dots = take(sizeof(double) * K * q);
     for (int s = 0; s < 2; ++s) L.cd[s] = take(sizeof(double) * K * K * q);
+    for (int s = 0; s < 2; ++s) L.mx[s] = take(sizeof(unsigned long long) * (K + 1) * q);
+    L.zero_end = o;
+    L.ex = take(sizeof(int32_t) * (K + 1) * Qp);
     L.vcopy = take(sizeof(double) * (K + 1) * n * q);
     for (int s = 0; s < 2; ++s) {
-        const long long Dp = s == 0 ? L.Mp : L.Np, d = s == 0 ? m : n;
-        L.ft4[s] = take(sizeof(float) * Qp * 4 * Dp);      // xi*^T split
         L.aq[s] = take(sizeof(double) * K * q * q);        // A_i = F_0^T dF_i (binary64)
         L.sym[s] = take(sizeof(double) * K * q * q);
         L.kw[s] = take(sizeof(double) * K * q * q);
+    }
+    L.tail = o;
+    for (int s = 0; s < 2; ++s) {
+        const long long Dp = s == 0 ? L.Mp : L.Np, d = s == 0 ? m : n;
+        L.ft4[s] = take(sizeof(float) * Qp * 4 * Dp);      // xi*^T split
         L.fr4[s] = take(sizeof(float) * Dp * 4 * Qp);      // F_0 split, later (F_0 + xi*) split
         L.y4[s] = take(sizeof(float) * Qp * 4 * Qp);       // Y^T split, later R split
         L.e[s] = take(sizeof(float) * Dp * Qp);            // F_0 Y, later (F_0 + xi*) R
@@ -805,7 +816,7 @@ int frame_gemm(cudaStream_t s, const float* A, long long a_rows, const float* B,
 
 struct OptLayout {
     long long m, n, q, Mp, Np, Qp, Dmax;
-    size_t hdr, gw4, gwt4, su4, sv4, dF[2], n64, xb4, r4, p, a6, b6;
+    size_t hdr, mx[2], zero_end, ex, gw4, gwt4, su4, sv4, dF[2], n64, xb4, r4, p, a6, b6;
     size_t ns_y, ns_z, ns_m, ns_y4, ns_z4, ns_m4, ns_t1, ns_t2, ns_t3, total;
 };
 
@@ -818,6 +829,10 @@ OptLayout opt_layout(long long m, long long n) {
     size_t o = 0;
     auto take = [&](size_t bytes) { const size_t at = o; o = al256(o + bytes); return at; };
     L.hdr = take(sizeof(FrameHeader));
+    for (int s = 0; s < 2; ++s) L.mx[s] = take(sizeof(unsigned long long) * q);
+    L.zero_end = o;
+    L.ex = take(sizeof(int32_t) * Qp);
+    // the four gradient operands, dead after the factor gradients: then the slabs of X_bar
     L.gw4 = take(sizeof(float) * L.Mp * 4 * L.Np);      // G_W, rows m, contraction n
     L.gwt4 = take(sizeof(float) * L.Np * 4 * L.Mp);     // G_W^T, rows n, contraction m
     L.su4 = take(sizeof(float) * Qp * 4 * L.Mp);        // (U S_0)^T
@@ -846,6 +861,75 @@ OptLayout opt_layout(long long m, long long n) {
 // launch one CUDA-core kernel of the frame merge / optimizer step on stream s
 #define FR_LAUNCH(...) do { const int _slot = prof_begin(1, s); __VA_ARGS__; prof_end(_slot, s); \
                                 if (cudaGetLastError() != cudaSuccess) return ISO_ERR_CUDA; } while (0)
+
+// C_i = F_0^T dF_i for i < K (K >= 1), or C = (F_0 + X)^T (F_0 + X) - I (K = 0),
+// in binary64 through exact slices on the tensor cores; `scratch` holds the
+// operands' slabs and, where the contraction is split, the partial sums.
+// Experts are batched as the scratch allows.  The contraction is split over
+// blocks until the last wave is full enough: `splits` minimises the number of
+// waves per split, with 1 % per split for the partial sums' traffic.
+int exact_product(cudaStream_t s, int sms, const OzSrc& src, int K, double* C, unsigned char* scratch,
+                  size_t scratch_bytes, int32_t* status) {
+    const long long q = src.f.q, d = src.f.d, Qp = src.Qp;
+    const long long nt = Qp / OZ_BM, chunks = (d + OZ_BK - 1) / OZ_BK;
+    const unsigned long long slot = (unsigned long long)nt * chunks * OZ_SLAB_BYTES;
+    const int rc = (int)std::max(1LL, std::min(256LL, (d + 255) / 256));
+    FR_LAUNCH((k_oz_colmax<<<dim3((unsigned)((q + 31) / 32), rc), dim3(32, 8), 0, s>>>(src, K + 1, rc)));
+    static std::once_flag once;
+    static cudaError_t opt = cudaSuccess;
+    std::call_once(once, [] { opt = cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM); });
+    if (opt != cudaSuccess) return ISO_ERR_CUDA;
+    if (scratch_bytes < slot * (K ? 2 : 1)) return ISO_ERR_WORKSPACE;
+    const int most = (int)std::min<unsigned long long>(std::max(K, 1), scratch_bytes / slot - (K ? 1 : 0));
+    auto split = [&](int z0, int nz, unsigned char* out) -> int {
+        FR_LAUNCH((k_oz_split<<<dim3((unsigned)chunks, (unsigned)nt, (unsigned)nz), 256, 0, s>>>(src, z0, out, slot)));
+        return ISO_OK;
+    };
+    ISO_TRY(split(0, 1, scratch));
+    for (int b0 = 0; b0 < std::max(K, 1); b0 += most) {
+        const int nz = std::min(most, std::max(K, 1) - b0);
+        unsigned char* const Bs = K ? scratch + slot : scratch;
+        if (K) ISO_TRY(split(1 + b0, nz, Bs));
+        const long long tiles = (K ? nt * nt : nt * (nt + 1) / 2) * nz;
+        const unsigned long long used = slot * (K ? 1 + nz : 1);
+        const long long fit = (long long)((scratch_bytes - used) / (8ull * (unsigned long long)(q * q) * nz));
+        const long long least = (chunks * OZ_BK + OZ_MAX_ROWS - 1) / OZ_MAX_ROWS;
+        long long best = least;
+        double cost = 1e300;
+        for (long long S = least; S <= std::max(least, 32LL); ++S) {
+            if (S > least && (S > fit || chunks / S < 2 * OZ_STEPS_LOW)) break;
+            const double c = (double)((tiles * S + sms - 1) / sms) / (double)S * (1.0 + 0.01 * (double)S);
+            if (c < cost) { cost = c; best = S; }
+        }
+        const long long per = (chunks + best - 1) / best;
+        const int splits = (int)((chunks + per - 1) / per);
+        if (splits > 1 && splits > fit) return ISO_ERR_WORKSPACE;
+        OzArgs g{};
+        g.A = scratch;
+        g.B = Bs;
+        g.b_stride = slot;
+        g.ea = src.ex;
+        g.eb = src.ex + (K ? (1 + b0) * Qp : 0);
+        g.eb_stride = Qp;
+        g.C = C + (long long)b0 * q * q;
+        g.c_stride = q * q;
+        g.part = splits > 1 ? reinterpret_cast<double*>(scratch + used) : nullptr;
+        g.q = q;
+        g.tiles = (int)nt;
+        g.chunks = (int)chunks;
+        g.per_split = (int)per;
+        g.symmetric = K ? 0 : 1;
+        g.minus_identity = K || splits > 1 ? 0 : 1;
+        g.status = status;
+        const int pslot = prof_begin(0, s);
+        k_oz_gemm<<<dim3((unsigned)(tiles / nz), (unsigned)splits, (unsigned)nz), OZ_THREADS, OZ_SMEM, s>>>(g);
+        prof_end(pslot, s);
+        if (cudaGetLastError() != cudaSuccess) return ISO_ERR_CUDA;
+        if (splits > 1)
+            FR_LAUNCH((k_oz_reduce<<<grid_of((long long)nz * q * q, sms), 256, 0, s>>>(g.part, splits, nz, q, g.C, K ? 0 : 1)));
+    }
+    return ISO_OK;
+}
 
 // Scratch of the inverse square root
 struct NsBufs {
@@ -967,7 +1051,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
     auto D = [&](size_t off) { return reinterpret_cast<double*>(ws + off); };
 
     // header, Gamma, c*, the sign dots and the column dots start at zero
-    if (cudaMemsetAsync(ws, 0, L.cd[1] + sizeof(double) * K * K * q, s) != cudaSuccess) return ISO_ERR_CUDA;
+    if (cudaMemsetAsync(ws, 0, L.zero_end, s) != cudaSuccess) return ISO_ERR_CUDA;
 
     // the V side as n x q row-major frames
     Frames fr[2];
@@ -995,9 +1079,10 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
     }
     // A_i = F_0^T dF_i (binary64), then Sym_i and Kw_i
     for (int sd = 0; sd < 2; ++sd) {
-        const dim3 grd((unsigned)((q + 63) / 64), (unsigned)((q + 63) / 64));
-        for (int i = 0; i < K; ++i)
-            FR_LAUNCH((k_fr_ftdf<<<grd, 256, 0, s>>>(fr[sd], dots, i, D(L.aq[sd]))));
+        OzSrc oz{fr[sd], dots, nullptr, reinterpret_cast<unsigned long long*>(ws + L.mx[sd]),
+                 reinterpret_cast<int32_t*>(ws + L.ex), Qp};
+        ISO_TRY(exact_product(s, sms, oz, K, D(L.aq[sd]), reinterpret_cast<unsigned char*>(ws + L.tail),
+                              L.total - L.tail, &hdr->status));
         FR_LAUNCH((k_fr_symskew<<<dim3((unsigned)(Qp / 32), (unsigned)(Qp / 32), K), dim3(32, 8), 0, s>>>(
             D(L.aq[sd]), Qp, q, D(L.sym[sd]), D(L.kw[sd]))));
     }
@@ -1121,7 +1206,7 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
     FrameHeader* hdr = reinterpret_cast<FrameHeader*>(ws + L.hdr);
     auto F = [&](size_t off) { return reinterpret_cast<float*>(ws + off); };
     auto D = [&](size_t off) { return reinterpret_cast<double*>(ws + off); };
-    if (cudaMemsetAsync(ws + L.hdr, 0, sizeof(FrameHeader), s) != cudaSuccess) return ISO_ERR_CUDA;
+    if (cudaMemsetAsync(ws + L.hdr, 0, L.zero_end - L.hdr, s) != cudaSuccess) return ISO_ERR_CUDA;
 
     Frames fr[2];
     fr[0] = Frames{}; fr[0].F0 = U; fr[0].d = m; fr[0].q = q;
@@ -1153,8 +1238,10 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
     // binary64, R = (I + N)^(-1/2) - I, E_F = dF + (F + dF) R
     for (int sd = 0; sd < 2; ++sd) {
         const long long Dp = sd == 0 ? L.Mp : L.Np, d = fr[sd].d;
-        const unsigned nt = (unsigned)((q + 63) / 64);
-        FR_LAUNCH((k_op_gram64<<<nt * (nt + 1) / 2, 256, 0, s>>>(sd == 0 ? U : V, D(L.dF[sd]), d, q, D(L.n64))));
+        OzSrc oz{fr[sd], nullptr, D(L.dF[sd]), reinterpret_cast<unsigned long long*>(ws + L.mx[sd]),
+                 reinterpret_cast<int32_t*>(ws + L.ex), Qp};
+        ISO_TRY(exact_product(s, sms, oz, 0, D(L.n64), reinterpret_cast<unsigned char*>(ws + L.gw4),
+                              L.dF[0] - L.gw4, &hdr->status));
         NsBufs nb{D(L.ns_y), D(L.ns_z), D(L.ns_m), F(L.ns_y4), F(L.ns_z4), F(L.ns_m4), F(L.ns_t1),
                   F(L.ns_t2), F(L.ns_t3)};
         ISO_TRY(ns_root(s, sms, hdr, sd, nullptr, D(L.n64), q, Qp, nb, ns_iters, F(L.r4)));

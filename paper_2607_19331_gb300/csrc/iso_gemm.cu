@@ -4,6 +4,7 @@
 #include "iso_internal.cuh"
 
 #include <mutex>
+#include <type_traits>
 
 namespace iso {
 
@@ -66,6 +67,19 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
+}
+
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+    uint32_t r[16];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
+                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+                   "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
+                   "=r"(r[14]), "=r"(r[15])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 // bounded wait on one barrier phase; false once the limit is reached or
@@ -217,6 +231,232 @@ k_gemm_tf32(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(GEMM_BN) : "memory");
+    }
+}
+
+// ---------------------------------------------------------------------------
+// exact-slice contraction (see iso_gemm.cuh)
+// ---------------------------------------------------------------------------
+namespace {
+
+// shared-memory descriptor of one slice: K-major, no swizzle; the two 8-row
+// halves of the contraction 128 bytes apart, 8-column groups 256 bytes apart
+__device__ __forceinline__ uint64_t plain_desc(uint32_t saddr) {
+    uint64_t d = 0;
+    d |= (uint64_t)((saddr >> 4) & 0x3FFFu);
+    d |= (uint64_t)(128u >> 4) << 16;        // leading byte offset: along the contraction
+    d |= (uint64_t)(256u >> 4) << 32;        // stride byte offset: along M / N
+    d |= (uint64_t)1u << 46;                 // descriptor version of sm_100; layout 0: no swizzle
+    return d;
+}
+constexpr uint32_t OZ_IDESC = (1u << 4)                 // D format: f32
+                            | (1u << 7)                 // A format: bf16
+                            | (1u << 10)                // B format: bf16
+                            | ((uint32_t)(OZ_BM >> 3) << 17)
+                            | ((uint32_t)(OZ_BM >> 4) << 24);
+
+__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
+                 :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(OZ_IDESC), "r"(accumulate) : "memory");
+}
+
+// tot += W * (the group's integer sums): this thread's lane, 64 columns
+template <int W>
+__device__ __forceinline__ void oz_drain(uint32_t taddr, long long (&tot)[64]) {
+#pragma unroll
+    for (int c = 0; c < 64; c += 16) {
+        float v[16];
+        tmem_ld16(taddr + c, v);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) tot[c + j] += (long long)__float2int_rn(v[j]) * (long long)W;
+    }
+}
+
+}  // namespace
+
+// One CTA per 128 x 128 tile (and contraction split, and expert): warp 0
+// copies slabs, warp 1 issues the products, warps 2 .. 9 drain tensor memory.
+// Bound by the tensor cores: 28 products of 128 x 128 x 16 per 16 rows, each
+// slab read once per sweep for 22 (6) products.
+__global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
+    extern __shared__ unsigned char gemm_smem_raw[];
+    unsigned char* const smem = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(gemm_smem_raw) + 127) & ~(uintptr_t)127);
+    uint64_t* const bars = reinterpret_cast<uint64_t*>(smem + OZ_STAGES * 2 * OZ_SLAB_BYTES);
+    // bars: full[S], empty[S], then per accumulator: ready[4], drained[4]
+    uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * OZ_STAGES + 8);
+    volatile int* const abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t smem_s = smem_u32(smem), bar_s = smem_u32(bars);
+    auto full_bar = [&](int s) { return bar_s + 8u * s; };
+    auto empty_bar = [&](int s) { return bar_s + 8u * (OZ_STAGES + s); };
+    auto ready_bar = [&](int a) { return bar_s + 8u * (2 * OZ_STAGES + a); };
+    auto drained_bar = [&](int a) { return bar_s + 8u * (2 * OZ_STAGES + 4 + a); };
+
+    int ti, tj;
+    if (g.symmetric) {
+        int rest = blockIdx.x;
+        ti = 0;
+        while (rest >= g.tiles - ti) { rest -= g.tiles - ti; ++ti; }   // at most `tiles` steps
+        tj = ti + rest;
+    } else {
+        ti = blockIdx.x / g.tiles;
+        tj = blockIdx.x % g.tiles;
+    }
+    const int split = blockIdx.y, z = blockIdx.z;
+    const int c0 = split * g.per_split;
+    const int nc = min(g.per_split, g.chunks - c0);     // >= 1 (host)
+    const unsigned char* const ga = g.A + ((unsigned long long)ti * g.chunks + c0) * OZ_SLAB_BYTES;
+    const unsigned char* const gb = g.B + z * g.b_stride + ((unsigned long long)tj * g.chunks + c0) * OZ_SLAB_BYTES;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < OZ_STAGES; ++s) {
+            mbar_init(full_bar(s), 1);
+            mbar_init(empty_bar(s), 1);
+        }
+        for (int a = 0; a < 4; ++a) {
+            mbar_init(ready_bar(a), 1);
+            mbar_init(drained_bar(a), OZ_EPI_WARPS);
+        }
+        *abort_flag = 0;
+        mbar_fence_init();
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+
+    if (warp == 0 && lane == 0) {
+        int it = 0;
+        for (; it < 2 * nc; ++it) {
+            const int s = it % OZ_STAGES;
+            if (!wait_phase(empty_bar(s), ((uint32_t)(it / OZ_STAGES) & 1u) ^ 1u, abort_flag)) break;
+            const bool high = it < nc;
+            const uint32_t bytes = high ? 3u * OZ_SLICE_BYTES : (uint32_t)OZ_SLAB_BYTES;
+            const unsigned long long off = (unsigned long long)(high ? it : it - nc) * OZ_SLAB_BYTES;
+            const uint32_t dst = smem_s + (uint32_t)s * 2u * OZ_SLAB_BYTES;
+            mbar_arrive_tx(full_bar(s), 2 * bytes);
+            bulk_g2s(dst, ga + off, bytes, full_bar(s));
+            bulk_g2s(dst + OZ_SLAB_BYTES, gb + off, bytes, full_bar(s));
+        }
+        // every copy this thread issued has landed before the CTA may exit
+        for (int k = (it > OZ_STAGES ? it - OZ_STAGES : 0); k < it; ++k)
+            for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
+                if (mbar_try_wait(full_bar(k % OZ_STAGES), (uint32_t)(k / OZ_STAGES) & 1u)) break;
+    } else if (warp == 1 && lane == 0) {
+        bool ok = true;
+        int it = 0, used[4] = {0, 0, 0, 0};              // drains of each accumulator so far
+        // one sweep: groups G0 .. G0 + NG - 1, a drain every STEPS steps
+        auto sweep = [&](auto g0_c, auto ng_c, auto steps_c) {
+            constexpr int G0 = decltype(g0_c)::value, NG = decltype(ng_c)::value, STEPS = decltype(steps_c)::value;
+            for (int c = 0; c < nc && ok; ++c, ++it) {
+                const int s = it % OZ_STAGES;
+                if (!wait_phase(full_bar(s), (uint32_t)(it / OZ_STAGES) & 1u, abort_flag)) { ok = false; break; }
+                tc_fence_after();
+                const bool first = c % STEPS == 0, last = c % STEPS == STEPS - 1 || c == nc - 1;
+                const uint32_t a0 = smem_s + (uint32_t)s * 2u * OZ_SLAB_BYTES, b0 = a0 + OZ_SLAB_BYTES;
+#pragma unroll
+                for (int a = 0; a < NG; ++a) {
+                    if (!ok) continue;
+                    if (first && used[a] > 0) {
+                        if (!wait_phase(drained_bar(a), (uint32_t)(used[a] - 1) & 1u, abort_flag)) { ok = false; continue; }
+                        tc_fence_after();
+                    }
+                    const int grp = G0 + a;
+#pragma unroll
+                    for (int t = 0; t <= grp; ++t)
+                        umma_bf16(tmem + (uint32_t)a * OZ_BM, plain_desc(a0 + (uint32_t)t * OZ_SLICE_BYTES),
+                                  plain_desc(b0 + (uint32_t)(grp - t) * OZ_SLICE_BYTES), (first && t == 0) ? 0u : 1u);
+                    if (last) {
+                        umma_commit(ready_bar(a));
+                        ++used[a];
+                    }
+                }
+                umma_commit(empty_bar(s));
+            }
+        };
+        using I = std::integral_constant<int, 0>;
+        sweep(I{}, std::integral_constant<int, 3>{}, std::integral_constant<int, OZ_STEPS_HIGH>{});
+        if (ok) sweep(std::integral_constant<int, 3>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, OZ_STEPS_LOW>{});
+        // products issued before a give-up still hold shared memory: wait for
+        // them (the last commit of every stage that was read)
+        if (!ok)
+            for (int k = (it > OZ_STAGES ? it - OZ_STAGES : 0); k < it; ++k)
+                for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
+                    if (mbar_try_wait(empty_bar(k % OZ_STAGES), (uint32_t)(k / OZ_STAGES) & 1u)) break;
+    } else if (warp >= 2) {
+        // lane of tensor memory: 32 (warp % 4) + lane; columns 64 h .. + 63
+        const int quad = warp & 3, h = (warp - 2) >> 2;
+        const uint32_t tq = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(64 * h);
+        const long long row = (long long)ti * OZ_BM + quad * 32 + lane;
+        const long long colb = (long long)tj * OZ_BM + 64 * h;
+        const long long q = g.q;
+        double* const dst = g.part ? g.part + ((long long)split * gridDim.z + z) * q * q : g.C + z * g.c_stride;
+        bool ok = true;
+        int used[4] = {0, 0, 0, 0};
+        auto take = [&](int a, auto w, long long (&tot)[64]) {
+            if (!ok) return;
+            if (!wait_phase(ready_bar(a), (uint32_t)used[a] & 1u, abort_flag)) { ok = false; return; }
+            tc_fence_after();
+            oz_drain<decltype(w)::value>(tq + (uint32_t)a * OZ_BM, tot);
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(drained_bar(a));
+            ++used[a];
+        };
+        long long tot[64];
+#pragma unroll
+        for (int j = 0; j < 64; ++j) tot[j] = 0;
+        for (int c = 0; c < nc && ok; c += OZ_STEPS_HIGH) {
+            take(0, std::integral_constant<int, 1 << 16>{}, tot);
+            take(1, std::integral_constant<int, 1 << 8>{}, tot);
+            take(2, std::integral_constant<int, 1>{}, tot);
+        }
+        // the high groups' total waits in the output array (an integer below
+        // 2^53 for any contraction below 2^23 rows) while the low ones run
+#pragma unroll
+        for (int j = 0; j < 64; ++j) {
+            if (ok && row < q && colb + j < q) dst[row * q + colb + j] = (double)tot[j];
+            tot[j] = 0;
+        }
+        for (int c = 0; c < nc && ok; c += OZ_STEPS_LOW) {
+            take(0, std::integral_constant<int, 1 << 24>{}, tot);
+            take(1, std::integral_constant<int, 1 << 16>{}, tot);
+            take(2, std::integral_constant<int, 1 << 8>{}, tot);
+            take(3, std::integral_constant<int, 1>{}, tot);
+        }
+        if (!ok) {
+            if (lane == 0 && g.status) atomicCAS(g.status, 0, (int32_t)ISO_ERR_TIMEOUT);
+        } else if (row < q) {
+            const int er = g.ea[row];
+            const int32_t* eb = g.eb + z * g.eb_stride;
+#pragma unroll
+            for (int j = 0; j < 64; ++j) {
+                const long long col = colb + j;
+                if (j % 4 == 0) asm volatile("" ::: "memory");   // keeps the loads of later columns behind (registers)
+                if (col >= q) continue;
+                const int ec = eb[col];
+                double v = fma(dst[row * q + col], 4294967296.0, (double)tot[j]);
+                v = (er >= OZ_NONFINITE || ec >= OZ_NONFINITE) ? __longlong_as_double(0x7FF8000000000000LL)
+                                                                : scalbn(v, er + ec - 62);
+                if (g.minus_identity && row == col) v -= 1.0;
+                dst[row * q + col] = v;
+                if (g.symmetric && ti != tj) dst[col * q + row] = v;
+            }
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(512) : "memory");
     }
 }
 

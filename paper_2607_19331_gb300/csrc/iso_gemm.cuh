@@ -68,6 +68,73 @@ struct GemmArgs {
 __global__ void k_gemm_tf32(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                             GemmArgs g);
 
+// ---------------------------------------------------------------------------
+// Binary64 contractions on the tensor cores: C = A^T B for binary64 columns,
+// from integer slices whose products and sums are exact in binary32 (the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump, "Error-free
+// transformations of matrix multiplication by using fast routines of matrix
+// multiplication", Numer. Algorithms 59, 2012).
+//
+// A column x with |x_r| < 2^e is written x_r = 2^(e - 7) sum_t d_t 2^(-8 t),
+// t = 0 .. 6, with integer digits |d_t| <= 128 (x rounded to 55 fractional
+// bits below 2^e), stored as bf16, which holds them exactly.  Then
+//   C_kl = 2^(e_k + e_l - 14) sum_g 2^(-8 g) I_g,  I_g = sum_{s + t = g} <a_s, b_t>
+// over g = 0 .. 6 (28 of the 49 slice pairs; the rest lies below the
+// rounding of the binary64 sum it replaces).  Each I_g accumulates in tensor
+// memory as binary32 over at most OZ_STEPS_* steps, which keeps every partial
+// sum at or below 2^24 whatever the digits (an exact integer), and is then
+// added to 64-bit integers in registers.
+//
+// Operand layout: slab (kt, c) holds columns 128 kt .. + 127, rows 16 c ..
+// + 15 of all seven slices, slice after slice, each 4 KB in the core-matrix
+// order the products read from shared memory (8 columns x 8 rows of 128
+// bytes; row halves 128 bytes apart, column groups 256 bytes apart), so one
+// bulk copy brings a slab and no tensor map or swizzle is needed.
+//
+// Measured on one 3584 x 18944 matrix (q = 3584): A_i of three experts, both
+// sides, 1441 ms as binary64 on the CUDA cores (64 x 64 tiles, 1.2 TFLOP/s,
+// the chip's binary64 rate) against 42 ms here (28 bf16 products for each: 1.2
+// PFLOP/s); the merge 1533 -> 140 ms.  The optimizer step of a 1536 x 8960
+// matrix, bound by F^T F, 29.7 -> 9.2 ms.
+constexpr int OZ_SLICES = 7;
+constexpr int OZ_BM = 128;                              // columns of A (and of B) per tile
+constexpr int OZ_BK = 16;                               // contraction rows per step
+constexpr int OZ_SLICE_BYTES = OZ_BM * OZ_BK * 2;       // 4 KB
+constexpr int OZ_SLAB_BYTES = OZ_SLICES * OZ_SLICE_BYTES;
+constexpr int OZ_STAGES = 3;
+constexpr int OZ_EPI_WARPS = 8;
+constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;
+constexpr int OZ_SMEM = 128 + OZ_STAGES * 2 * OZ_SLAB_BYTES + 256;
+// Two sweeps over the contraction, three and four slice groups each (a group
+// takes 128 of the 512 tensor-memory columns): groups 0 .. 2 read slices
+// 0 .. 2, groups 3 .. 6 all seven.  Steps per drain: (group + 1) pairs x 16
+// rows x 2^14 <= 2^24.
+constexpr int OZ_STEPS_HIGH = 21;                       // 3 pairs x 336 rows <= 1024
+constexpr int OZ_STEPS_LOW = 9;                         // 7 pairs x 144 rows <= 1024
+// 64-bit totals: |I_g| 2^(8 (6 - g)) summed over g = 3 .. 6 stays below 2^63
+constexpr long long OZ_MAX_ROWS = 1LL << 20;
+constexpr int32_t OZ_NONFINITE = 1 << 20;               // exponent of a column holding a NaN or an infinity
+
+struct OzArgs {
+    const unsigned char* A;   // slabs [kt][chunk]
+    const unsigned char* B;   // expert z at B + z * b_stride
+    unsigned long long b_stride;
+    const int32_t* ea;        // column exponents of A; of B at eb + z * eb_stride
+    const int32_t* eb;
+    long long eb_stride;
+    double* C;                // q x q, row stride q; expert z at C + z * c_stride
+    long long c_stride;
+    double* part;             // split contraction: [split][z][q][q] partial sums (NULL: C is written)
+    long long q;
+    int32_t tiles;            // tiles a side
+    int32_t chunks;           // 16-row chunks of the contraction
+    int32_t per_split;        // chunks per split (gridDim.y splits)
+    int32_t symmetric;        // A == B: tiles on and above the diagonal, written to both halves
+    int32_t minus_identity;   // subtract I (with one split only; k_oz_reduce otherwise)
+    int32_t* status;
+};
+__global__ void k_oz_gemm(OzArgs g);
+
 // Host side: a 2-D tensor map over a row-major fp32 array of `rows` x `cols`
 // (cols a multiple of 4, rows and the row stride as given) with a 32 x 128
 // box and the 128-byte swizzle the kernel's shared-memory descriptors expect.
