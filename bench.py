@@ -97,9 +97,9 @@ def algorithmic_bytes(shapes, K, inputs, op, scope="tensor", two_pass=False):
 # the source files each timed kernel kind is built from (besides the shared headers)
 KERNEL_SOURCES = {
     "count": ["iso_fused.cu", "iso_select.cu"],   # fused K = 1 pass, or the two-pass counting read
-    "apply": ["iso_apply.cu", "iso_merge.cu"],
-    "merge": ["iso_merge.cu"],                    # the apply pass of K >= 2 (and RAM) runs k_merge alone
-    "gram": ["iso_merge.cu"],
+    "apply": ["iso_apply.cu", "iso_merge.cu", "iso_merge.cuh"],
+    "merge": ["iso_merge.cu", "iso_merge.cuh"],   # the apply pass of K >= 2 (and RAM) runs k_merge alone
+    "gram": ["iso_gram.cu", "iso_merge.cuh"],
     "block_select": ["iso_block.cu"],
 }
 

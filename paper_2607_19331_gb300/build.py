@@ -15,9 +15,10 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libiso_gb300.so")
-SOURCES = ["iso_api.cu", "iso_select.cu", "iso_apply.cu", "iso_merge.cu", "iso_block.cu", "iso_fused.cu",
-           "iso_gemm.cu", "iso_frame.cu", "iso_range.cu"]
-HEADERS = ["iso_internal.cuh", "iso_kernels.cuh", "iso_gemm.cuh"]
+SOURCES = ["iso_merge.cu", "iso_merge_f32.cu", "iso_gram.cu", "iso_compact.cu", "iso_compact_f32.cu", "iso_select.cu",
+           "iso_api.cu", "iso_apply.cu", "iso_block.cu", "iso_fused.cu", "iso_gemm.cu", "iso_frame.cu", "iso_range.cu"]
+HEADERS = ["iso_internal.cuh", "iso_kernels.cuh", "iso_merge.cuh", "iso_gemm.cuh"]
+INCLUDED = {"iso_merge_f32.cu": ["iso_merge.cu"], "iso_compact_f32.cu": ["iso_compact.cu"]}   # sources that include others
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-static-global-template-stub=false", "-Xcompiler", "-fPIC,-ffp-contract=off",
          "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -45,7 +46,7 @@ def build(force: bool = False, verbose: bool = False, extra=None) -> str:
         s = os.path.join(CSRC, src)
         o = os.path.join(BUILD, src.replace(".cu", ".o"))
         objs.append(o)
-        if force or _stale(o, [s] + hdrs):
+        if force or _stale(o, [s] + hdrs + [os.path.join(CSRC, x) for x in INCLUDED.get(src, [])]):
             cmd = [nvcc(), *ARCH, *FLAGS, *(extra or []), "-c", s, "-o", o]
             jobs.append(cmd)
 

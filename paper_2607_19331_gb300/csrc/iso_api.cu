@@ -682,53 +682,64 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
             if (need_gram_pass) {
                 auto gram = [&](auto kc) {
                     constexpr int KC = decltype(kc)::value;
-                    if constexpr (KC >= 2) {
-                        if (c.ccv) {
-                            const int cs = compact_smem_bytes<BT, KC>();
-                            ISO_TRY(smem_optin(k_gramk_c<XT, BT, CK, KC>, cs));
-                            return launch(KD_GRAM, s, [&] { k_gramk_c<XT, BT, CK, KC><<<sms * 2, TPB, cs, s>>>(P); });
-                        }
-                    }
-                    const int ggrid = sms * gram_blocks_per_sm(KC);
-                    const int smem = gram_smem_bytes<XT, BT, KC>();
+                    const int smem = gram_smem_bytes<XT, BT, CK, KC>();
                     ISO_TRY(smem_optin(k_gramk<XT, BT, CK, KC>, smem));
-                    return launch(KD_GRAM, s, [&] { k_gramk<XT, BT, CK, KC><<<ggrid, TPB, smem, s>>>(P); });
+                    return launch(KD_GRAM, s, [&] { k_gramk<XT, BT, CK, KC><<<sms * MERGE_BLOCKS_PER_SM, TPB, smem, s>>>(P); });
                 };
-                if (K == 1) ISO_TRY(gram(std::integral_constant<int, 1>{}));
+                auto gram_c = [&](auto kc) {
+                    constexpr int KC = decltype(kc)::value;
+                    const int cs = compact_smem_bytes<BT, KC>();
+                    ISO_TRY(smem_optin(k_gramk_c<XT, BT, CK, KC>, cs));
+                    return launch(KD_GRAM, s, [&] { k_gramk_c<XT, BT, CK, KC><<<sms * 2, TPB, cs, s>>>(P); });
+                };
+                if (c.ccv) {
+                    if (K == 2) ISO_TRY(gram_c(std::integral_constant<int, 2>{}));
+                    else if (K <= 4) ISO_TRY(gram_c(std::integral_constant<int, 4>{}));
+                    else ISO_TRY(gram_c(std::integral_constant<int, 8>{}));
+                }
+                else if (K == 1) ISO_TRY(gram(std::integral_constant<int, 1>{}));
                 else if (K == 2) ISO_TRY(gram(std::integral_constant<int, 2>{}));
-                else if (K <= 4) ISO_TRY(gram(std::integral_constant<int, 4>{}));
+                else if (K == 3) ISO_TRY(gram(std::integral_constant<int, 3>{}));
+                else if (K == 4) ISO_TRY(gram(std::integral_constant<int, 4>{}));
                 else ISO_TRY(gram(std::integral_constant<int, 8>{}));
             }
             ISO_TRY(launch(KD_SOLVE, s, [&] { k_solve<<<(T + 127) / 128, 128, 0, s>>>(P, gram_mode); }));
         }
-        auto merge = [&](auto kc) {
+        auto merge_op = [&](auto kc, auto opf) {
+            constexpr int KC = decltype(kc)::value, OPF = decltype(opf)::value;
+            const int smem = merge_smem_bytes<XT, BT, KC>();
+            ISO_TRY(smem_optin(k_merge<XT, BT, CK, KC, OPF>, smem));
+            return launch(KD_APPLY, s, [&] { k_merge<XT, BT, CK, KC, OPF><<<sms * MERGE_BLOCKS_PER_SM, TPB, smem, s>>>(P); });
+        };
+        auto merge = [&](auto kc) -> int {
+            if (c.op == ISO_OP_TIES) return merge_op(kc, std::integral_constant<int, OPF_TIES>{});
+            if (c.op == ISO_OP_ISO) return merge_op(kc, std::integral_constant<int, OPF_ISO>{});
+            if (c.op == ISO_OP_RAM) return merge_op(kc, std::integral_constant<int, OPF_RAM>{});
+            return merge_op(kc, std::integral_constant<int, OPF_SUM>{});
+        };
+        auto merge_c = [&](auto kc) {
             constexpr int KC = decltype(kc)::value;
-            if (c.ccv) {
-                const int cs = compact_smem_bytes<BT, KC>();
-                if (c.op == ISO_OP_TIES) {
-                    ISO_TRY(smem_optin(k_merge_c<XT, BT, CK, KC, OPF_TIES>, cs));
-                    return launch(KD_APPLY, s, [&] { k_merge_c<XT, BT, CK, KC, OPF_TIES><<<sms * 2, TPB, cs, s>>>(P); });
-                }
-                ISO_TRY(smem_optin(k_merge_c<XT, BT, CK, KC, OPF_OTHER>, cs));
-                return launch(KD_APPLY, s, [&] { k_merge_c<XT, BT, CK, KC, OPF_OTHER><<<sms * 2, TPB, cs, s>>>(P); });
-            }
+            const int cs = compact_smem_bytes<BT, KC>();
             if (c.op == ISO_OP_TIES) {
-                const int smem = merge_smem_bytes<XT, BT, KC, OPF_TIES>();
-                const int mgrid = sms * merge_blocks_per_sm(KC, OPF_TIES);
-                ISO_TRY(smem_optin(k_merge<XT, BT, CK, KC, OPF_TIES>, smem));
-                return launch(KD_APPLY, s, [&] { k_merge<XT, BT, CK, KC, OPF_TIES><<<mgrid, TPB, smem, s>>>(P); });
+                ISO_TRY(smem_optin(k_merge_c<XT, BT, CK, KC, OPF_TIES>, cs));
+                return launch(KD_APPLY, s, [&] { k_merge_c<XT, BT, CK, KC, OPF_TIES><<<sms * 2, TPB, cs, s>>>(P); });
             }
-            const int smem = merge_smem_bytes<XT, BT, KC, OPF_OTHER>();
-            const int mgrid = sms * merge_blocks_per_sm(KC, OPF_OTHER);
-            ISO_TRY(smem_optin(k_merge<XT, BT, CK, KC, OPF_OTHER>, smem));
-            return launch(KD_APPLY, s, [&] { k_merge<XT, BT, CK, KC, OPF_OTHER><<<mgrid, TPB, smem, s>>>(P); });
+            ISO_TRY(smem_optin(k_merge_c<XT, BT, CK, KC, OPF_ISO>, cs));
+            return launch(KD_APPLY, s, [&] { k_merge_c<XT, BT, CK, KC, OPF_ISO><<<sms * 2, TPB, cs, s>>>(P); });
         };
         if (K == 1 && fuse_block) return ISO_OK;
         // RAM with one expert: the merge pass (its activity test lives there)
-        if (K == 1 && c.op == ISO_OP_RAM) ISO_TRY(merge(std::integral_constant<int, 2>{}));
+        if (c.ccv) {
+            if (K == 2) ISO_TRY(merge_c(std::integral_constant<int, 2>{}));
+            else if (K <= 4) ISO_TRY(merge_c(std::integral_constant<int, 4>{}));
+            else ISO_TRY(merge_c(std::integral_constant<int, 8>{}));
+        }
+        else if (K == 1 && c.op == ISO_OP_RAM)
+            ISO_TRY(merge_op(std::integral_constant<int, 1>{}, std::integral_constant<int, OPF_RAM>{}));
         else if (K == 1) ISO_TRY(launch(KD_APPLY, s, [&] { k_apply<XT, BT, CK, 1><<<pgrid, TPB, 0, s>>>(P); }));
         else if (K == 2) ISO_TRY(merge(std::integral_constant<int, 2>{}));
-        else if (K <= 4) ISO_TRY(merge(std::integral_constant<int, 4>{}));
+        else if (K == 3) ISO_TRY(merge(std::integral_constant<int, 3>{}));
+        else if (K == 4) ISO_TRY(merge(std::integral_constant<int, 4>{}));
         else ISO_TRY(merge(std::integral_constant<int, 8>{}));
         return ISO_OK;
     });

@@ -1,6 +1,6 @@
 // iso_kernels.cuh -- kernel declarations (definitions and explicit
 // instantiations live in iso_select.cu, iso_apply.cu, iso_merge.cu,
-// iso_block.cu and iso_fused.cu).
+// iso_gram.cu, iso_compact.cu, iso_block.cu and iso_fused.cu).
 #pragma once
 
 #include "iso_internal.cuh"
@@ -61,20 +61,17 @@ __global__ void k_fix_plan(Plan P);
 template <bool CK> __global__ void k_fix(Plan P);
 
 // apply: K = 1 (iso_apply.cu); K >= 2 with a compile-time bound KC >= K on
-// the expert count, and the Gram pass for any K (iso_merge.cu)
+// the expert count (iso_merge.cu), and the Gram pass for any K (iso_gram.cu)
 template <typename XT, typename BT, bool CK, int KC> __global__ void k_apply(Plan P);
-// k_merge is compiled for TIES alone and for the other operators (ISO, whose
-// 1-D tensors take the plain average, TA and RAM): TIES needs no coefficients
-enum MergeOpFamily : int { OPF_TIES = 0, OPF_OTHER = 1 };
+// k_merge is compiled per operator family (ISO's 1-D tensors take the plain
+// average, so OPF_ISO holds both forms; TA is OPF_SUM), two blocks per SM
+enum MergeOpFamily : int { OPF_TIES = 0, OPF_ISO = 1, OPF_RAM = 2, OPF_SUM = 3 };
 template <typename XT, typename BT, bool CK, int KC, int OPF> __global__ void k_merge(Plan P);
 template <typename XT, typename BT, bool CK, int KC> __global__ void k_gramk(Plan P);
-// k_merge: resident blocks of TPB threads per SM, two for every expert bound
-// and family (eight experts read their step from the stage entry by entry)
-constexpr int merge_blocks_per_sm(int KC, int OPF) { return 2; }
-// k_merge's dynamic shared memory (its per-warp staging ring)
-template <typename XT, typename BT, int KC, int OPF> int merge_smem_bytes();
-template <typename XT, typename BT, int KC> int gram_smem_bytes();
-constexpr int gram_blocks_per_sm(int KC) { return 2; }
+constexpr int MERGE_BLOCKS_PER_SM = 2;
+// their dynamic shared memory (the warps' chunk rings)
+template <typename XT, typename BT, int KC> int merge_smem_bytes();
+template <typename XT, typename BT, bool CK, int KC> int gram_smem_bytes();
 template <typename XT, typename BT, bool CK, int KC, int OPF> __global__ void k_merge_c(Plan P);
 template <typename XT, typename BT, bool CK, int KC> __global__ void k_gramk_c(Plan P);
 // the compact kernels' dynamic shared memory (one stage per warp)

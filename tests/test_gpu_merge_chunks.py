@@ -1,0 +1,62 @@
+"""The merge and Gram passes at the edges of what they stream: tensors one entry
+below, at and above a step, a chunk and a tile, every compile-time expert bound
+(1, 2, 3, 4, 8) and a count between bounds, both element types, checkpoints
+and task vectors, and the quotients by 3, 5, 6 and 7 of the disjoint mean.
+Values against the oracle within the parity bounds."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+import paper_2607_19331_gb300 as iso
+from parity_util import assert_values_close, to_np
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+OPS = {"ta": oracle.TA, "ties": oracle.TIES, "iso": oracle.ISO, "ram": oracle.RAM}
+SIZES = [1, 7, 8, 127, 128, 129, 255, 257, 511, 512, 513, 1023, 1024, 1025, 2049, 5000]
+
+
+def _set(dtype, seed, std, base=None):
+    g = torch.Generator().manual_seed(seed)
+    out = []
+    for q, n in enumerate(SIZES):
+        t = torch.randn(n, generator=g) * std
+        if base is not None:
+            t = t + base[q].float().reshape(-1)
+        out.append(t.to(dtype).reshape(1, n) if q % 3 else t.to(dtype))
+    return out
+
+
+@pytest.mark.parametrize("K", [1, 2, 3, 4, 5, 7, 8])
+@pytest.mark.parametrize("op", ["ta", "ties", "iso", "ram"])
+@pytest.mark.parametrize("bdt,xdt,ckpt", [(torch.bfloat16, torch.bfloat16, True), (torch.bfloat16, torch.float32, False),
+                                          (torch.float32, torch.float32, True), (torch.float32, torch.bfloat16, False)])
+def test_ragged_chunks(K, op, bdt, xdt, ckpt):
+    th0 = _set(bdt, 1, 0.02)
+    xs = [_set(xdt, 2 + i, 1e-3, th0 if ckpt else None) for i in range(K)]
+    one = [t.dim() == 1 for t in th0]
+    kw = dict(density=0.4, eps_act=5e-4)
+    out, st = iso.iso_merge([t.to(DEV) for t in th0], [[t.to(DEV) for t in x] for x in xs], op=op,
+                            experts_are_deltas=not ckpt, stats=True, **kw)
+    torch.cuda.synchronize()
+    assert int(st.status.item()) == 0
+    r = oracle.merge([to_np(t) for t in th0], [[to_np(t) for t in x] for x in xs], OPS[op],
+                     experts_are_deltas=not ckpt, shapes=[(1, n) for n in SIZES], is_1d=one, **kw)
+    for q in range(len(th0)):
+        assert_values_close(to_np(out[q]), r["out64"][q], r["mag"][q], f"chunks {op} K={K} tensor {q}", op=op, K=K)
+
+
+def test_mean_of_three_is_the_division():
+    # every quotient by 3 of a mantissa sweep, subnormal and overflowing sums
+    # included: identical experts s give (s + s + s) / 3 rounded as IEEE
+    u = torch.arange(0, 1 << 16, dtype=torch.int32) * 32749 % (0x7F000000 >> 2)
+    a = torch.cat([u, u + 0x3F000000 - (1 << 23), torch.tensor([1, 2, 3, 0x7F7FFFFF, 0x7F000000], dtype=torch.int32)])
+    a = a.view(torch.float32).clone()
+    a = a[torch.isfinite(a)]
+    th0 = [torch.zeros_like(a).to(DEV)]
+    out = iso.iso_merge(th0, [[a.to(DEV)], [a.to(DEV)], [a.to(DEV)]], op="ram", eps_act=0.0)
+    s = ((a.numpy() + a.numpy()) + a.numpy()).astype(np.float32)
+    ref = (s / np.float32(3)).astype(np.float32)
+    got = out[0].cpu().numpy()
+    assert np.array_equal(got.view(np.uint32), np.where(s == 0, np.float32(0), ref).view(np.uint32))
