@@ -140,12 +140,12 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
 
     // Full block of BLOCK_TPB x BFE entries in rows of a multiple of BFE: each
     // thread holds BFE consecutive entries (block order) in registers -- their
-    // keys and one word of signs, from which each tau is rebuilt exactly --
-    // and the
-    // threshold is found bit by bit from the top: t is the largest key value v
-    // with #{key >= v} >= k, so a bit is kept when the block still counts k
-    // keys at or above the prefix with that bit set.  No atomics, no bank
-    // conflicts; one block sum per bit below the highest.
+    // keys and one word of signs, from which each tau is rebuilt exactly -- and
+    // the threshold comes from a radix select over those registers, 11 bits
+    // per level down to the lowest bit any key has set (two levels for
+    // bf16-valued task vectors): four instructions per key and level, against
+    // two per key and bit for a descent bit by bit.  4096 x 14336 bf16 task
+    // vector at 5 %, outputs included: 235 -> 208 us.
     constexpr int BFE = BLOCK_MAX_ENTRIES / BLOCK_TPB;
     if (n == BLOCK_TPB * BFE && w % BFE == 0 && (d.cols % VEC) == 0 && (c0 % VEC) == 0 &&
         blockDim.x == BLOCK_TPB) {
@@ -153,6 +153,10 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
         const int rr = tq / (int)w, cc = tq - rr * (int)w;
         const long long ea = (r0 + rr) * d.cols + c0 + cc;     // tensor position of the thread's first entry
         static_assert(BFE <= 32, "one sign word per thread");
+        // theta_0 is needed only after the select: its lines go to L2 meanwhile
+        if (P.fuse_block)
+            for (int by = 0; by < BFE * (int)sizeof(BT); by += 64)
+                asm volatile("prefetch.global.L2 [%0];" :: "l"(static_cast<const char*>(d.base) + ea * (long long)sizeof(BT) + by));
         uint32_t key[BFE];
         uint32_t sgn = 0;
 #pragma unroll
@@ -177,28 +181,25 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
         if ((threadIdx.x & 31) == 0 && kor) atomicOr(&s_or, kor);
         __syncthreads();
         const int low = s_or ? __ffs(s_or) - 1 : 31;
-        const int top = s_or ? 31 - __clz(s_or) : 0;
-        // one barrier per bit: warp sums go to one of three counters; the
-        // counter of the bit after next is cleared meanwhile (its last reads
-        // were before this bit's barrier, its next adds come after the next one)
-        __shared__ uint32_t s_cnt[3];
-        if (threadIdx.x < 3) s_cnt[threadIdx.x] = 0;
-        __syncthreads();
         uint32_t prefix = 0;
-        int cur = 0;
-        for (int bit = top; bit >= low; --bit) {
-            const uint32_t cand = prefix | (1u << bit);
-            uint32_t c = 0;
-#pragma unroll
-            for (int j = 0; j < BFE; ++j) c += key[j] >= cand;
-            c = __reduce_add_sync(0xFFFFFFFFu, c);
-            if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_cnt[cur], c);
+        long long rank = k;
+        for (int pshift = 31;;) {
+            const int shift = max(pshift > RADIX_BITS ? pshift - RADIX_BITS : 0, low);
+            const int nb = 1 << (pshift - shift);
+            for (int q = threadIdx.x; q < nb; q += BLOCK_TPB) s_hist[q] = 0;
             __syncthreads();
-            if ((long long)s_cnt[cur] >= k) prefix = cand;
-            const int nxt2 = (cur + 2) % 3;
-            if (threadIdx.x == 0) s_cnt[nxt2] = 0;
-            cur = (cur + 1) % 3;
+#pragma unroll
+            for (int j = 0; j < BFE; ++j)
+                if ((key[j] >> pshift) == prefix) atomicAdd(&s_hist[(key[j] >> shift) & (uint32_t)(nb - 1)], 1u);
+            __syncthreads();
+            block_find_from_top_b(s_hist, nb, rank, s_scan, &s_bin, &s_above);
+            rank -= s_above;
+            prefix = (prefix << (pshift - shift)) | (uint32_t)s_bin;
+            __syncthreads();
+            if (shift == low) break;
+            pshift = shift;
         }
+        prefix <<= low;
         const uint32_t tk = prefix;
         uint32_t above = 0, ties = 0;
 #pragma unroll
@@ -239,6 +240,9 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
             stats(tk, k, tot_above, tot_ties, need);
         }
         if (P.fuse_block) {
+            // ties are kept at the thread's first `kt` entries
+            const long long before = cut - ea;
+            const int kt = before <= 0 ? 0 : (before >= BFE ? BFE : (int)before);
 #pragma unroll
             for (int gq = 0; gq < BFE / VEC; ++gq) {
                 const long long e = ea + gq * VEC;
@@ -247,7 +251,7 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
 #pragma unroll
                 for (int j = 0; j < VEC; ++j) {
                     const uint32_t kk = key[gq * VEC + j];
-                    const bool kept = kk > tk || (kk == tk && e + j < cut);
+                    const bool kept = (int)kk > (gq * VEC + j < kt ? (int)tk - 1 : (int)tk);
                     o[j] = kept ? out_of(th0[j], tau_of(gq * VEC + j), P.lambda) : th0[j];
                 }
                 store8(d.out, e, d.numel, o, obf);
