@@ -592,7 +592,7 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
             using XT = std::remove_pointer_t<decltype(xt)>;
             using BT = std::remove_pointer_t<decltype(bt)>;
             constexpr bool CK = decltype(ck)::value;
-            const int smem = (SAMPLE_MAX + SAMPLE_SEL_R * 256) * 4;
+            const int smem = (SAMPLE_MAX + SAMPLE_LIST + RADIX_BINS) * 4;
             ISO_TRY(smem_optin(k_sample<XT, BT, CK>, smem));
             ISO_TRY(launch(KD_SAMPLE, s, [&] { k_sample<XT, BT, CK><<<KU, SAMPLE_TPB, smem, s>>>(P); }));
             if (fused)

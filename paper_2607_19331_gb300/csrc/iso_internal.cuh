@@ -31,9 +31,10 @@ static_assert(WVEC * 32 * VEC == TILE, "tile geometry");
 constexpr int CHUNK_MAX = 1024;             // candidate slots a warp reserves at once
 constexpr int VCHUNK = 8192;                // compact-candidate value slots a warp reserves at most at once
 
-constexpr int SAMPLE_MAX = 24576;           // sampled keys per unit (96 KB of smem: two blocks per SM)
+constexpr int SAMPLE_MAX = 24576;           // sampled keys per unit (96 KB of smem)
 constexpr int SAMPLE_CHUNK = 256;           // contiguous entries per sample chunk
-constexpr int SAMPLE_TPB = 512;             // two sample blocks per SM
+constexpr int SAMPLE_TPB = 1024;            // one sample block per SM, three chunks per warp
+constexpr int SAMPLE_LIST = 8192;           // sampled keys gathered around the ranks
 constexpr int SAMPLE_SEL_R = 5;             // ranks selected at once from the sample
 constexpr int CUT_TPB = 1024;
 constexpr int CS_SPLIT = 4;                 // count-sample blocks per unit
@@ -629,6 +630,12 @@ __device__ __forceinline__ void add_rn2(float& d0, float& d1, float a0, float a1
     asm("{\n\t.reg .b64 pa, pb, pd;\n\tmov.b64 pa, {%2, %3};\n\tmov.b64 pb, {%4, %5};\n\t"
         "add.rn.f32x2 pd, pa, pb;\n\tmov.b64 {%0, %1}, pd;\n\t}"
         : "=f"(d0), "=f"(d1) : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+
+__device__ __forceinline__ void fma_rn2(float& d0, float& d1, float a0, float a1, float b0, float b1, float c0, float c1) {
+    asm("{\n\t.reg .b64 pa, pb, pc, pd;\n\tmov.b64 pa, {%2, %3};\n\tmov.b64 pb, {%4, %5};\n\tmov.b64 pc, {%6, %7};\n\t"
+        "fma.rn.f32x2 pd, pa, pb, pc;\n\tmov.b64 {%0, %1}, pd;\n\t}"
+        : "=f"(d0), "=f"(d1) : "f"(a0), "f"(a1), "f"(b0), "f"(b1), "f"(c0), "f"(c1));
 }
 
 // ---------------------------------------------------------------------------

@@ -100,31 +100,89 @@ __device__ void block_find_from_top(const uint32_t* hist, int nb, long long rank
 }
 
 // The rank[r]-th largest (1-based, 1 <= rank[r] <= n) of n keys in shared
-// memory for R <= SEL_R ranks at once.  The key is found one 8-bit digit at
-// a time from the top; ranks whose prefixes agree share a histogram, so one
-// pass over the keys per digit serves every rank (at most one histogram bin
-// per key), and each histogram is scanned by one warp.  `hist` holds
-// SEL_R * 256 zeroed counters on entry and is zero again on return.
+// memory for R <= SEL_R ranks at once, by the whole block (SAMPLE_TPB
+// threads).  One histogram of the top 11 bits; the keys of the bins that hold
+// the ranks (a few per cent of the sample) are gathered, and 7-bit digits of
+// those settle the rest, one histogram per distinct prefix, each scanned by
+// one warp.  More keys than the gather buffer holds (long runs of ties) are
+// read from the sample instead.  The exponent alone as a first digit put a
+// warp's keys into a handful of counters; on 11 bits a warp's 32 keys meet in
+// a few pairs (with every chunk loaded in one round, k_sample of two 1M-entry
+// binary32 units 36 -> 18 us, of 254 bf16 checkpoint tensors 131 -> 84 us).
+// `hist` holds RADIX_BINS counters, zero on entry; `list` SAMPLE_LIST keys.
+// On return *n_list is the number of gathered keys (all keys equal to a result
+// are among them), or -1.
 constexpr int SEL_R = SAMPLE_SEL_R;
-__device__ void block_select_ranks(const uint32_t* keys, int n, int R, const long long* rank,
-                                   uint32_t* hist, uint32_t* out) {
+constexpr int SEL_BITS = 7;
+static_assert(SEL_R << SEL_BITS <= RADIX_BINS, "digit histograms share the counters");
+__device__ void block_select_ranks(const uint32_t* keys, int n, int R, const long long* rank, uint32_t* hist,
+                                   uint32_t* list, int* n_list, uint32_t* out) {
     __shared__ uint32_t s_pref[SEL_R];
-    __shared__ long long s_rem[SEL_R];
+    __shared__ int s_rem[SEL_R];
+    __shared__ uint32_t s_scan[33];
+    __shared__ int s_n, s_b0, s_b1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x < R) { s_pref[threadIdx.x] = 0; s_rem[threadIdx.x] = rank[threadIdx.x]; }
+    constexpr int SH = 31 - RADIX_BITS;                       // shift of the first digit
+    for (int q = threadIdx.x; q < n; q += SAMPLE_TPB) atomicAdd(&hist[keys[q] >> SH], 1u);
+    if (threadIdx.x == 0) { s_n = 0; s_b0 = RADIX_BINS; s_b1 = -1; }
     __syncthreads();
+    {
+        // bins from the top, RADIX_BINS / SAMPLE_TPB per thread
+        constexpr int PER = RADIX_BINS / SAMPLE_TPB;
+        uint32_t h[PER], sum = 0, tot;
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            h[j] = hist[RADIX_BINS - 1 - (threadIdx.x * PER + j)];
+            sum += h[j];
+        }
+        const uint32_t excl = block_excl_scan(sum, s_scan, &tot);
+#pragma unroll
+        for (int r = 0; r < SEL_R; ++r) {
+            if (r >= R) continue;
+            const uint32_t rr = (uint32_t)rank[r];
+            if (excl < rr && rr <= excl + sum) {
+                uint32_t acc = excl;
+#pragma unroll
+                for (int j = 0; j < PER; ++j) {
+                    if (rr > acc && rr <= acc + h[j]) {
+                        const int bin = RADIX_BINS - 1 - (threadIdx.x * PER + j);
+                        s_pref[r] = (uint32_t)bin;
+                        s_rem[r] = (int)(rr - acc);
+                        atomicMin(&s_b0, bin);
+                        atomicMax(&s_b1, bin);
+                    }
+                    acc += h[j];
+                }
+            }
+        }
+    }
+    __syncthreads();
+    const uint32_t b0 = (uint32_t)s_b0, b1 = (uint32_t)s_b1;
+    for (int q = threadIdx.x; q < RADIX_BINS; q += SAMPLE_TPB) hist[q] = 0;
+    for (int q0 = 0; q0 < n; q0 += SAMPLE_TPB) {
+        const int q = q0 + threadIdx.x;
+        const uint32_t v = q < n ? keys[q] : 0;
+        const bool in = q < n && (v >> SH) >= b0 && (v >> SH) <= b1;
+        const unsigned m = __ballot_sync(0xFFFFFFFFu, in);
+        int at = 0;
+        if (lane == 0 && m) at = atomicAdd(&s_n, __popc(m));
+        at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(m & ((1u << lane) - 1u));
+        if (in && at < SAMPLE_LIST) list[at] = v;
+    }
+    __syncthreads();
+    const bool fits = s_n <= SAMPLE_LIST;
+    const uint32_t* src = fits ? list : keys;
+    const int ns = fits ? s_n : n;
+    if (threadIdx.x == 0) *n_list = fits ? s_n : -1;
 #pragma unroll 1
-    for (int lvl = 0; lvl < 4; ++lvl) {
-        const int dsh = 24 - 8 * lvl;                    // the digit's shift
+    for (int sh = SH; sh > 0;) {
+        const int bits = sh < SEL_BITS ? sh : SEL_BITS, dsh = sh - bits;
         // distinct prefixes in rank order (every thread alike)
         uint32_t gp[SEL_R];
         int grp[SEL_R];
         int ng = 0;
 #pragma unroll
-        for (int r = 0; r < SEL_R; ++r) {
-            gp[r] = 0;
-            grp[r] = -1;
-        }
+        for (int r = 0; r < SEL_R; ++r) { gp[r] = 0; grp[r] = -1; }
 #pragma unroll
         for (int r = 0; r < SEL_R; ++r) {
             if (r < R) {
@@ -140,62 +198,47 @@ __device__ void block_select_ranks(const uint32_t* keys, int n, int R, const lon
                 grp[r] = g;
             }
         }
-        // one histogram per distinct prefix; a thread's run of keys in one
-        // bin adds once (the keys near the threshold crowd into a few bins)
-        uint32_t run_slot = 0, run_cnt = 0;
-        for (int q = threadIdx.x; q < n; q += blockDim.x) {
-            const uint32_t v = keys[q];
-            const uint32_t top = lvl == 0 ? 0u : v >> (dsh + 8);
+        for (int q = threadIdx.x; q < ns; q += SAMPLE_TPB) {
+            const uint32_t v = src[q], top = v >> sh;
             int g = -1;
 #pragma unroll
             for (int j = SEL_R - 1; j >= 0; --j)
                 if (j < ng && gp[j] == top) g = j;
-            if (g < 0) continue;
-            const uint32_t slot = (uint32_t)g * 256u + ((v >> dsh) & 255u);
-            if (slot != run_slot) {
-                if (run_cnt) atomicAdd(&hist[run_slot], run_cnt);
-                run_slot = slot;
-                run_cnt = 0;
-            }
-            ++run_cnt;
+            if (g >= 0) atomicAdd(&hist[(g << SEL_BITS) + ((v >> dsh) & ((1u << bits) - 1u))], 1u);
         }
-        if (run_cnt) atomicAdd(&hist[run_slot], run_cnt);
         __syncthreads();
-        // warp g scans histogram g from the top bin: lane L holds bins 255-8L .. 248-8L
+        // warp g scans histogram g from the top bin: lane L holds bins 127 - 4 L ...
         if (warp < ng) {
-            uint32_t h[8];
-            uint32_t* hg = hist + warp * 256;
+            constexpr int PL = (1 << SEL_BITS) / 32;
+            uint32_t h[PL];
+            uint32_t* hg = hist + (warp << SEL_BITS);
             uint32_t sum = 0;
 #pragma unroll
-            for (int j = 0; j < 8; ++j) { h[j] = hg[255 - 8 * lane - j]; sum += h[j]; }
-            uint32_t incl = sum;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            const long long excl = (long long)(incl - sum);
+            for (int j = 0; j < PL; ++j) { h[j] = hg[(1 << SEL_BITS) - 1 - PL * lane - j]; sum += h[j]; }
+            uint32_t tot;
+            const uint32_t excl = warp_excl_scan(sum, &tot);
 #pragma unroll
             for (int r = 0; r < SEL_R; ++r) {
                 if (r >= R || grp[r] != warp) continue;
-                const long long rr = s_rem[r];
-                if (excl < rr && rr <= excl + (long long)sum) {
-                    long long acc = excl;
+                const uint32_t rr = (uint32_t)s_rem[r];
+                __syncwarp();
+                if (excl < rr && rr <= excl + sum) {
+                    uint32_t acc = excl;
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) {
-                        if (rr <= acc + (long long)h[j]) {
-                            s_pref[r] = (s_pref[r] << 8) | (uint32_t)(255 - 8 * lane - j);
-                            s_rem[r] = rr - acc;
-                            break;
+                    for (int j = 0; j < PL; ++j) {
+                        if (rr > acc && rr <= acc + h[j]) {
+                            s_pref[r] = (s_pref[r] << bits) | (uint32_t)((1 << SEL_BITS) - 1 - PL * lane - j);
+                            s_rem[r] = (int)(rr - acc);
                         }
                         acc += h[j];
                     }
                 }
             }
 #pragma unroll
-            for (int j = 0; j < 8; ++j) hg[255 - 8 * lane - j] = 0;
+            for (int j = 0; j < PL; ++j) hg[(1 << SEL_BITS) - 1 - PL * lane - j] = 0;
         }
         __syncthreads();
+        sh = dsh;
     }
     if (threadIdx.x < R) out[threadIdx.x] = s_pref[threadIdx.x];
     __syncthreads();
@@ -216,10 +259,12 @@ __device__ __forceinline__ int tensor_of_upos(const TensorDesc* tens, int n_tens
 }
 
 template <typename XT, typename BT, bool CKPT>
-__global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
+__global__ void __launch_bounds__(SAMPLE_TPB, 1) k_sample(Plan P) {
     extern __shared__ __align__(16) uint32_t s_keys[];
-    uint32_t* s_hist = s_keys + SAMPLE_MAX;          // SEL_R * 256 counters
+    uint32_t* s_list = s_keys + SAMPLE_MAX;          // SAMPLE_LIST keys
+    uint32_t* s_hist = s_list + SAMPLE_LIST;         // RADIX_BINS counters
     __shared__ long long s_scan[33];
+    __shared__ int s_nl;
 
     Unit& U = P.units[blockIdx.x];
     if (U.state != ST_SAMPLE) return;
@@ -227,80 +272,16 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
     const long long n = U.n;
     const int S = (int)(n < SAMPLE_MAX ? n : SAMPLE_MAX);
     constexpr int nch = SAMPLE_MAX / SAMPLE_CHUNK;
-    if (S < n && P.scope != ISO_SCOPE_GLOBAL) {
-        // chunks of 256 contiguous entries at evenly spaced, 8-aligned starts:
-        // one chunk per warp step, 8 entries per lane
-        const int t = U.tensor;
-        const void* x = P.xptr[i * P.n_tensors + t];
-        const void* b = P.tens[t].base;
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        // three chunks per warp at a time: their loads are in flight together
-        constexpr int CB = 3;
-        for (int c0 = warp; c0 < nch; c0 += CB * nw) {
-            float tau[CB][VEC];
-#pragma unroll
-            for (int m = 0; m < CB; ++m) {
-                const int c = c0 + m * nw;
-                // (n - 256) c / 95, rounded down (exact: integer arithmetic)
-                const long long start = (long long)(((unsigned long long)(n - SAMPLE_CHUNK) *
-                                                     (unsigned long long)(c < nch ? c : 0)) /
-                                                    (unsigned long long)(nch - 1)) & ~7LL;
-                TauSrc<XT, BT, CKPT>::load8(x, b, start + lane * VEC, n, tau[m]);
-            }
-#pragma unroll
-            for (int m = 0; m < CB; ++m) {
-                const int c = c0 + m * nw;
-                if (c < nch) {
-#pragma unroll
-                    for (int j = 0; j < VEC; ++j) s_keys[c * SAMPLE_CHUNK + lane * VEC + j] = key_of(tau[m][j]);
-                }
-            }
-        }
-    } else {
-        for (int q = threadIdx.x; q < S; q += blockDim.x) {
-            long long pos;
-            if (S == n) {
-                pos = q;
-            } else {
-                const int c = q / SAMPLE_CHUNK, j = q % SAMPLE_CHUNK;
-                pos = (long long)(((unsigned long long)(n - SAMPLE_CHUNK) * (unsigned long long)c) /
-                                  (unsigned long long)(nch - 1)) + j;
-            }
-            int t;
-            long long e;
-            if (P.scope == ISO_SCOPE_GLOBAL) {
-                t = tensor_of_upos(P.tens, P.n_tensors, pos);
-                e = pos - P.tens[t].uoff;
-            } else {
-                t = U.tensor;
-                e = pos;
-            }
-            const float tau = TauSrc<XT, BT, CKPT>::load1(P.xptr[i * P.n_tensors + t], P.tens[t].base, e);
-            s_keys[q] = key_of(tau);
-        }
-    }
-    for (int q = threadIdx.x; q < SEL_R * 256; q += blockDim.x) s_hist[q] = 0;
-    __syncthreads();
-    uint32_t lo, hi;
-    uint32_t that = 0;                       // fused pass: the estimate of the threshold
     const bool fused_t = P.fused && P.scope == ISO_SCOPE_TENSOR;
     const bool want_t = fused_t || !P.ccv;   // the counting pass sets a run of ties apart as well
     bool run_t = false;                      // ... when the sample shows one
     __shared__ long long s_rk[SEL_R];
     __shared__ uint32_t s_kv[SEL_R];
     __shared__ int s_edge[2];
-    if (S == n) {
-        // the sample is the whole unit: the band is the exact threshold
-        if (threadIdx.x == 0) s_rk[0] = U.k;
-        __syncthreads();
-        block_select_ranks(s_keys, S, 1, s_rk, s_hist, s_kv);
-        hi = lo = that = s_kv[0];
-        run_t = true;
-    } else {
+    if (S < n) {
         // the band's sample ranks, by one thread (binary64 is slow on this
-        // GPU), then every rank in one selection: the band edges and, for
-        // the fused pass, the rank of k and halfway to either edge
-        if (threadIdx.x == 0) {
+        // GPU) while the others load
+        if (threadIdx.x == SAMPLE_TPB - 1) {
             const double q = (double)U.k / (double)n;
             const double r = (double)U.k * (double)S / (double)n;
             const double delta = SAMPLE_Z * sqrt((double)S * q * (1.0 - q)) + 2.0;
@@ -315,8 +296,76 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
             s_edge[0] = ra >= 1;
             s_edge[1] = rb <= S;
         }
+        // chunks of 256 contiguous entries at evenly spaced starts: one chunk
+        // per warp step, 8 entries per lane, three chunks' loads in flight
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        constexpr int CB = nch / (SAMPLE_TPB / 32);
+        static_assert(CB * (SAMPLE_TPB / 32) == nch, "whole rounds of chunks");
+        float tau[CB][VEC];
+#pragma unroll
+        for (int m = 0; m < CB; ++m) {
+            const int c = warp + m * (SAMPLE_TPB / 32);
+            // (n - 256) c / 95, rounded down (exact: integer arithmetic)
+            long long start = (long long)(((unsigned long long)(n - SAMPLE_CHUNK) * (unsigned long long)c) /
+                                          (unsigned long long)(nch - 1));
+            int t = U.tensor;
+            bool vec = true;
+            if (P.scope == ISO_SCOPE_GLOBAL) {
+                // the tensor that holds the chunk's first entry; a chunk that
+                // runs past it is read entry by entry
+                t = tensor_of_upos(P.tens, P.n_tensors, start);
+                start -= P.tens[t].uoff;
+                vec = (start & ~7LL) + SAMPLE_CHUNK <= P.tens[t].numel;
+            }
+            if (vec) {
+                start &= ~7LL;
+                TauSrc<XT, BT, CKPT>::load8(P.xptr[i * P.n_tensors + t], P.tens[t].base, start + lane * VEC,
+                                            P.tens[t].numel, tau[m]);
+            } else {
+#pragma unroll
+                for (int j = 0; j < VEC; ++j) {
+                    const long long pos = P.tens[t].uoff + start + lane * VEC + j;
+                    const int tj = tensor_of_upos(P.tens, P.n_tensors, pos);
+                    tau[m][j] = TauSrc<XT, BT, CKPT>::load1(P.xptr[i * P.n_tensors + tj], P.tens[tj].base,
+                                                            pos - P.tens[tj].uoff);
+                }
+            }
+        }
+        for (int q = threadIdx.x; q < RADIX_BINS; q += SAMPLE_TPB) s_hist[q] = 0;
+#pragma unroll
+        for (int m = 0; m < CB; ++m) {
+            const int c = warp + m * (SAMPLE_TPB / 32);
+            uint4* d = reinterpret_cast<uint4*>(s_keys + c * SAMPLE_CHUNK + lane * VEC);
+            d[0] = make_uint4(key_of(tau[m][0]), key_of(tau[m][1]), key_of(tau[m][2]), key_of(tau[m][3]));
+            d[1] = make_uint4(key_of(tau[m][4]), key_of(tau[m][5]), key_of(tau[m][6]), key_of(tau[m][7]));
+        }
+    } else {
+        for (int q = threadIdx.x; q < S; q += SAMPLE_TPB) {
+            int t = U.tensor;
+            long long e = q;
+            if (P.scope == ISO_SCOPE_GLOBAL) {
+                t = tensor_of_upos(P.tens, P.n_tensors, q);
+                e = q - P.tens[t].uoff;
+            }
+            const float tau = TauSrc<XT, BT, CKPT>::load1(P.xptr[i * P.n_tensors + t], P.tens[t].base, e);
+            s_keys[q] = key_of(tau);
+        }
+        for (int q = threadIdx.x; q < RADIX_BINS; q += SAMPLE_TPB) s_hist[q] = 0;
+    }
+    __syncthreads();
+    uint32_t lo, hi;
+    uint32_t that = 0;                       // the estimate of the threshold
+    if (S == n) {
+        // the sample is the whole unit: the band is the exact threshold
+        if (threadIdx.x == 0) s_rk[0] = U.k;
         __syncthreads();
-        block_select_ranks(s_keys, S, want_t ? 5 : 2, s_rk, s_hist, s_kv);
+        block_select_ranks(s_keys, S, 1, s_rk, s_hist, s_list, &s_nl, s_kv);
+        hi = lo = that = s_kv[0];
+        run_t = true;
+    } else {
+        // every rank in one selection: the band edges and, for t^, the rank of
+        // k and halfway to either edge
+        block_select_ranks(s_keys, S, want_t ? 5 : 2, s_rk, s_hist, s_list, &s_nl, s_kv);
         // no two of the five ranks share a key: no run of ties worth setting apart
         const bool distinct = s_kv[0] != s_kv[3] && s_kv[3] != s_kv[2] && s_kv[2] != s_kv[4] && s_kv[4] != s_kv[1];
         hi = s_edge[0] ? s_kv[0] : KEY_MAX;
@@ -334,8 +383,10 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 2) k_sample(Plan P) {
             pv[3] = s_kv[4];
             pv[4] = s_kv[1];
             unsigned cnt[5] = {0, 0, 0, 0, 0};
-            for (int q = threadIdx.x; q < S; q += blockDim.x) {
-                const uint32_t v = s_keys[q];
+            const uint32_t* src = s_nl >= 0 ? s_list : s_keys;
+            const int ns = s_nl >= 0 ? s_nl : S;
+            for (int q = threadIdx.x; q < ns; q += blockDim.x) {
+                const uint32_t v = src[q];
 #pragma unroll
                 for (int j = 0; j < 5; ++j) cnt[j] += (v == pv[j]);
             }
@@ -528,16 +579,11 @@ __global__ void __launch_bounds__(CS_TPB, 4) k_csample(Plan P) {
 // Per entry the pass does only what every entry needs: tau, its key, the
 // count above the band and a band test.  Band keys (lo <= key <= hi, a few
 // per cent of the entries) are staged in shared memory -- lane L's j-th at
-// slot j*32 + L, conflict-free; every key is written and only a band key
-// advances the lane's slot -- and then copied, per lane, to the unit's
+// slot j*32 + L, conflict-free -- and then copied, per lane, to the unit's
 // candidate segment.  The radix select and the tie counts work on that set.
 //
 // The warp's tiles stream through two register buffers: the next tile's loads
-// are issued before the current tile is processed.  A non-finite tau has a key
-// above every finite key, so it is either above hi, where it turns the lane's
-// binary32 sum of tau^2 non-finite (then the tile is re-checked key by key),
-// or a band key, checked when the band keys are copied; lo itself is a sampled
-// key, so a non-finite lo is a band key of its own unit.
+// are issued before the current tile is processed.
 
 // consecutive items of one (expert, tensor) that the count pass visits (with
 // round-robin items, one item)
@@ -714,32 +760,34 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
             for (int j = 0; j < VEC; ++j) d[j] = tau[j];
         };
 
-        // pass 1: every entry.  In run mode (RUN: the sample's ranks around k
-        // share a key t^) the keys equal to t^ are counted apart and never
-        // staged.  Task vectors of bf16 checkpoints hold several per cent of
-        // their entries at t^: as candidates they cost more in the select
-        // (K = 3, 1.54G entries: histogram 2.92 -> 0.59 ms, ties 0.51 -> 0.25
-        // ms) than the extra compare here (4.14 -> 4.56 ms).  Task vectors
-        // without such a run keep the plain form.
-        uint32_t n_gt = 0, n_eq = 0;
-        float f_gg = 0.0f;                         // tau^2 above hi (also the non-finite detector)
+        // pass 1: every entry, with binary32 comparisons of |tau| (magnitudes
+        // order like their bits; hi = KEY_MAX is a NaN that nothing exceeds).
+        // In run mode (RUN: the sample's ranks around k share a key t^) the keys
+        // equal to t^ are counted apart and never staged.  Task vectors of
+        // bf16 checkpoints hold several per cent of their entries at t^: as
+        // candidates they cost more in the select (K = 3, 1.54G entries:
+        // histogram 2.92 -> 0.59 ms, ties 0.51 -> 0.25 ms) than the extra
+        // compare here.  Task vectors without such a run keep the plain form.
+        // 0 * tau finds non-finite entries, which the comparisons leave out.
+        uint32_t n_gt = 0, n_in = 0;               // keys above hi; keys in the band
+        float f_gg = 0.0f;                         // GAMMA: tau^2 above hi
+        float bad0 = 0.0f, bad1 = 0.0f;            // NaN once a tau was not finite
         uint32_t* sp = sbl;
-        auto entry = [&](float tau, auto run_c) {
-            constexpr bool RUN = decltype(run_c)::value;
-            const uint32_t kk = key_of(tau);
-            const bool gt = kk > hi;
+        const float hif = __uint_as_float(hi), lof = __uint_as_float(lo), thf = __uint_as_float(that);
+        auto entry = [&](float tau, auto run_c, auto gamma_c) {
+            constexpr bool RUN = decltype(run_c)::value, GAMMA = decltype(gamma_c)::value;
+            const float m = fabsf(tau);
+            const bool gt = m > hif;
+            const bool in = m >= lof && !gt;
             n_gt += gt;
-            f_gg = gt ? __fmaf_rn(tau, tau, f_gg) : f_gg;
-            *sp = kk;
-            if constexpr (RUN) {
-                const bool eq = kk == that;
-                n_eq += eq;
-                sp += (kk - lo <= span && !eq) ? 32 : 0;
-            } else {
-                sp += (kk - lo <= span) ? 32 : 0;
-            }
+            if (GAMMA) f_gg = gt ? __fmaf_rn(tau, tau, f_gg) : f_gg;
+            if (RUN) n_in += in;
+            // every key is written and only a band key advances the slot (a
+            // predicated store measured slower: it became a branch)
+            *sp = __float_as_uint(m);
+            sp += (RUN ? in && m != thf : in) ? 32 : 0;
         };
-        auto pass1 = [&](auto run_c) {
+        auto pass1 = [&](auto run_c, auto gamma_c) {
             if (rem >= TILE) {
 #pragma unroll
                 for (int v = 0; v < WVEC; ++v) {
@@ -747,7 +795,11 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
                     rt.tau(v, tau);
                     if (more) rt.load_step(v, r2.xp, r2.bp, ne0, nrem, lane);
 #pragma unroll
-                    for (int j = 0; j < VEC; ++j) entry(tau[j], run_c);
+                    for (int j = 0; j < VEC; j += 2) {
+                        fma_rn2(bad0, bad1, tau[j], tau[j + 1], 0.0f, 0.0f, bad0, bad1);
+                        entry(tau[j], run_c, gamma_c);
+                        entry(tau[j + 1], run_c, gamma_c);
+                    }
                     if constexpr (EMIT) stash(v, tau);
                 }
             } else {
@@ -758,29 +810,25 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
                     if (more) rt.load_step(v, r2.xp, r2.bp, ne0, nrem, lane);
                     const uint32_t o = (uint32_t)(v * (32 * VEC) + lane * VEC);
 #pragma unroll
-                    for (int j = 0; j < VEC; ++j)
-                        if (o + j < rem) entry(tau[j], run_c);
+                    for (int j = 0; j < VEC; ++j) {
+                        bad0 = __fmaf_rn(tau[j], 0.0f, bad0);
+                        if (o + j < rem) entry(tau[j], run_c, gamma_c);
+                    }
                     if constexpr (EMIT) stash(v, tau);
                 }
             }
         };
-        if (!EMIT && run) pass1(std::integral_constant<bool, true>{});
-        else pass1(std::integral_constant<bool, false>{});
-        const uint32_t nb = (uint32_t)(sp - sbl) >> 5;
-        if (__any_sync(FULL, !(fabsf(f_gg) <= 3.402823466e38f))) {
-            // a non-finite (or overflowing) sum: read the tile's keys again
-            uint32_t kmax = 0;
-            for (int v = 0; v < WVEC; ++v) {
-                const uint32_t o = (uint32_t)(v * (32 * VEC) + lane * VEC);
-                if (o >= rem) break;
-                float tau[VEC];
-                TauSrc<XT, BT, CK>::load8(rr.xp, rr.bp, (long long)e0 + o, (long long)rr.n, tau);
-#pragma unroll
-                for (int j = 0; j < VEC; ++j)
-                    if (o + j < rem) kmax = max(kmax, key_of(tau[j]));
-            }
-            if (__any_sync(FULL, kmax >= KEY_INF) && lane == 0) set_status(P.hdr, ISO_ERR_NONFINITE);
+        using T1 = std::integral_constant<bool, true>;
+        using T0 = std::integral_constant<bool, false>;
+        if (want_gamma) {
+            if (!EMIT && run) pass1(T1{}, T1{});
+            else pass1(T0{}, T1{});
+        } else {
+            if (!EMIT && run) pass1(T1{}, T0{});
+            else pass1(T0{}, T0{});
         }
+        if (__any_sync(FULL, !(bad0 + bad1 == 0.0f)) && lane == 0) set_status(P.hdr, ISO_ERR_NONFINITE);
+        const uint32_t nb = (uint32_t)(sp - sbl) >> 5;
         if (want_gamma) two_sum_add(s_gg, e_gg, f_gg);
         __syncwarp();
 
@@ -804,7 +852,7 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
             else { ch_pos = (uint32_t)start; ch_left = req; }
         }
         const bool store = t_int && !ovf;
-        uint32_t n_hi = 0, n_lo = 0, kbad = 0;
+        uint32_t n_hi = 0, n_lo = 0;
         float f_band = 0.0f;                      // tau^2 over the band keys above lo
         {
             uint32_t* dst = cseg + ch_pos + off;
@@ -813,15 +861,10 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
                 if (store) dst[q] = kk;
                 n_hi += run ? (kk > that) : (kk == hi);
                 n_lo += !run && (kk == lo) && (kk != hi);
-                kbad |= (kk >= KEY_INF);
                 if (want_gamma && (run ? kk > that : kk != lo)) { const float f = __uint_as_float(kk); f_band = __fmaf_rn(f, f, f_band); }
             }
         }
-        if (run) {
-            n_lo = n_eq;
-            kbad |= n_eq && that >= KEY_INF;
-        }
-        if (__any_sync(FULL, kbad) && lane == 0) set_status(P.hdr, ISO_ERR_NONFINITE);
+        if (run) n_lo = n_in - nb;                // the ties of t^
         if (want_gamma) two_sum_add(s_gb, e_gb, f_band);
         const uint32_t t_gt = __reduce_add_sync(FULL, n_gt);
         const uint32_t t_hi = __reduce_add_sync(FULL, n_hi);
