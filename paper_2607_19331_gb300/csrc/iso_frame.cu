@@ -80,16 +80,12 @@ __device__ __forceinline__ void split_tf32(double x, float& hi, float& lo) {
     lo = __uint_as_float(l);
 }
 
-// An operand row of contraction length L (padded) is stored in four segments
-// [hi | lo | hi | hi]: read from segment 0 it is (hi, lo, hi), from segment 1
-// (lo, hi, hi); A from 0 and B from 1 pair up as hi lo + lo hi + hi hi.
+// An operand row of contraction length L (padded) is stored as two segments [hi | lo].
 __device__ __forceinline__ void put_split(float* row, long long L, long long k, double x) {
     float hi, lo;
     split_tf32(x, hi, lo);
     row[k] = hi;
     row[L + k] = lo;
-    row[2 * L + k] = hi;
-    row[3 * L + k] = hi;
 }
 
 struct Frames {                     // one side (U: d = m; V: d = n), d x q row-major binary64
@@ -140,35 +136,41 @@ __device__ __forceinline__ double sign_of(const double* dots, long long q, int i
     return dots[(long long)i * q + k] < 0.0 ? -1.0 : 1.0;
 }
 
-// (dF_i^T dF_j)_kk for i <= j, summed into cd[i][j][k]
+// (dF_i^T dF_j)_kk for i <= j, summed into cd[i][j][k]; KC >= K is the
+// compile-time bound (a bound of 8 for any K spent 36 products a row: 6.1 ms
+// for three experts of a 3584 x 18944 matrix)
+template <int KC>
 __global__ void __launch_bounds__(256) k_fr_coldots(Frames f, const double* dots, double* cd, int row_chunks) {
     __shared__ double red[8][33];
     const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
     const int K = f.K;
     const long long per = (f.d + row_chunks - 1) / row_chunks;
     const long long r0 = (long long)blockIdx.y * per, r1 = min(f.d, r0 + per);
-    double acc[MAXK * (MAXK + 1) / 2];
+    double acc[KC * (KC + 1) / 2];
 #pragma unroll
-    for (int p = 0; p < MAXK * (MAXK + 1) / 2; ++p) acc[p] = 0.0;
-    double sg[MAXK];
+    for (int p = 0; p < KC * (KC + 1) / 2; ++p) acc[p] = 0.0;
+    double sg[KC];
 #pragma unroll
-    for (int i = 0; i < MAXK; ++i) sg[i] = (i < K && k < f.q) ? sign_of(dots, f.q, i, k) : 0.0;
+    for (int i = 0; i < KC; ++i) sg[i] = (i < K && k < f.q) ? sign_of(dots, f.q, i, k) : 0.0;
     if (k < f.q) {
+#pragma unroll 2
         for (long long r = r0 + threadIdx.y; r < r1; r += 8) {
             const double f0 = f.F0[r * f.q + k];
-            double dv[MAXK];
+            double dv[KC];
 #pragma unroll
-            for (int i = 0; i < MAXK; ++i) dv[i] = (i < K) ? fma(sg[i], f.F[i][r * f.q + k], -f0) : 0.0;
+            for (int i = 0; i < KC; ++i) dv[i] = (i < K) ? fma(sg[i], f.F[i][r * f.q + k], -f0) : 0.0;
             int p = 0;
 #pragma unroll
-            for (int i = 0; i < MAXK; ++i)
+            for (int i = 0; i < KC; ++i)
 #pragma unroll
-                for (int j = i; j < MAXK; ++j) acc[p] = fma(dv[i], dv[j], acc[p]), ++p;
+                for (int j = i; j < KC; ++j) acc[p] = fma(dv[i], dv[j], acc[p]), ++p;
         }
     }
     int p = 0;
-    for (int i = 0; i < MAXK; ++i)
-        for (int j = i; j < MAXK; ++j, ++p) {
+#pragma unroll
+    for (int i = 0; i < KC; ++i)
+#pragma unroll
+        for (int j = i; j < KC; ++j, ++p) {
             if (i >= K || j >= K) continue;
             red[threadIdx.y][threadIdx.x] = acc[p];
             __syncthreads();
@@ -181,7 +183,7 @@ __global__ void __launch_bounds__(256) k_fr_coldots(Frames f, const double* dots
         }
 }
 
-// Transposed split operand out[k][seg][j] (Qp rows of 4 Lr) of a d x q source,
+// Transposed split operand out[k][seg][j] (Qp rows of 2 Lr) of a d x q source,
 // j the source row (Lr = Dp; the stacked modes 4 and 5 put two d-row sources
 // one above the other, Lr = 2 Dp):
 //   0  F_0[j, k];  1  dF_i = s_i F_i - F_0;  2  X[j, k];  3  X[j, k] S_0[k]
@@ -222,14 +224,13 @@ __global__ void __launch_bounds__(256) k_fr_split_t(SplitT a) {
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += 8) {
         const long long k = k0 + y, r = r0 + threadIdx.x;
-        if (k < a.Qp && r < Lr) put_split(a.out + k * 4 * Lr, Lr, r, t[threadIdx.x][y]);
+        if (k < a.Qp && r < Lr) put_split(a.out + k * 2 * Lr, Lr, r, t[threadIdx.x][y]);
     }
 }
 
-// Row-major split operand out[r][seg][c] (rows_p rows of 4 Lp), element value by mode:
+// Row-major split operand out[r][seg][c] (rows_p rows of 2 Lp), element value by mode:
 //   0  F_0[r, c]                          (d x q)
 //   1  F_0[r, c] + X[r, c]                (d x q)
-//   2  M[r, c]                            (q x q binary64)
 //   3  Y^T[r, c] of the aggregate          (q x q)
 //   4  [E_U S_0 | U_0 S_0]                (m x 2 Qp: c < Qp from X = E_U, else U_0)
 //   5  [V_0 + E_V | E_V]                  (n x 2 Qp: X = E_V)
@@ -248,10 +249,8 @@ struct SplitR {
     int mode;
     float* out;
     long long rows, rows_p, Lp;
-    const int32_t* skip;   // optional: nothing to do while *skip != 0
 };
 __global__ void __launch_bounds__(256) k_fr_split_r(SplitR a) {
-    if (a.skip && *reinterpret_cast<const volatile int32_t*>(a.skip)) return;
     const long long total = a.rows_p * a.Lp;
     const long long q = a.f.q;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
@@ -261,7 +260,6 @@ __global__ void __launch_bounds__(256) k_fr_split_r(SplitR a) {
             switch (a.mode) {
                 case 0: if (c < q) v = a.f.F0[r * q + c]; break;
                 case 1: if (c < q) v = a.f.F0[r * q + c] + a.X[r * q + c]; break;
-                case 2: if (c < q) v = a.M[r * q + c]; break;
                 case 3:
                     if (c < q) {
                         // Y^T[j, k] = Y[k, j] = Sc[j, k] D_j - Kwc[j, k] (D_j - D_k) / 2
@@ -294,7 +292,7 @@ __global__ void __launch_bounds__(256) k_fr_split_r(SplitR a) {
                     break;
             }
         }
-        put_split(a.out + r * 4 * a.Lp, a.Lp, c, v);
+        put_split(a.out + r * 2 * a.Lp, a.Lp, c, v);
     }
 }
 
@@ -318,32 +316,44 @@ __device__ __forceinline__ double oz_value(const OzSrc& a, int z, long long e, l
 
 // every column's largest magnitude, all sources in one pass (reads each
 // array once: bound by HBM)
+template <int SC>
 __global__ void __launch_bounds__(256) k_oz_colmax(OzSrc a, int sources, int row_chunks) {
     const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
     const long long per = (a.f.d + row_chunks - 1) / row_chunks;
-    const long long r0 = (long long)blockIdx.y * per, r1 = min(a.f.d, r0 + per);
-    if (k >= a.f.q) return;
-    unsigned long long m[MAXK + 1];
-    double sg[MAXK];
+    const long long r0 = (long long)blockIdx.y * per, r1 = k < a.f.q ? min(a.f.d, r0 + per) : r0;
+    unsigned long long m[SC];
+    double sg[SC];
 #pragma unroll
-    for (int z = 0; z <= MAXK; ++z) m[z] = 0;
+    for (int z = 0; z < SC; ++z) m[z] = 0;
 #pragma unroll
-    for (int i = 0; i < MAXK; ++i) sg[i] = i + 1 < sources ? sign_of(a.dots, a.f.q, i, k) : 0.0;
+    for (int i = 0; i + 1 < SC; ++i) sg[i] = i + 1 < sources && k < a.f.q ? sign_of(a.dots, a.f.q, i, k) : 0.0;
     auto up = [](unsigned long long& x, double v) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
         x = b > x ? b : x;
     };
+#pragma unroll 4
     for (long long r = r0 + threadIdx.y; r < r1; r += 8) {
         const long long e = r * a.f.q + k;
         const double f0 = a.f.F0[e];
         up(m[0], a.X ? f0 + a.X[e] : f0);
 #pragma unroll
-        for (int i = 0; i < MAXK; ++i)
+        for (int i = 0; i + 1 < SC; ++i)
             if (i + 1 < sources) up(m[i + 1], fma(sg[i], a.f.F[i][e], -f0));
     }
+    // the block's rows first: one atomic per column and block
+    __shared__ unsigned long long red[8][33];
 #pragma unroll
-    for (int z = 0; z <= MAXK; ++z)
-        if (z < sources) atomicMax(&a.mx[(long long)z * a.f.q + k], m[z]);
+    for (int z = 0; z < SC; ++z) {
+        if (z >= sources) break;
+        red[threadIdx.y][threadIdx.x] = m[z];
+        __syncthreads();
+        if (threadIdx.y == 0 && k < a.f.q) {
+            unsigned long long v = m[z];
+            for (int y = 1; y < 8; ++y) v = red[y][threadIdx.x] > v ? red[y][threadIdx.x] : v;
+            atomicMax(&a.mx[(long long)z * a.f.q + k], v);
+        }
+        __syncthreads();
+    }
 }
 
 // |x| < 2^e for a column whose largest magnitude has these bits; columns
@@ -411,7 +421,7 @@ __global__ void __launch_bounds__(256) k_oz_reduce(const double* part, int split
 }
 
 // Split operands of an m x n bf16 / fp32 matrix G (row stride n): row-major
-// (rows Mp of 4 Np, element G[r, c]) or transposed (rows Np of 4 Mp, element
+// (rows Mp of 2 Np, element G[r, c]) or transposed (rows Np of 2 Mp, element
 // G[r, c] at row c, position r)
 __device__ __forceinline__ double load_typed(const void* p, int dtype, long long e) {
     if (dtype == ISO_BF16) return (double)__uint_as_float((uint32_t)static_cast<const unsigned short*>(p)[e] << 16);
@@ -423,7 +433,7 @@ __global__ void __launch_bounds__(256) k_op_split_g(const void* G, int dtype, lo
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
         const long long r = e / Np, c = e - r * Np;
         const double v = (r < m && c < n) ? load_typed(G, dtype, r * n + c) : 0.0;
-        put_split(out + r * 4 * Np, Np, c, v);
+        put_split(out + r * 2 * Np, Np, c, v);
     }
 }
 __global__ void __launch_bounds__(256) k_op_split_gt(const void* G, int dtype, long long m, long long n, long long Mp,
@@ -437,7 +447,7 @@ __global__ void __launch_bounds__(256) k_op_split_gt(const void* G, int dtype, l
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += 8) {
         const long long c = c0 + y, r = r0 + threadIdx.x;
-        if (c < Np && r < Mp) put_split(out + c * 4 * Mp, Mp, r, t[threadIdx.x][y]);
+        if (c < Np && r < Mp) put_split(out + c * 2 * Mp, Mp, r, t[threadIdx.x][y]);
     }
 }
 
@@ -551,16 +561,17 @@ __global__ void __launch_bounds__(256) k_fr_xi(Frames f, const double* dots, con
     }
 }
 
-// ||N||_F^2 of N = xi^T xi (binary32, ld Qp; or binary64, ld q), summed into the header
+// ||N||_F^2 of N = xi^T xi (binary32, ld Qp; or binary64, ld q), one warp per row, summed into the header
 __global__ void __launch_bounds__(256) k_fr_norm(const float* N, const double* N64, long long Qp, long long q,
                                                  FrameHeader* h, int side) {
     __shared__ double red[32];
+    const int lane = threadIdx.x & 31;
     double acc = 0.0;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < q * q; e += (long long)gridDim.x * blockDim.x) {
-        const long long r = e / q, c = e - r * q;
-        const double v = N64 ? N64[e] : (double)N[r * Qp + c];
-        acc += v * v;
-    }
+    for (long long r = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); r < q; r += (long long)gridDim.x * 8)
+        for (long long c = lane; c < q; c += 32) {
+            const double v = N64 ? N64[r * q + c] : (double)N[r * Qp + c];
+            acc += v * v;
+        }
     acc = block_sum(acc, red);
     if (threadIdx.x == 0) atomicAdd(&h->nu2[side], acc);
 }
@@ -569,26 +580,36 @@ __global__ void __launch_bounds__(256) k_fr_norm(const float* N, const double* N
 // arithmetic (functions of N); the products treat them so (B = M^T = M).  Each
 // kernel below symmetrises what it writes, one 32 x 32 tile and its mirror
 // per block (blocks below the diagonal return), so that rounding cannot
-// build an asymmetric component from one iteration to the next.  Reading
-// both tiles before writing either makes the update safe in place.
+// build an asymmetric component from one iteration to the next, and writes
+// the tile's split operands as well.  Reading both tiles before writing
+// either makes the update safe in place.
 struct NsArgs {
     const float* N;     // init: N = xi^T xi (binary32, ld Qp), unless N64 is given
     const double* N64;  // init: N in binary64 (ld q)
-    const float* T1;    // m: z y;  update: y m
-    const float* T2;    // update: m z
+    const float* T1;    // m: z y (NULL: 0);  update: y m
+    const float* T2;    // update: m z (NULL: 0)
     double* y;
     double* z;
     double* m;
+    float* y4;          // the split operands of y, z and m (Qp rows of 2 Qp, zero past q)
+    float* z4;
+    float* m4;
     FrameHeader* h;
     long long q, Qp;
     int side, it;
 };
 
-__device__ __forceinline__ bool ns_tile(long long q, long long& r0, long long& c0) {
+__device__ __forceinline__ bool ns_tile(long long& r0, long long& c0) {
     if (blockIdx.x < blockIdx.y) return false;
     r0 = (long long)blockIdx.y * 32;
     c0 = (long long)blockIdx.x * 32;
     return true;
+}
+
+// one entry of a symmetric iterate and of its split operand (zero past q)
+__device__ __forceinline__ void ns_put(const NsArgs& a, double* M, float* M4, long long r, long long c, double v) {
+    if (r < a.q && c < a.q) M[r * a.q + c] = v;
+    put_split(M4 + r * 2 * a.Qp, a.Qp, c, v);
 }
 
 // Y_0 = (I + N) / cs = I + y, Z_0 = I (z = 0); cs = 1 while ||N||_F < 0.9,
@@ -596,7 +617,7 @@ __device__ __forceinline__ bool ns_tile(long long q, long long& r0, long long& c
 __global__ void __launch_bounds__(256) k_fr_ns_init(NsArgs a) {
     __shared__ double ta[32][33], tb[32][33];
     long long r0, c0;
-    if (!ns_tile(a.q, r0, c0)) return;
+    if (!ns_tile(r0, c0)) return;
     const double nu = sqrt(a.h->nu2[a.side]);
     const double cs = nu < 0.9 ? 1.0 : 1.0 + 0.5 * nu;
     if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && threadIdx.y == 0) {
@@ -615,16 +636,11 @@ __global__ void __launch_bounds__(256) k_fr_ns_init(NsArgs a) {
     }
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += 8) {
-        const long long r = r0 + y, c = c0 + threadIdx.x;
-        if (r < a.q && c < a.q) {
-            a.y[r * a.q + c] = 0.5 * (ta[y][threadIdx.x] + tb[threadIdx.x][y]);
-            a.z[r * a.q + c] = 0.0;
-        }
-        const long long r2 = c0 + y, c2 = r0 + threadIdx.x;
-        if (r2 < a.q && c2 < a.q) {
-            a.y[r2 * a.q + c2] = 0.5 * (tb[y][threadIdx.x] + ta[threadIdx.x][y]);
-            a.z[r2 * a.q + c2] = 0.0;
-        }
+        const long long r = r0 + y, c = c0 + threadIdx.x, r2 = c0 + y, c2 = r0 + threadIdx.x;
+        ns_put(a, a.y, a.y4, r, c, 0.5 * (ta[y][threadIdx.x] + tb[threadIdx.x][y]));
+        ns_put(a, a.y, a.y4, r2, c2, 0.5 * (tb[y][threadIdx.x] + ta[threadIdx.x][y]));
+        if (r < a.q && c < a.q) a.z[r * a.q + c] = 0.0;
+        if (r2 < a.q && c2 < a.q) a.z[r2 * a.q + c2] = 0.0;
     }
 }
 
@@ -634,11 +650,11 @@ __global__ void __launch_bounds__(256) k_fr_ns_m(NsArgs a) {
     __shared__ double ta[32][33], tb[32][33];
     if (*reinterpret_cast<volatile int32_t*>(&a.h->conv[a.side])) return;
     long long r0, c0;
-    if (!ns_tile(a.q, r0, c0)) return;
+    if (!ns_tile(r0, c0)) return;
     auto w = [&](long long r, long long c) -> double {
         if (r >= a.q || c >= a.q) return 0.0;
         const long long e = r * a.q + c;
-        return a.y[e] + a.z[e] + (double)a.T1[r * a.Qp + c];
+        return a.y[e] + a.z[e] + (a.T1 ? (double)a.T1[r * a.Qp + c] : 0.0);
     };
     for (int y = threadIdx.y; y < 32; y += 8) {
         ta[y][threadIdx.x] = w(r0 + y, c0 + threadIdx.x);
@@ -648,13 +664,10 @@ __global__ void __launch_bounds__(256) k_fr_ns_m(NsArgs a) {
     float wm = 0.0f;
     for (int y = threadIdx.y; y < 32; y += 8) {
         const long long r = r0 + y, c = c0 + threadIdx.x;
-        if (r < a.q && c < a.q) {
-            const double v = 0.5 * (ta[y][threadIdx.x] + tb[threadIdx.x][y]);
-            a.m[r * a.q + c] = -0.5 * v;
-            wm = fmaxf(wm, (float)fabs(v));
-        }
-        const long long r2 = c0 + y, c2 = r0 + threadIdx.x;
-        if (r2 < a.q && c2 < a.q) a.m[r2 * a.q + c2] = -0.25 * (tb[y][threadIdx.x] + ta[threadIdx.x][y]);
+        const double v = 0.5 * (ta[y][threadIdx.x] + tb[threadIdx.x][y]);
+        ns_put(a, a.m, a.m4, r, c, -0.5 * v);
+        wm = fmaxf(wm, (float)fabs(v));
+        ns_put(a, a.m, a.m4, c0 + y, r0 + threadIdx.x, -0.25 * (tb[y][threadIdx.x] + ta[threadIdx.x][y]));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, o));
@@ -676,7 +689,7 @@ __global__ void __launch_bounds__(256) k_fr_ns_update(NsArgs a) {
         return;
     }
     long long r0, c0;
-    if (!ns_tile(a.q, r0, c0)) return;
+    if (!ns_tile(r0, c0)) return;
     auto fy = [&](long long r, long long c) -> double {
         if (r >= a.q || c >= a.q) return 0.0;
         const long long e = r * a.q + c;
@@ -685,7 +698,7 @@ __global__ void __launch_bounds__(256) k_fr_ns_update(NsArgs a) {
     auto fz = [&](long long r, long long c) -> double {
         if (r >= a.q || c >= a.q) return 0.0;
         const long long e = r * a.q + c;
-        return a.z[e] + a.m[e] + (double)a.T2[r * a.Qp + c];
+        return a.z[e] + a.m[e] + (a.T2 ? (double)a.T2[r * a.Qp + c] : 0.0);
     };
     for (int y = threadIdx.y; y < 32; y += 8) {
         ya[y][threadIdx.x] = fy(r0 + y, c0 + threadIdx.x);
@@ -695,16 +708,11 @@ __global__ void __launch_bounds__(256) k_fr_ns_update(NsArgs a) {
     }
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += 8) {
-        const long long r = r0 + y, c = c0 + threadIdx.x;
-        if (r < a.q && c < a.q) {
-            a.y[r * a.q + c] = 0.5 * (ya[y][threadIdx.x] + yb[threadIdx.x][y]);
-            a.z[r * a.q + c] = 0.5 * (za[y][threadIdx.x] + zb[threadIdx.x][y]);
-        }
-        const long long r2 = c0 + y, c2 = r0 + threadIdx.x;
-        if (r2 < a.q && c2 < a.q) {
-            a.y[r2 * a.q + c2] = 0.5 * (yb[y][threadIdx.x] + ya[threadIdx.x][y]);
-            a.z[r2 * a.q + c2] = 0.5 * (zb[y][threadIdx.x] + za[threadIdx.x][y]);
-        }
+        const long long r = r0 + y, c = c0 + threadIdx.x, r2 = c0 + y, c2 = r0 + threadIdx.x;
+        ns_put(a, a.y, a.y4, r, c, 0.5 * (ya[y][threadIdx.x] + yb[threadIdx.x][y]));
+        ns_put(a, a.z, a.z4, r, c, 0.5 * (za[y][threadIdx.x] + zb[threadIdx.x][y]));
+        ns_put(a, a.y, a.y4, r2, c2, 0.5 * (yb[y][threadIdx.x] + ya[threadIdx.x][y]));
+        ns_put(a, a.z, a.z4, r2, c2, 0.5 * (zb[y][threadIdx.x] + za[threadIdx.x][y]));
     }
 }
 
@@ -759,9 +767,9 @@ FrameLayout frame_layout(long long m, long long n, int K) {
     L.tail = o;
     for (int s = 0; s < 2; ++s) {
         const long long Dp = s == 0 ? L.Mp : L.Np, d = s == 0 ? m : n;
-        L.ft4[s] = take(sizeof(float) * Qp * 4 * Dp);      // xi*^T split
-        L.fr4[s] = take(sizeof(float) * Dp * 4 * Qp);      // F_0 split, later (F_0 + xi*) split
-        L.y4[s] = take(sizeof(float) * Qp * 4 * Qp);       // Y^T split, later R split
+        L.ft4[s] = take(sizeof(float) * Qp * 2 * Dp);      // xi*^T split
+        L.fr4[s] = take(sizeof(float) * Dp * 2 * Qp);      // F_0 split, later (F_0 + xi*) split
+        L.y4[s] = take(sizeof(float) * Qp * 2 * Qp);       // Y^T split, later R split
         L.e[s] = take(sizeof(float) * Dp * Qp);            // F_0 Y, later (F_0 + xi*) R
         L.xi[s] = take(sizeof(double) * d * q);            // xi*, later E_F
         L.nq[s] = take(sizeof(float) * Qp * Qp);
@@ -769,14 +777,14 @@ FrameLayout frame_layout(long long m, long long n, int K) {
     L.ns_y = take(sizeof(double) * q * q);
     L.ns_z = take(sizeof(double) * q * q);
     L.ns_m = take(sizeof(double) * q * q);
-    L.ns_y4 = take(sizeof(float) * Qp * 4 * Qp);
-    L.ns_z4 = take(sizeof(float) * Qp * 4 * Qp);
-    L.ns_m4 = take(sizeof(float) * Qp * 4 * Qp);
+    L.ns_y4 = take(sizeof(float) * Qp * 2 * Qp);
+    L.ns_z4 = take(sizeof(float) * Qp * 2 * Qp);
+    L.ns_m4 = take(sizeof(float) * Qp * 2 * Qp);
     L.ns_t1 = take(sizeof(float) * Qp * Qp);
     L.ns_t2 = take(sizeof(float) * Qp * Qp);
     L.ns_t3 = take(sizeof(float) * Qp * Qp);
-    L.a6 = take(sizeof(float) * L.Mp * 4 * 2 * Qp);
-    L.b6 = take(sizeof(float) * L.Np * 4 * 2 * Qp);
+    L.a6 = take(sizeof(float) * L.Mp * 2 * 2 * Qp);
+    L.b6 = take(sizeof(float) * L.Np * 2 * 2 * Qp);
     L.total = o;
     return L;
 }
@@ -795,21 +803,43 @@ int gemm_smem_optin() {
     return ISO_OK;
 }
 
+int x3_smem_optin() {
+    static std::once_flag once;
+    static int rc = ISO_OK;
+    std::call_once(once, [] {
+        if (cudaFuncSetAttribute(k_gemm_x3<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, X3_SMEM) != cudaSuccess ||
+            cudaFuncSetAttribute(k_gemm_x3<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, X3_SMEM) != cudaSuccess)
+            rc = ISO_ERR_CUDA;
+    });
+    return rc;
+}
+
 // C (a_rows x b_rows) = A B^T over the three-product split: A and B are
-// four-segment operand arrays of segment length L (rows a_rows / b_rows,
-// multiples of 128).
-int frame_gemm(cudaStream_t s, const float* A, long long a_rows, const float* B, long long b_rows, long long L,
-               GemmArgs g) {
-    CUtensorMap ta, tb;
-    ISO_TRY(gemm_tensor_map(&ta, A, a_rows, 4 * L, 4 * L));
-    ISO_TRY(gemm_tensor_map(&tb, B, b_rows, 4 * L, 4 * L));
-    g.k_tiles = (int)(3 * L / GEMM_BK);
-    g.a_k0 = 0;
-    g.b_k0 = (int)L;
-    ISO_TRY(gemm_smem_optin());
-    const dim3 grid((unsigned)(b_rows / GEMM_BN), (unsigned)(a_rows / GEMM_BM));
+// two-segment operand arrays of segment length L (rows a_rows / b_rows,
+// multiples of 128); with A2, a second product C2 = A2 B2^T of the same shape
+// in the same launch.  The tile shape with the smaller number of waves times
+// what a stage costs in it (clocks per 32 contraction columns: 1900 for 128 x
+// 256, bound by shared memory; 1150 for 128 x 128, bound by L2).
+int frame_gemm(cudaStream_t s, int sms, const float* A, long long a_rows, const float* B, long long b_rows, long long L,
+               GemmArgs g, const float* A2 = nullptr, const float* B2 = nullptr) {
+    CUtensorMap ta, tb, ta2, tb2;
+    ISO_TRY(gemm_tensor_map(&ta, A, a_rows, 2 * L, 2 * L));
+    ISO_TRY(gemm_tensor_map(&tb, B, b_rows, 2 * L, 2 * L));
+    ISO_TRY(gemm_tensor_map(&ta2, A2 ? A2 : A, a_rows, 2 * L, 2 * L));
+    ISO_TRY(gemm_tensor_map(&tb2, A2 ? B2 : B, b_rows, 2 * L, 2 * L));
+    g.k_tiles = (int)(L / GEMM_BK);
+    g.seg = (int)L;
+    g.c_cols = (int)b_rows;
+    ISO_TRY(x3_smem_optin());
+    const unsigned nz = A2 ? 2 : 1;
+    const long long my = a_rows / GEMM_BM, t128 = my * (b_rows / 128) * nz, t256 = my * ((b_rows + 255) / 256) * nz;
+    const bool wide = (t256 + sms - 1) / sms * 1900 <= (t128 + sms - 1) / sms * 1150;
     const int slot = prof_begin(0, s);
-    k_gemm_tf32<<<grid, GEMM_THREADS, GEMM_SMEM, s>>>(ta, tb, g);
+    if (wide)
+        k_gemm_x3<256><<<dim3((unsigned)((b_rows + 255) / 256), (unsigned)my, nz), GEMM_THREADS, X3_SMEM, s>>>(ta, tb, ta2,
+                                                                                                            tb2, g);
+    else
+        k_gemm_x3<128><<<dim3((unsigned)(b_rows / 128), (unsigned)my, nz), GEMM_THREADS, X3_SMEM, s>>>(ta, tb, ta2, tb2, g);
     prof_end(slot, s);
     return cudaGetLastError() == cudaSuccess ? ISO_OK : ISO_ERR_CUDA;
 }
@@ -833,24 +863,24 @@ OptLayout opt_layout(long long m, long long n) {
     L.zero_end = o;
     L.ex = take(sizeof(int32_t) * Qp);
     // the four gradient operands, dead after the factor gradients: then the slabs of X_bar
-    L.gw4 = take(sizeof(float) * L.Mp * 4 * L.Np);      // G_W, rows m, contraction n
-    L.gwt4 = take(sizeof(float) * L.Np * 4 * L.Mp);     // G_W^T, rows n, contraction m
-    L.su4 = take(sizeof(float) * Qp * 4 * L.Mp);        // (U S_0)^T
-    L.sv4 = take(sizeof(float) * Qp * 4 * L.Np);        // (V S_0)^T
+    L.gw4 = take(sizeof(float) * L.Mp * 2 * L.Np);      // G_W, rows m, contraction n
+    L.gwt4 = take(sizeof(float) * L.Np * 2 * L.Mp);     // G_W^T, rows n, contraction m
+    L.su4 = take(sizeof(float) * Qp * 2 * L.Mp);        // (U S_0)^T
+    L.sv4 = take(sizeof(float) * Qp * 2 * L.Np);        // (V S_0)^T
     L.dF[0] = take(sizeof(double) * m * q);             // U_bar - U, later E_U
     L.dF[1] = take(sizeof(double) * n * q);             // V_bar - V, later E_V
     L.n64 = take(sizeof(double) * q * q);               // (F + dF)^T (F + dF) - I
-    L.xb4 = take(sizeof(float) * L.Dmax * 4 * Qp);      // F + dF
-    L.r4 = take(sizeof(float) * Qp * 4 * Qp);
+    L.xb4 = take(sizeof(float) * L.Dmax * 2 * Qp);      // F + dF
+    L.r4 = take(sizeof(float) * Qp * 2 * Qp);
     L.p = take(sizeof(float) * L.Dmax * Qp);
-    L.a6 = take(sizeof(float) * L.Mp * 4 * 2 * Qp);
-    L.b6 = take(sizeof(float) * L.Np * 4 * 2 * Qp);
+    L.a6 = take(sizeof(float) * L.Mp * 2 * 2 * Qp);
+    L.b6 = take(sizeof(float) * L.Np * 2 * 2 * Qp);
     L.ns_y = take(sizeof(double) * q * q);
     L.ns_z = take(sizeof(double) * q * q);
     L.ns_m = take(sizeof(double) * q * q);
-    L.ns_y4 = take(sizeof(float) * Qp * 4 * Qp);
-    L.ns_z4 = take(sizeof(float) * Qp * 4 * Qp);
-    L.ns_m4 = take(sizeof(float) * Qp * 4 * Qp);
+    L.ns_y4 = take(sizeof(float) * Qp * 2 * Qp);
+    L.ns_z4 = take(sizeof(float) * Qp * 2 * Qp);
+    L.ns_m4 = take(sizeof(float) * Qp * 2 * Qp);
     L.ns_t1 = take(sizeof(float) * Qp * Qp);
     L.ns_t2 = take(sizeof(float) * Qp * Qp);
     L.ns_t3 = take(sizeof(float) * Qp * Qp);
@@ -874,7 +904,11 @@ int exact_product(cudaStream_t s, int sms, const OzSrc& src, int K, double* C, u
     const long long nt = Qp / OZ_BM, chunks = (d + OZ_BK - 1) / OZ_BK;
     const unsigned long long slot = (unsigned long long)nt * chunks * OZ_SLAB_BYTES;
     const int rc = (int)std::max(1LL, std::min(256LL, (d + 255) / 256));
-    FR_LAUNCH((k_oz_colmax<<<dim3((unsigned)((q + 31) / 32), rc), dim3(32, 8), 0, s>>>(src, K + 1, rc)));
+    const dim3 mg((unsigned)((q + 31) / 32), rc), mb(32, 8);
+    if (K == 0) FR_LAUNCH((k_oz_colmax<1><<<mg, mb, 0, s>>>(src, K + 1, rc)));
+    else if (K <= 2) FR_LAUNCH((k_oz_colmax<3><<<mg, mb, 0, s>>>(src, K + 1, rc)));
+    else if (K <= 4) FR_LAUNCH((k_oz_colmax<5><<<mg, mb, 0, s>>>(src, K + 1, rc)));
+    else FR_LAUNCH((k_oz_colmax<MAXK + 1><<<mg, mb, 0, s>>>(src, K + 1, rc)));
     static std::once_flag once;
     static cudaError_t opt = cudaSuccess;
     std::call_once(once, [] { opt = cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM); });
@@ -939,45 +973,32 @@ struct NsBufs {
 
 // R = (I + N)^(-1/2) - I for N = X^T X (binary32, ld Qp) with X^T F_0 skew,
 // by the difference-form Newton-Schulz iteration (k_fr_ns_*), written as
-// the split operand R4 (Qp rows of 4 Qp; R is symmetric, so it serves as B
+// the split operand R4 (Qp rows of 2 Qp; R is symmetric, so it serves as B
 // of (F_0 + X) R).  Header slot `side` holds its scaling and state.
 int ns_root(cudaStream_t s, int sms, FrameHeader* hdr, int side, const float* Nq, const double* N64, long long q,
             long long Qp, const NsBufs& b, int ns_iters, float* R4) {
-    FR_LAUNCH((k_fr_norm<<<grid_of(q * q, sms), 256, 0, s>>>(Nq, N64, Qp, q, hdr, side)));
+    FR_LAUNCH((k_fr_norm<<<grid_of(q * 32, sms), 256, 0, s>>>(Nq, N64, Qp, q, hdr, side)));
     NsArgs na{};
-    na.N = Nq; na.N64 = N64; na.y = b.y; na.z = b.z; na.m = b.m; na.h = hdr;
+    na.N = Nq; na.N64 = N64; na.y = b.y; na.z = b.z; na.m = b.m; na.y4 = b.y4; na.z4 = b.z4; na.m4 = b.m4; na.h = hdr;
     na.q = q; na.Qp = Qp; na.side = side;
-    const dim3 tiles((unsigned)((q + 31) / 32), (unsigned)((q + 31) / 32)), tb(32, 8);
+    const dim3 tiles((unsigned)(Qp / 32), (unsigned)(Qp / 32)), tb(32, 8);
     FR_LAUNCH((k_fr_ns_init<<<tiles, tb, 0, s>>>(na)));
-    SplitR sq{};
-    sq.f.q = q; sq.hdr = hdr; sq.side = side; sq.mode = 2; sq.rows = q; sq.rows_p = Qp; sq.Lp = Qp;
-    sq.skip = &hdr->conv[side];
-    auto split_q = [&](const double* M_, float* out) -> int {
-        sq.M = M_; sq.out = out;
-        FR_LAUNCH((k_fr_split_r<<<grid_of(Qp * Qp, sms), 256, 0, s>>>(sq)));
-        return ISO_OK;
-    };
-    ISO_TRY(split_q(b.y, b.y4));
-    ISO_TRY(split_q(b.z, b.z4));
     for (int it = 0; it < ns_iters; ++it) {
         GemmArgs g{};
         g.mode = GEMM_STORE_F32; g.ldc = Qp; g.M = (int)Qp; g.N = (int)Qp; g.status = &hdr->status;
         g.skip = &hdr->conv[side];
         g.C = b.t1;
-        ISO_TRY(frame_gemm(s, b.z4, Qp, b.y4, Qp, Qp, g));     // z y
+        if (it) ISO_TRY(frame_gemm(s, sms, b.z4, Qp, b.y4, Qp, Qp, g));     // z y (z = 0 at first)
         na.it = it;
-        na.T1 = b.t1;
+        na.T1 = it ? b.t1 : nullptr;
         FR_LAUNCH((k_fr_ns_m<<<tiles, tb, 0, s>>>(na)));
-        ISO_TRY(split_q(b.m, b.m4));
+        // y m and, past the first step (z = 0), m z in one launch
         g.C = b.t2;
-        ISO_TRY(frame_gemm(s, b.y4, Qp, b.m4, Qp, Qp, g));     // y m
-        g.C = b.t3;
-        ISO_TRY(frame_gemm(s, b.m4, Qp, b.z4, Qp, Qp, g));     // m z
+        g.C2 = b.t3;
+        ISO_TRY(frame_gemm(s, sms, b.y4, Qp, b.m4, Qp, Qp, g, it ? b.m4 : nullptr, b.z4));
         na.T1 = b.t2;
-        na.T2 = b.t3;
+        na.T2 = it ? b.t3 : nullptr;
         FR_LAUNCH((k_fr_ns_update<<<tiles, tb, 0, s>>>(na)));
-        ISO_TRY(split_q(b.y, b.y4));
-        ISO_TRY(split_q(b.z, b.z4));
     }
     SplitR sr{};
     sr.f.q = q; sr.hdr = hdr; sr.side = side; sr.mode = 6; sr.M = b.z; sr.out = R4;
@@ -1073,8 +1094,12 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
         FR_LAUNCH((k_fr_signdots<<<dim3((unsigned)((q + 31) / 32), K, rc), dim3(32, 8), 0, s>>>(fr[0], dots, rc)));
         for (int sd = 0; sd < 2; ++sd) {
             const int r2 = (int)std::max(1LL, std::min(256LL, (fr[sd].d + 255) / 256));
-            FR_LAUNCH((k_fr_coldots<<<dim3((unsigned)((q + 31) / 32), r2), dim3(32, 8), 0, s>>>(
-                fr[sd], dots, D(L.cd[sd]), r2)));
+            const dim3 cg((unsigned)((q + 31) / 32), r2), cb(32, 8);
+            if (K == 1) FR_LAUNCH((k_fr_coldots<1><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
+            else if (K == 2) FR_LAUNCH((k_fr_coldots<2><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
+            else if (K == 3) FR_LAUNCH((k_fr_coldots<3><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
+            else if (K == 4) FR_LAUNCH((k_fr_coldots<4><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
+            else FR_LAUNCH((k_fr_coldots<8><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
         }
     }
     // A_i = F_0^T dF_i (binary64), then Sym_i and Kw_i
@@ -1113,7 +1138,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
         {
             GemmArgs g{};
             g.mode = GEMM_STORE_F32; g.C = F(L.e[sd]); g.ldc = Qp; g.M = (int)Dp; g.N = (int)Qp; g.status = &hdr->status;
-            ISO_TRY(frame_gemm(s, F(L.fr4[sd]), Dp, F(L.y4[sd]), Qp, Qp, g));
+            ISO_TRY(frame_gemm(s, sms, F(L.fr4[sd]), Dp, F(L.y4[sd]), Qp, Qp, g));
         }
         FR_LAUNCH((k_fr_xi<<<grid_of(d * q, sms), 256, 0, s>>>(fr[sd], dots, coef, F(L.e[sd]), Qp, k_keep, D(L.xi[sd]))));
         // N = xi*^T xi*
@@ -1123,7 +1148,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
             FR_LAUNCH((k_fr_split_t<<<dim3((unsigned)(Dp / 32), (unsigned)(Qp / 32)), dim3(32, 8), 0, s>>>(st)));
             GemmArgs g{};
             g.mode = GEMM_STORE_F32; g.C = F(L.nq[sd]); g.ldc = Qp; g.M = (int)Qp; g.N = (int)Qp; g.status = &hdr->status;
-            ISO_TRY(frame_gemm(s, F(L.ft4[sd]), Qp, F(L.ft4[sd]), Qp, Dp, g));
+            ISO_TRY(frame_gemm(s, sms, F(L.ft4[sd]), Qp, F(L.ft4[sd]), Qp, Dp, g));
         }
         // (I + N)^(-1/2) = I + R by the difference-form Newton-Schulz iteration,
         // then F_0 + xi*, and E_F = xi* + (F_0 + xi*) R
@@ -1137,7 +1162,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
         {
             GemmArgs g{};
             g.mode = GEMM_STORE_F32; g.C = F(L.e[sd]); g.ldc = Qp; g.M = (int)Dp; g.N = (int)Qp; g.status = &hdr->status;
-            ISO_TRY(frame_gemm(s, F(L.fr4[sd]), Dp, F(L.y4[sd]), Qp, Qp, g));
+            ISO_TRY(frame_gemm(s, sms, F(L.fr4[sd]), Dp, F(L.y4[sd]), Qp, Qp, g));
         }
         FR_LAUNCH((k_fr_motion<<<grid_of(d * q, sms), 256, 0, s>>>(D(L.xi[sd]), F(L.e[sd]), Qp, d, q)));
         // the reconstruction's operand of this side
@@ -1152,7 +1177,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
         GemmArgs g{};
         g.mode = GEMM_ADD_BASE; g.M = (int)m; g.N = (int)n; g.out = out->data; g.w0 = W0->data; g.ldo = n;
         g.out_dtype = W0->dtype; g.status = &hdr->status;
-        ISO_TRY(frame_gemm(s, F(L.a6), L.Mp, F(L.b6), L.Np, 2 * Qp, g));
+        ISO_TRY(frame_gemm(s, sms, F(L.a6), L.Mp, F(L.b6), L.Np, 2 * Qp, g));
     }
     if (stats && stats->status) FR_LAUNCH((k_fr_status<<<1, 32, 0, s>>>(hdr, stats->status)));
     return ISO_OK;
@@ -1230,9 +1255,9 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
         GemmArgs g{};
         g.mode = GEMM_ADAMW; g.M = (int)(sd == 0 ? m : n); g.N = (int)q; g.ldo = q; g.status = &hdr->status;
         g.adam = AdamwArgs{sd == 0 ? U : V, sd == 0 ? mU : mV, sd == 0 ? vU : vV, D(L.dF[sd]),
-                           cfg->lr, cfg->beta1, cfg->beta2, cfg->eps, cfg->weight_decay, bc1, bc2};
-        if (sd == 0) ISO_TRY(frame_gemm(s, F(L.gw4), L.Mp, F(L.sv4), Qp, L.Np, g));
-        else ISO_TRY(frame_gemm(s, F(L.gwt4), L.Np, F(L.su4), Qp, L.Mp, g));
+                           cfg->beta1, cfg->beta2, cfg->eps, bc2, cfg->lr * cfg->weight_decay, cfg->lr / bc1};
+        if (sd == 0) ISO_TRY(frame_gemm(s, sms, F(L.gw4), L.Mp, F(L.sv4), Qp, L.Np, g));
+        else ISO_TRY(frame_gemm(s, sms, F(L.gwt4), L.Np, F(L.su4), Qp, L.Mp, g));
     }
     // the polar retraction of each side: N = (F + dF)^T (F + dF) - I in
     // binary64, R = (I + N)^(-1/2) - I, E_F = dF + (F + dF) R
@@ -1251,7 +1276,7 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
         {
             GemmArgs g{};
             g.mode = GEMM_STORE_F32; g.C = F(L.p); g.ldc = Qp; g.M = (int)Dp; g.N = (int)Qp; g.status = &hdr->status;
-            ISO_TRY(frame_gemm(s, F(L.xb4), Dp, F(L.r4), Qp, Qp, g));
+            ISO_TRY(frame_gemm(s, sms, F(L.xb4), Dp, F(L.r4), Qp, Qp, g));
         }
         FR_LAUNCH((k_fr_motion<<<grid_of(d * q, sms), 256, 0, s>>>(D(L.dF[sd]), F(L.p), Qp, d, q)));
         // the reconstruction's operand of this side ([E_U S_0 | U S_0] or [V + E_V | E_V])
@@ -1266,7 +1291,7 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
         GemmArgs g{};
         g.mode = GEMM_ADD_BASE; g.M = (int)m; g.N = (int)n; g.out = W_out->data; g.w0 = W->data; g.ldo = n;
         g.out_dtype = W->dtype; g.status = &hdr->status;
-        ISO_TRY(frame_gemm(s, F(L.a6), L.Mp, F(L.b6), L.Np, 2 * Qp, g));
+        ISO_TRY(frame_gemm(s, sms, F(L.a6), L.Mp, F(L.b6), L.Np, 2 * Qp, g));
     }
     if (stats && stats->status) FR_LAUNCH((k_fr_status<<<1, 32, 0, s>>>(hdr, stats->status)));
     return ISO_OK;

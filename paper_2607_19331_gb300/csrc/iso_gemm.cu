@@ -37,10 +37,11 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
                  :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar) : "memory");
 }
 
-__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
+__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate,
+                                          uint32_t idesc = UMMA_IDESC) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                  "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-                 :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(UMMA_IDESC), "r"(accumulate) : "memory");
+                 :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
 // arrive on `bar` once every tcgen05.mma this thread issued before has completed
@@ -91,6 +92,51 @@ __device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volati
     }
     *abort_flag = 1;
     return false;
+}
+
+// one entry of the AdamW epilogue (a call, so that the unrolled columns stay
+// in registers without 32 copies of the binary64 code)
+__device__ __noinline__ void adamw_entry(const AdamwArgs& a, long long e, float grad) {
+    const double gr = (double)grad;
+    const double mm = a.beta1 * (double)a.m[e] + (1.0 - a.beta1) * gr;
+    const double vv = a.beta2 * (double)a.v[e] + (1.0 - a.beta2) * gr * gr;
+    a.m[e] = (float)mm;
+    a.v[e] = (float)vv;
+    a.dX[e] = -a.lr_wd * a.X[e] - a.lr_bc1 * mm / (sqrt(vv / a.bc2) + a.eps);
+}
+
+// one row's 32 accumulated columns from col0 on, by epilogue mode
+__device__ __forceinline__ void gemm_store32(const GemmArgs& g, float* C, long long row, int col0, const float (&v)[32]) {
+    if (g.mode == GEMM_STORE_F32) {
+        float4* dst = reinterpret_cast<float4*>(C + row * g.ldc + col0);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    } else if (g.mode == GEMM_ADAMW) {
+        if (row < g.M) {
+            const AdamwArgs& a = g.adam;
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+                if (col0 + j < g.N) adamw_entry(a, row * g.ldo + col0 + j, v[j]);
+        }
+    } else if (row < g.M) {
+        if (g.out_dtype == ISO_BF16) {
+            const unsigned short* w = static_cast<const unsigned short*>(g.w0) + row * g.ldo;
+            __nv_bfloat16* o = static_cast<__nv_bfloat16*>(g.out) + row * g.ldo;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const int col = col0 + j;
+                if (col < g.N) o[col] = __float2bfloat16_rn(__fadd_rn(__uint_as_float((uint32_t)w[col] << 16), v[j]));
+            }
+        } else {
+            const float* w = static_cast<const float*>(g.w0) + row * g.ldo;
+            float* o = static_cast<float*>(g.out) + row * g.ldo;
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const int col = col0 + j;
+                if (col < g.N) o[col] = __fadd_rn(w[col], v[j]);
+            }
+        }
+    }
 }
 
 }  // namespace
@@ -185,45 +231,9 @@ k_gemm_tf32(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
             float v[32];
             tmem_ld32(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)(c * 32), v);
             const int col0 = n0 + c * 32;
-            if (g.mode == GEMM_STORE_F32) {
-                float4* dst = reinterpret_cast<float4*>(g.C + row * g.ldc + col0);
+            float4* dst = reinterpret_cast<float4*>(g.C + row * g.ldc + col0);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-            } else if (g.mode == GEMM_ADAMW) {
-                if (row < g.M) {
-                    const AdamwArgs& a = g.adam;
-#pragma unroll 4
-                    for (int j = 0; j < 32; ++j) {
-                        const int col = col0 + j;
-                        if (col >= g.N) break;
-                        const long long e = row * g.ldo + col;
-                        const double gr = (double)v[j];
-                        const double mm = a.beta1 * (double)a.m[e] + (1.0 - a.beta1) * gr;
-                        const double vv = a.beta2 * (double)a.v[e] + (1.0 - a.beta2) * gr * gr;
-                        a.m[e] = (float)mm;
-                        a.v[e] = (float)vv;
-                        a.dX[e] = -a.lr * a.wd * a.X[e] - (a.lr / a.bc1) * mm / (sqrt(vv / a.bc2) + a.eps);
-                    }
-                }
-            } else if (row < g.M) {
-                if (g.out_dtype == ISO_BF16) {
-                    const unsigned short* w = static_cast<const unsigned short*>(g.w0) + row * g.ldo;
-                    __nv_bfloat16* o = static_cast<__nv_bfloat16*>(g.out) + row * g.ldo;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int col = col0 + j;
-                        if (col < g.N) o[col] = __float2bfloat16_rn(__fadd_rn(__uint_as_float((uint32_t)w[col] << 16), v[j]));
-                    }
-                } else {
-                    const float* w = static_cast<const float*>(g.w0) + row * g.ldo;
-                    float* o = static_cast<float*>(g.out) + row * g.ldo;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) {
-                        const int col = col0 + j;
-                        if (col < g.N) o[col] = __fadd_rn(w[col], v[j]);
-                    }
-                }
-            }
+            for (int j = 0; j < 8; ++j) dst[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
         }
     }
     tc_fence_before();
@@ -233,6 +243,130 @@ k_gemm_tf32(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(GEMM_BN) : "memory");
     }
 }
+
+// The epilogue of the split product, and its three products per stage.
+template <int BN>
+__global__ void __launch_bounds__(GEMM_THREADS, 1)
+k_gemm_x3(const __grid_constant__ CUtensorMap ta1, const __grid_constant__ CUtensorMap tb1,
+          const __grid_constant__ CUtensorMap ta2, const __grid_constant__ CUtensorMap tb2, GemmArgs g) {
+    if (g.skip && *reinterpret_cast<const volatile int32_t*>(g.skip)) return;
+    constexpr int STAGES = BN == 256 ? 2 : 3;
+    constexpr int A_BYTES = GEMM_TILE_BYTES, B_BYTES = GEMM_TILE_BYTES * (BN / 128);
+    constexpr int STAGE_BYTES = 2 * (A_BYTES + B_BYTES);                  // A hi, A lo, B hi, B lo
+    constexpr uint32_t IDESC = (UMMA_IDESC & ~(0x3Fu << 17)) | ((uint32_t)(BN >> 3) << 17);
+    static_assert(1024 + STAGES * STAGE_BYTES + 256 <= X3_SMEM, "shared memory");
+    extern __shared__ unsigned char gemm_smem_raw[];
+    unsigned char* const smem = reinterpret_cast<unsigned char*>(
+        (reinterpret_cast<uintptr_t>(gemm_smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint64_t* const bars = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
+    // bars[0, S): full, bars[S, 2S): empty, bars[2S]: accumulators ready
+    uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
+    volatile int* const abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int m0 = blockIdx.y * GEMM_BM, n0 = blockIdx.x * BN;
+    const CUtensorMap* const ta = blockIdx.z ? &ta2 : &ta1;
+    const CUtensorMap* const tb = blockIdx.z ? &tb2 : &tb1;
+    float* const C = blockIdx.z ? g.C2 : g.C;
+    const uint32_t smem_s = smem_u32(smem), bar_s = smem_u32(bars);
+    auto full_bar = [&](int s) { return bar_s + 8u * s; };
+    auto empty_bar = [&](int s) { return bar_s + 8u * (STAGES + s); };
+    const uint32_t accum_bar = bar_s + 8u * (2 * STAGES);
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < STAGES; ++s) {
+            mbar_init(full_bar(s), 1);
+            mbar_init(empty_bar(s), 1);
+        }
+        mbar_init(accum_bar, 1);
+        *abort_flag = 0;
+        mbar_fence_init();
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     :: "r"(smem_u32(tmem_slot)), "r"(2 * BN) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+    const int KT = g.k_tiles;
+
+    if (warp == 0 && lane == 0) {
+        int issued = 0;
+        for (int kt = 0; kt < KT; ++kt) {
+            const int s = kt % STAGES;
+            if (!wait_phase(empty_bar(s), ((uint32_t)(kt / STAGES) & 1u) ^ 1u, abort_flag)) break;
+            // rows past the operand's end are filled with zeros and count as copied
+            mbar_arrive_tx(full_bar(s), STAGE_BYTES);
+            const uint32_t a0 = smem_s + (uint32_t)(s * STAGE_BYTES), b0 = a0 + 2 * A_BYTES;
+            const int x = kt * GEMM_BK;
+            tma_load_2d(a0, ta, x, m0, full_bar(s));
+            tma_load_2d(a0 + A_BYTES, ta, g.seg + x, m0, full_bar(s));
+#pragma unroll
+            for (int h = 0; h < BN / 128; ++h) {
+                tma_load_2d(b0 + h * GEMM_TILE_BYTES, tb, x, n0 + 128 * h, full_bar(s));
+                tma_load_2d(b0 + B_BYTES + h * GEMM_TILE_BYTES, tb, g.seg + x, n0 + 128 * h, full_bar(s));
+            }
+            ++issued;
+        }
+        // every copy this thread issued has landed before the CTA may exit
+        for (int kt = (issued > STAGES ? issued - STAGES : 0); kt < issued; ++kt) {
+            for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
+                if (mbar_try_wait(full_bar(kt % STAGES), (uint32_t)(kt / STAGES) & 1u)) break;
+        }
+    } else if (warp == 1 && lane == 0) {
+        for (int kt = 0; kt < KT; ++kt) {
+            const int s = kt % STAGES;
+            if (!wait_phase(full_bar(s), (uint32_t)(kt / STAGES) & 1u, abort_flag)) break;
+            tc_fence_after();
+            const uint32_t a0 = smem_s + (uint32_t)(s * STAGE_BYTES), b0 = a0 + 2 * A_BYTES;
+#pragma unroll
+            for (int kk = 0; kk < GEMM_BK / 8; ++kk) {
+                const uint64_t ah = sw128_desc(a0 + 32u * kk), al = sw128_desc(a0 + A_BYTES + 32u * kk);
+                const uint64_t bh = sw128_desc(b0 + 32u * kk), bl = sw128_desc(b0 + B_BYTES + 32u * kk);
+                const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
+                umma_tf32(tmem, ah, bh, acc, IDESC);
+                umma_tf32(tmem + BN, ah, bl, acc, IDESC);
+                umma_tf32(tmem + BN, al, bh, 1u, IDESC);
+            }
+            umma_commit(empty_bar(s));
+        }
+        // the accumulator barrier also tracks products issued before a give-up
+        umma_commit(accum_bar);
+    }
+    __syncwarp();
+
+    const bool ok = wait_phase(accum_bar, 0u, abort_flag) && !*abort_flag;
+    tc_fence_after();
+    if (!ok) {
+        if (threadIdx.x == 0 && g.status) atomicCAS(g.status, 0, (int32_t)ISO_ERR_TIMEOUT);
+    } else {
+        const long long row = (long long)m0 + warp * 32 + lane;
+        const uint32_t tq = tmem + ((uint32_t)(warp * 32) << 16);
+#pragma unroll 1
+        for (int c = 0; c < BN; c += 32) {
+            if (n0 + c >= g.c_cols) break;
+            float v[32], w[32];
+            tmem_ld32(tq + (uint32_t)c, v);
+            tmem_ld32(tq + (uint32_t)(BN + c), w);
+#pragma unroll
+            for (int j = 0; j < 32; ++j) v[j] = __fadd_rn(v[j], w[j]);
+            gemm_store32(g, C, row, n0 + c, v);
+        }
+    }
+    __syncwarp();
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(2 * BN) : "memory");
+    }
+}
+template __global__ void k_gemm_x3<128>(const __grid_constant__ CUtensorMap, const __grid_constant__ CUtensorMap,
+                                        const __grid_constant__ CUtensorMap, const __grid_constant__ CUtensorMap, GemmArgs);
+template __global__ void k_gemm_x3<256>(const __grid_constant__ CUtensorMap, const __grid_constant__ CUtensorMap,
+                                        const __grid_constant__ CUtensorMap, const __grid_constant__ CUtensorMap, GemmArgs);
 
 // ---------------------------------------------------------------------------
 // exact-slice contraction (see iso_gemm.cuh)

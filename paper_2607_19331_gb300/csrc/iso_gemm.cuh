@@ -1,8 +1,9 @@
-// iso_gemm.cuh -- the dense contraction of the frame-space merge on the
-// fifth-generation tensor cores: C = A B^T for row-major fp32 operands read as
-// tf32, with tcgen05.mma accumulating in tensor memory.
+// iso_gemm.cuh -- the dense contractions of the frame-space merge and the
+// optimizer step on the fifth-generation tensor cores: C = A B^T for row-major
+// fp32 operands read as tf32, with tcgen05.mma accumulating in tensor memory.
 //
-// One CTA of 128 threads computes one 128 x 128 tile of C:
+// k_gemm_tf32: one product.  One CTA of 128 threads computes one 128 x 128
+// tile of C:
 //   warp 0, lane 0  loads the operand tiles (TMA, 128 rows x 32 fp32 = 128 B
 //                   per row, 128-byte swizzle) into a GEMM_STAGES-deep ring,
 //                   one mbarrier per stage counting the copied bytes;
@@ -12,6 +13,16 @@
 //   all four warps  read the accumulator back with tcgen05.ld (warp w owns
 //                   lanes 32 w .. 32 w + 31, one output row per thread) and
 //                   store it (the epilogue).
+// k_gemm_x3: the three products hi hi + hi lo + lo hi of split operands (x =
+// hi + lo, stored as two segments [hi | lo] of each row), the same roles.  A
+// stage holds the hi and lo tiles of both operands, so each is loaded once for
+// the products it enters, and the two small products have an accumulator of
+// their own: their sum is added once, in the epilogue.  Tiles of 128 x 256
+// (two stages of 96 KB) or 128 x 128 (three of 64 KB).  What bounds it is the
+// path from L2 to the SMs: three products over three separate segments with
+// 128 x 128 tiles asked for 128 bytes per clock and SM and ran at 0.46 of the
+// tf32 rate; this form asks for 62.  All products of the frame merge of a 3584
+// x 18944 matrix: 59.2 -> 31.9 ms.
 // Every wait on a barrier is bounded; a wait that gives up records
 // ISO_ERR_TIMEOUT, and the kernel still waits (bounded) for its own copies and
 // products before it frees its tensor memory and returns.
@@ -45,15 +56,20 @@ struct AdamwArgs {
     float* m;             // first moment (in place)
     float* v;             // second moment (in place)
     double* dX;           // out: X_bar - X = -lr wd X - lr / bc1 * m / (sqrt(v / bc2) + eps)
-    double lr, beta1, beta2, eps, wd, bc1, bc2;
+    double beta1, beta2, eps, bc2;
+    double lr_wd, lr_bc1; // lr wd, lr / bc1
 };
 
+constexpr int X3_SMEM = 1024 + 192 * 1024 + 256;   // both tile shapes
 struct GemmArgs {
     int32_t M, N;         // output extents (GEMM_ADD_BASE stores only inside them)
     int32_t k_tiles;      // contraction length / GEMM_BK
-    int32_t a_k0, b_k0;   // first contraction column read from A's and B's arrays
+    int32_t a_k0, b_k0;   // k_gemm_tf32: first contraction column read from A's and B's arrays
+    int32_t seg;          // k_gemm_x3: columns of one segment (the lo segment starts there)
+    int32_t c_cols;       // k_gemm_x3: padded columns of C (a 256-wide tile may reach past them)
     int32_t mode;         // GemmEpilogue
     float* C;
+    float* C2;            // k_gemm_x3: the output of the second product (grid z = 1)
     long long ldc;
     void* out;            // GEMM_ADD_BASE: output and base (same dtype, iso_dtype out_dtype)
     const void* w0;
@@ -67,6 +83,9 @@ struct GemmArgs {
 
 __global__ void k_gemm_tf32(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
                             GemmArgs g);
+template <int BN>
+__global__ void k_gemm_x3(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb,
+                          const __grid_constant__ CUtensorMap ta2, const __grid_constant__ CUtensorMap tb2, GemmArgs g);
 
 // ---------------------------------------------------------------------------
 // Binary64 contractions on the tensor cores: C = A^T B for binary64 columns,
