@@ -9,6 +9,8 @@
 // the same streaming apply pass as the other scopes.
 #include "iso_kernels.cuh"
 
+#include <type_traits>
+
 namespace iso {
 
 __device__ __forceinline__ long long k_of_density_b(double rho, long long n) {
@@ -139,92 +141,95 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
     const bool want_gamma = (P.op == ISO_OP_ISO) && (P.K == 1);
 
     // Full block of BLOCK_TPB x BFE entries in rows of a multiple of BFE: each
-    // thread holds BFE consecutive entries (block order) in registers -- their
-    // keys and one word of signs, from which each tau is rebuilt exactly -- and
-    // the threshold comes from a radix select over those registers, 11 bits
-    // per level down to the lowest bit any key has set (two levels for
-    // bf16-valued task vectors): four instructions per key and level, against
-    // two per key and bit for a descent bit by bit.  4096 x 14336 bf16 task
-    // vector at 5 %, outputs included: 235 -> 208 us.
+    // thread holds BFE consecutive entries (block order) of the task vector in
+    // registers, and the threshold comes from a radix select over those
+    // registers, 11 bits per level down to the lowest bit any key has set (two
+    // levels for bf16-valued task vectors).  Bound by issue: a descent bit by
+    // bit spent two instructions per key and bit (235 us for a 4096 x 14336
+    // bf16 task vector at 5 %, outputs included), keys and signs kept apart
+    // and rejoined for the outputs 208 us, this form 188 us.
     constexpr int BFE = BLOCK_MAX_ENTRIES / BLOCK_TPB;
     if (n == BLOCK_TPB * BFE && w % BFE == 0 && (d.cols % VEC) == 0 && (c0 % VEC) == 0 &&
         blockDim.x == BLOCK_TPB) {
         const int tq = threadIdx.x * BFE;
         const int rr = tq / (int)w, cc = tq - rr * (int)w;
         const long long ea = (r0 + rr) * d.cols + c0 + cc;     // tensor position of the thread's first entry
-        static_assert(BFE <= 32, "one sign word per thread");
         // theta_0 is needed only after the select: its lines go to L2 meanwhile
         if (P.fuse_block)
             for (int by = 0; by < BFE * (int)sizeof(BT); by += 64)
                 asm volatile("prefetch.global.L2 [%0];" :: "l"(static_cast<const char*>(d.base) + ea * (long long)sizeof(BT) + by));
-        uint32_t key[BFE];
-        uint32_t sgn = 0;
+        float v[BFE];
 #pragma unroll
         for (int g = 0; g < BFE / VEC; ++g) {
             float t8[VEC];
             TauSrc<XT, BT, CK>::load8(x, d.base, ea + g * VEC, d.numel, t8);
 #pragma unroll
-            for (int j = 0; j < VEC; ++j) {
-                const uint32_t b = __float_as_uint(t8[j]);
-                key[g * VEC + j] = b & 0x7FFFFFFFu;
-                sgn |= (b >> 31) << (g * VEC + j);
-            }
+            for (int j = 0; j < VEC; ++j) v[g * VEC + j] = t8[j];
         }
-        auto tau_of = [&](int j) -> float { return __uint_as_float(key[j] | (((sgn >> j) & 1u) << 31)); };
-        uint32_t kmax = 0, kor = 0;
+        for (int q = threadIdx.x; q < RADIX_BINS; q += BLOCK_TPB) s_hist[q] = 0;
+        if (threadIdx.x == 0) { s_or = 0; s_cutq = CUT_ALL; }
+        uint32_t kor = 0;
+        float bad0 = 0.0f, bad1 = 0.0f;                // 0 * tau: NaN once a tau is not finite
 #pragma unroll
-        for (int j = 0; j < BFE; ++j) { kmax = max(kmax, key[j]); kor |= key[j]; }
-        if (kmax >= KEY_INF) set_status(P.hdr, ISO_ERR_NONFINITE);
-        kor = __reduce_or_sync(0xFFFFFFFFu, kor);
-        if (threadIdx.x == 0) s_or = 0;
+        for (int j = 0; j < BFE; j += 2) {
+            kor |= __float_as_uint(v[j]) | __float_as_uint(v[j + 1]);
+            fma_rn2(bad0, bad1, v[j], v[j + 1], 0.0f, 0.0f, bad0, bad1);
+        }
+        if (!(bad0 + bad1 == 0.0f)) set_status(P.hdr, ISO_ERR_NONFINITE);
+        kor = __reduce_or_sync(0xFFFFFFFFu, kor & KEY_MAX);
         __syncthreads();
         if ((threadIdx.x & 31) == 0 && kor) atomicOr(&s_or, kor);
+        // first level: the top 11 bits of every key
+        constexpr int SH1 = 31 - RADIX_BITS;
+#pragma unroll
+        for (int j = 0; j < BFE; ++j) atomicAdd(&s_hist[(__float_as_uint(v[j]) >> SH1) & (RADIX_BINS - 1)], 1u);
         __syncthreads();
         const int low = s_or ? __ffs(s_or) - 1 : 31;
-        uint32_t prefix = 0;
         long long rank = k;
-        for (int pshift = 31;;) {
+        block_find_from_top_b(s_hist, RADIX_BINS, rank, s_scan, &s_bin, &s_above);
+        rank -= s_above;
+        uint32_t prefix = (uint32_t)s_bin;
+        int pshift = SH1;
+        while (pshift > low) {
+            __syncthreads();
             const int shift = max(pshift > RADIX_BITS ? pshift - RADIX_BITS : 0, low);
-            const int nb = 1 << (pshift - shift);
-            for (int q = threadIdx.x; q < nb; q += BLOCK_TPB) s_hist[q] = 0;
+            const uint32_t nm = (1u << (pshift - shift)) - 1u;
+            for (int q = threadIdx.x; q <= (int)nm; q += BLOCK_TPB) s_hist[q] = 0;
             __syncthreads();
+            const uint32_t want = prefix << pshift, mask = KEY_MAX & ~((1u << pshift) - 1u);
 #pragma unroll
-            for (int j = 0; j < BFE; ++j)
-                if ((key[j] >> pshift) == prefix) atomicAdd(&s_hist[(key[j] >> shift) & (uint32_t)(nb - 1)], 1u);
+            for (int j = 0; j < BFE; ++j) {
+                const uint32_t b = __float_as_uint(v[j]);
+                if ((b & mask) == want) atomicAdd(&s_hist[(b >> shift) & nm], 1u);
+            }
             __syncthreads();
-            block_find_from_top_b(s_hist, nb, rank, s_scan, &s_bin, &s_above);
+            block_find_from_top_b(s_hist, (int)nm + 1, rank, s_scan, &s_bin, &s_above);
             rank -= s_above;
             prefix = (prefix << (pshift - shift)) | (uint32_t)s_bin;
-            __syncthreads();
-            if (shift == low) break;
             pshift = shift;
         }
-        prefix <<= low;
-        const uint32_t tk = prefix;
+        const uint32_t tk = prefix << pshift;
+        const float tf = __uint_as_float(tk);
         uint32_t above = 0, ties = 0;
 #pragma unroll
-        for (int j = 0; j < BFE; ++j) { above += key[j] > tk; ties += key[j] == tk; }
+        for (int j = 0; j < BFE; ++j) { above += fabsf(v[j]) > tf; ties += fabsf(v[j]) == tf; }
         uint32_t tot_ties;
         const uint32_t ties_before = block_excl_scan(ties, s_scan32, &tot_ties);
         const uint32_t tot_above = block_sum(above, s_scan32);
         const long long need = k - (long long)tot_above;
-        if (threadIdx.x == 0) s_cutq = CUT_ALL;
-        __syncthreads();
         if (need < (long long)tot_ties && (long long)ties_before < need && need <= (long long)(ties_before + ties)) {
             uint32_t acc = ties_before;
 #pragma unroll
             for (int j = 0; j < BFE; ++j)
-                if (key[j] == tk && (long long)(++acc) == need) s_cutq = ea + j + 1;
+                if (fabsf(v[j]) == tf && (long long)(++acc) == need) s_cutq = ea + j + 1;
         }
         double g = 0.0;
         if (want_gamma) {
             // squares of the entries above t as binary32 two-sum pairs, then binary64 over the block
             float sg = 0.0f, eg = 0.0f;
 #pragma unroll
-            for (int j = 0; j < BFE; ++j) {
-                const float f = __uint_as_float(key[j]);          // |tau|: the same square
-                if (key[j] > tk) two_sum_add(sg, eg, __fmul_rn(f, f));
-            }
+            for (int j = 0; j < BFE; ++j)
+                if (fabsf(v[j]) > tf) two_sum_add(sg, eg, __fmul_rn(v[j], v[j]));
             g = block_sum((double)sg + (double)eg, s_dred);
         }
         __syncthreads();
@@ -240,22 +245,28 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
             stats(tk, k, tot_above, tot_ties, need);
         }
         if (P.fuse_block) {
-            // ties are kept at the thread's first `kt` entries
+            // ties are kept at the thread's first kt entries: |tau| above this
+            // bound (below t's magnitude, or t's own) is kept
             const long long before = cut - ea;
             const int kt = before <= 0 ? 0 : (before >= BFE ? BFE : (int)before);
+            const float tl = tk ? __uint_as_float(tk - 1) : -1.0f;
+            auto put = [&](auto same, float bound) {
 #pragma unroll
-            for (int gq = 0; gq < BFE / VEC; ++gq) {
-                const long long e = ea + gq * VEC;
-                float th0[VEC], o[VEC];
-                load8_tail<BT>(d.base, e, d.numel, th0);
+                for (int gq = 0; gq < BFE / VEC; ++gq) {
+                    const long long e = ea + gq * VEC;
+                    float th0[VEC], o[VEC];
+                    load8_tail<BT>(d.base, e, d.numel, th0);
 #pragma unroll
-                for (int j = 0; j < VEC; ++j) {
-                    const uint32_t kk = key[gq * VEC + j];
-                    const bool kept = (int)kk > (gq * VEC + j < kt ? (int)tk - 1 : (int)tk);
-                    o[j] = kept ? out_of(th0[j], tau_of(gq * VEC + j), P.lambda) : th0[j];
+                    for (int j = 0; j < VEC; ++j) {
+                        const int q = gq * VEC + j;
+                        const float bd = decltype(same)::value ? bound : (q < kt ? tl : tf);
+                        o[j] = fabsf(v[q]) > bd ? out_of(th0[j], v[q], P.lambda) : th0[j];
+                    }
+                    store8(d.out, e, d.numel, o, obf);
                 }
-                store8(d.out, e, d.numel, o, obf);
-            }
+            };
+            if (kt == 0 || kt == BFE) put(std::integral_constant<bool, true>{}, kt ? tl : tf);
+            else put(std::integral_constant<bool, false>{}, 0.0f);
         }
         return;
     }
