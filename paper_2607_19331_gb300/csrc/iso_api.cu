@@ -442,7 +442,7 @@ int upload(cudaStream_t s, char* dst_dev, const std::vector<char>& blob) {
         ch.pad = 0;
         std::memset(ch.data, 0, sizeof(ch.data));
         std::memcpy(ch.data, blob.data() + off, nb);
-        ISO_TRY(launch(KD_UPLOAD, s, [&] { k_upload<<<1, 256, 0, s>>>(ch); }));
+        ISO_TRY(launch(KD_UPLOAD, s, [&] { pdl_launch(k_upload, 1, 256, 0, s, ch); }));
         off += nb;
     }
     return ISO_OK;
@@ -584,49 +584,49 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
     int rc = ISO_OK;
     if (!select && !c.mask_only && (c.op == ISO_OP_TIES || c.op == ISO_OP_ISO) && P.st_units && KU > 0)
         ISO_TRY(launch(KD_INIT, s, [&] {
-            k_units_off<<<(KU + 255) / 256, 256, 0, s>>>(P.st_units, P.st_units_stride, P.st_unit_base, L.n_units, K);
+            pdl_launch(k_units_off, (KU + 255) / 256, 256, 0, s, P.st_units, P.st_units_stride, P.st_unit_base, L.n_units, K);
         }));
     if (select && c.topk.scope != ISO_SCOPE_BLOCK) {
-        ISO_TRY(launch(KD_INIT, s, [&] { k_init_units<<<(KU + 255) / 256, 256, 0, s>>>(P, L.global_n); }));
+        ISO_TRY(launch(KD_INIT, s, [&] { pdl_launch(k_init_units, (KU + 255) / 256, 256, 0, s, P, L.global_n); }));
         rc = dispatch_src(c.xdt, c.bdt, c.ckpt, [&](auto* xt, auto* bt, auto ck) -> int {
             using XT = std::remove_pointer_t<decltype(xt)>;
             using BT = std::remove_pointer_t<decltype(bt)>;
             constexpr bool CK = decltype(ck)::value;
             const int smem = (SAMPLE_MAX + SAMPLE_LIST + RADIX_BINS) * 4;
             ISO_TRY(smem_optin(k_sample<XT, BT, CK>, smem));
-            ISO_TRY(launch(KD_SAMPLE, s, [&] { k_sample<XT, BT, CK><<<KU, SAMPLE_TPB, smem, s>>>(P); }));
+            ISO_TRY(launch(KD_SAMPLE, s, [&] { pdl_launch(k_sample<XT, BT, CK>, KU, SAMPLE_TPB, smem, s, P); }));
             if (fused)
-                ISO_TRY(launch(KD_SAMPLE, s, [&] { k_csample<XT, BT, CK><<<KU * CS_SPLIT, CS_TPB, 0, s>>>(P); }));
+                ISO_TRY(launch(KD_SAMPLE, s, [&] { pdl_launch(k_csample<XT, BT, CK>, KU * CS_SPLIT, CS_TPB, 0, s, P); }));
             if (fused) {
                 if (CK) {
                     ISO_TRY(smem_optin(k_count_apply<true>, FUSED_SMEM));
-                    ISO_TRY(launch(KD_COUNT, s, [&] { k_count_apply<true><<<sms * FUSED_GRID_PER_SM, TPB, FUSED_SMEM, s>>>(P); }));
+                    ISO_TRY(launch(KD_COUNT, s, [&] { pdl_launch(k_count_apply<true>, sms * FUSED_GRID_PER_SM, TPB, FUSED_SMEM, s, P); }));
                 } else {
                     ISO_TRY(smem_optin(k_count_apply<false>, FUSED_SMEM));
-                    ISO_TRY(launch(KD_COUNT, s, [&] { k_count_apply<false><<<sms * FUSED_GRID_PER_SM, TPB, FUSED_SMEM, s>>>(P); }));
+                    ISO_TRY(launch(KD_COUNT, s, [&] { pdl_launch(k_count_apply<false>, sms * FUSED_GRID_PER_SM, TPB, FUSED_SMEM, s, P); }));
                 }
             } else {
                 if (c.ccv) {
                     ISO_TRY(smem_optin(k_count<XT, BT, CK, true>, COUNT_EMIT_SMEM));
                     ISO_TRY(launch(KD_COUNT, s, [&] {
-                        k_count<XT, BT, CK, true><<<sms * COUNT_GRID_PER_SM, TPB, COUNT_EMIT_SMEM, s>>>(P);
+                        pdl_launch(k_count<XT, BT, CK, true>, sms * COUNT_GRID_PER_SM, TPB, COUNT_EMIT_SMEM, s, P);
                     }));
                 }
                 else
-                    ISO_TRY(launch(KD_COUNT, s, [&] { k_count<XT, BT, CK, false><<<sms * COUNT_GRID_PER_SM, TPB, 0, s>>>(P); }));
+                    ISO_TRY(launch(KD_COUNT, s, [&] { pdl_launch(k_count<XT, BT, CK, false>, sms * COUNT_GRID_PER_SM, TPB, 0, s, P); }));
             }
-            ISO_TRY(launch(KD_DECIDE, s, [&] { k_decide<<<(KU + 255) / 256, 256, 0, s>>>(P); }));
+            ISO_TRY(launch(KD_DECIDE, s, [&] { pdl_launch(k_decide, (KU + 255) / 256, 256, 0, s, P); }));
             if (c.topk.scope == ISO_SCOPE_GLOBAL) ISO_TRY(smem_optin(k_radix_flat, RADIX_FLAT_SMEM));
             for (int level = 0; level < 3; ++level) {
                 if (c.topk.scope == ISO_SCOPE_GLOBAL)
-                    ISO_TRY(launch(KD_RADIX_FLAT, s, [&] { k_radix_flat<<<sms * 2, TPB, RADIX_FLAT_SMEM, s>>>(P); }));
-                ISO_TRY(launch(KD_RADIX_HIST, s, [&] { k_radix_hist<XT, BT, CK><<<pgrid, TPB, 0, s>>>(P); }));
-                ISO_TRY(launch(KD_RADIX_PICK, s, [&] { k_radix_pick<<<KU, TPB, 0, s>>>(P); }));
+                    ISO_TRY(launch(KD_RADIX_FLAT, s, [&] { pdl_launch(k_radix_flat, sms * 2, TPB, RADIX_FLAT_SMEM, s, P); }));
+                ISO_TRY(launch(KD_RADIX_HIST, s, [&] { pdl_launch(k_radix_hist<XT, BT, CK>, pgrid, TPB, 0, s, P); }));
+                ISO_TRY(launch(KD_RADIX_PICK, s, [&] { pdl_launch(k_radix_pick, KU, TPB, 0, s, P); }));
             }
-            ISO_TRY(launch(KD_TIE, s, [&] { k_tie<XT, BT, CK><<<pgrid, TPB, 0, s>>>(P); }));
+            ISO_TRY(launch(KD_TIE, s, [&] { pdl_launch(k_tie<XT, BT, CK>, pgrid, TPB, 0, s, P); }));
             if (c.topk.scope == ISO_SCOPE_GLOBAL)
-                ISO_TRY(launch(KD_CUT_PART, s, [&] { k_cut_part<<<pgrid, TPB, 0, s>>>(P); }));
-            ISO_TRY(launch(KD_CUT, s, [&] { k_cut<XT, BT, CK><<<KU, CUT_TPB, 0, s>>>(P); }));
+                ISO_TRY(launch(KD_CUT_PART, s, [&] { pdl_launch(k_cut_part, pgrid, TPB, 0, s, P); }));
+            ISO_TRY(launch(KD_CUT, s, [&] { pdl_launch(k_cut<XT, BT, CK>, KU, CUT_TPB, 0, s, P); }));
             return ISO_OK;
         });
         ISO_TRY(rc);
@@ -638,7 +638,7 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
             const int smem = BLOCK_KEYS_WORDS * 4;
             ISO_TRY(smem_optin(k_block_select<XT, BT, CK>, smem));
             if (KU > 0)
-                ISO_TRY(launch(KD_BLOCK_SELECT, s, [&] { k_block_select<XT, BT, CK><<<KU, BLOCK_TPB, smem, s>>>(P); }));
+                ISO_TRY(launch(KD_BLOCK_SELECT, s, [&] { pdl_launch(k_block_select<XT, BT, CK>, KU, BLOCK_TPB, smem, s, P); }));
             return ISO_OK;
         });
         ISO_TRY(rc);
@@ -647,28 +647,28 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
     if (c.mask_only) {
         uint32_t* const* mdev = reinterpret_cast<uint32_t* const*>(ws + L.mptr);
         if (c.xdt == ISO_BF16)
-            ISO_TRY(launch(KD_MASK, s, [&] { k_mask<__nv_bfloat16><<<pgrid, TPB, 0, s>>>(P, mdev); }));
+            ISO_TRY(launch(KD_MASK, s, [&] { pdl_launch(k_mask<__nv_bfloat16>, pgrid, TPB, 0, s, P, mdev); }));
         else
-            ISO_TRY(launch(KD_MASK, s, [&] { k_mask<float><<<pgrid, TPB, 0, s>>>(P, mdev); }));
+            ISO_TRY(launch(KD_MASK, s, [&] { pdl_launch(k_mask<float>, pgrid, TPB, 0, s, P, mdev); }));
         return ISO_OK;
     }
 
     if (fused) {
         // exact coefficients and repair flags, then the kept band entries, then
         // the full exact apply of any flagged tensor
-        ISO_TRY(launch(KD_SOLVE, s, [&] { k_solve<<<(T + 127) / 128, 128, 0, s>>>(P, gram_mode); }));
-        ISO_TRY(launch(KD_REPAIR, s, [&] { k_fix_plan<<<1, 1024, 0, s>>>(P); }));
+        ISO_TRY(launch(KD_SOLVE, s, [&] { pdl_launch(k_solve, (T + 127) / 128, 128, 0, s, P, gram_mode); }));
+        ISO_TRY(launch(KD_REPAIR, s, [&] { pdl_launch(k_fix_plan, 1, 1024, 0, s, P); }));
         int ggrid = 0, fgrid = 0;
         if (c.ckpt) {
             ISO_TRY(resident_grid(k_patch<true>, TPB, 0, sms, &ggrid));
             ISO_TRY(resident_grid(k_fix<true>, TPB, 0, sms, &fgrid));
-            ISO_TRY(launch(KD_PATCH, s, [&] { k_patch<true><<<ggrid, TPB, 0, s>>>(P); }));
-            ISO_TRY(launch(KD_REPAIR, s, [&] { k_fix<true><<<fgrid, TPB, 0, s>>>(P); }));
+            ISO_TRY(launch(KD_PATCH, s, [&] { pdl_launch(k_patch<true>, ggrid, TPB, 0, s, P); }));
+            ISO_TRY(launch(KD_REPAIR, s, [&] { pdl_launch(k_fix<true>, fgrid, TPB, 0, s, P); }));
         } else {
             ISO_TRY(resident_grid(k_patch<false>, TPB, 0, sms, &ggrid));
             ISO_TRY(resident_grid(k_fix<false>, TPB, 0, sms, &fgrid));
-            ISO_TRY(launch(KD_PATCH, s, [&] { k_patch<false><<<ggrid, TPB, 0, s>>>(P); }));
-            ISO_TRY(launch(KD_REPAIR, s, [&] { k_fix<false><<<fgrid, TPB, 0, s>>>(P); }));
+            ISO_TRY(launch(KD_PATCH, s, [&] { pdl_launch(k_patch<false>, ggrid, TPB, 0, s, P); }));
+            ISO_TRY(launch(KD_REPAIR, s, [&] { pdl_launch(k_fix<false>, fgrid, TPB, 0, s, P); }));
         }
         return ISO_OK;
     }
@@ -684,13 +684,13 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
                     constexpr int KC = decltype(kc)::value;
                     const int smem = gram_smem_bytes<XT, BT, CK, KC>();
                     ISO_TRY(smem_optin(k_gramk<XT, BT, CK, KC>, smem));
-                    return launch(KD_GRAM, s, [&] { k_gramk<XT, BT, CK, KC><<<sms * MERGE_BLOCKS_PER_SM, TPB, smem, s>>>(P); });
+                    return launch(KD_GRAM, s, [&] { pdl_launch(k_gramk<XT, BT, CK, KC>, sms * MERGE_BLOCKS_PER_SM, TPB, smem, s, P); });
                 };
                 auto gram_c = [&](auto kc) {
                     constexpr int KC = decltype(kc)::value;
                     const int cs = compact_smem_bytes<BT, KC>();
                     ISO_TRY(smem_optin(k_gramk_c<XT, BT, CK, KC>, cs));
-                    return launch(KD_GRAM, s, [&] { k_gramk_c<XT, BT, CK, KC><<<sms * 2, TPB, cs, s>>>(P); });
+                    return launch(KD_GRAM, s, [&] { pdl_launch(k_gramk_c<XT, BT, CK, KC>, sms * 2, TPB, cs, s, P); });
                 };
                 if (c.ccv) {
                     if (K == 2) ISO_TRY(gram_c(std::integral_constant<int, 2>{}));
@@ -703,13 +703,13 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
                 else if (K == 4) ISO_TRY(gram(std::integral_constant<int, 4>{}));
                 else ISO_TRY(gram(std::integral_constant<int, 8>{}));
             }
-            ISO_TRY(launch(KD_SOLVE, s, [&] { k_solve<<<(T + 127) / 128, 128, 0, s>>>(P, gram_mode); }));
+            ISO_TRY(launch(KD_SOLVE, s, [&] { pdl_launch(k_solve, (T + 127) / 128, 128, 0, s, P, gram_mode); }));
         }
         auto merge_op = [&](auto kc, auto opf) {
             constexpr int KC = decltype(kc)::value, OPF = decltype(opf)::value;
             const int smem = merge_smem_bytes<XT, BT, KC>();
             ISO_TRY(smem_optin(k_merge<XT, BT, CK, KC, OPF>, smem));
-            return launch(KD_APPLY, s, [&] { k_merge<XT, BT, CK, KC, OPF><<<sms * MERGE_BLOCKS_PER_SM, TPB, smem, s>>>(P); });
+            return launch(KD_APPLY, s, [&] { pdl_launch(k_merge<XT, BT, CK, KC, OPF>, sms * MERGE_BLOCKS_PER_SM, TPB, smem, s, P); });
         };
         auto merge = [&](auto kc) -> int {
             if (c.op == ISO_OP_TIES) return merge_op(kc, std::integral_constant<int, OPF_TIES>{});
@@ -722,10 +722,10 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
             const int cs = compact_smem_bytes<BT, KC>();
             if (c.op == ISO_OP_TIES) {
                 ISO_TRY(smem_optin(k_merge_c<XT, BT, CK, KC, OPF_TIES>, cs));
-                return launch(KD_APPLY, s, [&] { k_merge_c<XT, BT, CK, KC, OPF_TIES><<<sms * 2, TPB, cs, s>>>(P); });
+                return launch(KD_APPLY, s, [&] { pdl_launch(k_merge_c<XT, BT, CK, KC, OPF_TIES>, sms * 2, TPB, cs, s, P); });
             }
             ISO_TRY(smem_optin(k_merge_c<XT, BT, CK, KC, OPF_ISO>, cs));
-            return launch(KD_APPLY, s, [&] { k_merge_c<XT, BT, CK, KC, OPF_ISO><<<sms * 2, TPB, cs, s>>>(P); });
+            return launch(KD_APPLY, s, [&] { pdl_launch(k_merge_c<XT, BT, CK, KC, OPF_ISO>, sms * 2, TPB, cs, s, P); });
         };
         if (K == 1 && fuse_block) return ISO_OK;
         // RAM with one expert: the merge pass (its activity test lives there)
@@ -736,7 +736,7 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
         }
         else if (K == 1 && c.op == ISO_OP_RAM)
             ISO_TRY(merge_op(std::integral_constant<int, 1>{}, std::integral_constant<int, OPF_RAM>{}));
-        else if (K == 1) ISO_TRY(launch(KD_APPLY, s, [&] { k_apply<XT, BT, CK, 1><<<pgrid, TPB, 0, s>>>(P); }));
+        else if (K == 1) ISO_TRY(launch(KD_APPLY, s, [&] { pdl_launch(k_apply<XT, BT, CK, 1>, pgrid, TPB, 0, s, P); }));
         else if (K == 2) ISO_TRY(merge(std::integral_constant<int, 2>{}));
         else if (K == 3) ISO_TRY(merge(std::integral_constant<int, 3>{}));
         else if (K == 4) ISO_TRY(merge(std::integral_constant<int, 4>{}));
@@ -784,7 +784,7 @@ int run_call(Call& c, void* workspace, size_t ws_bytes, const iso_merge_stats* s
     }
     if (st && st->status) {
         if (c.n > 0)
-            ISO_TRY(launch(KD_STATUS, s, [&] { k_status<<<1, 32, 0, s>>>(reinterpret_cast<const Header*>(ws), st->status); }));
+            ISO_TRY(launch(KD_STATUS, s, [&] { pdl_launch(k_status, 1, 32, 0, s, reinterpret_cast<const Header*>(ws), st->status); }));
         else
             ISO_TRY(launch(KD_MEMSET, s, [&] { cudaMemsetAsync(st->status, 0, 4, s); }));
     }
@@ -1187,6 +1187,7 @@ namespace iso {
 namespace {
 
 __global__ void k_status_first(const int32_t* st, int n, int32_t* out) {
+    pdl_enter();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     int32_t v = ISO_OK;
     for (int g = 0; g < n && v == ISO_OK; ++g) v = st[g];
@@ -1425,7 +1426,7 @@ int32_t iso_update_host(const iso_tensor* theta_0, const iso_tensor* update, int
     for (int b = 0; b < 2 && b < G; ++b)
         if (cudaStreamWaitEvent(comp, ev[FREED][(G - 1 - b) & 1], 0) != cudaSuccess) return ISO_ERR_CUDA;
     if (stats && stats->status)
-        return launch(KD_STATUS, comp, [&] { k_status_first<<<1, 32, 0, comp>>>(gstat, G, stats->status); });
+        return launch(KD_STATUS, comp, [&] { pdl_launch(k_status_first, 1, 32, 0, comp, gstat, G, stats->status); });
     return ISO_OK;
 }
 

@@ -95,6 +95,7 @@ __device__ __forceinline__ SelParam block_param(const Plan& P, const TensorDesc&
 
 template <typename XT, typename BT, bool CK, int KC>
 __global__ void __launch_bounds__(TPB) k_apply(Plan P) {
+    pdl_enter();
     static_assert(KC == 1, "K >= 2 merges run in k_merge");
     const int K = 1;
     const int lane = threadIdx.x & 31;
@@ -201,6 +202,7 @@ __global__ void __launch_bounds__(TPB) k_apply(Plan P) {
 // retention coefficients: one thread per tensor
 // ---------------------------------------------------------------------------
 __global__ void k_solve(Plan P, int gram_mode) {
+    pdl_enter();
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= P.n_tensors) return;
     const int K = P.K;
@@ -248,6 +250,7 @@ __global__ void k_solve(Plan P, int gram_mode) {
 // ---------------------------------------------------------------------------
 template <typename XT>
 __global__ void __launch_bounds__(TPB) k_mask(Plan P, uint32_t* const* mptr) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const long long W = (long long)gridDim.x * WPB;
     for (long long g = (long long)blockIdx.x * WPB + (threadIdx.x >> 5); g < P.n_tiles; g += W) {
@@ -295,6 +298,7 @@ __global__ void __launch_bounds__(TPB) k_mask(Plan P, uint32_t* const* mptr) {
 }
 
 __global__ void k_status(const Header* h, int32_t* out) {
+    pdl_enter();
     if (threadIdx.x == 0 && blockIdx.x == 0) *out = h->status;
 }
 
@@ -303,6 +307,7 @@ __global__ void k_status(const Header* h, int32_t* out) {
 // selection pass runs for such a group, so their records are written here,
 // the same record the selection writes for an untrimmed unit.
 __global__ void k_units_off(iso_unit_stats* st, long long stride, long long base, int n_units, int K) {
+    pdl_enter();
     const long long n = (long long)K * n_units;
     for (long long idx = blockIdx.x * (long long)blockDim.x + threadIdx.x; idx < n;
          idx += (long long)gridDim.x * blockDim.x) {
@@ -319,6 +324,7 @@ __global__ void k_units_off(iso_unit_stats* st, long long stride, long long base
 }
 
 __global__ void k_upload(UploadChunk c) {
+    pdl_enter();
     uint4* dst = reinterpret_cast<uint4*>(c.dst);
     for (uint32_t q = threadIdx.x; q < c.nbytes / 16; q += blockDim.x) dst[q] = c.data[q];
 }

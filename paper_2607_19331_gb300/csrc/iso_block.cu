@@ -46,6 +46,7 @@ __device__ __forceinline__ int kpad(int q) { return q + (q >> 5); }
 
 template <typename XT, typename BT, bool CK>
 __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(Plan P) {
+    pdl_enter();
     extern __shared__ __align__(16) uint32_t s_keys[];      // kpad(BLOCK_MAX_ENTRIES)
     __shared__ uint32_t s_hist[RADIX_BINS];
     __shared__ long long s_scan[33];

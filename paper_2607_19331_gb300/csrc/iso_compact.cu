@@ -153,6 +153,7 @@ __device__ __forceinline__ void compact_step(const CompactParams<KC>& cp, const 
 
 template <typename XT, typename BT, bool CK, int KC, int OPF>
 __global__ void __launch_bounds__(TPB, 2) k_merge_c(Plan P) {
+    pdl_enter();
     constexpr int E = 4, SPT = TILE / (32 * E);
     const int K = P.K;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -223,6 +224,7 @@ __global__ void __launch_bounds__(TPB, 2) k_merge_c(Plan P) {
 // warp sums per tile, binary32 two-sum pairs per tensor, one atomic per pair.
 template <typename XT, typename BT, bool CK, int KC>
 __global__ void __launch_bounds__(TPB, 2) k_gramk_c(Plan P) {
+    pdl_enter();
     constexpr int E = 4, SPT = TILE / (32 * E);
     constexpr int NP = KC * (KC + 1) / 2;
     static_assert(NP <= 64, "two pair sums per lane");

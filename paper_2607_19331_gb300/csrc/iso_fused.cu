@@ -86,6 +86,7 @@ __device__ __forceinline__ void fused_fast_tile(const unsigned char* sx, const u
 // arrived on without transactions and the tile is read from global memory.
 template <bool CK>
 __global__ void __launch_bounds__(TPB, FUSED_BLOCKS_PER_SM) k_count_apply(Plan P) {
+    pdl_enter();
     extern __shared__ __align__(128) unsigned char s_ring[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     unsigned char* const ring = s_ring + (size_t)warp * FUSED_STAGES * FUSED_STAGE_BYTES;
@@ -438,6 +439,7 @@ __global__ void __launch_bounds__(TPB, FUSED_BLOCKS_PER_SM) k_count_apply(Plan P
 // skipped.
 template <bool CK>
 __global__ void __launch_bounds__(TPB) k_patch(Plan P) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const uint32_t W = gridDim.x * WPB;
     const uint32_t wid = blockIdx.x * WPB + (threadIdx.x >> 5);
@@ -501,6 +503,7 @@ __global__ void __launch_bounds__(TPB) k_patch(Plan P) {
 // units of its tile counts, so that k_fix can spread all ranges evenly over
 // the GPU.  One block; the total goes to the header.
 __global__ void __launch_bounds__(1024) k_fix_plan(Plan P) {
+    pdl_enter();
     __shared__ long long s_scan[33];
     long long base = 0;
     for (int t0 = 0; t0 < P.n_tensors; t0 += blockDim.x) {
@@ -561,6 +564,7 @@ struct FixRange {
 
 template <bool CK>
 __global__ void __launch_bounds__(TPB) k_fix(Plan P) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const long long total = *(volatile int32_t*)&P.hdr->fix_tiles;
     const long long W = (long long)gridDim.x * WPB;

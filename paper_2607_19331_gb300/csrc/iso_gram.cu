@@ -15,6 +15,7 @@ namespace iso {
 // see k_merge for what changed.
 template <typename XT, typename BT, bool CK, int KC>
 __global__ void __launch_bounds__(TPB, 2) k_gramk(Plan P) {
+    pdl_enter();
     using G = ChunkGeom<XT, BT, KC, CK>;
     constexpr int E = G::E;
     constexpr int NP = KC * (KC + 1) / 2;

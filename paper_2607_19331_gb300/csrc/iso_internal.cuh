@@ -225,6 +225,35 @@ struct Plan {
     double* st_coef;
 };
 
+// First statement of every kernel launched with pdl_launch: wait until the
+// stream's earlier work is complete and visible, then let the next kernel be
+// set up while this one runs.  Every kernel of a chain has to wait (also one
+// that returns at once), since the next kernel's wait covers only this one.
+__device__ __forceinline__ void pdl_enter() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Launch with programmatic stream serialization: the kernel's set-up overlaps
+// the end of the stream's previous kernel (its pdl_enter holds it back until
+// that one is complete).  A call is a chain of a dozen short kernels: two
+// 1M-entry units, TIES, 104 -> 80 us; one decoder layer's update 199 -> 160 us;
+// a mask 323 -> 291 us.
+template <typename... KArgs, typename... Args>
+inline cudaError_t pdl_launch(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+
 // ---------------------------------------------------------------------------
 // element access
 // ---------------------------------------------------------------------------

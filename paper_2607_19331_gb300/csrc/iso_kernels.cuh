@@ -7,8 +7,6 @@
 
 namespace iso {
 
-
-
 // the streaming passes over (expert, tile) items deal them round-robin over
 // the warps (1) or give each warp one contiguous range (0).  Contiguous ranges
 // measured faster for these passes on the 7B K = 8 merges (round-robin: every

@@ -121,6 +121,7 @@ __device__ __forceinline__ void merge_pair(const float (&t0)[KC], const float (&
 // TIES: 5.03 -> 4.60 ms (5.5 TB/s).
 template <typename XT, typename BT, bool CK, int KC, int OPF>
 __global__ void __launch_bounds__(TPB, 2) k_merge(Plan P) {
+    pdl_enter();
     using G = ChunkGeom<XT, BT, KC, true>;
     constexpr int E = G::E;
     extern __shared__ __align__(128) unsigned char s_ring[];

@@ -31,6 +31,7 @@ namespace iso {
 // unit table
 // ---------------------------------------------------------------------------
 __global__ void k_init_units(Plan P, long long global_n) {
+    pdl_enter();
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= P.K * P.n_units) return;
     const int i = idx / P.n_units, u = idx % P.n_units;
@@ -260,6 +261,7 @@ __device__ __forceinline__ int tensor_of_upos(const TensorDesc* tens, int n_tens
 
 template <typename XT, typename BT, bool CKPT>
 __global__ void __launch_bounds__(SAMPLE_TPB, 1) k_sample(Plan P) {
+    pdl_enter();
     extern __shared__ __align__(16) uint32_t s_keys[];
     uint32_t* s_list = s_keys + SAMPLE_MAX;          // SAMPLE_LIST keys
     uint32_t* s_hist = s_list + SAMPLE_LIST;         // RADIX_BINS counters
@@ -463,6 +465,7 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 1) k_sample(Plan P) {
 // interpolates inside it.
 template <typename XT, typename BT, bool CKPT>
 __global__ void __launch_bounds__(CS_TPB, 4) k_csample(Plan P) {
+    pdl_enter();
     const int u = blockIdx.x / CS_SPLIT, part = blockIdx.x % CS_SPLIT;
     Unit& U = P.units[u];
     // uniform over the unit's blocks: all of them return here, or none
@@ -633,6 +636,7 @@ __device__ __forceinline__ bool count_run_at(const Plan& P, uint32_t it, uint32_
 // and writes the row's candidates in position order.
 template <typename XT, typename BT, bool CK, bool EMIT>
 __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
+    pdl_enter();
     __shared__ uint32_t s_band[WPB][TILE + 32];
     extern __shared__ float s_vst[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -933,6 +937,7 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
 // decide: where is rank k relative to the band?
 // ---------------------------------------------------------------------------
 __global__ void k_decide(Plan P) {
+    pdl_enter();
     int idx = blockIdx.x * blockDim.x + threadIdx.x;
     if (idx >= P.K * P.n_units) return;
     Unit& U = P.units[idx];
@@ -1033,6 +1038,7 @@ __device__ __forceinline__ bool radix_flat(const Plan& P, const Unit& U) {
 // another key was seen: what the pick needs to tell a single-key bin.  RADIX_FLAT_SMEM bytes of dynamic shared
 // memory: WPB count arrays, the first keys, the flags.
 __global__ void __launch_bounds__(TPB) k_radix_flat(Plan P) {
+    pdl_enter();
     extern __shared__ uint32_t fsm[];
     if (*(volatile int32_t*)&P.hdr->n_radix == 0) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1110,17 +1116,19 @@ __global__ void __launch_bounds__(TPB) k_radix_flat(Plan P) {
 
 template <typename XT, typename BT, bool CK>
 __global__ void __launch_bounds__(TPB, 4) k_radix_hist(Plan P) {
+    pdl_enter();
     __shared__ uint32_t s_hist[RADIX_BINS];
     __shared__ uint32_t s_key[RADIX_BINS];     // the bin's first key
     __shared__ uint32_t s_mixed[RADIX_BINS];   // another key was seen
     if (*(volatile int32_t*)&P.hdr->n_radix == 0) return;
-    for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) { s_hist[b] = 0; s_key[b] = KEY_NONE; s_mixed[b] = 0; }
-    __syncthreads();
     const long long items = (long long)P.K * P.n_tiles;
     const long long per = (items + gridDim.x - 1) / gridDim.x;
     const long long beg = blockIdx.x * per;
     const long long end = (beg + per < items) ? beg + per : items;
+    if (beg >= items) return;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int b = threadIdx.x; b < RADIX_BINS; b += blockDim.x) { s_hist[b] = 0; s_key[b] = KEY_NONE; s_mixed[b] = 0; }
+    __syncthreads();
     long long it = beg;
     while (it < end) {
         Cursor c;
@@ -1213,6 +1221,7 @@ __global__ void __launch_bounds__(TPB, 4) k_radix_hist(Plan P) {
 }
 
 __global__ void __launch_bounds__(TPB) k_radix_pick(Plan P) {
+    pdl_enter();
     __shared__ long long s_scan[33];
     __shared__ int s_bin;
     __shared__ long long s_above;
@@ -1256,6 +1265,7 @@ __global__ void __launch_bounds__(TPB) k_radix_pick(Plan P) {
 // ---------------------------------------------------------------------------
 template <typename XT, typename BT, bool CK>
 __global__ void __launch_bounds__(TPB) k_tie(Plan P) {
+    pdl_enter();
     if (*(volatile int32_t*)&P.hdr->n_tknown == 0) return;
     const long long items = (long long)P.K * P.n_tiles;
     const long long per = (items + gridDim.x - 1) / gridDim.x;
@@ -1366,6 +1376,7 @@ __device__ __forceinline__ bool cut_split(const Plan& P, const Unit& U) {
 // unit's histogram row (free once the radix select is over).  One warp per
 // chunk, consecutive loads.
 __global__ void __launch_bounds__(TPB) k_cut_part(Plan P) {
+    pdl_enter();
     const int lane = threadIdx.x & 31;
     const long long gw = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const long long nw = ((long long)gridDim.x * blockDim.x) >> 5;
@@ -1389,6 +1400,7 @@ __global__ void __launch_bounds__(TPB) k_cut_part(Plan P) {
 
 template <typename XT, typename BT, bool CKPT>
 __global__ void __launch_bounds__(CUT_TPB) k_cut(Plan P) {
+    pdl_enter();
     __shared__ long long s_scan[33];
     __shared__ uint32_t s_scan32[33];
     __shared__ long long s_tile;
