@@ -67,16 +67,42 @@ struct FrameHeader {
     uint32_t wmax[2][FR_MAX_NS];    // per side and iteration: max |w| as binary32 bits
 };
 
+// Conversions between binary64 and binary32 / tf32 in integer arithmetic: the
+// conversion instructions run at the binary64 rate, a thirtieth of the integer
+// rate here, and the element-wise kernels below were bound by them.
+// The nearest tf32 value (ties away) of a binary64 value with high word hw: as
+// the high word of a binary64 number (the low word is 0) and as binary32 bits.
+// Magnitudes below 2^-126 give 0; from 2^128 on an infinity (or a NaN).
+__device__ __forceinline__ void tf32_of(uint32_t hw, uint32_t& hw_out, uint32_t& f32) {
+    const uint32_t sg = hw & 0x80000000u;
+    uint32_t r = ((hw & 0x7FFFFFFFu) + 0x200u) & ~0x3FFu;          // 10 of the 20 mantissa bits
+    r = r < 0x38100000u ? 0u : r;
+    hw_out = sg | r;
+    f32 = sg | (r ? (r - 0x38000000u) << 3 : 0u);
+    if (r >= 0x47F00000u) f32 = sg | ((hw & 0x7FFFFFFFu) > 0x7FF00000u ? 0x7FC00000u : 0x7F800000u);
+}
+// binary32 -> binary64 (subnormals give 0)
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x), m = u & 0x7FFFFFFFu;
+    if (m >= 0x7F800000u) return (double)x;
+    const uint32_t h = m < 0x00800000u ? 0u : (m >> 3) + 0x38000000u;
+    return __hiloint2double((int)((u & 0x80000000u) | h), m < 0x00800000u ? 0 : (int)(m << 29));
+}
+// x / 2 (subnormal results give 0)
+__device__ __forceinline__ double halve(double x) {
+    const uint32_t h = (uint32_t)__double2hiint(x), m = h & 0x7FFFFFFFu;
+    if (m >= 0x7FF00000u) return x;
+    return m < 0x00200000u ? 0.0 : __hiloint2double((int)(h - 0x00100000u), __double2loint(x));
+}
+
 // binary64 -> (hi, lo) with hi a tf32 value (round to nearest, ties away) and
-// lo the binary32 rest, so that hi + lo = x to about 2^-22 |x|
+// lo the tf32 value nearest to the rest, so that hi + lo = x to about 2^-22 |x|
 __device__ __forceinline__ void split_tf32(double x, float& hi, float& lo) {
-    const float x32 = (float)x;
-    uint32_t h;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(h) : "f"(x32));
-    hi = __uint_as_float(h);
-    const float l32 = (float)(x - (double)hi);
-    uint32_t l;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(l) : "f"(l32));
+    uint32_t hw, f;
+    tf32_of((uint32_t)__double2hiint(x), hw, f);
+    hi = __uint_as_float(f);
+    uint32_t lw, l;
+    tf32_of((uint32_t)__double2hiint(x - __hiloint2double((int)hw, 0)), lw, l);
     lo = __uint_as_float(l);
 }
 
@@ -100,6 +126,7 @@ struct Frames {                     // one side (U: d = m; V: d = n), d x q row-
 // ---------------------------------------------------------------------------
 // out (C x R) = in (R x C)^T, binary64, 32 x 32 tiles
 __global__ void __launch_bounds__(256) k_fr_transpose(const double* in, double* out, long long R, long long C) {
+    pdl_enter();
     __shared__ double t[32][33];
     const long long r0 = (long long)blockIdx.y * 32, c0 = (long long)blockIdx.x * 32;
     for (int y = threadIdx.y; y < 32; y += 8) {
@@ -115,6 +142,7 @@ __global__ void __launch_bounds__(256) k_fr_transpose(const double* in, double* 
 
 // s_ik = sign(<u_0k, u_ik>): the column dot products (U side), summed into dots[i][k]
 __global__ void __launch_bounds__(256) k_fr_signdots(Frames f, double* dots, int row_chunks) {
+    pdl_enter();
     __shared__ double red[8][33];
     const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
     const int i = blockIdx.y;
@@ -141,6 +169,7 @@ __device__ __forceinline__ double sign_of(const double* dots, long long q, int i
 // for three experts of a 3584 x 18944 matrix)
 template <int KC>
 __global__ void __launch_bounds__(256) k_fr_coldots(Frames f, const double* dots, double* cd, int row_chunks) {
+    pdl_enter();
     __shared__ double red[8][33];
     const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
     const int K = f.K;
@@ -198,6 +227,7 @@ struct SplitT {
     long long Dp, Qp;
 };
 __global__ void __launch_bounds__(256) k_fr_split_t(SplitT a) {
+    pdl_enter();
     __shared__ double t[32][33];
     const long long Lr = (a.mode >= 4) ? 2 * a.Dp : a.Dp;
     const long long r0 = (long long)blockIdx.x * 32, k0 = (long long)blockIdx.y * 32;
@@ -251,10 +281,10 @@ struct SplitR {
     long long rows, rows_p, Lp;
 };
 __global__ void __launch_bounds__(256) k_fr_split_r(SplitR a) {
-    const long long total = a.rows_p * a.Lp;
+    pdl_enter();
     const long long q = a.f.q;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const long long r = e / a.Lp, c = e - r * a.Lp;
+    for (long long r = blockIdx.x; r < a.rows_p; r += gridDim.x)
+    for (long long c = threadIdx.x; c < a.Lp; c += blockDim.x) {
         double v = 0.0;
         if (r < a.rows) {
             switch (a.mode) {
@@ -318,6 +348,7 @@ __device__ __forceinline__ double oz_value(const OzSrc& a, int z, long long e, l
 // array once: bound by HBM)
 template <int SC>
 __global__ void __launch_bounds__(256) k_oz_colmax(OzSrc a, int sources, int row_chunks) {
+    pdl_enter();
     const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
     const long long per = (a.f.d + row_chunks - 1) / row_chunks;
     const long long r0 = (long long)blockIdx.y * per, r1 = k < a.f.q ? min(a.f.d, r0 + per) : r0;
@@ -369,6 +400,7 @@ __device__ __forceinline__ int oz_exponent(unsigned long long bits) {
 // its signed base-256 digits from the bottom, one 16-byte store per slice
 // (consecutive columns consecutive).
 __global__ void __launch_bounds__(256) k_oz_split(OzSrc a, int z0, unsigned char* out, unsigned long long slot_bytes) {
+    pdl_enter();
     const int z = z0 + blockIdx.z;
     const int kl = threadIdx.x & 127, half = threadIdx.x >> 7;
     const long long k = (long long)blockIdx.y * OZ_BM + kl;
@@ -408,6 +440,7 @@ __global__ void __launch_bounds__(256) k_oz_split(OzSrc a, int z0, unsigned char
 // C (qq entries per z) = the sum of the splits' partial sums, in split order
 __global__ void __launch_bounds__(256) k_oz_reduce(const double* part, int splits, int nz, long long q, double* C,
                                                    int minus_identity) {
+    pdl_enter();
     const long long total = (long long)nz * q * q;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
         double s = part[e];
@@ -424,20 +457,21 @@ __global__ void __launch_bounds__(256) k_oz_reduce(const double* part, int split
 // (rows Mp of 2 Np, element G[r, c]) or transposed (rows Np of 2 Mp, element
 // G[r, c] at row c, position r)
 __device__ __forceinline__ double load_typed(const void* p, int dtype, long long e) {
-    if (dtype == ISO_BF16) return (double)__uint_as_float((uint32_t)static_cast<const unsigned short*>(p)[e] << 16);
-    return (double)static_cast<const float*>(p)[e];
+    if (dtype == ISO_BF16) return widen(__uint_as_float((uint32_t)static_cast<const unsigned short*>(p)[e] << 16));
+    return widen(static_cast<const float*>(p)[e]);
 }
 __global__ void __launch_bounds__(256) k_op_split_g(const void* G, int dtype, long long m, long long n, long long Mp,
                                                     long long Np, float* out) {
-    const long long total = Mp * Np;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const long long r = e / Np, c = e - r * Np;
+    pdl_enter();
+    for (long long r = blockIdx.x; r < Mp; r += gridDim.x)
+    for (long long c = threadIdx.x; c < Np; c += blockDim.x) {
         const double v = (r < m && c < n) ? load_typed(G, dtype, r * n + c) : 0.0;
         put_split(out + r * 2 * Np, Np, c, v);
     }
 }
 __global__ void __launch_bounds__(256) k_op_split_gt(const void* G, int dtype, long long m, long long n, long long Mp,
                                                      long long Np, float* out) {
+    pdl_enter();
     __shared__ double t[32][33];
     const long long r0 = (long long)blockIdx.x * 32, c0 = (long long)blockIdx.y * 32;
     for (int y = threadIdx.y; y < 32; y += 8) {
@@ -453,12 +487,14 @@ __global__ void __launch_bounds__(256) k_op_split_gt(const void* G, int dtype, l
 
 // F += E (binary64, d x q)
 __global__ void __launch_bounds__(256) k_op_add(double* F, const double* E, long long total) {
+    pdl_enter();
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x)
         F[e] += E[e];
 }
 
 // Sym_i = sym(A_i), Kw_i = A_i - Sym_i (binary64; A is K arrays q x q)
 __global__ void __launch_bounds__(256) k_fr_symskew(const double* A, long long Qp, long long q, double* sym, double* kw) {
+    pdl_enter();
     __shared__ double ta[32][33], tb[32][33];
     const int i = blockIdx.z;
     const double* Ai = A + (long long)i * q * q;
@@ -479,7 +515,7 @@ __global__ void __launch_bounds__(256) k_fr_symskew(const double* A, long long Q
     }
 }
 
-// Gamma_ij (i <= j), summed into gram[i][j]; block y covers a slice of the q x q entries
+// Gamma_ij (i <= j), summed into gram[i][j]; block y takes rows y, y + gridDim.y, ... of the q x q entries
 struct GramArgs {
     const double* A[2];         // per side: K arrays q x q
     const double* sym[2];
@@ -491,6 +527,7 @@ struct GramArgs {
     int K;
 };
 __global__ void __launch_bounds__(256) k_fr_gram(GramArgs g) {
+    pdl_enter();
     __shared__ double red[32];
     // pair (i, j), i <= j, from blockIdx.x
     int i = 0, j = 0, p = blockIdx.x;
@@ -499,27 +536,27 @@ __global__ void __launch_bounds__(256) k_fr_gram(GramArgs g) {
         p -= g.K - i;
     }
     const long long q = g.q, qq = q * q;
-    const long long per = (qq + gridDim.y - 1) / gridDim.y;
-    const long long e0 = (long long)blockIdx.y * per, e1 = min(qq, e0 + per);
     double acc = 0.0;
-    for (long long e = e0 + threadIdx.x; e < e1; e += blockDim.x) {
-        const long long r = e / q, c = e - r * q;
-        const double sr = g.S0[r], sc = g.S0[c];
-        const double Dr = r < g.k_keep ? 1.0 : 0.0, Dc = c < g.k_keep ? 1.0 : 0.0;
-        // column terms (row l = r, column k = c), both sides
-        double colt = 0.0;
+    for (long long r = blockIdx.y; r < q; r += gridDim.y) {
+        const double sr = g.S0[r], Dr = r < g.k_keep ? 1.0 : 0.0;
+        for (long long c = threadIdx.x; c < q; c += blockDim.x) {
+            const long long e = r * q + c;
+            const double sc = g.S0[c], Dc = c < g.k_keep ? 1.0 : 0.0;
+            // column terms (row l = r, column k = c), both sides
+            double colt = 0.0;
 #pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            const double ai = g.A[s][(long long)i * qq + e];
-            const double aj = g.A[s][(long long)j * qq + e];
-            const double si = g.sym[s][(long long)i * qq + e], sj = g.sym[s][(long long)j * qq + e];
-            colt += ai * sj + si * aj - si * sj;
+            for (int s = 0; s < 2; ++s) {
+                const double ai = g.A[s][(long long)i * qq + e];
+                const double aj = g.A[s][(long long)j * qq + e];
+                const double si = g.sym[s][(long long)i * qq + e], sj = g.sym[s][(long long)j * qq + e];
+                colt += ai * sj + si * aj - si * sj;
+            }
+            acc -= sc * sc * Dc * colt;
+            // cross terms (k = r, l = c)
+            const double kui = g.kw[0][(long long)i * qq + e], kuj = g.kw[0][(long long)j * qq + e];
+            const double kvi = g.kw[1][(long long)i * qq + e], kvj = g.kw[1][(long long)j * qq + e];
+            acc -= sr * sc * Dr * Dc * (kui * kvj + kuj * kvi);
         }
-        acc -= sc * sc * Dc * colt;
-        // cross terms (k = r, l = c)
-        const double kui = g.kw[0][(long long)i * qq + e], kuj = g.kw[0][(long long)j * qq + e];
-        const double kvi = g.kw[1][(long long)i * qq + e], kvj = g.kw[1][(long long)j * qq + e];
-        acc -= sr * sc * Dr * Dc * (kui * kvj + kuj * kvi);
     }
     if (blockIdx.y == 0)
         for (long long k = threadIdx.x; k < min(q, g.k_keep); k += blockDim.x)
@@ -532,6 +569,7 @@ __global__ void __launch_bounds__(256) k_fr_gram(GramArgs g) {
 // c* from Gamma (upper triangle), then the caller's stats
 __global__ void k_fr_solve(double* gram, double* coef, int K, double ridge, double c_min, double c_max,
                            double* st_gram, double* st_coef) {
+    pdl_enter();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     double G[MAXK * MAXK], c[MAXK];
     for (int a = 0; a < K; ++a)
@@ -549,21 +587,23 @@ __global__ void k_fr_solve(double* gram, double* coef, int K, double ridge, doub
 // xi* = D dF_c - E (E = F_0 Y from the GEMM, ld Qp)
 __global__ void __launch_bounds__(256) k_fr_xi(Frames f, const double* dots, const double* coef, const float* E,
                                                long long Qp, long long k_keep, double* xi) {
-    const long long total = f.d * f.q;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const long long r = e / f.q, k = e - r * f.q;
+    pdl_enter();
+    for (long long r = blockIdx.x; r < f.d; r += gridDim.x)
+    for (long long k = threadIdx.x; k < f.q; k += blockDim.x) {
+        const long long e = r * f.q + k;
         double v = 0.0;
         if (k < k_keep) {
             const double f0 = f.F0[e];
             for (int i = 0; i < f.K; ++i) v = fma(coef[i], fma(sign_of(dots, f.q, i, k), f.F[i][e], -f0), v);
         }
-        xi[e] = v - (double)E[r * Qp + k];
+        xi[e] = v - widen(E[r * Qp + k]);
     }
 }
 
 // ||N||_F^2 of N = xi^T xi (binary32, ld Qp; or binary64, ld q), one warp per row, summed into the header
 __global__ void __launch_bounds__(256) k_fr_norm(const float* N, const double* N64, long long Qp, long long q,
                                                  FrameHeader* h, int side) {
+    pdl_enter();
     __shared__ double red[32];
     const int lane = threadIdx.x & 31;
     double acc = 0.0;
@@ -615,6 +655,7 @@ __device__ __forceinline__ void ns_put(const NsArgs& a, double* M, float* M4, lo
 // Y_0 = (I + N) / cs = I + y, Z_0 = I (z = 0); cs = 1 while ||N||_F < 0.9,
 // else 1 + ||N||_F / 2, so that the eigenvalues of Y_0 lie in (0, 2)
 __global__ void __launch_bounds__(256) k_fr_ns_init(NsArgs a) {
+    pdl_enter();
     __shared__ double ta[32][33], tb[32][33];
     long long r0, c0;
     if (!ns_tile(r0, c0)) return;
@@ -637,8 +678,8 @@ __global__ void __launch_bounds__(256) k_fr_ns_init(NsArgs a) {
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += 8) {
         const long long r = r0 + y, c = c0 + threadIdx.x, r2 = c0 + y, c2 = r0 + threadIdx.x;
-        ns_put(a, a.y, a.y4, r, c, 0.5 * (ta[y][threadIdx.x] + tb[threadIdx.x][y]));
-        ns_put(a, a.y, a.y4, r2, c2, 0.5 * (tb[y][threadIdx.x] + ta[threadIdx.x][y]));
+        ns_put(a, a.y, a.y4, r, c, halve(ta[y][threadIdx.x] + tb[threadIdx.x][y]));
+        ns_put(a, a.y, a.y4, r2, c2, halve(tb[y][threadIdx.x] + ta[threadIdx.x][y]));
         if (r < a.q && c < a.q) a.z[r * a.q + c] = 0.0;
         if (r2 < a.q && c2 < a.q) a.z[r2 * a.q + c2] = 0.0;
     }
@@ -647,6 +688,7 @@ __global__ void __launch_bounds__(256) k_fr_ns_init(NsArgs a) {
 // w = y + z + z y (the residual Z Y - I), m = -w / 2; the largest |w| of the
 // iteration goes to the header
 __global__ void __launch_bounds__(256) k_fr_ns_m(NsArgs a) {
+    pdl_enter();
     __shared__ double ta[32][33], tb[32][33];
     if (*reinterpret_cast<volatile int32_t*>(&a.h->conv[a.side])) return;
     long long r0, c0;
@@ -654,21 +696,24 @@ __global__ void __launch_bounds__(256) k_fr_ns_m(NsArgs a) {
     auto w = [&](long long r, long long c) -> double {
         if (r >= a.q || c >= a.q) return 0.0;
         const long long e = r * a.q + c;
-        return a.y[e] + a.z[e] + (a.T1 ? (double)a.T1[r * a.Qp + c] : 0.0);
+        const double v = a.y[e] + a.z[e];
+        return a.T1 ? v + widen(a.T1[r * a.Qp + c]) : v;
     };
     for (int y = threadIdx.y; y < 32; y += 8) {
         ta[y][threadIdx.x] = w(r0 + y, c0 + threadIdx.x);
         tb[y][threadIdx.x] = w(c0 + y, r0 + threadIdx.x);
     }
     __syncthreads();
-    float wm = 0.0f;
+    unsigned long long most = 0;                   // largest |w| as binary64 bits
     for (int y = threadIdx.y; y < 32; y += 8) {
         const long long r = r0 + y, c = c0 + threadIdx.x;
-        const double v = 0.5 * (ta[y][threadIdx.x] + tb[threadIdx.x][y]);
-        ns_put(a, a.m, a.m4, r, c, -0.5 * v);
-        wm = fmaxf(wm, (float)fabs(v));
-        ns_put(a, a.m, a.m4, c0 + y, r0 + threadIdx.x, -0.25 * (tb[y][threadIdx.x] + ta[threadIdx.x][y]));
+        const double v = halve(ta[y][threadIdx.x] + tb[threadIdx.x][y]);
+        ns_put(a, a.m, a.m4, r, c, -halve(v));
+        const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
+        most = b > most ? b : most;
+        ns_put(a, a.m, a.m4, c0 + y, r0 + threadIdx.x, -halve(halve(tb[y][threadIdx.x] + ta[threadIdx.x][y])));
     }
+    float wm = (float)__longlong_as_double((long long)most);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) wm = fmaxf(wm, __shfl_xor_sync(0xFFFFFFFFu, wm, o));
     if ((threadIdx.x & 31) == 0) atomicMax(&a.h->wmax[a.side][a.it], __float_as_uint(wm));
@@ -679,6 +724,7 @@ __global__ void __launch_bounds__(256) k_fr_ns_m(NsArgs a) {
 // stopped its quadratic fall below 1e-2 (the rounding floor of the products),
 // or has grown.
 __global__ void __launch_bounds__(256) k_fr_ns_update(NsArgs a) {
+    pdl_enter();
     __shared__ double ya[32][33], yb[32][33], za[32][33], zb[32][33];
     if (*reinterpret_cast<volatile int32_t*>(&a.h->conv[a.side])) return;
     const double wc = (double)__uint_as_float(a.h->wmax[a.side][a.it]);
@@ -693,12 +739,13 @@ __global__ void __launch_bounds__(256) k_fr_ns_update(NsArgs a) {
     auto fy = [&](long long r, long long c) -> double {
         if (r >= a.q || c >= a.q) return 0.0;
         const long long e = r * a.q + c;
-        return a.y[e] + a.m[e] + (double)a.T1[r * a.Qp + c];
+        return a.y[e] + a.m[e] + widen(a.T1[r * a.Qp + c]);
     };
     auto fz = [&](long long r, long long c) -> double {
         if (r >= a.q || c >= a.q) return 0.0;
         const long long e = r * a.q + c;
-        return a.z[e] + a.m[e] + (a.T2 ? (double)a.T2[r * a.Qp + c] : 0.0);
+        const double v = a.z[e] + a.m[e];
+        return a.T2 ? v + widen(a.T2[r * a.Qp + c]) : v;
     };
     for (int y = threadIdx.y; y < 32; y += 8) {
         ya[y][threadIdx.x] = fy(r0 + y, c0 + threadIdx.x);
@@ -709,22 +756,22 @@ __global__ void __launch_bounds__(256) k_fr_ns_update(NsArgs a) {
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += 8) {
         const long long r = r0 + y, c = c0 + threadIdx.x, r2 = c0 + y, c2 = r0 + threadIdx.x;
-        ns_put(a, a.y, a.y4, r, c, 0.5 * (ya[y][threadIdx.x] + yb[threadIdx.x][y]));
-        ns_put(a, a.z, a.z4, r, c, 0.5 * (za[y][threadIdx.x] + zb[threadIdx.x][y]));
-        ns_put(a, a.y, a.y4, r2, c2, 0.5 * (yb[y][threadIdx.x] + ya[threadIdx.x][y]));
-        ns_put(a, a.z, a.z4, r2, c2, 0.5 * (zb[y][threadIdx.x] + za[threadIdx.x][y]));
+        ns_put(a, a.y, a.y4, r, c, halve(ya[y][threadIdx.x] + yb[threadIdx.x][y]));
+        ns_put(a, a.z, a.z4, r, c, halve(za[y][threadIdx.x] + zb[threadIdx.x][y]));
+        ns_put(a, a.y, a.y4, r2, c2, halve(yb[y][threadIdx.x] + ya[threadIdx.x][y]));
+        ns_put(a, a.z, a.z4, r2, c2, halve(zb[y][threadIdx.x] + za[threadIdx.x][y]));
     }
 }
 
 // E_F = xi* + (F_0 + xi*) R (P from the GEMM, ld Qp), in place over xi*
 __global__ void __launch_bounds__(256) k_fr_motion(double* xi, const float* P, long long Qp, long long d, long long q) {
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < d * q; e += (long long)gridDim.x * blockDim.x) {
-        const long long r = e / q, c = e - r * q;
-        xi[e] += (double)P[r * Qp + c];
-    }
+    pdl_enter();
+    for (long long r = blockIdx.x; r < d; r += gridDim.x)
+        for (long long c = threadIdx.x; c < q; c += blockDim.x) xi[r * q + c] += widen(P[r * Qp + c]);
 }
 
 __global__ void k_fr_status(const FrameHeader* h, int32_t* out) {
+    pdl_enter();
     if (threadIdx.x == 0 && blockIdx.x == 0) *out = h->status;
 }
 
@@ -836,10 +883,10 @@ int frame_gemm(cudaStream_t s, int sms, const float* A, long long a_rows, const 
     const bool wide = (t256 + sms - 1) / sms * 1900 <= (t128 + sms - 1) / sms * 1150;
     const int slot = prof_begin(0, s);
     if (wide)
-        k_gemm_x3<256><<<dim3((unsigned)((b_rows + 255) / 256), (unsigned)my, nz), GEMM_THREADS, X3_SMEM, s>>>(ta, tb, ta2,
+        pdl_launch(k_gemm_x3<256>, dim3((unsigned)((b_rows + 255) / 256), (unsigned)my, nz), GEMM_THREADS, X3_SMEM, s, ta, tb, ta2,
                                                                                                             tb2, g);
     else
-        k_gemm_x3<128><<<dim3((unsigned)(b_rows / 128), (unsigned)my, nz), GEMM_THREADS, X3_SMEM, s>>>(ta, tb, ta2, tb2, g);
+        pdl_launch(k_gemm_x3<128>, dim3((unsigned)(b_rows / 128), (unsigned)my, nz), GEMM_THREADS, X3_SMEM, s, ta, tb, ta2, tb2, g);
     prof_end(slot, s);
     return cudaGetLastError() == cudaSuccess ? ISO_OK : ISO_ERR_CUDA;
 }
@@ -905,10 +952,10 @@ int exact_product(cudaStream_t s, int sms, const OzSrc& src, int K, double* C, u
     const unsigned long long slot = (unsigned long long)nt * chunks * OZ_SLAB_BYTES;
     const int rc = (int)std::max(1LL, std::min(256LL, (d + 255) / 256));
     const dim3 mg((unsigned)((q + 31) / 32), rc), mb(32, 8);
-    if (K == 0) FR_LAUNCH((k_oz_colmax<1><<<mg, mb, 0, s>>>(src, K + 1, rc)));
-    else if (K <= 2) FR_LAUNCH((k_oz_colmax<3><<<mg, mb, 0, s>>>(src, K + 1, rc)));
-    else if (K <= 4) FR_LAUNCH((k_oz_colmax<5><<<mg, mb, 0, s>>>(src, K + 1, rc)));
-    else FR_LAUNCH((k_oz_colmax<MAXK + 1><<<mg, mb, 0, s>>>(src, K + 1, rc)));
+    if (K == 0) FR_LAUNCH((pdl_launch(k_oz_colmax<1>, mg, mb, 0, s, src, K + 1, rc)));
+    else if (K <= 2) FR_LAUNCH((pdl_launch(k_oz_colmax<3>, mg, mb, 0, s, src, K + 1, rc)));
+    else if (K <= 4) FR_LAUNCH((pdl_launch(k_oz_colmax<5>, mg, mb, 0, s, src, K + 1, rc)));
+    else FR_LAUNCH((pdl_launch(k_oz_colmax<MAXK + 1>, mg, mb, 0, s, src, K + 1, rc)));
     static std::once_flag once;
     static cudaError_t opt = cudaSuccess;
     std::call_once(once, [] { opt = cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM); });
@@ -916,7 +963,7 @@ int exact_product(cudaStream_t s, int sms, const OzSrc& src, int K, double* C, u
     if (scratch_bytes < slot * (K ? 2 : 1)) return ISO_ERR_WORKSPACE;
     const int most = (int)std::min<unsigned long long>(std::max(K, 1), scratch_bytes / slot - (K ? 1 : 0));
     auto split = [&](int z0, int nz, unsigned char* out) -> int {
-        FR_LAUNCH((k_oz_split<<<dim3((unsigned)chunks, (unsigned)nt, (unsigned)nz), 256, 0, s>>>(src, z0, out, slot)));
+        FR_LAUNCH((pdl_launch(k_oz_split, dim3((unsigned)chunks, (unsigned)nt, (unsigned)nz), 256, 0, s, src, z0, out, slot)));
         return ISO_OK;
     };
     ISO_TRY(split(0, 1, scratch));
@@ -956,11 +1003,11 @@ int exact_product(cudaStream_t s, int sms, const OzSrc& src, int K, double* C, u
         g.minus_identity = K || splits > 1 ? 0 : 1;
         g.status = status;
         const int pslot = prof_begin(0, s);
-        k_oz_gemm<<<dim3((unsigned)(tiles / nz), (unsigned)splits, (unsigned)nz), OZ_THREADS, OZ_SMEM, s>>>(g);
+        pdl_launch(k_oz_gemm, dim3((unsigned)(tiles / nz), (unsigned)splits, (unsigned)nz), OZ_THREADS, OZ_SMEM, s, g);
         prof_end(pslot, s);
         if (cudaGetLastError() != cudaSuccess) return ISO_ERR_CUDA;
         if (splits > 1)
-            FR_LAUNCH((k_oz_reduce<<<grid_of((long long)nz * q * q, sms), 256, 0, s>>>(g.part, splits, nz, q, g.C, K ? 0 : 1)));
+            FR_LAUNCH((pdl_launch(k_oz_reduce, grid_of((long long)nz * q * q, sms), 256, 0, s, g.part, splits, nz, q, g.C, K ? 0 : 1)));
     }
     return ISO_OK;
 }
@@ -977,12 +1024,12 @@ struct NsBufs {
 // of (F_0 + X) R).  Header slot `side` holds its scaling and state.
 int ns_root(cudaStream_t s, int sms, FrameHeader* hdr, int side, const float* Nq, const double* N64, long long q,
             long long Qp, const NsBufs& b, int ns_iters, float* R4) {
-    FR_LAUNCH((k_fr_norm<<<grid_of(q * 32, sms), 256, 0, s>>>(Nq, N64, Qp, q, hdr, side)));
+    FR_LAUNCH((pdl_launch(k_fr_norm, grid_of(q * 32, sms), 256, 0, s, Nq, N64, Qp, q, hdr, side)));
     NsArgs na{};
     na.N = Nq; na.N64 = N64; na.y = b.y; na.z = b.z; na.m = b.m; na.y4 = b.y4; na.z4 = b.z4; na.m4 = b.m4; na.h = hdr;
     na.q = q; na.Qp = Qp; na.side = side;
     const dim3 tiles((unsigned)(Qp / 32), (unsigned)(Qp / 32)), tb(32, 8);
-    FR_LAUNCH((k_fr_ns_init<<<tiles, tb, 0, s>>>(na)));
+    FR_LAUNCH((pdl_launch(k_fr_ns_init, tiles, tb, 0, s, na)));
     for (int it = 0; it < ns_iters; ++it) {
         GemmArgs g{};
         g.mode = GEMM_STORE_F32; g.ldc = Qp; g.M = (int)Qp; g.N = (int)Qp; g.status = &hdr->status;
@@ -991,19 +1038,19 @@ int ns_root(cudaStream_t s, int sms, FrameHeader* hdr, int side, const float* Nq
         if (it) ISO_TRY(frame_gemm(s, sms, b.z4, Qp, b.y4, Qp, Qp, g));     // z y (z = 0 at first)
         na.it = it;
         na.T1 = it ? b.t1 : nullptr;
-        FR_LAUNCH((k_fr_ns_m<<<tiles, tb, 0, s>>>(na)));
+        FR_LAUNCH((pdl_launch(k_fr_ns_m, tiles, tb, 0, s, na)));
         // y m and, past the first step (z = 0), m z in one launch
         g.C = b.t2;
         g.C2 = b.t3;
         ISO_TRY(frame_gemm(s, sms, b.y4, Qp, b.m4, Qp, Qp, g, it ? b.m4 : nullptr, b.z4));
         na.T1 = b.t2;
         na.T2 = it ? b.t3 : nullptr;
-        FR_LAUNCH((k_fr_ns_update<<<tiles, tb, 0, s>>>(na)));
+        FR_LAUNCH((pdl_launch(k_fr_ns_update, tiles, tb, 0, s, na)));
     }
     SplitR sr{};
     sr.f.q = q; sr.hdr = hdr; sr.side = side; sr.mode = 6; sr.M = b.z; sr.out = R4;
     sr.rows = q; sr.rows_p = Qp; sr.Lp = Qp;
-    FR_LAUNCH((k_fr_split_r<<<grid_of(Qp * Qp, sms), 256, 0, s>>>(sr)));
+    FR_LAUNCH((pdl_launch(k_fr_split_r, grid_of(Qp * Qp, sms), 256, 0, s, sr)));
     return ISO_OK;
 }
 
@@ -1084,22 +1131,22 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
     }
     {
         const dim3 blk(32, 8), grd((unsigned)((n + 31) / 32), (unsigned)((q + 31) / 32));
-        FR_LAUNCH((k_fr_transpose<<<grd, blk, 0, s>>>(Vt0, D(L.vcopy), q, n)));
+        FR_LAUNCH((pdl_launch(k_fr_transpose, grd, blk, 0, s, Vt0, D(L.vcopy), q, n)));
         for (int i = 0; i < K; ++i)
-            FR_LAUNCH((k_fr_transpose<<<grd, blk, 0, s>>>(Vt[i], D(L.vcopy) + (size_t)(i + 1) * n * q, q, n)));
+            FR_LAUNCH((pdl_launch(k_fr_transpose, grd, blk, 0, s, Vt[i], D(L.vcopy) + (size_t)(i + 1) * n * q, q, n)));
     }
     // signs (from the U frames), then the column dot products of each side
     {
         const int rc = (int)std::max(1LL, std::min(64LL, ((long long)m + 511) / 512));
-        FR_LAUNCH((k_fr_signdots<<<dim3((unsigned)((q + 31) / 32), K, rc), dim3(32, 8), 0, s>>>(fr[0], dots, rc)));
+        FR_LAUNCH((pdl_launch(k_fr_signdots, dim3((unsigned)((q + 31) / 32), K, rc), dim3(32, 8), 0, s, fr[0], dots, rc)));
         for (int sd = 0; sd < 2; ++sd) {
             const int r2 = (int)std::max(1LL, std::min(256LL, (fr[sd].d + 255) / 256));
             const dim3 cg((unsigned)((q + 31) / 32), r2), cb(32, 8);
-            if (K == 1) FR_LAUNCH((k_fr_coldots<1><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
-            else if (K == 2) FR_LAUNCH((k_fr_coldots<2><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
-            else if (K == 3) FR_LAUNCH((k_fr_coldots<3><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
-            else if (K == 4) FR_LAUNCH((k_fr_coldots<4><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
-            else FR_LAUNCH((k_fr_coldots<8><<<cg, cb, 0, s>>>(fr[sd], dots, D(L.cd[sd]), r2)));
+            if (K == 1) FR_LAUNCH((pdl_launch(k_fr_coldots<1>, cg, cb, 0, s, fr[sd], dots, D(L.cd[sd]), r2)));
+            else if (K == 2) FR_LAUNCH((pdl_launch(k_fr_coldots<2>, cg, cb, 0, s, fr[sd], dots, D(L.cd[sd]), r2)));
+            else if (K == 3) FR_LAUNCH((pdl_launch(k_fr_coldots<3>, cg, cb, 0, s, fr[sd], dots, D(L.cd[sd]), r2)));
+            else if (K == 4) FR_LAUNCH((pdl_launch(k_fr_coldots<4>, cg, cb, 0, s, fr[sd], dots, D(L.cd[sd]), r2)));
+            else FR_LAUNCH((pdl_launch(k_fr_coldots<8>, cg, cb, 0, s, fr[sd], dots, D(L.cd[sd]), r2)));
         }
     }
     // A_i = F_0^T dF_i (binary64), then Sym_i and Kw_i
@@ -1108,7 +1155,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
                  reinterpret_cast<int32_t*>(ws + L.ex), Qp};
         ISO_TRY(exact_product(s, sms, oz, K, D(L.aq[sd]), reinterpret_cast<unsigned char*>(ws + L.tail),
                               L.total - L.tail, &hdr->status));
-        FR_LAUNCH((k_fr_symskew<<<dim3((unsigned)(Qp / 32), (unsigned)(Qp / 32), K), dim3(32, 8), 0, s>>>(
+        FR_LAUNCH((pdl_launch(k_fr_symskew, dim3((unsigned)(Qp / 32), (unsigned)(Qp / 32), K), dim3(32, 8), 0, s, 
             D(L.aq[sd]), Qp, q, D(L.sym[sd]), D(L.kw[sd]))));
     }
     // Gamma and c*
@@ -1119,9 +1166,9 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
         }
         ga.S0 = S0; ga.gram = gram; ga.q = q; ga.Qp = Qp; ga.k_keep = k_keep; ga.K = K;
         const int pairs = K * (K + 1) / 2;
-        const int slices = (int)std::max(1LL, std::min((long long)sms * 4, (q * q + 4095) / 4096));
-        FR_LAUNCH((k_fr_gram<<<dim3(pairs, slices), 256, 0, s>>>(ga)));
-        FR_LAUNCH((k_fr_solve<<<1, 32, 0, s>>>(gram, coef, K, cfg->ridge, cfg->c_min, cfg->c_max,
+        const int slices = (int)std::max(1LL, std::min((long long)sms * 4, q));
+        FR_LAUNCH((pdl_launch(k_fr_gram, dim3(pairs, slices), 256, 0, s, ga)));
+        FR_LAUNCH((pdl_launch(k_fr_solve, 1, 32, 0, s, gram, coef, K, cfg->ridge, cfg->c_min, cfg->c_max,
                                                 stats ? stats->gram : nullptr, stats ? stats->coef : nullptr)));
     }
     // per side: aggregate tangent, polar factor, motion E_F
@@ -1132,20 +1179,20 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
         sr.side = sd; sr.k_keep = k_keep;
         // Y^T, F_0, then E = F_0 Y
         sr.mode = 3; sr.out = F(L.y4[sd]); sr.rows = q; sr.rows_p = Qp; sr.Lp = Qp;
-        FR_LAUNCH((k_fr_split_r<<<grid_of(Qp * Qp, sms), 256, 0, s>>>(sr)));
+        FR_LAUNCH((pdl_launch(k_fr_split_r, grid_of(Qp * Qp, sms), 256, 0, s, sr)));
         sr.mode = 0; sr.out = F(L.fr4[sd]); sr.rows = d; sr.rows_p = Dp; sr.Lp = Qp;
-        FR_LAUNCH((k_fr_split_r<<<grid_of(Dp * Qp, sms), 256, 0, s>>>(sr)));
+        FR_LAUNCH((pdl_launch(k_fr_split_r, grid_of(Dp * Qp, sms), 256, 0, s, sr)));
         {
             GemmArgs g{};
             g.mode = GEMM_STORE_F32; g.C = F(L.e[sd]); g.ldc = Qp; g.M = (int)Dp; g.N = (int)Qp; g.status = &hdr->status;
             ISO_TRY(frame_gemm(s, sms, F(L.fr4[sd]), Dp, F(L.y4[sd]), Qp, Qp, g));
         }
-        FR_LAUNCH((k_fr_xi<<<grid_of(d * q, sms), 256, 0, s>>>(fr[sd], dots, coef, F(L.e[sd]), Qp, k_keep, D(L.xi[sd]))));
+        FR_LAUNCH((pdl_launch(k_fr_xi, grid_of(d * q, sms), 256, 0, s, fr[sd], dots, coef, F(L.e[sd]), Qp, k_keep, D(L.xi[sd]))));
         // N = xi*^T xi*
         {
             SplitT st{};
             st.f = fr[sd]; st.dots = dots; st.X = D(L.xi[sd]); st.mode = 2; st.out = F(L.ft4[sd]); st.Dp = Dp; st.Qp = Qp;
-            FR_LAUNCH((k_fr_split_t<<<dim3((unsigned)(Dp / 32), (unsigned)(Qp / 32)), dim3(32, 8), 0, s>>>(st)));
+            FR_LAUNCH((pdl_launch(k_fr_split_t, dim3((unsigned)(Dp / 32), (unsigned)(Qp / 32)), dim3(32, 8), 0, s, st)));
             GemmArgs g{};
             g.mode = GEMM_STORE_F32; g.C = F(L.nq[sd]); g.ldc = Qp; g.M = (int)Qp; g.N = (int)Qp; g.status = &hdr->status;
             ISO_TRY(frame_gemm(s, sms, F(L.ft4[sd]), Qp, F(L.ft4[sd]), Qp, Dp, g));
@@ -1158,19 +1205,19 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
             ISO_TRY(ns_root(s, sms, hdr, sd, F(L.nq[sd]), nullptr, q, Qp, nb, ns_iters, F(L.y4[sd])));
         }
         sr.mode = 1; sr.X = D(L.xi[sd]); sr.out = F(L.fr4[sd]); sr.rows = d; sr.rows_p = Dp; sr.Lp = Qp;
-        FR_LAUNCH((k_fr_split_r<<<grid_of(Dp * Qp, sms), 256, 0, s>>>(sr)));
+        FR_LAUNCH((pdl_launch(k_fr_split_r, grid_of(Dp * Qp, sms), 256, 0, s, sr)));
         {
             GemmArgs g{};
             g.mode = GEMM_STORE_F32; g.C = F(L.e[sd]); g.ldc = Qp; g.M = (int)Dp; g.N = (int)Qp; g.status = &hdr->status;
             ISO_TRY(frame_gemm(s, sms, F(L.fr4[sd]), Dp, F(L.y4[sd]), Qp, Qp, g));
         }
-        FR_LAUNCH((k_fr_motion<<<grid_of(d * q, sms), 256, 0, s>>>(D(L.xi[sd]), F(L.e[sd]), Qp, d, q)));
+        FR_LAUNCH((pdl_launch(k_fr_motion, grid_of(d * q, sms), 256, 0, s, D(L.xi[sd]), F(L.e[sd]), Qp, d, q)));
         // the reconstruction's operand of this side
         sr.X = D(L.xi[sd]);
         sr.mode = sd == 0 ? 4 : 5;
         sr.out = F(sd == 0 ? L.a6 : L.b6);
         sr.rows = d; sr.rows_p = Dp; sr.Lp = 2 * Qp;
-        FR_LAUNCH((k_fr_split_r<<<grid_of(Dp * 2 * Qp, sms), 256, 0, s>>>(sr)));
+        FR_LAUNCH((pdl_launch(k_fr_split_r, grid_of(Dp * 2 * Qp, sms), 256, 0, s, sr)));
     }
     // W* = W_0 + [E_U S_0 | U_0 S_0] [V* | E_V]^T
     {
@@ -1179,7 +1226,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
         g.out_dtype = W0->dtype; g.status = &hdr->status;
         ISO_TRY(frame_gemm(s, sms, F(L.a6), L.Mp, F(L.b6), L.Np, 2 * Qp, g));
     }
-    if (stats && stats->status) FR_LAUNCH((k_fr_status<<<1, 32, 0, s>>>(hdr, stats->status)));
+    if (stats && stats->status) FR_LAUNCH((pdl_launch(k_fr_status, 1, 32, 0, s, hdr, stats->status)));
     return ISO_OK;
 }
 
@@ -1237,15 +1284,15 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
     fr[0] = Frames{}; fr[0].F0 = U; fr[0].d = m; fr[0].q = q;
     fr[1] = Frames{}; fr[1].F0 = V; fr[1].d = n; fr[1].q = q;
     // operands of the factor gradients G_U = G_W (V S_0), G_V = G_W^T (U S_0)
-    FR_LAUNCH((k_op_split_g<<<grid_of(L.Mp * L.Np, sms), 256, 0, s>>>(G_W->data, G_W->dtype, m, n, L.Mp, L.Np,
+    FR_LAUNCH((pdl_launch(k_op_split_g, grid_of(L.Mp * L.Np, sms), 256, 0, s, G_W->data, G_W->dtype, m, n, L.Mp, L.Np,
                                                                       F(L.gw4))));
-    FR_LAUNCH((k_op_split_gt<<<dim3((unsigned)(L.Mp / 32), (unsigned)(L.Np / 32)), dim3(32, 8), 0, s>>>(
+    FR_LAUNCH((pdl_launch(k_op_split_gt, dim3((unsigned)(L.Mp / 32), (unsigned)(L.Np / 32)), dim3(32, 8), 0, s, 
         G_W->data, G_W->dtype, m, n, L.Mp, L.Np, F(L.gwt4))));
     for (int sd = 0; sd < 2; ++sd) {
         SplitT st{};
         st.f = fr[sd]; st.X = sd == 0 ? U : V; st.S0 = S0; st.mode = 3; st.Dp = sd == 0 ? L.Mp : L.Np; st.Qp = Qp;
         st.out = F(sd == 0 ? L.su4 : L.sv4);
-        FR_LAUNCH((k_fr_split_t<<<dim3((unsigned)(st.Dp / 32), (unsigned)(Qp / 32)), dim3(32, 8), 0, s>>>(st)));
+        FR_LAUNCH((pdl_launch(k_fr_split_t, dim3((unsigned)(st.Dp / 32), (unsigned)(Qp / 32)), dim3(32, 8), 0, s, st)));
     }
     // the factor gradients on the tensor cores with AdamW in the epilogue:
     // dF = F_bar - F, the moments updated in place
@@ -1272,28 +1319,28 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
         ISO_TRY(ns_root(s, sms, hdr, sd, nullptr, D(L.n64), q, Qp, nb, ns_iters, F(L.r4)));
         SplitR sr{};
         sr.f = fr[sd]; sr.X = D(L.dF[sd]); sr.mode = 1; sr.out = F(L.xb4); sr.rows = d; sr.rows_p = Dp; sr.Lp = Qp;
-        FR_LAUNCH((k_fr_split_r<<<grid_of(Dp * Qp, sms), 256, 0, s>>>(sr)));
+        FR_LAUNCH((pdl_launch(k_fr_split_r, grid_of(Dp * Qp, sms), 256, 0, s, sr)));
         {
             GemmArgs g{};
             g.mode = GEMM_STORE_F32; g.C = F(L.p); g.ldc = Qp; g.M = (int)Dp; g.N = (int)Qp; g.status = &hdr->status;
             ISO_TRY(frame_gemm(s, sms, F(L.xb4), Dp, F(L.r4), Qp, Qp, g));
         }
-        FR_LAUNCH((k_fr_motion<<<grid_of(d * q, sms), 256, 0, s>>>(D(L.dF[sd]), F(L.p), Qp, d, q)));
+        FR_LAUNCH((pdl_launch(k_fr_motion, grid_of(d * q, sms), 256, 0, s, D(L.dF[sd]), F(L.p), Qp, d, q)));
         // the reconstruction's operand of this side ([E_U S_0 | U S_0] or [V + E_V | E_V])
         sr.S0 = S0; sr.X = D(L.dF[sd]); sr.mode = sd == 0 ? 4 : 5; sr.out = F(sd == 0 ? L.a6 : L.b6);
         sr.rows = d; sr.rows_p = Dp; sr.Lp = 2 * Qp;
-        FR_LAUNCH((k_fr_split_r<<<grid_of(Dp * 2 * Qp, sms), 256, 0, s>>>(sr)));
+        FR_LAUNCH((pdl_launch(k_fr_split_r, grid_of(Dp * 2 * Qp, sms), 256, 0, s, sr)));
     }
     // F+ = F + E_F, then W+ = W + [E_U S_0 | U S_0] [V+ | E_V]^T
-    FR_LAUNCH((k_op_add<<<grid_of(m * q, sms), 256, 0, s>>>(U, D(L.dF[0]), m * q)));
-    FR_LAUNCH((k_op_add<<<grid_of(n * q, sms), 256, 0, s>>>(V, D(L.dF[1]), n * q)));
+    FR_LAUNCH((pdl_launch(k_op_add, grid_of(m * q, sms), 256, 0, s, U, D(L.dF[0]), m * q)));
+    FR_LAUNCH((pdl_launch(k_op_add, grid_of(n * q, sms), 256, 0, s, V, D(L.dF[1]), n * q)));
     {
         GemmArgs g{};
         g.mode = GEMM_ADD_BASE; g.M = (int)m; g.N = (int)n; g.out = W_out->data; g.w0 = W->data; g.ldo = n;
         g.out_dtype = W->dtype; g.status = &hdr->status;
         ISO_TRY(frame_gemm(s, sms, F(L.a6), L.Mp, F(L.b6), L.Np, 2 * Qp, g));
     }
-    if (stats && stats->status) FR_LAUNCH((k_fr_status<<<1, 32, 0, s>>>(hdr, stats->status)));
+    if (stats && stats->status) FR_LAUNCH((pdl_launch(k_fr_status, 1, 32, 0, s, hdr, stats->status)));
     return ISO_OK;
 }
 

@@ -249,6 +249,7 @@ template <int BN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 k_gemm_x3(const __grid_constant__ CUtensorMap ta1, const __grid_constant__ CUtensorMap tb1,
           const __grid_constant__ CUtensorMap ta2, const __grid_constant__ CUtensorMap tb2, GemmArgs g) {
+    pdl_enter();
     if (g.skip && *reinterpret_cast<const volatile int32_t*>(g.skip)) return;
     constexpr int STAGES = BN == 256 ? 2 : 3;
     constexpr int A_BYTES = GEMM_TILE_BYTES, B_BYTES = GEMM_TILE_BYTES * (BN / 128);
@@ -414,6 +415,7 @@ __device__ __forceinline__ void oz_drain(uint32_t taddr, long long (&tot)[64]) {
 // Bound by the tensor cores: 28 products of 128 x 128 x 16 per 16 rows, each
 // slab read once per sweep for 22 (6) products.
 __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
+    pdl_enter();
     extern __shared__ unsigned char gemm_smem_raw[];
     unsigned char* const smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(gemm_smem_raw) + 127) & ~(uintptr_t)127);
