@@ -40,6 +40,36 @@ __device__ void block_find_from_top_b(const uint32_t* hist, int nb, long long ra
     __syncthreads();
 }
 
+// Among the nb <= RADIX_BINS counters from the top, the bin that holds rank
+// (1 <= rank <= their sum): its index, the count above it and its own count,
+// in res.  Two barriers; every thread of the block calls it.
+struct BinHit { int bin; uint32_t above, count; };
+__device__ __forceinline__ void block_find32(const uint32_t* hist, int nb, uint32_t rank, uint32_t* sm, BinHit* res) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int PER = RADIX_BINS / BLOCK_TPB;
+    const int j0 = threadIdx.x * PER;
+    uint32_t h[PER], sum = 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+        h[j] = j0 + j < nb ? hist[nb - 1 - j0 - j] : 0u;
+        sum += h[j];
+    }
+    uint32_t tot;
+    uint32_t excl = warp_excl_scan(sum, &tot);
+    if (lane == 0) sm[warp] = tot;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < BLOCK_TPB / 32; ++w) excl += w < warp ? sm[w] : 0u;
+    if (excl < rank && rank <= excl + sum) {
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            if (rank > excl && rank <= excl + h[j]) { res->bin = nb - 1 - j0 - j; res->above = excl; res->count = h[j]; }
+            excl += h[j];
+        }
+    }
+    __syncthreads();
+}
+
 // keys sit at q + q / 32: a thread walking its own contiguous range and a
 // warp walking consecutive entries are both free of bank conflicts
 __device__ __forceinline__ int kpad(int q) { return q + (q >> 5); }
@@ -56,6 +86,7 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
     __shared__ long long s_above;
     __shared__ long long s_cutq;
     __shared__ uint32_t s_or;
+    __shared__ BinHit s_hit;
 
     const int idx = blockIdx.x;
     const int i = idx / P.n_units, u = idx % P.n_units;
@@ -148,7 +179,8 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
     // levels for bf16-valued task vectors).  Bound by issue: a descent bit by
     // bit spent two instructions per key and bit (235 us for a 4096 x 14336
     // bf16 task vector at 5 %, outputs included), keys and signs kept apart
-    // and rejoined for the outputs 208 us, this form 188 us.
+    // and rejoined for the outputs 208 us, separate passes for the counts above
+    // and at the threshold 188 us, this form 169 us.
     constexpr int BFE = BLOCK_MAX_ENTRIES / BLOCK_TPB;
     if (n == BLOCK_TPB * BFE && w % BFE == 0 && (d.cols % VEC) == 0 && (c0 % VEC) == 0 &&
         blockDim.x == BLOCK_TPB) {
@@ -168,7 +200,7 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
             for (int j = 0; j < VEC; ++j) v[g * VEC + j] = t8[j];
         }
         for (int q = threadIdx.x; q < RADIX_BINS; q += BLOCK_TPB) s_hist[q] = 0;
-        if (threadIdx.x == 0) { s_or = 0; s_cutq = CUT_ALL; }
+        if (threadIdx.x == 0) { s_or = 0; s_cutq = CUT_ALL; s_hit = BinHit{0, 0u, 0u}; }
         uint32_t kor = 0;
         float bad0 = 0.0f, bad1 = 0.0f;                // 0 * tau: NaN once a tau is not finite
 #pragma unroll
@@ -186,13 +218,12 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
         for (int j = 0; j < BFE; ++j) atomicAdd(&s_hist[(__float_as_uint(v[j]) >> SH1) & (RADIX_BINS - 1)], 1u);
         __syncthreads();
         const int low = s_or ? __ffs(s_or) - 1 : 31;
-        long long rank = k;
-        block_find_from_top_b(s_hist, RADIX_BINS, rank, s_scan, &s_bin, &s_above);
-        rank -= s_above;
-        uint32_t prefix = (uint32_t)s_bin;
+        uint32_t rank = (uint32_t)k;
+        block_find32(s_hist, RADIX_BINS, rank, s_scan32, &s_hit);
+        rank -= s_hit.above;
+        uint32_t prefix = (uint32_t)s_hit.bin;
         int pshift = SH1;
         while (pshift > low) {
-            __syncthreads();
             const int shift = max(pshift > RADIX_BITS ? pshift - RADIX_BITS : 0, low);
             const uint32_t nm = (1u << (pshift - shift)) - 1u;
             for (int q = threadIdx.x; q <= (int)nm; q += BLOCK_TPB) s_hist[q] = 0;
@@ -204,25 +235,27 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
                 if ((b & mask) == want) atomicAdd(&s_hist[(b >> shift) & nm], 1u);
             }
             __syncthreads();
-            block_find_from_top_b(s_hist, (int)nm + 1, rank, s_scan, &s_bin, &s_above);
-            rank -= s_above;
-            prefix = (prefix << (pshift - shift)) | (uint32_t)s_bin;
+            block_find32(s_hist, (int)nm + 1, rank, s_scan32, &s_hit);
+            rank -= s_hit.above;
+            prefix = (prefix << (pshift - shift)) | (uint32_t)s_hit.bin;
             pshift = shift;
         }
         const uint32_t tk = prefix << pshift;
         const float tf = __uint_as_float(tk);
-        uint32_t above = 0, ties = 0;
+        // what is left of the rank are the ties to keep, of as many as the last bin holds
+        const long long need = (long long)rank, tot_above = k - need;
+        const uint32_t tot_ties = s_hit.count;
+        if (need < (long long)tot_ties) {
+            uint32_t ties = 0, all;
 #pragma unroll
-        for (int j = 0; j < BFE; ++j) { above += fabsf(v[j]) > tf; ties += fabsf(v[j]) == tf; }
-        uint32_t tot_ties;
-        const uint32_t ties_before = block_excl_scan(ties, s_scan32, &tot_ties);
-        const uint32_t tot_above = block_sum(above, s_scan32);
-        const long long need = k - (long long)tot_above;
-        if (need < (long long)tot_ties && (long long)ties_before < need && need <= (long long)(ties_before + ties)) {
-            uint32_t acc = ties_before;
+            for (int j = 0; j < BFE; ++j) ties += fabsf(v[j]) == tf;
+            const uint32_t ties_before = block_excl_scan(ties, s_scan32, &all);
+            if ((long long)ties_before < need && need <= (long long)(ties_before + ties)) {
+                uint32_t acc = ties_before;
 #pragma unroll
-            for (int j = 0; j < BFE; ++j)
-                if (fabsf(v[j]) == tf && (long long)(++acc) == need) s_cutq = ea + j + 1;
+                for (int j = 0; j < BFE; ++j)
+                    if (fabsf(v[j]) == tf && (long long)(++acc) == need) s_cutq = ea + j + 1;
+            }
         }
         double g = 0.0;
         if (want_gamma) {
