@@ -598,7 +598,7 @@ __global__ void __launch_bounds__(TPB) k_fix(Plan P) {
     RawTile<__nv_bfloat16, __nv_bfloat16, true> rt;   // x in rt.x, theta_0 in rt.b
 #pragma unroll
     for (int v = 0; v < WVEC; ++v)
-        rt.load_step(v, P.xptr[cur.t], P.tens[cur.t].base, e0, (uint32_t)P.tens[cur.t].numel - e0, lane);
+        rt.load_step(v, P.xptr[cur.t], P.tens[cur.t].base, e0, (uint32_t)P.tens[cur.t].numel - e0, lane, v);
     for (long long f = fb; f < fe; ++f) {
         if (cur.t != pt) {
             pt = cur.t;
@@ -633,7 +633,7 @@ __global__ void __launch_bounds__(TPB) k_fix(Plan P) {
             float th0[VEC], tau[VEC];
             raw_to_f32<__nv_bfloat16>(rt.b[v], th0);
             if (CK) rt.tau(v, tau); else raw_to_f32<__nv_bfloat16>(rt.x[v], tau);
-            if (more) rt.load_step(v, nxp, nbp, ne0, nrem, lane);
+            if (more) rt.load_step(v, nxp, nbp, ne0, nrem, lane, v);
             if (e >= n) continue;
 #pragma unroll
             for (int j = 0; j < VEC; ++j) {

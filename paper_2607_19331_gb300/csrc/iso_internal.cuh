@@ -37,7 +37,7 @@ constexpr int SAMPLE_TPB = 1024;            // one sample block per SM, three ch
 constexpr int SAMPLE_LIST = 8192;           // sampled keys gathered around the ranks
 constexpr int SAMPLE_SEL_R = 5;             // ranks selected at once from the sample
 constexpr int CUT_TPB = 1024;
-constexpr int CS_SPLIT = 4;                 // count-sample blocks per unit
+constexpr int CS_SPLIT = 16;                // count-sample blocks per unit: one round of loads per warp
 constexpr int CS_TPB = 256;
 constexpr double SAMPLE_Z = 5.0;            // band half-width in sample standard deviations
 constexpr int COUNT_CHUNKS = 512;           // fused K = 1 pass: 256-entry chunks counted for the cut estimate
@@ -172,7 +172,7 @@ struct Unit {
 struct Header {             // first bytes of the workspace
     int32_t status;
     int32_t n_radix;        // units in ST_RADIX after the last pick
-    int32_t n_tknown;
+    int32_t n_tie;          // units whose tie counts (or sums above t) k_tie takes from their candidates
     int32_t fix_tiles;      // fused K = 1 pass: tiles k_fix re-applies (k_fix_plan)
 };
 
@@ -384,12 +384,13 @@ __device__ __forceinline__ void raw_to_f32(const uint4 (&w)[Lanes<T>::N], float 
 
 // One lane's share of a tile of a task-vector source, as raw words, so the
 // next tile's loads can be in flight while the current one is processed.
-template <typename XT, typename BT, bool CK>
+// NV < WVEC: only NV of its vector steps are held at a time (load_step's slot).
+template <typename XT, typename BT, bool CK, int NV = WVEC>
 struct RawTile {
     static constexpr int NX = Lanes<XT>::N;
     static constexpr int NB = CK ? Lanes<BT>::N : 1;
-    uint4 x[WVEC][NX];
-    uint4 b[WVEC][NB];
+    uint4 x[NV][NX];
+    uint4 b[NV][NB];
     __device__ __forceinline__ void load(const void* xp, const void* bp, long long e0, long long n, int lane) {
 #pragma unroll
         for (int v = 0; v < WVEC; ++v) {
@@ -406,28 +407,28 @@ struct RawTile {
         }
     }
     // vector step v of the tile starting at tensor entry e0, with rem = numel - e0
-    // entries left in the tensor (32-bit offsets; no bounds tests on a whole tile)
+    // entries left in the tensor (32-bit offsets; no bounds tests on a whole tile), into `slot`
     __device__ __forceinline__ void load_step(int v, const void* xp, const void* bp, uint32_t e0,
-                                              uint32_t rem, int lane) {
+                                              uint32_t rem, int lane, int slot) {
         const uint32_t o = (uint32_t)(v * (32 * VEC) + lane * VEC);
         if (rem >= TILE) {
             const char* xq = static_cast<const char*>(xp) + ((size_t)e0 + o) * sizeof(XT);
 #pragma unroll
-            for (int q = 0; q < NX; ++q) x[v][q] = ld_stream(xq + 16 * q);
+            for (int q = 0; q < NX; ++q) x[slot][q] = ld_stream(xq + 16 * q);
             if (CK) {
                 const char* bq = static_cast<const char*>(bp) + ((size_t)e0 + o) * sizeof(BT);
 #pragma unroll
-                for (int q = 0; q < NB; ++q) b[v][q] = ld_stream(bq + 16 * q);
+                for (int q = 0; q < NB; ++q) b[slot][q] = ld_stream(bq + 16 * q);
             }
         } else if (o < rem) {
-            load_raw8<XT>(xp, (long long)e0 + o, (long long)e0 + rem, x[v]);
+            load_raw8<XT>(xp, (long long)e0 + o, (long long)e0 + rem, x[slot]);
             if (CK) load_raw8<BT>(bp, (long long)e0 + o, (long long)e0 + rem,
-                                  reinterpret_cast<uint4(&)[Lanes<BT>::N]>(b[v]));
+                                  reinterpret_cast<uint4(&)[Lanes<BT>::N]>(b[slot]));
         } else {
 #pragma unroll
-            for (int q = 0; q < NX; ++q) x[v][q] = make_uint4(0, 0, 0, 0);
+            for (int q = 0; q < NX; ++q) x[slot][q] = make_uint4(0, 0, 0, 0);
 #pragma unroll
-            for (int q = 0; q < NB; ++q) b[v][q] = make_uint4(0, 0, 0, 0);
+            for (int q = 0; q < NB; ++q) b[slot][q] = make_uint4(0, 0, 0, 0);
         }
     }
     // tau = x (delta) or x - base (checkpoint), binary32

@@ -637,6 +637,7 @@ __device__ __forceinline__ bool count_run_at(const Plan& P, uint32_t it, uint32_
 template <typename XT, typename BT, bool CK, bool EMIT>
 __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
     pdl_enter();
+    constexpr bool RUNS = !EMIT;
     __shared__ uint32_t s_band[WPB][TILE + 32];
     extern __shared__ float s_vst[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -706,7 +707,10 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
     // step is converted to tau, its registers are refilled with the same step
     // of the next tile (item it2 of run r2), so a whole tile of loads is in
     // flight while this one is counted.
-    RawTile<XT, BT, CK> rt;
+    // Binary32 checkpoints hold half a tile of loads (up to 64 bytes per lane
+    // and step): a whole one spilled (41M entries: 79 us, 70 us so).
+    constexpr int DV = (CK && sizeof(XT) + sizeof(BT) > 4) ? 2 : WVEC;
+    RawTile<XT, BT, CK, DV> rt;
     // the unused slots of the warp's chunk get KEY_NONE, so that a large
     // unit's pool can be read as one flat array (k_radix_hist)
     auto seal = [&]() {
@@ -723,7 +727,7 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
             lo = au->lo;
             hi = au->hi;
             span = hi - lo;
-            run = !EMIT && au->mode_t;
+            run = RUNS && au->mode_t;
             that = au->that;
             want_gamma = au->want_gamma != 0;
             cap = (uint32_t)au->cand_cap;
@@ -791,13 +795,18 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
             *sp = __float_as_uint(m);
             sp += (RUN ? in && m != thf : in) ? 32 : 0;
         };
+        // the registers of step v take the step DV ahead: of this tile, or of the next
+        auto refill = [&](int v) {
+            if (v + DV < WVEC) rt.load_step(v + DV, rr.xp, rr.bp, e0, rem, lane, v % DV);
+            else if (more) rt.load_step(v + DV - WVEC, r2.xp, r2.bp, ne0, nrem, lane, v % DV);
+        };
         auto pass1 = [&](auto run_c, auto gamma_c) {
             if (rem >= TILE) {
 #pragma unroll
                 for (int v = 0; v < WVEC; ++v) {
                     float tau[VEC];
-                    rt.tau(v, tau);
-                    if (more) rt.load_step(v, r2.xp, r2.bp, ne0, nrem, lane);
+                    rt.tau(v % DV, tau);
+                    refill(v);
 #pragma unroll
                     for (int j = 0; j < VEC; j += 2) {
                         fma_rn2(bad0, bad1, tau[j], tau[j + 1], 0.0f, 0.0f, bad0, bad1);
@@ -810,8 +819,8 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
 #pragma unroll
                 for (int v = 0; v < WVEC; ++v) {
                     float tau[VEC];
-                    rt.tau(v, tau);
-                    if (more) rt.load_step(v, r2.xp, r2.bp, ne0, nrem, lane);
+                    rt.tau(v % DV, tau);
+                    refill(v);
                     const uint32_t o = (uint32_t)(v * (32 * VEC) + lane * VEC);
 #pragma unroll
                     for (int j = 0; j < VEC; ++j) {
@@ -825,10 +834,10 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
         using T1 = std::integral_constant<bool, true>;
         using T0 = std::integral_constant<bool, false>;
         if (want_gamma) {
-            if (!EMIT && run) pass1(T1{}, T1{});
+            if (RUNS && run) pass1(std::integral_constant<bool, RUNS>{}, T1{});
             else pass1(T0{}, T1{});
         } else {
-            if (!EMIT && run) pass1(T1{}, T0{});
+            if (RUNS && run) pass1(std::integral_constant<bool, RUNS>{}, T0{});
             else pass1(T0{}, T0{});
         }
         if (__any_sync(FULL, !(bad0 + bad1 == 0.0f)) && lane == 0) set_status(P.hdr, ISO_ERR_NONFINITE);
@@ -913,7 +922,7 @@ __global__ void __launch_bounds__(TPB, COUNT_BLOCKS_PER_SM) k_count(Plan P) {
     {
         const uint32_t e0 = r.e0;
 #pragma unroll
-        for (int v = 0; v < WVEC; ++v) rt.load_step(v, r.xp, r.bp, e0, r.n - e0, lane);
+        for (int v = 0; v < DV; ++v) rt.load_step(v, r.xp, r.bp, e0, r.n - e0, lane, v);
     }
     for (;;) {
         // the next item: the same run, or the next counted run
@@ -1008,7 +1017,6 @@ __global__ void k_decide(Plan P) {
     // in the band (t >= lo) and the unit's value segment did not overflow
     U.v_ok = (P.ccv && !U.fallback && U.v_alloc <= U.v_cap) ? 1 : 0;
     if (U.state == ST_RADIX) atomicAdd(&P.hdr->n_radix, 1);
-    else atomicAdd(&P.hdr->n_tknown, 1);
 }
 
 // ---------------------------------------------------------------------------
@@ -1251,7 +1259,7 @@ __global__ void __launch_bounds__(TPB) k_radix_pick(Plan P) {
             U.tie_src = TIE_ARRAY;
             U.state = ST_TKNOWN;
             atomicSub(&P.hdr->n_radix, 1);
-            atomicAdd(&P.hdr->n_tknown, 1);
+            if (U.need < U.ties || U.want_gamma) atomicAdd(&P.hdr->n_tie, 1);
         } else {
             U.r_prefix = (U.r_prefix << (pshift - shift)) | (uint32_t)b;
             U.r_pshift = shift;
@@ -1266,7 +1274,7 @@ __global__ void __launch_bounds__(TPB) k_radix_pick(Plan P) {
 template <typename XT, typename BT, bool CK>
 __global__ void __launch_bounds__(TPB) k_tie(Plan P) {
     pdl_enter();
-    if (*(volatile int32_t*)&P.hdr->n_tknown == 0) return;
+    if (*(volatile int32_t*)&P.hdr->n_tie == 0) return;
     const long long items = (long long)P.K * P.n_tiles;
     const long long per = (items + gridDim.x - 1) / gridDim.x;
     const long long beg = blockIdx.x * per;
