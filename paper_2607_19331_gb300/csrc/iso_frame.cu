@@ -70,16 +70,19 @@ struct FrameHeader {
 // Conversions between binary64 and binary32 / tf32 in integer arithmetic: the
 // conversion instructions run at the binary64 rate, a thirtieth of the integer
 // rate here, and the element-wise kernels below were bound by them.
-// The nearest tf32 value (ties away) of a binary64 value with high word hw: as
-// the high word of a binary64 number (the low word is 0) and as binary32 bits.
-// Magnitudes below 2^-126 give 0; from 2^128 on an infinity (or a NaN).
-__device__ __forceinline__ void tf32_of(uint32_t hw, uint32_t& hw_out, uint32_t& f32) {
-    const uint32_t sg = hw & 0x80000000u;
-    uint32_t r = ((hw & 0x7FFFFFFFu) + 0x200u) & ~0x3FFu;          // 10 of the 20 mantissa bits
+// x rounded to binary32 (nearest even) and then to tf32 (nearest, ties away),
+// as the two conversions give it: as the high word of a binary64 number (the
+// low word is 0) and as binary32 bits.  The first rounding matters only where
+// it carries into the high word, from a low word of 0xF0000000 on.  Magnitudes
+// below 2^-126 give 0; from 2^128 on an infinity (or a NaN).
+__device__ __forceinline__ void tf32_of(double x, uint32_t& hw_out, uint32_t& f32) {
+    const uint32_t hw = (uint32_t)__double2hiint(x);
+    const uint32_t sg = hw & 0x80000000u, m = hw & 0x7FFFFFFFu;
+    uint32_t r = (m + 0x200u + ((uint32_t)__double2loint(x) >= 0xF0000000u ? 1u : 0u)) & ~0x3FFu;   // 10 of 20 mantissa bits
     r = r < 0x38100000u ? 0u : r;
     hw_out = sg | r;
     f32 = sg | (r ? (r - 0x38000000u) << 3 : 0u);
-    if (r >= 0x47F00000u) f32 = sg | ((hw & 0x7FFFFFFFu) > 0x7FF00000u ? 0x7FC00000u : 0x7F800000u);
+    if (r >= 0x47F00000u) f32 = sg | (m > 0x7FF00000u ? 0x7FC00000u : 0x7F800000u);
 }
 // binary32 -> binary64 (subnormals give 0)
 __device__ __forceinline__ double widen(float x) {
@@ -99,11 +102,10 @@ __device__ __forceinline__ double halve(double x) {
 // lo the tf32 value nearest to the rest, so that hi + lo = x to about 2^-22 |x|
 __device__ __forceinline__ void split_tf32(double x, float& hi, float& lo) {
     uint32_t hw, f;
-    tf32_of((uint32_t)__double2hiint(x), hw, f);
+    tf32_of(x, hw, f);
     hi = __uint_as_float(f);
-    uint32_t lw, l;
-    tf32_of((uint32_t)__double2hiint(x - __hiloint2double((int)hw, 0)), lw, l);
-    lo = __uint_as_float(l);
+    tf32_of(x - __hiloint2double((int)hw, 0), hw, f);
+    lo = __uint_as_float(f);
 }
 
 // An operand row of contraction length L (padded) is stored as two segments [hi | lo].
@@ -1302,7 +1304,7 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
         GemmArgs g{};
         g.mode = GEMM_ADAMW; g.M = (int)(sd == 0 ? m : n); g.N = (int)q; g.ldo = q; g.status = &hdr->status;
         g.adam = AdamwArgs{sd == 0 ? U : V, sd == 0 ? mU : mV, sd == 0 ? vU : vV, D(L.dF[sd]),
-                           cfg->beta1, cfg->beta2, cfg->eps, bc2, cfg->lr * cfg->weight_decay, cfg->lr / bc1};
+                           cfg->beta1, cfg->beta2, cfg->eps, cfg->lr * cfg->weight_decay, cfg->lr / bc1, 1.0 / bc2};
         if (sd == 0) ISO_TRY(frame_gemm(s, sms, F(L.gw4), L.Mp, F(L.sv4), Qp, L.Np, g));
         else ISO_TRY(frame_gemm(s, sms, F(L.gwt4), L.Np, F(L.su4), Qp, L.Mp, g));
     }

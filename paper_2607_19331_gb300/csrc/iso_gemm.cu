@@ -94,6 +94,26 @@ __device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volati
     return false;
 }
 
+// c / (sqrt(x) + eps) in binary64.  The division and square root instructions'
+// sequences made up most of the epilogue's binary64 work; here a binary32
+// reciprocal square root and reciprocal are refined (Newton-Raphson; the last
+// step of each forms the residual exactly, as in Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", 1990), which
+// leaves root and quotient within two units in the last place.  x outside
+// binary32's comfortable range takes the library's.
+__device__ __forceinline__ double over_root(double c, double x, double eps) {
+    const float xf = (float)x;
+    if (!(xf > 1e-30f && xf < 1e30f)) return c / (sqrt(x) + eps);
+    const double r0 = (double)rsqrtf(xf);
+    const double r1 = fma(0.5 * r0, fma(-x * r0, r0, 1.0), r0);       // 1 / sqrt(x) to about 2^-43
+    const double s0 = x * r1;
+    const double d = fma(fma(-s0, s0, x), 0.5 * r1, s0) + eps;
+    const double i0 = (double)__frcp_rn((float)d);
+    const double i1 = fma(fma(-d, i0, 1.0), i0, i0);                  // 1 / d to about 2^-46
+    const double q = c * i1;
+    return fma(fma(-d, q, c), i1, q);
+}
+
 // one entry of the AdamW epilogue (a call, so that the unrolled columns stay
 // in registers without 32 copies of the binary64 code)
 __device__ __noinline__ void adamw_entry(const AdamwArgs& a, long long e, float grad) {
@@ -102,7 +122,7 @@ __device__ __noinline__ void adamw_entry(const AdamwArgs& a, long long e, float 
     const double vv = a.beta2 * (double)a.v[e] + (1.0 - a.beta2) * gr * gr;
     a.m[e] = (float)mm;
     a.v[e] = (float)vv;
-    a.dX[e] = -a.lr_wd * a.X[e] - a.lr_bc1 * mm / (sqrt(vv / a.bc2) + a.eps);
+    a.dX[e] = -a.lr_wd * a.X[e] - over_root(a.lr_bc1 * mm, vv * a.ibc2, a.eps);
 }
 
 // one row's 32 accumulated columns from col0 on, by epilogue mode

@@ -56,8 +56,8 @@ struct AdamwArgs {
     float* m;             // first moment (in place)
     float* v;             // second moment (in place)
     double* dX;           // out: X_bar - X = -lr wd X - lr / bc1 * m / (sqrt(v / bc2) + eps)
-    double beta1, beta2, eps, bc2;
-    double lr_wd, lr_bc1; // lr wd, lr / bc1
+    double beta1, beta2, eps;
+    double lr_wd, lr_bc1, ibc2;   // lr wd, lr / bc1, 1 / bc2
 };
 
 constexpr int X3_SMEM = 1024 + 192 * 1024 + 256;   // both tile shapes
