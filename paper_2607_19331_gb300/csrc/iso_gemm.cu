@@ -37,11 +37,37 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map
                  :: "r"(dst), "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar) : "memory");
 }
 
-__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate,
-                                          uint32_t idesc = UMMA_IDESC) {
+__device__ __forceinline__ void umma_tf32(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
     asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
                  "tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n\t}"
-                 :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate) : "memory");
+                 :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(UMMA_IDESC), "r"(accumulate) : "memory");
+}
+
+// The products of one warp run in warp-uniform control flow with one elected
+// lane issuing them: descriptors and accumulator addresses then live in
+// uniform registers.  A single-lane branch around the whole loop moved each of
+// them there per product, and a 64-clock product took 100 (k_gemm_x3<128>) to
+// 140 clocks (k_oz_gemm).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+// KIND 0: tf32, 1: bf16; descriptors as their low words (the high word is
+// the same for both operands)
+template <int KIND>
+__device__ __forceinline__ void umma_lo(uint32_t tmem_d, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t idesc,
+                                        uint32_t accumulate) {
+    if (KIND == 0)
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+                     "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+                     "tcgen05.mma.cta_group::1.kind::tf32 [%0], da, db, %4, p;\n\t}"
+                     :: "r"(tmem_d), "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\tsetp.ne.b32 p, %5, 0;\n\t"
+                     "mov.b64 da, {%1, %3};\n\tmov.b64 db, {%2, %3};\n\t"
+                     "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+                     :: "r"(tmem_d), "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate) : "memory");
 }
 
 // arrive on `bar` once every tcgen05.mma this thread issued before has completed
@@ -70,17 +96,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
     for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-                 "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-                   "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-                   "=r"(r[14]), "=r"(r[15])
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
+    uint32_t r[8];
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                  : "r"(taddr));
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
-    for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(r[j]);
+    for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(r[j]);
 }
 
 // bounded wait on one barrier phase; false once the limit is reached or
@@ -283,7 +306,7 @@ k_gemm_x3(const __grid_constant__ CUtensorMap ta1, const __grid_constant__ CUten
     // bars[0, S): full, bars[S, 2S): empty, bars[2S]: accumulators ready
     uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * STAGES + 1);
     volatile int* const abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const int m0 = blockIdx.y * GEMM_BM, n0 = blockIdx.x * BN;
     const CUtensorMap* const ta = blockIdx.z ? &ta2 : &ta1;
     const CUtensorMap* const tb = blockIdx.z ? &tb2 : &tb1;
@@ -310,7 +333,7 @@ k_gemm_x3(const __grid_constant__ CUtensorMap ta1, const __grid_constant__ CUten
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *reinterpret_cast<volatile uint32_t*>(tmem_slot), 0);
     const int KT = g.k_tiles;
 
     if (warp == 0 && lane == 0) {
@@ -336,25 +359,28 @@ k_gemm_x3(const __grid_constant__ CUtensorMap ta1, const __grid_constant__ CUten
             for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
                 if (mbar_try_wait(full_bar(kt % STAGES), (uint32_t)(kt / STAGES) & 1u)) break;
         }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        const bool lead = elect_one();
+        const uint32_t hi = (uint32_t)(sw128_desc(smem_s) >> 32), lo0 = (uint32_t)sw128_desc(smem_s);
         for (int kt = 0; kt < KT; ++kt) {
             const int s = kt % STAGES;
-            if (!wait_phase(full_bar(s), (uint32_t)(kt / STAGES) & 1u, abort_flag)) break;
+            if (!__all_sync(0xFFFFFFFFu, wait_phase(full_bar(s), (uint32_t)(kt / STAGES) & 1u, abort_flag))) break;
             tc_fence_after();
-            const uint32_t a0 = smem_s + (uint32_t)(s * STAGE_BYTES), b0 = a0 + 2 * A_BYTES;
+            const uint32_t a0 = lo0 + (uint32_t)(s * (STAGE_BYTES >> 4)), b0 = a0 + (2 * A_BYTES >> 4);
 #pragma unroll
             for (int kk = 0; kk < GEMM_BK / 8; ++kk) {
-                const uint64_t ah = sw128_desc(a0 + 32u * kk), al = sw128_desc(a0 + A_BYTES + 32u * kk);
-                const uint64_t bh = sw128_desc(b0 + 32u * kk), bl = sw128_desc(b0 + B_BYTES + 32u * kk);
+                const uint32_t ah = a0 + 2 * kk, al = ah + (A_BYTES >> 4), bh = b0 + 2 * kk, bl = bh + (B_BYTES >> 4);
                 const uint32_t acc = (kt > 0 || kk > 0) ? 1u : 0u;
-                umma_tf32(tmem, ah, bh, acc, IDESC);
-                umma_tf32(tmem + BN, ah, bl, acc, IDESC);
-                umma_tf32(tmem + BN, al, bh, 1u, IDESC);
+                if (lead) {
+                    umma_lo<0>(tmem, ah, bh, hi, IDESC, acc);
+                    umma_lo<0>(tmem + BN, ah, bl, hi, IDESC, acc);
+                    umma_lo<0>(tmem + BN, al, bh, hi, IDESC, 1u);
+                }
             }
-            umma_commit(empty_bar(s));
+            if (lead) umma_commit(empty_bar(s));
         }
         // the accumulator barrier also tracks products issued before a give-up
-        umma_commit(accum_bar);
+        if (lead) umma_commit(accum_bar);
     }
     __syncwarp();
 
@@ -410,21 +436,15 @@ constexpr uint32_t OZ_IDESC = (1u << 4)                 // D format: f32
                             | ((uint32_t)(OZ_BM >> 3) << 17)
                             | ((uint32_t)(OZ_BM >> 4) << 24);
 
-__device__ __forceinline__ void umma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t accumulate) {
-    asm volatile("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                 "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-                 :: "r"(tmem_d), "l"(adesc), "l"(bdesc), "r"(OZ_IDESC), "r"(accumulate) : "memory");
-}
-
 // tot += W * (the group's integer sums): this thread's lane, 64 columns
 template <int W>
 __device__ __forceinline__ void oz_drain(uint32_t taddr, long long (&tot)[64]) {
 #pragma unroll
-    for (int c = 0; c < 64; c += 16) {
-        float v[16];
-        tmem_ld16(taddr + c, v);
+    for (int c = 0; c < 64; c += 8) {
+        float v[8];
+        tmem_ld8(taddr + c, v);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) tot[c + j] += (long long)__float2int_rn(v[j]) * (long long)W;
+        for (int j = 0; j < 8; ++j) tot[c + j] += (long long)__float2int_rn(v[j]) * (long long)W;
     }
 }
 
@@ -443,7 +463,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
     // bars: full[S], empty[S], then per accumulator: ready[4], drained[4]
     uint32_t* const tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * OZ_STAGES + 8);
     volatile int* const abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = __shfl_sync(0xFFFFFFFFu, (int)threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
     const uint32_t smem_s = smem_u32(smem), bar_s = smem_u32(bars);
     auto full_bar = [&](int s) { return bar_s + 8u * s; };
     auto empty_bar = [&](int s) { return bar_s + 8u * (OZ_STAGES + s); };
@@ -486,7 +506,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+    const uint32_t tmem = __shfl_sync(0xFFFFFFFFu, *reinterpret_cast<volatile uint32_t*>(tmem_slot), 0);
 
     if (warp == 0 && lane == 0) {
         int it = 0;
@@ -505,7 +525,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
         for (int k = (it > OZ_STAGES ? it - OZ_STAGES : 0); k < it; ++k)
             for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
                 if (mbar_try_wait(full_bar(k % OZ_STAGES), (uint32_t)(k / OZ_STAGES) & 1u)) break;
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
+        const bool lead = elect_one();
+        const uint32_t hi = (uint32_t)(plain_desc(smem_s) >> 32), lo0 = (uint32_t)plain_desc(smem_s);
         bool ok = true;
         int it = 0, used[4] = {0, 0, 0, 0};              // drains of each accumulator so far
         // one sweep: groups G0 .. G0 + NG - 1, a drain every STEPS steps
@@ -513,28 +535,30 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
             constexpr int G0 = decltype(g0_c)::value, NG = decltype(ng_c)::value, STEPS = decltype(steps_c)::value;
             for (int c = 0; c < nc && ok; ++c, ++it) {
                 const int s = it % OZ_STAGES;
-                if (!wait_phase(full_bar(s), (uint32_t)(it / OZ_STAGES) & 1u, abort_flag)) { ok = false; break; }
+                if (!__all_sync(0xFFFFFFFFu, wait_phase(full_bar(s), (uint32_t)(it / OZ_STAGES) & 1u, abort_flag))) { ok = false; break; }
                 tc_fence_after();
                 const bool first = c % STEPS == 0, last = c % STEPS == STEPS - 1 || c == nc - 1;
-                const uint32_t a0 = smem_s + (uint32_t)s * 2u * OZ_SLAB_BYTES, b0 = a0 + OZ_SLAB_BYTES;
+                const uint32_t a0 = lo0 + (uint32_t)s * (2u * OZ_SLAB_BYTES >> 4), b0 = a0 + (OZ_SLAB_BYTES >> 4);
 #pragma unroll
                 for (int a = 0; a < NG; ++a) {
                     if (!ok) continue;
                     if (first && used[a] > 0) {
-                        if (!wait_phase(drained_bar(a), (uint32_t)(used[a] - 1) & 1u, abort_flag)) { ok = false; continue; }
+                        if (!__all_sync(0xFFFFFFFFu, wait_phase(drained_bar(a), (uint32_t)(used[a] - 1) & 1u, abort_flag))) { ok = false; continue; }
                         tc_fence_after();
                     }
                     const int grp = G0 + a;
 #pragma unroll
                     for (int t = 0; t <= grp; ++t)
-                        umma_bf16(tmem + (uint32_t)a * OZ_BM, plain_desc(a0 + (uint32_t)t * OZ_SLICE_BYTES),
-                                  plain_desc(b0 + (uint32_t)(grp - t) * OZ_SLICE_BYTES), (first && t == 0) ? 0u : 1u);
+                        if (lead)
+                            umma_lo<1>(tmem + (uint32_t)a * OZ_BM, a0 + (uint32_t)t * (OZ_SLICE_BYTES >> 4),
+                                       b0 + (uint32_t)(grp - t) * (OZ_SLICE_BYTES >> 4), hi, OZ_IDESC,
+                                       (first && t == 0) ? 0u : 1u);
                     if (last) {
-                        umma_commit(ready_bar(a));
+                        if (lead) umma_commit(ready_bar(a));
                         ++used[a];
                     }
                 }
-                umma_commit(empty_bar(s));
+                if (lead) umma_commit(empty_bar(s));
             }
         };
         using I = std::integral_constant<int, 0>;
