@@ -453,7 +453,7 @@ __device__ __forceinline__ void oz_drain(uint32_t taddr, long long (&tot)[64]) {
 // One CTA per 128 x 128 tile (and contraction split, and expert): warp 0
 // copies slabs, warp 1 issues the products, warps 2 .. 9 drain tensor memory.
 // Bound by the tensor cores: 28 products of 128 x 128 x 16 per 16 rows, each
-// slab read once per sweep for 22 (6) products.
+// slab read once per sweep for 18 (10) products.
 __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
     pdl_enter();
     extern __shared__ unsigned char gemm_smem_raw[];
@@ -514,7 +514,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
             const int s = it % OZ_STAGES;
             if (!wait_phase(empty_bar(s), ((uint32_t)(it / OZ_STAGES) & 1u) ^ 1u, abort_flag)) break;
             const bool high = it < nc;
-            const uint32_t bytes = high ? 3u * OZ_SLICE_BYTES : (uint32_t)OZ_SLAB_BYTES;
+            const uint32_t bytes = high ? (uint32_t)(OZ_HIGH * OZ_SLICE_BYTES) : (uint32_t)OZ_SLAB_BYTES;
             const unsigned long long off = (unsigned long long)(high ? it : it - nc) * OZ_SLAB_BYTES;
             const uint32_t dst = smem_s + (uint32_t)s * 2u * OZ_SLAB_BYTES;
             mbar_arrive_tx(full_bar(s), 2 * bytes);
@@ -528,8 +528,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
     } else if (warp == 1) {
         const bool lead = elect_one();
         const uint32_t hi = (uint32_t)(plain_desc(smem_s) >> 32), lo0 = (uint32_t)plain_desc(smem_s);
+        // Every group of a drain interval takes the next of the four
+        // accumulators in turn (use u: accumulator u % 4), so in the low sweep,
+        // with three groups, one is drained ahead of the products that need it
         bool ok = true;
-        int it = 0, used[4] = {0, 0, 0, 0};              // drains of each accumulator so far
+        int it = 0, use = 0;
         // one sweep: groups G0 .. G0 + NG - 1, a drain every STEPS steps
         auto sweep = [&](auto g0_c, auto ng_c, auto steps_c) {
             constexpr int G0 = decltype(g0_c)::value, NG = decltype(ng_c)::value, STEPS = decltype(steps_c)::value;
@@ -542,28 +545,28 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
 #pragma unroll
                 for (int a = 0; a < NG; ++a) {
                     if (!ok) continue;
-                    if (first && used[a] > 0) {
-                        if (!__all_sync(0xFFFFFFFFu, wait_phase(drained_bar(a), (uint32_t)(used[a] - 1) & 1u, abort_flag))) { ok = false; continue; }
+                    const int u = use + a;
+                    const uint32_t acc = (uint32_t)u & 3u;
+                    if (first && u >= 4) {
+                        if (!__all_sync(0xFFFFFFFFu, wait_phase(drained_bar(acc), (uint32_t)((u >> 2) - 1) & 1u, abort_flag))) { ok = false; continue; }
                         tc_fence_after();
                     }
                     const int grp = G0 + a;
 #pragma unroll
                     for (int t = 0; t <= grp; ++t)
                         if (lead)
-                            umma_lo<1>(tmem + (uint32_t)a * OZ_BM, a0 + (uint32_t)t * (OZ_SLICE_BYTES >> 4),
+                            umma_lo<1>(tmem + acc * OZ_BM, a0 + (uint32_t)t * (OZ_SLICE_BYTES >> 4),
                                        b0 + (uint32_t)(grp - t) * (OZ_SLICE_BYTES >> 4), hi, OZ_IDESC,
                                        (first && t == 0) ? 0u : 1u);
-                    if (last) {
-                        if (lead) umma_commit(ready_bar(a));
-                        ++used[a];
-                    }
+                    if (last && lead) umma_commit(ready_bar(acc));
                 }
+                if (last) use += NG;
                 if (lead) umma_commit(empty_bar(s));
             }
         };
-        using I = std::integral_constant<int, 0>;
-        sweep(I{}, std::integral_constant<int, 3>{}, std::integral_constant<int, OZ_STEPS_HIGH>{});
-        if (ok) sweep(std::integral_constant<int, 3>{}, std::integral_constant<int, 4>{}, std::integral_constant<int, OZ_STEPS_LOW>{});
+        sweep(std::integral_constant<int, 0>{}, std::integral_constant<int, OZ_HIGH>{}, std::integral_constant<int, OZ_STEPS_HIGH>{});
+        if (ok) sweep(std::integral_constant<int, OZ_HIGH>{}, std::integral_constant<int, OZ_SLICES - OZ_HIGH>{},
+                      std::integral_constant<int, OZ_STEPS_LOW>{});
         // products issued before a give-up still hold shared memory: wait for
         // them (the last commit of every stage that was read)
         if (!ok)
@@ -579,37 +582,38 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
         const long long q = g.q;
         double* const dst = g.part ? g.part + ((long long)split * gridDim.z + z) * q * q : g.C + z * g.c_stride;
         bool ok = true;
-        int used[4] = {0, 0, 0, 0};
-        auto take = [&](int a, auto w, long long (&tot)[64]) {
+        int use = 0;
+        auto take = [&](auto w, long long (&tot)[64]) {
             if (!ok) return;
-            if (!wait_phase(ready_bar(a), (uint32_t)used[a] & 1u, abort_flag)) { ok = false; return; }
+            const int acc = use & 3;
+            if (!wait_phase(ready_bar(acc), (uint32_t)(use >> 2) & 1u, abort_flag)) { ok = false; return; }
             tc_fence_after();
-            oz_drain<decltype(w)::value>(tq + (uint32_t)a * OZ_BM, tot);
+            oz_drain<decltype(w)::value>(tq + (uint32_t)acc * OZ_BM, tot);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(drained_bar(a));
-            ++used[a];
+            if (lane == 0) mbar_arrive(drained_bar(acc));
+            ++use;
         };
         long long tot[64];
 #pragma unroll
         for (int j = 0; j < 64; ++j) tot[j] = 0;
         for (int c = 0; c < nc && ok; c += OZ_STEPS_HIGH) {
-            take(0, std::integral_constant<int, 1 << 16>{}, tot);
-            take(1, std::integral_constant<int, 1 << 8>{}, tot);
-            take(2, std::integral_constant<int, 1>{}, tot);
+            take(std::integral_constant<int, 1 << 24>{}, tot);
+            take(std::integral_constant<int, 1 << 16>{}, tot);
+            take(std::integral_constant<int, 1 << 8>{}, tot);
+            take(std::integral_constant<int, 1>{}, tot);
         }
-        // the high groups' total waits in the output array (an integer below
-        // 2^53 for any contraction below 2^23 rows) while the low ones run
+        // the high groups' total waits in the output array (rounded once to
+        // binary64) while the low ones run
 #pragma unroll
         for (int j = 0; j < 64; ++j) {
             if (ok && row < q && colb + j < q) dst[row * q + colb + j] = (double)tot[j];
             tot[j] = 0;
         }
         for (int c = 0; c < nc && ok; c += OZ_STEPS_LOW) {
-            take(0, std::integral_constant<int, 1 << 24>{}, tot);
-            take(1, std::integral_constant<int, 1 << 16>{}, tot);
-            take(2, std::integral_constant<int, 1 << 8>{}, tot);
-            take(3, std::integral_constant<int, 1>{}, tot);
+            take(std::integral_constant<int, 1 << 16>{}, tot);
+            take(std::integral_constant<int, 1 << 8>{}, tot);
+            take(std::integral_constant<int, 1>{}, tot);
         }
         if (!ok) {
             if (lane == 0 && g.status) atomicCAS(g.status, 0, (int32_t)ISO_ERR_TIMEOUT);
@@ -622,7 +626,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
                 if (j % 4 == 0) asm volatile("" ::: "memory");   // keeps the loads of later columns behind (registers)
                 if (col >= q) continue;
                 const int ec = eb[col];
-                double v = fma(dst[row * q + col], 4294967296.0, (double)tot[j]);
+                double v = fma(dst[row * q + col], 16777216.0, (double)tot[j]);
                 v = (er >= OZ_NONFINITE || ec >= OZ_NONFINITE) ? __longlong_as_double(0x7FF8000000000000LL)
                                                                 : scalbn(v, er + ec - 62);
                 if (g.minus_identity && row == col) v -= 1.0;

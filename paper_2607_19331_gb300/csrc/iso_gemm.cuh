@@ -112,9 +112,9 @@ __global__ void k_gemm_x3(const __grid_constant__ CUtensorMap ta, const __grid_c
 //
 // Measured on one 3584 x 18944 matrix (q = 3584): A_i of three experts, both
 // sides, 1441 ms as binary64 on the CUDA cores (64 x 64 tiles, 1.2 TFLOP/s,
-// the chip's binary64 rate) against 42 ms here (28 bf16 products for each: 1.2
-// PFLOP/s); the merge 1533 -> 140 ms.  The optimizer step of a 1536 x 8960
-// matrix, bound by F^T F, 29.7 -> 9.2 ms.
+// the chip's binary64 rate) against 34 ms here (28 bf16 products for each: 1.4
+// PFLOP/s).  The optimizer step of a 1536 x 8960
+// matrix was bound by F^T F: 22.6 -> 1.0 ms.
 constexpr int OZ_SLICES = 7;
 constexpr int OZ_BM = 128;                              // columns of A (and of B) per tile
 constexpr int OZ_BK = 16;                               // contraction rows per step
@@ -124,13 +124,15 @@ constexpr int OZ_STAGES = 3;
 constexpr int OZ_EPI_WARPS = 8;
 constexpr int OZ_THREADS = 64 + 32 * OZ_EPI_WARPS;
 constexpr int OZ_SMEM = 128 + OZ_STAGES * 2 * OZ_SLAB_BYTES + 256;
-// Two sweeps over the contraction, three and four slice groups each (a group
-// takes 128 of the 512 tensor-memory columns): groups 0 .. 2 read slices
-// 0 .. 2, groups 3 .. 6 all seven.  Steps per drain: (group + 1) pairs x 16
-// rows x 2^14 <= 2^24.
-constexpr int OZ_STEPS_HIGH = 21;                       // 3 pairs x 336 rows <= 1024
+// Two sweeps over the contraction (a group takes 128 of the 512 tensor-memory
+// columns): groups 0 .. 3 read slices 0 .. 3, groups 4 .. 6 all seven, which
+// leaves the sweep with most of the work a fourth accumulator to drain into
+// registers behind the products.  Steps per drain: (group + 1) pairs x 16 rows
+// x 2^14 <= 2^24.
+constexpr int OZ_HIGH = 4;                              // groups of the first sweep
+constexpr int OZ_STEPS_HIGH = 16;                       // 4 pairs x 256 rows <= 1024
 constexpr int OZ_STEPS_LOW = 9;                         // 7 pairs x 144 rows <= 1024
-// 64-bit totals: |I_g| 2^(8 (6 - g)) summed over g = 3 .. 6 stays below 2^63
+// 64-bit totals: |I_g| 2^(8 (3 - g)) summed over g = 0 .. 3 stays below 2^63
 constexpr long long OZ_MAX_ROWS = 1LL << 20;
 constexpr int32_t OZ_NONFINITE = 1 << 20;               // exponent of a column holding a NaN or an infinity
 
