@@ -678,6 +678,8 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
         using BT = std::remove_pointer_t<decltype(bt)>;
         constexpr bool CK = decltype(ck)::value;
 
+        if (gram_mode == GRAM_ACCUM && !need_gram_pass)
+            ISO_TRY(launch(KD_SOLVE, s, [&] { pdl_launch(k_block_gamma, T, TPB, 0, s, P); }));
         if (gram_mode != GRAM_NONE) {
             if (need_gram_pass) {
                 auto gram = [&](auto kc) {

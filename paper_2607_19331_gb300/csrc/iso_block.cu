@@ -274,7 +274,7 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
             U.state = ST_DONE;
             if (want_gamma) {
                 const double ft = (double)__uint_as_float(tk);
-                atomicAdd(&P.gram[t], g + (double)need * ft * ft);
+                U.gamma = g + (double)need * ft * ft;
             }
             stats(tk, k, tot_above, tot_ties, need);
         }
@@ -404,11 +404,23 @@ __global__ void __launch_bounds__(BLOCK_TPB, BLOCK_CTAS_PER_SM) k_block_select(P
         U.state = ST_DONE;
         if (want_gamma) {
             const double ft = (double)__uint_as_float(tk);
-            atomicAdd(&P.gram[t], g + (double)need * ft * ft);
+            U.gamma = g + (double)need * ft * ft;
         }
         stats(tk, k, tot_above, tot_ties, need);
     }
     if (P.fuse_block) apply_block(tk, cut, false);
+}
+
+// K = 1 ISO: a tensor's Gamma from its units' sums, in a fixed order (one block
+// per tensor)
+__global__ void __launch_bounds__(TPB) k_block_gamma(Plan P) {
+    pdl_enter();
+    __shared__ double red[33];
+    const TensorDesc& d = P.tens[blockIdx.x];
+    double g = 0.0;
+    for (int b = threadIdx.x; b < d.nblocks; b += TPB) g += P.units[d.unit + b].gamma;
+    g = block_sum(g, red);
+    if (threadIdx.x == 0) P.gram[blockIdx.x] = g;
 }
 
 #define ISO_BLOCK_INST(XT, BT, CK) template __global__ void k_block_select<XT, BT, CK>(Plan);

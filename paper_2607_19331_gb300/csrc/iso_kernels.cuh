@@ -35,6 +35,7 @@ __global__ void k_radix_flat(Plan P);
 constexpr int BLOCK_TPB = 512;             // k_block_select: threads per unit (32 keys each on the fast path)
 constexpr int BLOCK_CTAS_PER_SM = 2;       // two units in flight per SM
 template <typename XT, typename BT, bool CK> __global__ void k_block_select(Plan P);
+__global__ void k_block_gamma(Plan P);
 
 // fused K = 1 pass (bf16 base and update)
 #ifndef ISO_FUSED_BLOCKS_PER_SM
