@@ -42,8 +42,10 @@ __device__ __forceinline__ float div_count(float a, int cnt, const float2* tab) 
 
 // outputs of two neighbouring entries in a tile with per-tile bounds; the
 // same operations in the same order as merged_fast, an unselected term left
-// out instead of added as +0 (the sums start at +0 and never become -0)
-template <int OPK, int KC>
+// out instead of added as +0 (the sums start at +0 and never become -0).
+// ALL: an untrimmed TIES tensor, every expert's value taken as it is (no pass
+// has looked at it, so a NaN, which no bound admits, is to reach the sum).
+template <int OPK, bool ALL, int KC>
 __device__ __forceinline__ void merge_pair(const float (&t0)[KC], const float (&t1)[KC], float a0, float a1,
                                            const float (&cf)[KC], const float (&bound)[KC], float lambda, int K,
                                            bool iso1d, const float2* tab, float& bad0, float& bad1, float& o0,
@@ -53,8 +55,8 @@ __device__ __forceinline__ void merge_pair(const float (&t0)[KC], const float (&
         float x0[KC], x1[KC], s0 = 0.0f, s1 = 0.0f;
 #pragma unroll
         for (int q = 0; q < KC; ++q) {
-            x0[q] = fabsf(t0[q]) > bound[q] ? t0[q] : 0.0f;
-            x1[q] = fabsf(t1[q]) > bound[q] ? t1[q] : 0.0f;
+            x0[q] = (ALL ? q < K : fabsf(t0[q]) > bound[q]) ? t0[q] : 0.0f;
+            x1[q] = (ALL ? q < K : fabsf(t1[q]) > bound[q]) ? t1[q] : 0.0f;
             add_rn2(s0, s1, s0, s1, x0[q], x1[q]);
         }
         const uint32_t b0 = __float_as_uint(s0) & 0x80000000u, b1 = __float_as_uint(s1) & 0x80000000u;
@@ -118,7 +120,7 @@ __device__ __forceinline__ void merge_pair(const float (&t0)[KC], const float (&
 // K = 3; 76 for ISO), now by HBM.  1.54G entries, bf16 checkpoints: RAM K = 3
 // 8.54 -> 2.91 ms (5.3 TB/s of 10 B per entry), ISO K = 3 4.71 -> 2.51 ms (6.1
 // TB/s), TIES K = 2 5.00 -> 2.35 ms; 0.70G entries, eight binary32 task vectors,
-// TIES: 5.03 -> 4.60 ms (5.5 TB/s).
+// TIES: 5.03 -> 4.66 ms (5.4 TB/s).
 template <typename XT, typename BT, bool CK, int KC, int OPF>
 __global__ void __launch_bounds__(TPB, 2) k_merge(Plan P) {
     pdl_enter();
@@ -177,7 +179,7 @@ __global__ void __launch_bounds__(TPB, 2) k_merge(Plan P) {
                 store_out<BT, E>(d.out, e, n, o);
             }
         };
-        auto fast = [&](auto opk_c) {
+        auto fast = [&](auto opk_c, auto all_c) {
             steps([&](long long, const Words<XT, E> (&x)[KC], const Words<BT, E>& b, float (&o)[E]) {
 #pragma unroll
                 for (int j = 0; j < E; j += 2) {
@@ -189,8 +191,8 @@ __global__ void __launch_bounds__(TPB, 2) k_merge(Plan P) {
                         t1[q] = word_f32<XT, E>(x[q], j + 1);
                         if (CK) sub_rn2(t0[q], t1[q], t0[q], t1[q], a0, a1);
                     }
-                    merge_pair<decltype(opk_c)::value, KC>(t0, t1, a0, a1, cf, bound, P.lambda, K, mp.iso1d, s_tab,
-                                                           bad0, bad1, o[j], o[j + 1]);
+                    merge_pair<decltype(opk_c)::value, decltype(all_c)::value, KC>(
+                        t0, t1, a0, a1, cf, bound, P.lambda, K, mp.iso1d, s_tab, bad0, bad1, o[j], o[j + 1]);
                 }
             });
         };
@@ -212,13 +214,14 @@ __global__ void __launch_bounds__(TPB, 2) k_merge(Plan P) {
                 }
             });
         } else if (OPF == OPF_TIES) {
-            fast(std::integral_constant<int, OPK_TIES>{});
+            if (mp.sel == SEL_ALL) fast(std::integral_constant<int, OPK_TIES>{}, std::true_type{});
+            else fast(std::integral_constant<int, OPK_TIES>{}, std::false_type{});
         } else if (OPF == OPF_RAM) {
-            fast(std::integral_constant<int, OPK_RAM>{});
+            fast(std::integral_constant<int, OPK_RAM>{}, std::false_type{});
         } else if (OPF == OPF_SUM || opk == OPK_SUM) {
-            fast(std::integral_constant<int, OPK_SUM>{});
+            fast(std::integral_constant<int, OPK_SUM>{}, std::false_type{});
         } else {
-            fast(std::integral_constant<int, OPK_ISO>{});
+            fast(std::integral_constant<int, OPK_ISO>{}, std::false_type{});
         }
     });
     // RAM reads every entry's magnitude: a NaN or infinity is reported

@@ -132,7 +132,7 @@ __device__ __forceinline__ void merge_params(const Plan& P, int t, int K, MergeP
     const int opk = (P.op == ISO_OP_TA || iso1d) ? OPK_SUM
                   : (P.op == ISO_OP_TIES ? OPK_TIES : (P.op == ISO_OP_RAM ? OPK_RAM : OPK_ISO));
     int sel;
-    if (opk == OPK_SUM || opk == OPK_RAM) sel = SEL_ALL;
+    if (opk == OPK_SUM || opk == OPK_RAM || (opk == OPK_TIES && !trim)) sel = SEL_ALL;
     else if (trim && P.scope == ISO_SCOPE_BLOCK) sel = SEL_BLOCK;
     else sel = SEL_PACKED;
     if (lane == 0) {
@@ -163,8 +163,6 @@ __device__ __forceinline__ void merge_params(const Plan& P, int t, int K, MergeP
     }
     __syncwarp();
 }
-
-__device__ __forceinline__ int sgnf(float v) { return (v > 0.0f) - (v < 0.0f); }
 
 // selection bits of the K experts at entry e (tensor-local), bit i for expert i
 template <int KC>
@@ -334,15 +332,6 @@ __device__ __forceinline__ float merged_fast(int opk, bool iso1d, float lambda, 
     return (upd == 0.0f) ? th0 : __fadd_rn(th0, upd);
 }
 
-template <int KC>
-__device__ __forceinline__ uint32_t fast_bits(const int (&T)[KC], int K, const float (&tau)[KC]) {
-    uint32_t bits = 0;
-#pragma unroll
-    for (int i = 0; i < KC; ++i)
-        if (i < K && (int)key_of(tau[i]) > T[i]) bits |= 1u << i;
-    return bits;
-}
-
 // the warp's tiles: beg, beg + step, ... below end -- dealt round-robin over
 // the warps (all warps sweep one window of the tensors together, for DRAM
 // page locality) or one contiguous range per warp
@@ -376,9 +365,6 @@ __device__ __forceinline__ long long tensor_tile_end(const Plan& P, int t) {
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, uint32_t src_bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" :: "r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async8(uint32_t dst, const void* src, uint32_t src_bytes) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" :: "r"(dst), "l"(src), "r"(src_bytes) : "memory");
 }
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>

@@ -60,3 +60,26 @@ def test_mean_of_three_is_the_division():
     ref = (s / np.float32(3)).astype(np.float32)
     got = out[0].cpu().numpy()
     assert np.array_equal(got.view(np.uint32), np.where(s == 0, np.float32(0), ref).view(np.uint32))
+
+
+@pytest.mark.parametrize("K", [2, 3, 4, 6])
+def test_untrimmed_ties_vector_with_nonfinite_values(K):
+    # a TIES vector left untrimmed is read by no counting pass: the call
+    # reports nothing, an infinity stays one, and next to a NaN (its sum has
+    # no sign) the agreeing set is the positive values.  The neighbouring
+    # entries are untouched by it: small whole numbers, every sum exact.
+    n = 1500
+    g = torch.Generator().manual_seed(7)
+    x = torch.randint(-4, 5, (K, n), generator=g).float()
+    x[0, 3::10] = float("nan")
+    x[1, 5::10] = float("inf")
+    th0 = torch.zeros(n)
+    out, st = iso.iso_merge([th0.to(DEV)], [[v.to(DEV)] for v in x], op="ties", density=0.2, lam=1.0, mask_1d=False, stats=True)
+    torch.cuda.synchronize()
+    assert int(st.status.item()) == 0
+    s = x.sum(0)
+    sign = torch.where(s.isnan(), torch.ones(n), s.sign())
+    agree = (x * sign > 0)
+    cnt = agree.sum(0)
+    m = torch.where(agree, x, torch.zeros_like(x)).sum(0) / cnt.clamp(min=1)
+    assert torch.equal(out[0].cpu(), m)
