@@ -9,7 +9,7 @@
 //              ISO   2-D: a = c, the tensor's retention coefficient (Sec. 4.2)
 //                    1-D: a = 1/K = 1, no mask                 (App. E, Algorithm 1)
 //            An update of exactly zero leaves theta_0 untouched.
-//            (K >= 2 and the Gram pass: iso_merge.cu)
+//            (K >= 2: iso_merge.cu; the Gram pass: iso_gram.cu)
 //   k_solve  (Gamma + ridge I) c = diag Gamma on the non-zero experts, clip
 //   k_mask   the mask itself as a packed bitmask
 //   k_delta  tau = theta_i - theta_0 in binary32

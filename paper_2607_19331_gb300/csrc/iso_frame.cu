@@ -28,23 +28,24 @@
 // * W* = W_0 + [E_U S_0 | U_0 S_0] [V* | E_V]^T with E_F = F* - F_0: the
 //   difference form keeps the low-precision products on the small motion;
 //   W_0 itself (the caller's matrix) replaces U_0 S_0 V_0^T.
-// * Precision.  A_i = F_0^T dF_i is binary64 on the CUDA cores: on dense
-//   spectra the frames rotate far inside near-degenerate singular subspaces
-//   while the proxies stay small, so Gamma is a difference of terms up to
-//   thousands of times larger than itself (the paper takes the merge in
-//   binary64 throughout).  The other large contractions (F_0 Y, xi*^T xi*,
-//   the Newton-Schulz products, (F_0 + xi*) R and the reconstruction) run on
-//   the tensor cores (k_gemm_tf32) as three tf32 products per pair (hi hi +
-//   hi lo + lo hi, x = hi + lo split in binary64) with binary32 accumulation,
-//   about 2^-22 relative per product; what they feed is the merged frame,
-//   whose error reaches W* only through products with the small motion.
-//   Everything else is binary64 on the CUDA cores.
+// * Precision.  A_i = F_0^T dF_i to binary64: on dense spectra the frames
+//   rotate far inside near-degenerate singular subspaces while the proxies
+//   stay small, so Gamma is a difference of terms up to thousands of times
+//   larger than itself (the paper takes the merge in binary64 throughout).
+//   It runs on the tensor cores all the same, from exact 8-bit slices of the
+//   columns (k_oz_gemm), as the optimizer step's F^T F does.  The other large
+//   contractions (F_0 Y, xi*^T xi*, the Newton-Schulz products,
+//   (F_0 + xi*) R and the reconstruction) are three tf32 products per pair
+//   (hi hi + hi lo + lo hi, x = hi + lo split in binary64; k_gemm_x3) with
+//   binary32 accumulation, about 2^-22 relative per product; what they feed
+//   is the merged frame, whose error reaches W* only through products with
+//   the small motion.  Everything else is binary64 on the CUDA cores.
 #include "iso_gemm.cuh"
 #include "iso_internal.cuh"
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
-#include <mutex>
 #include <vector>
 
 namespace iso {
@@ -214,49 +215,32 @@ __global__ void __launch_bounds__(256) k_fr_coldots(Frames f, const double* dots
         }
 }
 
-// Transposed split operand out[k][seg][j] (Qp rows of 2 Lr) of a d x q source,
-// j the source row (Lr = Dp; the stacked modes 4 and 5 put two d-row sources
-// one above the other, Lr = 2 Dp):
-//   0  F_0[j, k];  1  dF_i = s_i F_i - F_0;  2  X[j, k];  3  X[j, k] S_0[k]
-//   4  [F_0 ; X];  5  [X ; F_0 + X]
+// Transposed split operand out[k][seg][j] (Qp rows of 2 Dp) of the d x q
+// matrix X, j its row, or of X S_0 (S0 given)
 struct SplitT {
-    Frames f;
-    const double* dots;
+    long long d, q;
     const double* X;
-    const double* S0;
-    int mode, i;
+    const double* S0;      // optional column factors
     float* out;
     long long Dp, Qp;
 };
 __global__ void __launch_bounds__(256) k_fr_split_t(SplitT a) {
     pdl_enter();
     __shared__ double t[32][33];
-    const long long Lr = (a.mode >= 4) ? 2 * a.Dp : a.Dp;
     const long long r0 = (long long)blockIdx.x * 32, k0 = (long long)blockIdx.y * 32;
-    const long long d = a.f.d, q = a.f.q;
     for (int y = threadIdx.y; y < 32; y += 8) {
-        long long r = r0 + y;
-        const long long k = k0 + threadIdx.x;
-        int half = 0;
-        if (a.mode >= 4 && r >= a.Dp) { half = 1; r -= a.Dp; }
+        const long long r = r0 + y, k = k0 + threadIdx.x;
         double v = 0.0;
-        if (r < d && k < q) {
-            const long long e = r * q + k;
-            switch (a.mode) {
-                case 0: v = a.f.F0[e]; break;
-                case 1: v = fma(sign_of(a.dots, q, a.i, k), a.f.F[a.i][e], -a.f.F0[e]); break;
-                case 2: v = a.X[e]; break;
-                case 3: v = a.X[e] * a.S0[k]; break;
-                case 4: v = half ? a.X[e] : a.f.F0[e]; break;
-                case 5: v = half ? a.f.F0[e] + a.X[e] : a.X[e]; break;
-            }
+        if (r < a.d && k < a.q) {
+            v = a.X[r * a.q + k];
+            if (a.S0) v *= a.S0[k];
         }
         t[y][threadIdx.x] = v;
     }
     __syncthreads();
     for (int y = threadIdx.y; y < 32; y += 8) {
         const long long k = k0 + y, r = r0 + threadIdx.x;
-        if (k < a.Qp && r < Lr) put_split(a.out + k * 2 * Lr, Lr, r, t[threadIdx.x][y]);
+        if (k < a.Qp && r < a.Dp) put_split(a.out + k * 2 * a.Dp, a.Dp, r, t[threadIdx.x][y]);
     }
 }
 
@@ -843,24 +827,17 @@ int grid_of(long long work, int sms) {
     return (int)std::max(1LL, std::min(b, (long long)sms * 8));
 }
 
-int gemm_smem_optin() {
-    static int done = 0;
-    if (done) return ISO_OK;
-    if (cudaFuncSetAttribute(k_gemm_tf32, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM) != cudaSuccess)
-        return ISO_ERR_CUDA;
-    done = 1;
+// Large dynamic shared memory must be opted into once per kernel and device.
+template <auto Kernel>
+int smem_optin(int bytes) {
+    static std::atomic<unsigned long long> done{0};       // a bit per device
+    int d = 0;
+    if (cudaGetDevice(&d) != cudaSuccess) return ISO_ERR_CUDA;
+    const unsigned long long bit = d < 64 ? 1ull << d : 0;
+    if (done.load(std::memory_order_relaxed) & bit) return ISO_OK;
+    if (cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return ISO_ERR_CUDA;
+    done.fetch_or(bit, std::memory_order_relaxed);
     return ISO_OK;
-}
-
-int x3_smem_optin() {
-    static std::once_flag once;
-    static int rc = ISO_OK;
-    std::call_once(once, [] {
-        if (cudaFuncSetAttribute(k_gemm_x3<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, X3_SMEM) != cudaSuccess ||
-            cudaFuncSetAttribute(k_gemm_x3<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, X3_SMEM) != cudaSuccess)
-            rc = ISO_ERR_CUDA;
-    });
-    return rc;
 }
 
 // C (a_rows x b_rows) = A B^T over the three-product split: A and B are
@@ -879,7 +856,8 @@ int frame_gemm(cudaStream_t s, int sms, const float* A, long long a_rows, const 
     g.k_tiles = (int)(L / GEMM_BK);
     g.seg = (int)L;
     g.c_cols = (int)b_rows;
-    ISO_TRY(x3_smem_optin());
+    ISO_TRY(smem_optin<k_gemm_x3<128>>(X3_SMEM));
+    ISO_TRY(smem_optin<k_gemm_x3<256>>(X3_SMEM));
     const unsigned nz = A2 ? 2 : 1;
     const long long my = a_rows / GEMM_BM, t128 = my * (b_rows / 128) * nz, t256 = my * ((b_rows + 255) / 256) * nz;
     const bool wide = (t256 + sms - 1) / sms * 1900 <= (t128 + sms - 1) / sms * 1150;
@@ -958,10 +936,7 @@ int exact_product(cudaStream_t s, int sms, const OzSrc& src, int K, double* C, u
     else if (K <= 2) FR_LAUNCH((pdl_launch(k_oz_colmax<3>, mg, mb, 0, s, src, K + 1, rc)));
     else if (K <= 4) FR_LAUNCH((pdl_launch(k_oz_colmax<5>, mg, mb, 0, s, src, K + 1, rc)));
     else FR_LAUNCH((pdl_launch(k_oz_colmax<MAXK + 1>, mg, mb, 0, s, src, K + 1, rc)));
-    static std::once_flag once;
-    static cudaError_t opt = cudaSuccess;
-    std::call_once(once, [] { opt = cudaFuncSetAttribute(k_oz_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM); });
-    if (opt != cudaSuccess) return ISO_ERR_CUDA;
+    ISO_TRY(smem_optin<k_oz_gemm>(OZ_SMEM));
     if (scratch_bytes < slot * (K ? 2 : 1)) return ISO_ERR_WORKSPACE;
     const int most = (int)std::min<unsigned long long>(std::max(K, 1), scratch_bytes / slot - (K ? 1 : 0));
     auto split = [&](int z0, int nz, unsigned char* out) -> int {
@@ -1193,7 +1168,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
         // N = xi*^T xi*
         {
             SplitT st{};
-            st.f = fr[sd]; st.dots = dots; st.X = D(L.xi[sd]); st.mode = 2; st.out = F(L.ft4[sd]); st.Dp = Dp; st.Qp = Qp;
+            st.d = fr[sd].d; st.q = q; st.X = D(L.xi[sd]); st.out = F(L.ft4[sd]); st.Dp = Dp; st.Qp = Qp;
             FR_LAUNCH((pdl_launch(k_fr_split_t, dim3((unsigned)(Dp / 32), (unsigned)(Qp / 32)), dim3(32, 8), 0, s, st)));
             GemmArgs g{};
             g.mode = GEMM_STORE_F32; g.C = F(L.nq[sd]); g.ldc = Qp; g.M = (int)Qp; g.N = (int)Qp; g.status = &hdr->status;
@@ -1292,7 +1267,7 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
         G_W->data, G_W->dtype, m, n, L.Mp, L.Np, F(L.gwt4))));
     for (int sd = 0; sd < 2; ++sd) {
         SplitT st{};
-        st.f = fr[sd]; st.X = sd == 0 ? U : V; st.S0 = S0; st.mode = 3; st.Dp = sd == 0 ? L.Mp : L.Np; st.Qp = Qp;
+        st.d = fr[sd].d; st.q = q; st.X = sd == 0 ? U : V; st.S0 = S0; st.Dp = sd == 0 ? L.Mp : L.Np; st.Qp = Qp;
         st.out = F(sd == 0 ? L.su4 : L.sv4);
         FR_LAUNCH((pdl_launch(k_fr_split_t, dim3((unsigned)(st.Dp / 32), (unsigned)(Qp / 32)), dim3(32, 8), 0, s, st)));
     }
@@ -1360,7 +1335,7 @@ int32_t iso_gemm_tf32(const float* A, int64_t lda, const float* B, int64_t ldb, 
     CUtensorMap ta, tb;
     ISO_TRY(gemm_tensor_map(&ta, A, M, lda, lda));
     ISO_TRY(gemm_tensor_map(&tb, B, N, ldb, ldb));
-    ISO_TRY(gemm_smem_optin());
+    ISO_TRY(smem_optin<k_gemm_tf32>(GEMM_SMEM));
     GemmArgs g{};
     g.mode = GEMM_STORE_F32; g.C = C; g.ldc = ldc; g.M = (int)M; g.N = (int)N;
     g.k_tiles = (int)(Kc / GEMM_BK); g.a_k0 = (int)a_k0; g.b_k0 = (int)b_k0;
