@@ -240,9 +240,11 @@ def run_frame(args):
     projection (3584 x 18944, bf16 base ~ N(0, 0.02^2), K RL experts = base +
     N(0, (5e-4)^2), seeded).  The thin SVDs (torch.linalg, binary64, the one
     library step) are timed once and reported apart; a step is one
-    iso_frame_merge call on resident factors.  The roofline is that of the
-    dominant kernel, the tcgen05 product, timed live on the reconstruction's
-    shape (M = 3584, N = 18944, a contraction of 3 x 2 x 3584 tf32 terms)."""
+    iso_frame_merge call on resident factors.  The roofline is that of
+    the plain tcgen05 product (k_gemm_tf32), timed live on the
+    reconstruction's shape (M = 3584, N = 18944, a contraction of 3 x 2 x 3584
+    tf32 terms); the merge's own products (k_gemm_x3, k_oz_gemm) are among the
+    step's kernels."""
     import torch
     import paper_2607_19331_gb300 as iso
     dev = torch.device("cuda", 0)
@@ -288,7 +290,7 @@ def run_frame(args):
     torch.cuda.synchronize()
     prof = iso.profile_read()
     iso.profile_enable(False)
-    # the dominant kernel alone, on the reconstruction's shape
+    # the plain product alone, on the reconstruction's shape
     pad = lambda x: (x + 127) // 128 * 128
     Mp, Np, L = pad(m), pad(n), 2 * pad(min(m, n))
     A = torch.randn(Mp, 4 * L, device=dev)
@@ -335,9 +337,10 @@ def run_opt(args):
     """One ISO[AdamW] step (Sec. 4.3) of a Qwen2.5-7B gate/up projection
     (3584 x 18944, bf16 weights, binary64 frames from the weights' thin SVD,
     a seeded synthetic gradient ~ N(0, 1e-3^2)) at the paper's learning rate
-    7.5e-7.  A step is one iso_opt_step call; the roofline is that of the
-    step's tcgen05 factor-gradient product (M = 18944, N = 3584, a
-    contraction of 3 x 3584 tf32 terms), timed live."""
+    7.5e-7.  A step is one iso_opt_step call; the roofline is that of
+    the plain tcgen05 product (k_gemm_tf32) on the factor-gradient shape
+    (M = 18944, N = 3584, a contraction of 3 x 3584 tf32 terms), timed live;
+    the step's own products (k_gemm_x3, k_oz_gemm) are among its kernels."""
     import torch
     import paper_2607_19331_gb300 as iso
     dev = torch.device("cuda", 0)
