@@ -245,21 +245,16 @@ __global__ void __launch_bounds__(TPB, FUSED_BLOCKS_PER_SM) k_count_apply(Plan P
     for (uint32_t g = beg; g < end; g += step) {
         {
             const uint32_t bar = bar_s + 8u * s;
-            const uint32_t par = (phases >> s) & 1u;
-            int spin = 0;
-            while (!mbar_try_wait(bar, par)) {
-                if (++spin >= MBAR_SPIN_LIMIT) {
-                    // give up: report, then wait (bounded) for the copies this
-                    // warp still has in flight before the block may exit
-                    if (lane == 0) set_status(P.hdr, ISO_ERR_TIMEOUT);
-                    const uint32_t pend = min((end - g + step - 1) / step, (uint32_t)FUSED_STAGES);
-                    for (uint32_t j = 0; j < pend; ++j) {
-                        const int sj = (s + (int)j) % FUSED_STAGES;
-                        for (int r = 0; r < MBAR_SPIN_LIMIT; ++r)
-                            if (mbar_try_wait(bar_s + 8u * sj, (phases >> sj) & 1u)) break;
-                    }
-                    return;
+            if (!mbar_wait_warp(bar, (phases >> s) & 1u)) {
+                // give up: report, then wait (bounded) for the copies this
+                // warp still has in flight before the block may exit
+                if (lane == 0) set_status(P.hdr, ISO_ERR_TIMEOUT);
+                const uint32_t pend = min((end - g + step - 1) / step, (uint32_t)FUSED_STAGES);
+                for (uint32_t j = 0; j < pend; ++j) {
+                    const int sj = (s + (int)j) % FUSED_STAGES;
+                    mbar_wait(bar_s + 8u * sj, (phases >> sj) & 1u);
                 }
+                return;
             }
             phases ^= 1u << s;
         }

@@ -116,6 +116,11 @@ __device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volati
     *abort_flag = 1;
     return false;
 }
+// The same for a whole warp, with one answer for all of its lanes: what
+// follows (tensor-memory loads, products, shuffles) takes every lane.
+__device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
+    return __all_sync(0xFFFFFFFFu, wait_phase(bar, parity, abort_flag));
+}
 
 // c / (sqrt(x) + eps) in binary64.  The division and square root instructions'
 // sequences made up most of the epilogue's binary64 work; here a binary32
@@ -238,8 +243,7 @@ k_gemm_tf32(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
         // every copy this thread issued has landed before the CTA may exit
         for (int kt = (issued > GEMM_STAGES ? issued - GEMM_STAGES : 0); kt < issued; ++kt) {
             const int s = kt % GEMM_STAGES;
-            for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
-                if (mbar_try_wait(full_bar(s), (uint32_t)(kt / GEMM_STAGES) & 1u)) break;
+            mbar_wait(full_bar(s), (uint32_t)(kt / GEMM_STAGES) & 1u);
         }
     } else if (warp == 1 && lane == 0) {
         // products: four K = 8 steps per 128-byte stage, the descriptor's start
@@ -262,10 +266,14 @@ k_gemm_tf32(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
     __syncwarp();
 
     // epilogue: one accumulator row per thread, 32 columns per tensor-memory load
-    const bool ok = wait_phase(accum_bar, 0u, abort_flag) && !*abort_flag;
+    const bool ok = __all_sync(0xFFFFFFFFu, wait_phase(accum_bar, 0u, abort_flag) && !*abort_flag);
     tc_fence_after();
     if (!ok) {
-        if (threadIdx.x == 0 && g.status) atomicCAS(g.status, 0, (int32_t)ISO_ERR_TIMEOUT);
+        if (lane == 0 && g.status) atomicCAS(g.status, 0, (int32_t)ISO_ERR_TIMEOUT);
+        // tensor memory is freed only when no product writes to it any more
+        // (the abort flag cuts the wait above short)
+        mbar_wait(accum_bar, 0u);
+        __syncwarp();
     } else {
         const int r = warp * 32 + lane;
         const long long row = (long long)m0 + r;
@@ -355,16 +363,14 @@ k_gemm_x3(const __grid_constant__ CUtensorMap ta1, const __grid_constant__ CUten
             ++issued;
         }
         // every copy this thread issued has landed before the CTA may exit
-        for (int kt = (issued > STAGES ? issued - STAGES : 0); kt < issued; ++kt) {
-            for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
-                if (mbar_try_wait(full_bar(kt % STAGES), (uint32_t)(kt / STAGES) & 1u)) break;
-        }
+        for (int kt = (issued > STAGES ? issued - STAGES : 0); kt < issued; ++kt)
+            mbar_wait(full_bar(kt % STAGES), (uint32_t)(kt / STAGES) & 1u);
     } else if (warp == 1) {
         const bool lead = elect_one();
         const uint32_t hi = (uint32_t)(sw128_desc(smem_s) >> 32), lo0 = (uint32_t)sw128_desc(smem_s);
         for (int kt = 0; kt < KT; ++kt) {
             const int s = kt % STAGES;
-            if (!__all_sync(0xFFFFFFFFu, wait_phase(full_bar(s), (uint32_t)(kt / STAGES) & 1u, abort_flag))) break;
+            if (!wait_phase_warp(full_bar(s), (uint32_t)(kt / STAGES) & 1u, abort_flag)) break;
             tc_fence_after();
             const uint32_t a0 = lo0 + (uint32_t)(s * (STAGE_BYTES >> 4)), b0 = a0 + (2 * A_BYTES >> 4);
 #pragma unroll
@@ -384,10 +390,14 @@ k_gemm_x3(const __grid_constant__ CUtensorMap ta1, const __grid_constant__ CUten
     }
     __syncwarp();
 
-    const bool ok = wait_phase(accum_bar, 0u, abort_flag) && !*abort_flag;
+    const bool ok = __all_sync(0xFFFFFFFFu, wait_phase(accum_bar, 0u, abort_flag) && !*abort_flag);
     tc_fence_after();
     if (!ok) {
-        if (threadIdx.x == 0 && g.status) atomicCAS(g.status, 0, (int32_t)ISO_ERR_TIMEOUT);
+        if (lane == 0 && g.status) atomicCAS(g.status, 0, (int32_t)ISO_ERR_TIMEOUT);
+        // tensor memory is freed only when no product writes to it any more
+        // (the abort flag cuts the wait above short)
+        mbar_wait(accum_bar, 0u);
+        __syncwarp();
     } else {
         const long long row = (long long)m0 + warp * 32 + lane;
         const uint32_t tq = tmem + ((uint32_t)(warp * 32) << 16);
@@ -522,9 +532,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
             bulk_g2s(dst + OZ_SLAB_BYTES, gb + off, bytes, full_bar(s));
         }
         // every copy this thread issued has landed before the CTA may exit
+#pragma unroll 1
         for (int k = (it > OZ_STAGES ? it - OZ_STAGES : 0); k < it; ++k)
-            for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
-                if (mbar_try_wait(full_bar(k % OZ_STAGES), (uint32_t)(k / OZ_STAGES) & 1u)) break;
+            mbar_wait(full_bar(k % OZ_STAGES), (uint32_t)(k / OZ_STAGES) & 1u);
     } else if (warp == 1) {
         const bool lead = elect_one();
         const uint32_t hi = (uint32_t)(plain_desc(smem_s) >> 32), lo0 = (uint32_t)plain_desc(smem_s);
@@ -538,7 +548,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
             constexpr int G0 = decltype(g0_c)::value, NG = decltype(ng_c)::value, STEPS = decltype(steps_c)::value;
             for (int c = 0; c < nc && ok; ++c, ++it) {
                 const int s = it % OZ_STAGES;
-                if (!__all_sync(0xFFFFFFFFu, wait_phase(full_bar(s), (uint32_t)(it / OZ_STAGES) & 1u, abort_flag))) { ok = false; break; }
+                if (!wait_phase_warp(full_bar(s), (uint32_t)(it / OZ_STAGES) & 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 const bool first = c % STEPS == 0, last = c % STEPS == STEPS - 1 || c == nc - 1;
                 const uint32_t a0 = lo0 + (uint32_t)s * (2u * OZ_SLAB_BYTES >> 4), b0 = a0 + (OZ_SLAB_BYTES >> 4);
@@ -548,7 +558,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
                     const int u = use + a;
                     const uint32_t acc = (uint32_t)u & 3u;
                     if (first && u >= 4) {
-                        if (!__all_sync(0xFFFFFFFFu, wait_phase(drained_bar(acc), (uint32_t)((u >> 2) - 1) & 1u, abort_flag))) { ok = false; continue; }
+                        if (!wait_phase_warp(drained_bar(acc), (uint32_t)((u >> 2) - 1) & 1u, abort_flag)) { ok = false; continue; }
                         tc_fence_after();
                     }
                     const int grp = G0 + a;
@@ -567,12 +577,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
         sweep(std::integral_constant<int, 0>{}, std::integral_constant<int, OZ_HIGH>{}, std::integral_constant<int, OZ_STEPS_HIGH>{});
         if (ok) sweep(std::integral_constant<int, OZ_HIGH>{}, std::integral_constant<int, OZ_SLICES - OZ_HIGH>{},
                       std::integral_constant<int, OZ_STEPS_LOW>{});
-        // products issued before a give-up still hold shared memory: wait for
-        // them (the last commit of every stage that was read)
-        if (!ok)
-            for (int k = (it > OZ_STAGES ? it - OZ_STAGES : 0); k < it; ++k)
-                for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
-                    if (mbar_try_wait(empty_bar(k % OZ_STAGES), (uint32_t)(k / OZ_STAGES) & 1u)) break;
+        // the products use shared and tensor memory until they complete, also
+        // where this warp or a drain gave up: wait for them (the last commit of
+        // every stage that was read)
+#pragma unroll 1
+        for (int k = (it > OZ_STAGES ? it - OZ_STAGES : 0); k < it; ++k)
+            mbar_wait(empty_bar(k % OZ_STAGES), (uint32_t)(k / OZ_STAGES) & 1u);
+        __syncwarp();
     } else if (warp >= 2) {
         // lane of tensor memory: 32 (warp % 4) + lane; columns 64 h .. + 63
         const int quad = warp & 3, h = (warp - 2) >> 2;
@@ -586,7 +597,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) k_oz_gemm(OzArgs g) {
         auto take = [&](auto w, long long (&tot)[64]) {
             if (!ok) return;
             const int acc = use & 3;
-            if (!wait_phase(ready_bar(acc), (uint32_t)(use >> 2) & 1u, abort_flag)) { ok = false; return; }
+            ok = wait_phase_warp(ready_bar(acc), (uint32_t)(use >> 2) & 1u, abort_flag);
+            if (!ok) return;
             tc_fence_after();
             oz_drain<decltype(w)::value>(tq + (uint32_t)acc * OZ_BM, tot);
             tc_fence_before();

@@ -713,6 +713,16 @@ __device__ __forceinline__ void fence_proxy_async_smem() {
 // probes of one barrier phase before a wait gives up: at most about four
 // seconds of suspension in all
 constexpr int MBAR_SPIN_LIMIT = 1 << 22;
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
+    for (int spin = 0; spin < MBAR_SPIN_LIMIT; ++spin)
+        if (mbar_try_wait(bar, parity)) return true;
+    return false;
+}
+// The same for a whole warp, with one answer for all of its lanes: what
+// follows a wait (shuffles, votes, tensor-memory loads) takes every lane.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity) {
+    return __all_sync(0xFFFFFFFFu, mbar_wait(bar, parity));
+}
 
 // Retention coefficients (Sec. 4.2; App. E, Retention coefficients): on the
 // experts with Gamma_ii > 0, (Gamma + ridge I) c = diag(Gamma) by Gaussian

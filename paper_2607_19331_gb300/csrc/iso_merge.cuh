@@ -456,20 +456,17 @@ __device__ __forceinline__ bool stream_chunks(const Plan& P, int K, const WarpRa
 #pragma unroll 1
     for (long long i = 0; i < NC; ++i) {
         const uint32_t bar = bar_s + 8u * s;
-        int spin = 0;
-        while (!mbar_try_wait(bar, (phases >> s) & 1u)) {
-            if (++spin >= MBAR_SPIN_LIMIT) {
-                // give up: report, then wait (bounded) for the copies this
-                // warp still has in flight before the block may exit
-                if (lane == 0) set_status(P.hdr, ISO_ERR_TIMEOUT);
-                const int pend = (int)(NC - i < D ? NC - i : D);
-                for (int j = 0; j < pend; ++j) {
-                    const int sj = (s + j) % D;
-                    for (int r = 0; r < MBAR_SPIN_LIMIT; ++r)
-                        if (mbar_try_wait(bar_s + 8u * sj, (phases >> sj) & 1u)) break;
-                }
-                return false;
+        if (!mbar_wait_warp(bar, (phases >> s) & 1u)) {
+            // give up: report, then wait (bounded) for the copies this
+            // warp still has in flight before the block may exit
+            if (lane == 0) set_status(P.hdr, ISO_ERR_TIMEOUT);
+            const int pend = (int)(NC - i < D ? NC - i : D);
+            for (int j = 0; j < pend; ++j) {
+                const int sj = (s + j) % D;
+                mbar_wait(bar_s + 8u * sj, (phases >> sj) & 1u);
             }
+            __syncwarp();
+            return false;
         }
         phases ^= 1u << s;
         body(wr.tile(i / G::CPT), (int)(i % G::CPT), ring + s * G::BYTES);
