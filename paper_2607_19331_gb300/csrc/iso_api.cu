@@ -224,11 +224,9 @@ long long blocks_of(const iso_tensor& t, const iso_topk_cfg& c) {
     return ((t.rows + c.block_rows - 1) / c.block_rows) * ((t.cols + c.block_cols - 1) / c.block_cols);
 }
 
-// candidate capacity of one unit of n entries at density rho, a multiple of
-// four slots (k_tie reads the segment 16 bytes at a time)
+// candidate capacity of one unit of n entries at density rho
 unsigned long long cand_cap_of(long long n, double rho, bool quantized) {
-    auto up4 = [](unsigned long long v) { return (v + 3) & ~3ull; };
-    if (n <= SAMPLE_MAX) return up4((unsigned long long)n);   // exact band: its ties
+    if (n <= SAMPLE_MAX) return (unsigned long long)n;   // exact band: its ties
     double kk = std::floor(rho * (double)n + 0.5);
     kk = std::min(std::max(kk, 0.0), (double)n);
     const double q = kk / (double)n;
@@ -242,7 +240,7 @@ unsigned long long cand_cap_of(long long n, double rho, bool quantized) {
     // (few significant bits) and binary32 ones essentially do not
     const double ties = quantized ? 0.08 : 0.004;
     const double cap = 8192.0 + std::ceil((2.0 * band + ties) * (double)n) + waste;
-    return up4((unsigned long long)std::min(cap, (double)n));
+    return (unsigned long long)std::min(cap, (double)n);
 }
 
 // Value slots of one unit's compact candidates (keys >= lo, about the kept

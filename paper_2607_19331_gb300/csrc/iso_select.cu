@@ -1296,23 +1296,23 @@ __global__ void __launch_bounds__(TPB) k_tie(Plan P) {
         uint32_t* tc = P.tcnt + (long long)c.i * P.n_tiles + c.g;
         double g_warp = 0.0;
         if (U->r_src == SRC_CAND) {
-            // one tile's candidate list per thread, 16-byte loads (segments
-            // start at and are padded to multiples of four slots)
-            const uint32_t* cs = P.cand + U->cand_off;
+            // one tile's candidate list per thread, by whole 16-byte words of
+            // the candidate array (which starts and ends at a 256-byte
+            // boundary); slots of neighbouring lists and units are passed over
             for (long long q0 = 0; q0 < ntile; q0 += blockDim.x) {
                 const long long q = q0 + threadIdx.x;
                 uint32_t cnt = 0;
                 float fg = 0.0f;
                 if (q < ntile) {
                     const uint2 r = P.tcand[(long long)c.i * P.n_tiles + c.g + q];
-                    const uint32_t r1 = r.x + r.y;
-                    auto one = [&](uint32_t j, uint32_t kk) {
-                        if (j < r.x || j >= r1) return;
+                    const unsigned long long r0 = U->cand_off + r.x, r1 = r0 + r.y;
+                    auto one = [&](unsigned long long j, uint32_t kk) {
+                        if (j < r0 || j >= r1) return;
                         cnt += (kk == tk);
                         if (want_g && kk > tk) { const float f = __uint_as_float(kk); fg = __fmaf_rn(f, f, fg); }
                     };
-                    for (uint32_t j = r.x & ~3u; j < r1; j += 4) {
-                        const uint4 w = *reinterpret_cast<const uint4*>(cs + j);
+                    for (unsigned long long j = r0 & ~3ull; j < r1; j += 4) {
+                        const uint4 w = *reinterpret_cast<const uint4*>(P.cand + j);
                         one(j, w.x); one(j + 1, w.y); one(j + 2, w.z); one(j + 3, w.w);
                     }
                     if (want_cnt) tc[q] = cnt;

@@ -378,3 +378,19 @@ def test_range_selection_argument_errors():
     assert L.iso_range_mask(x, base, 0, 10_000, 5, 0, mask, None, 80, None) == _abi.ISO_ERR_WORKSPACE
     assert L.iso_range_mask(x, base, 0, 10_000, 5, 0, None, ws, 80, None) == _abi.ISO_ERR_ARG
     assert L.iso_range_mask(x, base, 7, 7, 5, 0, None, None, 0, None) == 0     # an empty range is a no-op
+
+
+def test_candidate_segments_take_no_padding():
+    # units of at most the sample's size reserve one 4-byte candidate slot per
+    # entry: 64 tensors of 4097 and of 4100 entries (the same tiles) differ by
+    # 64 * 3 slots and nothing else, for one expert and for three
+    L = _abi.lib()
+
+    def minimum(n, K):
+        ts = _arr(*[_fake(1, n, is_1d=1, dtype=_abi.ISO_F32) for _ in range(64)])
+        mn, full = ctypes.c_size_t(), ctypes.c_size_t()
+        assert L.iso_workspace_size(ts, 64, K, ctypes.byref(iso.merge_cfg("ties", 0.2)), ctypes.byref(mn),
+                                    ctypes.byref(full)) == 0
+        return full.value
+    for K in (1, 3):
+        assert minimum(4100, K) - minimum(4097, K) == K * 64 * 3 * 4
