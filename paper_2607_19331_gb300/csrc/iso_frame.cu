@@ -324,50 +324,72 @@ struct OzSrc {
     unsigned long long* mx;          // [1 + K][q] largest |bits| of each column (zeroed by the caller)
     int32_t* ex;                     // [1 + K][Qp] column exponents
     long long Qp;
+    int32_t* peaked;                 // [1 + K][1 + q]: how many columns are left to binary64, and which
 };
-__device__ __forceinline__ double oz_value(const OzSrc& a, int z, long long e, long long k) {
+// entry e of source z (sg: the column's sign s_ik, for z > 0)
+__device__ __forceinline__ double oz_signed(const OzSrc& a, int z, long long e, double sg) {
     if (z == 0) return a.X ? a.f.F0[e] + a.X[e] : a.f.F0[e];
-    return fma(sign_of(a.dots, a.f.q, z - 1, k), a.f.F[z - 1][e], -a.f.F0[e]);
+    return fma(sg, a.f.F[z - 1][e], -a.f.F0[e]);
+}
+__device__ __forceinline__ double oz_value(const OzSrc& a, int z, long long e, long long k) {
+    return oz_signed(a, z, e, z ? sign_of(a.dots, a.f.q, z - 1, k) : 0.0);
 }
 
 // every column's largest magnitude, all sources in one pass (reads each
-// array once: bound by HBM)
+// array once: bound by HBM), and its sum of squares in binary32, one partial
+// per row chunk (part[chunk][source][column]; summed in order by
+// k_oz_columns, so that the same input always gives the same sum)
 template <int SC>
-__global__ void __launch_bounds__(256) k_oz_colmax(OzSrc a, int sources, int row_chunks) {
+__global__ void __launch_bounds__(256) k_oz_colmax(OzSrc a, int sources, int row_chunks, float* part) {
     pdl_enter();
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.y == 0 && (int)threadIdx.x < sources)
+        a.peaked[threadIdx.x * (1 + a.f.q)] = 0;
     const long long k = (long long)blockIdx.x * 32 + threadIdx.x;
     const long long per = (a.f.d + row_chunks - 1) / row_chunks;
     const long long r0 = (long long)blockIdx.y * per, r1 = k < a.f.q ? min(a.f.d, r0 + per) : r0;
     unsigned long long m[SC];
+    float ss[SC];
     double sg[SC];
 #pragma unroll
-    for (int z = 0; z < SC; ++z) m[z] = 0;
+    for (int z = 0; z < SC; ++z) { m[z] = 0; ss[z] = 0.0f; }
 #pragma unroll
     for (int i = 0; i + 1 < SC; ++i) sg[i] = i + 1 < sources && k < a.f.q ? sign_of(a.dots, a.f.q, i, k) : 0.0;
-    auto up = [](unsigned long long& x, double v) {
+    // the square from the value cut to binary32 by integer arithmetic (20
+    // mantissa bits; below 2^-63 zero, which only ever makes the sum smaller)
+    auto up = [](unsigned long long& x, float& s, double v) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
         x = b > x ? b : x;
+        const uint32_t h = (uint32_t)(b >> 32);
+        const float f = __uint_as_float(h < 0x3C000000u ? 0u : (h - 0x38000000u) << 3);
+        s = __fmaf_rn(f, f, s);
     };
 #pragma unroll 4
     for (long long r = r0 + threadIdx.y; r < r1; r += 8) {
         const long long e = r * a.f.q + k;
         const double f0 = a.f.F0[e];
-        up(m[0], a.X ? f0 + a.X[e] : f0);
+        up(m[0], ss[0], a.X ? f0 + a.X[e] : f0);
 #pragma unroll
         for (int i = 0; i + 1 < SC; ++i)
-            if (i + 1 < sources) up(m[i + 1], fma(sg[i], a.f.F[i][e], -f0));
+            if (i + 1 < sources) up(m[i + 1], ss[i + 1], fma(sg[i], a.f.F[i][e], -f0));
     }
     // the block's rows first: one atomic per column and block
     __shared__ unsigned long long red[8][33];
+    __shared__ float reds[8][33];
 #pragma unroll
     for (int z = 0; z < SC; ++z) {
         if (z >= sources) break;
         red[threadIdx.y][threadIdx.x] = m[z];
+        reds[threadIdx.y][threadIdx.x] = ss[z];
         __syncthreads();
         if (threadIdx.y == 0 && k < a.f.q) {
             unsigned long long v = m[z];
-            for (int y = 1; y < 8; ++y) v = red[y][threadIdx.x] > v ? red[y][threadIdx.x] : v;
+            float s = ss[z];
+            for (int y = 1; y < 8; ++y) {
+                v = red[y][threadIdx.x] > v ? red[y][threadIdx.x] : v;
+                s += reds[y][threadIdx.x];
+            }
             atomicMax(&a.mx[(long long)z * a.f.q + k], v);
+            part[((long long)blockIdx.y * sources + z) * a.f.q + k] = s;
         }
         __syncthreads();
     }
@@ -379,6 +401,108 @@ __device__ __forceinline__ int oz_exponent(unsigned long long bits) {
     const int be = (int)(bits >> 52);
     if (be >= 0x7FF) return OZ_NONFINITE;
     return max(be - 1022, -900);
+}
+
+// Which columns the slices cannot hold well enough: an entry of the product is
+// off by about sqrt(d) 2^-56.3 2^(e_a + e_b) (the slice pairs left out), a
+// binary64 sum by about 2^-55 |a| |b|, so the slices are the nearer ones while
+// 2^e <= 1.6 d^(-1/4) |x| for both columns.  Dense columns are (random ones
+// from d = 200 on: 2^e is at most 8 |x| / sqrt(d)); a column with an entry that
+// holds much of its norm is not, and its entries come from k_oz_f64.  RMS error
+// over |a| |b| of the slices and of the binary64 sum, d = 3584: dense 9e-18 and
+// 4e-17; a peak of 0.2 of the norm in each column, on different rows, 4.9e-17
+// and 4.1e-17 (ratio 1.94); of 0.5, 6.6e-16 and 3.2e-17.  Columns outside
+// 2^-55 .. 2^50, where the binary32 sum of squares does not reach, are left to
+// binary64 as well; zero columns are exact, and non-finite ones NaN either way.
+__global__ void __launch_bounds__(256) k_oz_columns(OzSrc a, int sources, int row_chunks, const float* part) {
+    pdl_enter();
+    const long long q = a.f.q, k = (long long)blockIdx.x * 256 + threadIdx.x;
+    const int z = blockIdx.y;
+    if (k >= q) return;
+    const unsigned long long bits = a.mx[(long long)z * q + k];
+    const int e = oz_exponent(bits);
+    if (bits == 0 || e >= OZ_NONFINITE) return;
+    float s = 0.0f;
+    for (int c = 0; c < row_chunks; ++c) s += part[((long long)c * sources + z) * q + k];
+    const float lim = 1.6f * 1.6f * rsqrtf((float)a.f.d);            // of (2^e / |x|)^2
+    if (e < -55 || e > 50 || !(exp2f((float)(2 * e)) <= lim * s)) {
+        int32_t* const list = a.peaked + z * (1 + q);
+        list[1 + atomicAdd(&list[0], 1)] = (int32_t)k;
+    }
+}
+
+// The product's entries of those columns, summed in binary64 on the CUDA cores
+// in row order: peaked columns of the first operand against every column of
+// the second, and every column of the first against peaked ones of the second
+// (an entry of both is written twice, the same sum).  A block takes a group of
+// 8 listed columns, one per warp, against 32 columns of the other operand, one
+// entry per thread: the binary64 rate (two sums a clock and SM) is what bounds
+// it, so a few listed columns are better spread over many blocks than tiled
+// (one column of a 1216 x 576 frame: 670 us in 64 x 64 tiles).  32 rows a
+// step, the next ones' loads in flight.  Without such columns, the usual
+// case, the blocks return at once.
+constexpr int OZF_LIST = 8, OZF_COLS = 32, OZF_ROWS = 32;
+__global__ void __launch_bounds__(256) k_oz_f64(OzSrc a, int K, double* C) {
+    pdl_enter();
+    __shared__ double sl[OZF_ROWS][OZF_LIST], so[OZF_ROWS][OZF_COLS];
+    const long long q = a.f.q, d = a.f.d;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long nt = (q + OZF_COLS - 1) / OZF_COLS;
+    auto groups = [&](int z) { return (long long)(a.peaked[z * (1 + q)] + OZF_LIST - 1) / OZF_LIST; };
+    const long long ga = groups(0) * nt;              // work items of the first operand's columns, per pair
+    long long first = 0;                              // first work item of this pair
+    for (int i = 0; i < (K ? K : 1); ++i) {
+        const int zb = K ? 1 + i : 0;
+        const long long items = ga + (K ? groups(zb) * nt : 0);
+        // this block's items, counted over all pairs
+        long long w = ((long long)blockIdx.x - first % gridDim.x + gridDim.x) % gridDim.x;
+        for (; w < items; w += gridDim.x) {
+            const bool rows = w < ga;                 // the listed column is the product's row
+            const int zl = rows ? 0 : zb, zo = rows ? zb : 0;
+            const long long v = rows ? w : w - ga;
+            const int32_t* const list = a.peaked + zl * (1 + q);
+            auto listed = [&](int x) { const long long at = v / nt * OZF_LIST + x; return at < list[0] ? (long long)list[1 + at] : -1LL; };
+            const long long kl = listed(threadIdx.x & (OZF_LIST - 1));    // the column this thread loads from
+            const long long kw = listed(warp), ko = v % nt * OZF_COLS + lane;
+            const double gl = zl && kl >= 0 ? sign_of(a.dots, q, zl - 1, kl) : 0.0;
+            const double go = zo && ko < q ? sign_of(a.dots, q, zo - 1, ko) : 0.0;
+            double nl, no[OZF_ROWS / 8];
+            auto load = [&](long long r0) {
+                const long long rl = r0 + threadIdx.x / OZF_LIST;
+                nl = rl < d && kl >= 0 ? oz_signed(a, zl, rl * q + kl, gl) : 0.0;
+#pragma unroll
+                for (int y = 0; y < OZF_ROWS / 8; ++y) {
+                    const long long ro = r0 + 8 * y + warp;
+                    no[y] = ro < d && ko < q ? oz_signed(a, zo, ro * q + ko, go) : 0.0;
+                }
+            };
+            double acc = 0.0;
+            load(0);
+            for (long long r0 = 0; r0 < d; r0 += OZF_ROWS) {
+                __syncthreads();
+                sl[threadIdx.x / OZF_LIST][threadIdx.x & (OZF_LIST - 1)] = nl;
+#pragma unroll
+                for (int y = 0; y < OZF_ROWS / 8; ++y) so[8 * y + warp][lane] = no[y];
+                __syncthreads();
+                load(r0 + OZF_ROWS);
+                if (kw >= 0) {
+#pragma unroll
+                    for (int r = 0; r < OZF_ROWS; ++r) acc = fma(sl[r][warp], so[r][lane], acc);
+                }
+            }
+            if (kw >= 0 && ko < q) {
+                const long long k = rows ? kw : ko, l = rows ? ko : kw;
+                if (K) {
+                    C[((long long)i * q + k) * q + l] = acc;
+                } else {
+                    acc -= k == l ? 1.0 : 0.0;
+                    C[k * q + l] = acc;
+                    C[l * q + k] = acc;
+                }
+            }
+        }
+        first += items;
+    }
 }
 
 // The slabs of source z0 + blockIdx.z (slot blockIdx.z of `out`): thread =
@@ -770,6 +894,7 @@ struct FrameLayout {
     long long m, n, q, Mp, Np, Qp, K;
     size_t hdr, gram, coef, dots, mx[2], zero_end, ex, vcopy;
     size_t tail;      // from here on: unused until A_i is formed (its operands' slabs)
+                      // (sym[side] holds the side's list of peaked columns until then)
     size_t cd[2], ft4[2], aq[2], sym[2], kw[2], fr4[2], y4[2], e[2], xi[2], nq[2];
     size_t ns_y, ns_z, ns_m, ns_y4, ns_z4, ns_m4, ns_t1, ns_t2, ns_t3;
     size_t a6, b6, total;
@@ -920,8 +1045,9 @@ OptLayout opt_layout(long long m, long long n) {
                                 if (cudaGetLastError() != cudaSuccess) return ISO_ERR_CUDA; } while (0)
 
 // C_i = F_0^T dF_i for i < K (K >= 1), or C = (F_0 + X)^T (F_0 + X) - I (K = 0),
-// in binary64 through exact slices on the tensor cores; `scratch` holds the
-// operands' slabs and, where the contraction is split, the partial sums.
+// in binary64 through exact slices on the tensor cores (peaked columns summed
+// in binary64); `scratch` holds the operands' slabs and, where the contraction
+// is split, the partial sums.
 // Experts are batched as the scratch allows.  The contraction is split over
 // blocks until the last wave is full enough: `splits` minimises the number of
 // waves per split, with 1 % per split for the partial sums' traffic.
@@ -932,10 +1058,13 @@ int exact_product(cudaStream_t s, int sms, const OzSrc& src, int K, double* C, u
     const unsigned long long slot = (unsigned long long)nt * chunks * OZ_SLAB_BYTES;
     const int rc = (int)std::max(1LL, std::min(256LL, (d + 255) / 256));
     const dim3 mg((unsigned)((q + 31) / 32), rc), mb(32, 8);
-    if (K == 0) FR_LAUNCH((pdl_launch(k_oz_colmax<1>, mg, mb, 0, s, src, K + 1, rc)));
-    else if (K <= 2) FR_LAUNCH((pdl_launch(k_oz_colmax<3>, mg, mb, 0, s, src, K + 1, rc)));
-    else if (K <= 4) FR_LAUNCH((pdl_launch(k_oz_colmax<5>, mg, mb, 0, s, src, K + 1, rc)));
-    else FR_LAUNCH((pdl_launch(k_oz_colmax<MAXK + 1>, mg, mb, 0, s, src, K + 1, rc)));
+    float* const part = reinterpret_cast<float*>(scratch);      // read before the slabs are written
+    if (scratch_bytes / sizeof(float) < (size_t)rc * (K + 1) * q) return ISO_ERR_WORKSPACE;
+    if (K == 0) FR_LAUNCH((pdl_launch(k_oz_colmax<1>, mg, mb, 0, s, src, K + 1, rc, part)));
+    else if (K <= 2) FR_LAUNCH((pdl_launch(k_oz_colmax<3>, mg, mb, 0, s, src, K + 1, rc, part)));
+    else if (K <= 4) FR_LAUNCH((pdl_launch(k_oz_colmax<5>, mg, mb, 0, s, src, K + 1, rc, part)));
+    else FR_LAUNCH((pdl_launch(k_oz_colmax<MAXK + 1>, mg, mb, 0, s, src, K + 1, rc, part)));
+    FR_LAUNCH((pdl_launch(k_oz_columns, dim3((unsigned)((q + 255) / 256), (unsigned)(K + 1)), 256, 0, s, src, K + 1, rc, part)));
     ISO_TRY(smem_optin<k_oz_gemm>(OZ_SMEM));
     if (scratch_bytes < slot * (K ? 2 : 1)) return ISO_ERR_WORKSPACE;
     const int most = (int)std::min<unsigned long long>(std::max(K, 1), scratch_bytes / slot - (K ? 1 : 0));
@@ -986,6 +1115,7 @@ int exact_product(cudaStream_t s, int sms, const OzSrc& src, int K, double* C, u
         if (splits > 1)
             FR_LAUNCH((pdl_launch(k_oz_reduce, grid_of((long long)nz * q * q, sms), 256, 0, s, g.part, splits, nz, q, g.C, K ? 0 : 1)));
     }
+    FR_LAUNCH((pdl_launch(k_oz_f64, 4 * sms, 256, 0, s, src, K, C)));
     return ISO_OK;
 }
 
@@ -1129,7 +1259,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
     // A_i = F_0^T dF_i (binary64), then Sym_i and Kw_i
     for (int sd = 0; sd < 2; ++sd) {
         OzSrc oz{fr[sd], dots, nullptr, reinterpret_cast<unsigned long long*>(ws + L.mx[sd]),
-                 reinterpret_cast<int32_t*>(ws + L.ex), Qp};
+                 reinterpret_cast<int32_t*>(ws + L.ex), Qp, reinterpret_cast<int32_t*>(ws + L.sym[sd])};
         ISO_TRY(exact_product(s, sms, oz, K, D(L.aq[sd]), reinterpret_cast<unsigned char*>(ws + L.tail),
                               L.total - L.tail, &hdr->status));
         FR_LAUNCH((pdl_launch(k_fr_symskew, dim3((unsigned)(Qp / 32), (unsigned)(Qp / 32), K), dim3(32, 8), 0, s, 
@@ -1288,7 +1418,7 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
     for (int sd = 0; sd < 2; ++sd) {
         const long long Dp = sd == 0 ? L.Mp : L.Np, d = fr[sd].d;
         OzSrc oz{fr[sd], nullptr, D(L.dF[sd]), reinterpret_cast<unsigned long long*>(ws + L.mx[sd]),
-                 reinterpret_cast<int32_t*>(ws + L.ex), Qp};
+                 reinterpret_cast<int32_t*>(ws + L.ex), Qp, reinterpret_cast<int32_t*>(ws + L.ns_y)};
         ISO_TRY(exact_product(s, sms, oz, 0, D(L.n64), reinterpret_cast<unsigned char*>(ws + L.gw4),
                               L.dF[0] - L.gw4, &hdr->status));
         NsBufs nb{D(L.ns_y), D(L.ns_z), D(L.ns_m), F(L.ns_y4), F(L.ns_z4), F(L.ns_m4), F(L.ns_t1),

@@ -98,8 +98,15 @@ __global__ void k_gemm_x3(const __grid_constant__ CUtensorMap ta, const __grid_c
 // t = 0 .. 6, with integer digits |d_t| <= 128 (x rounded to 55 fractional
 // bits below 2^e), stored as bf16, which holds them exactly.  Then
 //   C_kl = 2^(e_k + e_l - 14) sum_g 2^(-8 g) I_g,  I_g = sum_{s + t = g} <a_s, b_t>
-// over g = 0 .. 6 (28 of the 49 slice pairs; the rest lies below the
-// rounding of the binary64 sum it replaces).  Each I_g accumulates in tensor
+// over g = 0 .. 6 (28 of the 49 slice pairs).  Over d rows the pairs left out
+// come to about sqrt(d) 2^-56.3 2^(e_k + e_l), at most 6.1 d 2^-56 2^(e_k +
+// e_l), and the rounding of the columns to 2^-56.8 (2^e_k |b| + 2^e_l |a|): for
+// dense columns less than the rounding of a binary64 sum, for columns whose
+// largest entry holds much of their norm more.  Those are told apart by
+// k_oz_columns, which has the figures, and summed in binary64 by k_oz_f64.
+// The bounds are on the columns' norms: where two dense columns hardly overlap,
+// their product is off by that much of |a| |b|, not of sum |a_r b_r|.
+// Each I_g accumulates in tensor
 // memory as binary32 over at most OZ_STEPS_* steps, which keeps every partial
 // sum at or below 2^24 whatever the digits (an exact integer), and is then
 // added to 64-bit integers in registers.

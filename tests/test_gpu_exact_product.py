@@ -49,7 +49,7 @@ def _gamma(U0, Us, V0, Vs, S):
 
 
 # (m, n): one 16-row chunk and a ragged one, several tiles, the drain every 9
-# and 21 chunks crossed, a contraction split over blocks
+# and 16 chunks crossed, a contraction split over blocks
 @pytest.mark.parametrize("m,n,K", [(16, 40, 1), (17, 5, 2), (130, 129, 2), (336, 337, 1), (2500, 64, 3), (70, 1000, 2)])
 @pytest.mark.parametrize("kind", ["random", "scaled", "extreme"])
 def test_gram_of_exact_products(m, n, K, kind):
@@ -90,3 +90,63 @@ def test_nonfinite_column_reaches_the_gram():
     _, st = iso.frame_merge_factors(U0, S, U0, [U1], [U0], W0, ns_iters=1, stats=True)
     torch.cuda.synchronize()
     assert not torch.isfinite(st.gram).all()
+
+
+def _peaked(rng, d, q, peak, rest, shift):
+    """Columns with one entry `peak`, the others about `rest`; every fourth
+    column dense."""
+    F = rest * rng.normal(size=(d, q))
+    k = np.arange(q)
+    F[(k * 7 + shift) % d, k] = peak
+    F[:, 3::4] = rng.normal(size=(d, len(k[3::4]))) / np.sqrt(d)
+    return F
+
+
+# columns whose largest entry holds most of their norm (more than one tile of
+# 64 of them, a remainder, a few), on different rows in the two operands
+@pytest.mark.parametrize("m,n,K", [(130, 129, 2), (336, 337, 1), (2048, 96, 1), (70, 1000, 3), (2500, 5, 2)])
+@pytest.mark.parametrize("rest", [1e-3, 1e-5])
+def test_gram_of_peaked_columns(m, n, K, rest):
+    rng = np.random.default_rng(m + n + K)
+    q = min(m, n)
+    U0, V0 = _peaked(rng, m, q, 1.0, rest, 0), _peaked(rng, n, q, 1.0, rest, 0)
+    Us = [U0 + _peaked(rng, m, q, 1.0, rest, m // 2 + i) for i in range(K)]
+    Vs = [V0 + _peaked(rng, n, q, 1.0, rest, n // 2 + i) for i in range(K)]
+    S = np.linspace(1.0, 0.1, q)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+    W0 = torch.zeros(m, n, device=DEV)
+    _, st = iso.frame_merge_factors(dev(U0), dev(S), dev(V0.T), [dev(U) for U in Us], [dev(V.T) for V in Vs], W0,
+                                    rho_keep=1.0, ns_iters=1, stats=True)
+    torch.cuda.synchronize()
+    ref, mag = _gamma(U0, Us, V0, Vs, S)
+    err = np.abs(st.gram.cpu().numpy() - ref.astype(np.float64)) / mag.astype(np.float64)
+    # binary64 sums: d 2^-53 of the magnitudes at worst
+    assert err.max() <= 2.0 ** -49, (m, n, rest, err)
+
+
+@pytest.mark.parametrize("d,seed", [(1 << 18, s) for s in range(4)] + [(8960, 4), (333, 5)])
+@pytest.mark.parametrize("tall", [True, False])
+def test_one_small_entry_of_peaked_columns(d, seed, tall):
+    """Two modes: one side moved along one peaked column, the other by a
+    rotation of 0.7.  Gamma = |dF_2|^2 + 2 0.7^2 - A_12^2 - ... - 1.4 A_12,
+    about 2, where A_12 = <F_01, dF_2> is a sum of terms below 0.01 that a
+    binary64 sum holds to a few 1e-17; the slices alone leave it off by some
+    sqrt(d) 2^-56.3, 6e-15 at d = 2^18.  Bound: 2^-49, eight roundings of
+    numbers up to 2 in the sums that follow."""
+    rng = np.random.default_rng(seed)
+    F0 = np.sqrt(1 - 0.81) / np.sqrt(d) * rng.normal(size=(d, 2))
+    dF = np.zeros((d, 2))
+    dF[:, 1] = np.sqrt(1 - 0.81) / np.sqrt(d) * rng.normal(size=d)
+    F0[1, 0] = F0[d // 2, 1] = dF[d - 2, 1] = 0.9
+    O0 = np.eye(2)
+    O1 = O0 + np.array([[0.0, 0.7], [-0.7, 0.0]])
+    U0, V0, U1, V1 = (F0, O0, F0 + dF, O1) if tall else (O0, F0, O1, F0 + dF)
+    S = np.ones(2)
+    dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+    W0 = torch.zeros(U0.shape[0], V0.shape[0], device=DEV)
+    _, st = iso.frame_merge_factors(dev(U0), dev(S), dev(V0.T), [dev(U1)], [dev(V1.T)], W0, rho_keep=1.0, ns_iters=1,
+                                    stats=True)
+    torch.cuda.synchronize()
+    ref, _ = _gamma(U0, [U1], V0, [V1], S)
+    err = abs(float(np.longdouble(st.gram.cpu().item()) - ref[0, 0]))
+    assert err <= 2.0 ** -49, (d, tall, err)
