@@ -188,3 +188,26 @@ def test_opt_step_full_size_projection_paper_learning_rate():
     # one Qwen2.5-7B gate projection (3584 x 18944, bf16 weights) at the
     # paper's ISO-AdamW learning rate 7.5e-7, first step
     _run_and_check(3584, 18944, 1, 0.0, "bf16", lr=7.5e-7, gscale=1e-3, seed=23)
+
+
+@pytest.mark.parametrize("e", [-100, -118, -124, -128, -132])
+@pytest.mark.parametrize("dtype", [torch.float32, torch.bfloat16])
+def test_opt_step_gradients_near_the_smallest_normal_number(e, dtype):
+    # gradient entries of about 2^e, spectrum of about 2^40, so that the factor
+    # gradients are normal numbers again.  As two tf32 values an entry is held
+    # to 2^-137 (the last place of tf32's subnormals is 2^-136), the products
+    # to 2^-20 as elsewhere.
+    rng = np.random.default_rng(-e)
+    m, n = 192, 128
+    U, V = _orth(rng, m, n), _orth(rng, n, n)
+    S = np.linspace(2.0, 1.0, n) * 2.0 ** 40
+    G = torch.from_numpy((rng.normal(size=(m, n)) * 2.0 ** e).astype(np.float32)).to(dtype)
+    to = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(DEV)
+    mom = [torch.zeros(x, n, device=DEV) for x in (m, m, n, n)]
+    W = torch.zeros(m, n, device=DEV)
+    iso.opt_step(to(U), to(V), to(S), G.to(DEV), *mom, W, W_out=torch.empty_like(W), lr=0.0, step=1)
+    torch.cuda.synchronize()
+    G = G.double().numpy()
+    for got, g in ((mom[0], G @ (V * S)), (mom[2], G.T @ (U * S))):
+        err = np.linalg.norm(got.cpu().double().numpy() - 0.1 * g) / np.linalg.norm(0.1 * g)
+        assert err <= 2.0 ** (-137 - e) + 2.0 ** -20, (e, err)
