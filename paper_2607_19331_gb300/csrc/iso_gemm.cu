@@ -125,13 +125,20 @@ __device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, v
 // c / (sqrt(x) + eps) in binary64.  The division and square root instructions'
 // sequences made up most of the epilogue's binary64 work; here a binary32
 // reciprocal square root and reciprocal are refined (Newton-Raphson; the last
-// step of each forms the residual exactly, as in Markstein, "Computation of
-// elementary functions on the IBM RISC System/6000 processor", 1990), which
-// leaves root and quotient within two units in the last place.  x outside
-// binary32's comfortable range takes the library's.
+// step of each forms the residual and adds the correction with one rounding,
+// as in Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor", 1990).  The approximation entering the last step is
+// good to 2^-43, so root and quotient are off by at most half an ulp + 2^-30
+// ulp: the rounded values but for near-ties.  That holds while x and the
+// divisor are in binary32's comfortable range and c is far from binary64's
+// ends; everything else takes the library's.
 __device__ __forceinline__ double over_root(double c, double x, double eps) {
     const float xf = (float)x;
-    if (!(xf > 1e-30f && xf < 1e30f)) return c / (sqrt(x) + eps);
+    const uint32_t hc = (uint32_t)__double2hiint(c) & 0x7FFFFFFFu;
+    const bool plain = xf > 1e-30f && xf < 1e30f && (uint32_t)__double2hiint(eps) < 0x46300000u     // eps < 2^100
+                       && (hc - 0x07B00000u < 0x78300000u - 0x07B00000u                             // 2^-900 <= |c| < 2^900
+                           || (hc | (uint32_t)__double2loint(c)) == 0);
+    if (!plain) return c / (sqrt(x) + eps);
     const double r0 = (double)rsqrtf(xf);
     const double r1 = fma(0.5 * r0, fma(-x * r0, r0, 1.0), r0);       // 1 / sqrt(x) to about 2^-43
     const double s0 = x * r1;

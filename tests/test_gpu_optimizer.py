@@ -211,3 +211,10 @@ def test_opt_step_gradients_near_the_smallest_normal_number(e, dtype):
     for got, g in ((mom[0], G @ (V * S)), (mom[2], G.T @ (U * S))):
         err = np.linalg.norm(got.cpu().double().numpy() - 0.1 * g) / np.linalg.norm(0.1 * g)
         assert err <= 2.0 ** (-137 - e) + 2.0 ** -20, (e, err)
+
+
+@pytest.mark.parametrize("eps,lr", [(1e20, 1e20), (1e39, 1e39), (1e200, 1e200)])
+def test_opt_step_with_a_dominant_eps(eps, lr):
+    # eps far above sqrt(v), also beyond binary32's range: a momentum step of
+    # lr / eps, as the definition has it
+    _run_and_check(96, 64, 5, 0.0, "f32", lr=lr, eps=eps, seed=31)
