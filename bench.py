@@ -240,11 +240,10 @@ def run_frame(args):
     projection (3584 x 18944, bf16 base ~ N(0, 0.02^2), K RL experts = base +
     N(0, (5e-4)^2), seeded).  The thin SVDs (torch.linalg, binary64, the one
     library step) are timed once and reported apart; a step is one
-    iso_frame_merge call on resident factors.  The roofline is that of
-    the plain tcgen05 product (k_gemm_tf32), timed live on the
-    reconstruction's shape (M = 3584, N = 18944, a contraction of 3 x 2 x 3584
-    tf32 terms); the merge's own products (k_gemm_x3, k_oz_gemm) are among the
-    step's kernels."""
+    iso_frame_merge call on resident factors.  The roofline is that of the
+    merge's split product (k_gemm_x3), timed live on the reconstruction's shape
+    (M = 3584, N = 18944, a contraction of 3 x 2 x 3584 tf32 terms, binary32
+    outputs); the exact slices (k_oz_gemm) are among the step's kernels."""
     import torch
     import paper_2607_19331_gb300 as iso
     dev = torch.device("cuda", 0)
@@ -290,20 +289,20 @@ def run_frame(args):
     torch.cuda.synchronize()
     prof = iso.profile_read()
     iso.profile_enable(False)
-    # the plain product alone, on the reconstruction's shape
+    # the split product alone, on the reconstruction's shape
     pad = lambda x: (x + 127) // 128 * 128
     Mp, Np, L = pad(m), pad(n), 2 * pad(min(m, n))
-    A = torch.randn(Mp, 4 * L, device=dev)
-    B = torch.randn(Np, 4 * L, device=dev)
+    A = torch.randn(Mp, 2 * L, device=dev)
+    B = torch.randn(Np, 2 * L, device=dev)
     C = torch.empty(Mp, Np, device=dev)
     for _ in range(3):
-        iso.gemm_tf32(A, B, C, 3 * L, 0, L)
+        iso.gemm_x3(A, B, C)
     torch.cuda.synchronize()
     f0, f1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     reps = 10
     f0.record(stream)
     for _ in range(reps):
-        iso.gemm_tf32(A, B, C, 3 * L, 0, L)
+        iso.gemm_x3(A, B, C)
     f1.record(stream)
     torch.cuda.synchronize()
     g_ms = f0.elapsed_time(f1) / reps
@@ -324,7 +323,7 @@ def run_frame(args):
                    "svd_seconds_library": round(svd_s, 2),
                    "l2": "operands larger than L2 (129 MB); no flush needed"},
         "kernels": {k: {"launches": v[0] // 3, "ms_per_step": round(v[1] / 3, 3)} for k, v in prof.items()},
-        "roofline": {"bound": "tensor", "kernel": "k_gemm_tf32 (reconstruction shape)", "achieved": round(achieved, 1),
+        "roofline": {"bound": "tensor", "kernel": "k_gemm_x3 (reconstruction shape)", "achieved": round(achieved, 1),
                      "peak": round(peak, 1), "peak_source": src, "unit": "TFLOP/s",
                      "frac": round(achieved / peak, 4), "traffic": None, "avg_launch_ms": round(g_ms, 3),
                      "algorithmic_flops_per_launch": flops},
@@ -337,10 +336,10 @@ def run_opt(args):
     """One ISO[AdamW] step (Sec. 4.3) of a Qwen2.5-7B gate/up projection
     (3584 x 18944, bf16 weights, binary64 frames from the weights' thin SVD,
     a seeded synthetic gradient ~ N(0, 1e-3^2)) at the paper's learning rate
-    7.5e-7.  A step is one iso_opt_step call; the roofline is that of
-    the plain tcgen05 product (k_gemm_tf32) on the factor-gradient shape
-    (M = 18944, N = 3584, a contraction of 3 x 3584 tf32 terms), timed live;
-    the step's own products (k_gemm_x3, k_oz_gemm) are among its kernels."""
+    7.5e-7.  A step is one iso_opt_step call; the roofline is that of the
+    split product (k_gemm_x3) on the factor-gradient shape (M = 18944, N =
+    3584, a contraction of 3 x 3584 tf32 terms, binary32 outputs), timed live;
+    the exact slices (k_oz_gemm) are among the step's kernels."""
     import torch
     import paper_2607_19331_gb300 as iso
     dev = torch.device("cuda", 0)
@@ -389,16 +388,16 @@ def run_opt(args):
     iso.profile_enable(False)
     pad = lambda x: (x + 127) // 128 * 128
     Np, L = pad(n), pad(m)
-    A = torch.randn(Np, 4 * L, device=dev)
-    B = torch.randn(pad(min(m, n)), 4 * L, device=dev)
+    A = torch.randn(Np, 2 * L, device=dev)
+    B = torch.randn(pad(min(m, n)), 2 * L, device=dev)
     C = torch.empty(Np, pad(min(m, n)), device=dev)
     for _ in range(3):
-        iso.gemm_tf32(A, B, C, 3 * L, 0, L)
+        iso.gemm_x3(A, B, C)
     torch.cuda.synchronize()
     f0, f1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     f0.record(stream)
     for _ in range(10):
-        iso.gemm_tf32(A, B, C, 3 * L, 0, L)
+        iso.gemm_x3(A, B, C)
     f1.record(stream)
     torch.cuda.synchronize()
     g_ms = f0.elapsed_time(f1) / 10
@@ -417,7 +416,7 @@ def run_opt(args):
         "config": {"workload": args.workload, "m": m, "n": n, "lr": 7.5e-7, "svd_seconds_library_once": round(svd_s, 2),
                    "l2": "operands larger than L2 (129 MB); no flush needed"},
         "kernels": {k: {"launches": v[0] // 3, "ms_per_step": round(v[1] / 3, 3)} for k, v in prof.items()},
-        "roofline": {"bound": "tensor", "kernel": "k_gemm_tf32 (factor-gradient shape)", "achieved": round(achieved, 1),
+        "roofline": {"bound": "tensor", "kernel": "k_gemm_x3 (factor-gradient shape)", "achieved": round(achieved, 1),
                      "peak": round(peak, 1), "peak_source": src, "unit": "TFLOP/s", "frac": round(achieved / peak, 4),
                      "traffic": None, "avg_launch_ms": round(g_ms, 3), "algorithmic_flops_per_launch": flops},
         "gpu_launches": int(launches), "clocks": ck, "e2e": None, "cpu_baseline": None,

@@ -422,8 +422,22 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
                      const iso_adamw_cfg* cfg, void* workspace, size_t ws_bytes, const iso_merge_stats* stats,
                      void* stream);
 
-/* The frame merge's dense product on the tensor cores, for tests of the
- * contraction alone: C (M x N, row stride ldc) = A[:, a_k0 : a_k0 + Kc]
+/* The dense product of the frame merge and the optimizer step on its own, for
+ * tests and timing: C (M x N) = A B^T over split operands, x = hi + lo with hi
+ * and lo tf32 values.  A is M rows and B N rows of 2 Kc binary32 entries, Kc
+ * hi and then Kc lo ones; three products (hi hi, hi lo, lo hi) with binary32
+ * accumulation, the latter two summed apart and added once.  With A2, B2 and
+ * C2 (all or none), C2 = A2 B2^T in the same launch.  With W0 and out (both
+ * or neither, in place of C; at most M x N entries, one dtype) out = W0 + A
+ * B^T instead of C.  M and N multiples of 128 below 2^23, Kc a multiple of 32 below 2^28;
+ * width: columns of C per tile, 128 or 256, or 0 for the merge's own choice.
+ * Device pointers, 16-byte aligned; enqueued on stream. */
+int32_t iso_gemm_x3(const float* A, const float* B, const float* A2, const float* B2, float* C, float* C2,
+                    const iso_tensor* W0, const iso_tensor* out, int64_t M, int64_t N, int64_t Kc, int32_t width,
+                    void* stream);
+
+/* A plain product on the tensor cores, one tf32 contraction (no other call
+ * runs it): C (M x N, row stride ldc) = A[:, a_k0 : a_k0 + Kc]
  * B[:, b_k0 : b_k0 + Kc]^T, A (M rows, stride lda) and B (N rows, stride
  * ldb) row-major binary32 read as tf32, binary32 accumulation.  M and N
  * multiples of 128; Kc, a_k0 and b_k0 multiples of 32; strides multiples of

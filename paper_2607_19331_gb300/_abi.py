@@ -97,6 +97,7 @@ PROTOTYPES = [
     ("iso_frame_merge", I32, [P, P, P, P, P, I32, I64, I64, PT, PT, ctypes.POINTER(IsoFrameCfg), P, SZ,
                               ctypes.POINTER(IsoMergeStats), P]),
     ("iso_gemm_tf32", I32, [P, I64, P, I64, P, I64, I64, I64, I64, I64, I64, P]),
+    ("iso_gemm_x3", I32, [P, P, P, P, P, P, PT, PT, I64, I64, I64, I32, P]),
     ("iso_opt_workspace_size", I32, [I64, I64, ctypes.POINTER(SZ)]),
     ("iso_opt_step", I32, [P, P, P, PT, P, P, P, P, PT, PT, I64, I64, ctypes.POINTER(IsoAdamwCfg), P, SZ,
                            ctypes.POINTER(IsoMergeStats), P]),

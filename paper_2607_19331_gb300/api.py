@@ -496,6 +496,20 @@ def gemm_tf32(A: torch.Tensor, B: torch.Tensor, C: torch.Tensor, Kc: int, a_k0=0
     return C
 
 
+def gemm_x3(A, B, C=None, A2=None, B2=None, C2=None, W0=None, out=None, width=0, stream=None):
+    """iso_gemm_x3: C = A B^T (or out = W0 + A B^T) over operands split as [hi | lo] along
+    their columns, three tf32 products; C2 = A2 B2^T in the same launch."""
+    for t in (A, B, C, A2, B2, C2):
+        if t is not None and (t.dtype != torch.float32 or not t.is_contiguous() or t.dim() != 2):
+            raise ValueError("gemm_x3 takes contiguous 2-D float32 tensors")
+    p = lambda t: None if t is None else t.data_ptr()
+    d = lambda t: None if t is None else describe([t])
+    rc = lib().iso_gemm_x3(p(A), p(B), p(A2), p(B2), p(C), p(C2), d(W0), d(out), A.shape[0], B.shape[0],
+                           A.shape[1] // 2, int(width), _stream(stream))
+    check(rc, "iso_gemm_x3")
+    return C if out is None else out
+
+
 # ---------------------------------------------------------------------------
 # ISO-Optimizer step ISO[AdamW] on one matrix (Sec. 4.3)
 # ---------------------------------------------------------------------------

@@ -998,9 +998,9 @@ int smem_optin(int bytes) {
 // multiples of 128); with A2, a second product C2 = A2 B2^T of the same shape
 // in the same launch.  The tile shape with the smaller number of waves times
 // what a stage costs in it (clocks per 32 contraction columns: 1900 for 128 x
-// 256, bound by shared memory; 1150 for 128 x 128, bound by L2).
+// 256, bound by shared memory; 1150 for 128 x 128, bound by L2), or the given one.
 int frame_gemm(cudaStream_t s, int sms, const float* A, long long a_rows, const float* B, long long b_rows, long long L,
-               GemmArgs g, const float* A2 = nullptr, const float* B2 = nullptr) {
+               GemmArgs g, const float* A2 = nullptr, const float* B2 = nullptr, int width = 0) {
     CUtensorMap ta, tb, ta2, tb2;
     ISO_TRY(gemm_tensor_map(&ta, A, a_rows, 2 * L, 2 * L));
     ISO_TRY(gemm_tensor_map(&tb, B, b_rows, 2 * L, 2 * L));
@@ -1013,7 +1013,7 @@ int frame_gemm(cudaStream_t s, int sms, const float* A, long long a_rows, const 
     ISO_TRY(smem_optin<k_gemm_x3<256>>(X3_SMEM));
     const unsigned nz = A2 ? 2 : 1;
     const long long my = a_rows / GEMM_BM, t128 = my * (b_rows / 128) * nz, t256 = my * ((b_rows + 255) / 256) * nz;
-    const bool wide = (t256 + sms - 1) / sms * 1900 <= (t128 + sms - 1) / sms * 1150;
+    const bool wide = width ? width == 256 : (t256 + sms - 1) / sms * 1900 <= (t128 + sms - 1) / sms * 1150;
     const int slot = prof_begin(0, s);
     if (wide)
         pdl_launch(k_gemm_x3<256>, dim3((unsigned)((b_rows + 255) / 256), (unsigned)my, nz), GEMM_THREADS, X3_SMEM, s, ta, tb, ta2,
@@ -1479,7 +1479,35 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
     return ISO_OK;
 }
 
-// The tcgen05 product on its own, for tests of the contraction: C (M x N,
+// The split product on its own, for tests and timing
+int32_t iso_gemm_x3(const float* A, const float* B, const float* A2, const float* B2, float* C, float* C2,
+                    const iso_tensor* W0, const iso_tensor* out, int64_t M, int64_t N, int64_t Kc, int32_t width,
+                    void* stream) {
+    if (!A || !B || !A2 != !B2 || !A2 != !C2 || !W0 != !out || !C == !out || (out && A2)) return ISO_ERR_ARG;
+    if (M <= 0 || N <= 0 || Kc <= 0 || (width != 0 && width != 128 && width != 256)) return ISO_ERR_ARG;
+    if (M % GEMM_BM || N % GEMM_BN || Kc % GEMM_BK) return ISO_ERR_SHAPE;
+    if (M >= (1LL << 23) || N >= (1LL << 23) || Kc >= (1LL << 28)) return ISO_ERR_UNSUPPORTED;
+    for (const float* p : {A, B, A2, B2, static_cast<const float*>(C), static_cast<const float*>(C2)})
+        if ((uintptr_t)p & 15u) return ISO_ERR_ALIGN;
+    GemmArgs g{};
+    g.mode = GEMM_STORE_F32; g.C = C; g.C2 = C2; g.ldc = N; g.M = (int)M; g.N = (int)N;
+    if (out) {
+        if (W0->rows != out->rows || W0->cols != out->cols || out->rows < 1 || out->cols < 1 || out->rows > M || out->cols > N)
+            return ISO_ERR_SHAPE;
+        if ((W0->dtype != ISO_BF16 && W0->dtype != ISO_F32) || out->dtype != W0->dtype) return ISO_ERR_DTYPE;
+        if (!W0->data || !out->data) return ISO_ERR_ARG;
+        if (((uintptr_t)W0->data & 15u) || ((uintptr_t)out->data & 15u)) return ISO_ERR_ALIGN;
+        g.mode = GEMM_ADD_BASE; g.M = (int)out->rows; g.N = (int)out->cols; g.out = out->data; g.w0 = W0->data;
+        g.ldo = out->cols; g.out_dtype = out->dtype;
+    }
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return ISO_ERR_CUDA;
+    return frame_gemm(static_cast<cudaStream_t>(stream), sms, A, M, B, N, Kc, g, A2, B2, width);
+}
+
+// A plain tcgen05 product on its own: C (M x N,
 // ldc) = A[:, a_k0 : a_k0 + Kc] B[:, b_k0 : b_k0 + Kc]^T with A (M x lda) and
 // B (N x ldb) row-major binary32 read as tf32.
 int32_t iso_gemm_tf32(const float* A, int64_t lda, const float* B, int64_t ldb, float* C, int64_t ldc, int64_t M,

@@ -394,3 +394,21 @@ def test_candidate_segments_take_no_padding():
         return full.value
     for K in (1, 3):
         assert minimum(4100, K) - minimum(4097, K) == K * 64 * 3 * 4
+
+
+def test_split_product_rejects_before_launch():
+    L = _abi.lib()
+    A, B, C = 0x10000, 0x20000, 0x30000
+    w, o = _arr(_fake(128, 128, ptr=0x40000)), _arr(_fake(128, 128, ptr=0x50000))
+
+    def call(A=A, B=B, A2=None, B2=None, C=C, C2=None, W0=None, out=None, M=128, N=128, Kc=32, width=0):
+        return L.iso_gemm_x3(A, B, A2, B2, C, C2, W0, out, M, N, Kc, width, None)
+    for kw in (dict(A=None), dict(C=None), dict(A2=A), dict(A2=A, B2=B), dict(W0=w), dict(W0=w, out=o), dict(M=0),
+               dict(width=64), dict(C=None, W0=w, out=o, A2=A, B2=B, C2=C)):
+        assert call(**kw) == _abi.ISO_ERR_ARG, kw
+    for kw in (dict(M=127), dict(N=130), dict(Kc=16), dict(C=None, W0=w, out=_arr(_fake(128, 64, ptr=0x50000))),
+               dict(C=None, W0=_arr(_fake(129, 128, ptr=0x40000)), out=_arr(_fake(129, 128, ptr=0x50000)))):
+        assert call(**kw) == _abi.ISO_ERR_SHAPE, kw
+    assert call(A=0x10004) == _abi.ISO_ERR_ALIGN
+    assert call(C=None, W0=w, out=_arr(_fake(128, 128, ptr=0x50000, dtype=_abi.ISO_F32))) == _abi.ISO_ERR_DTYPE
+    assert call(M=1 << 23) == _abi.ISO_ERR_UNSUPPORTED
