@@ -62,6 +62,41 @@ def test_mean_of_three_is_the_division():
     assert np.array_equal(got.view(np.uint32), np.where(s == 0, np.float32(0), ref).view(np.uint32))
 
 
+# values whose sum in order is 0, so that the sum with x appended is x
+ZERO_SUMS = {3: (1, -1), 5: (1, -1, 1, -1), 6: (1, 1, -2, 1, -1), 7: (1, -1, 1, -1, 1, -1), 8: (1, 1, -2, 1, -1, 1, -1)}
+
+
+@pytest.mark.parametrize("K", [3, 5, 6, 7, 8])
+def test_quotients_are_the_division(K):
+    # x / K for every mantissa of one binade, and for magnitudes through the
+    # lower edge of the fast form (2^-120), the subnormals and the top: RAM over
+    # experts that sum to x, all active
+    m = torch.arange(0, 1 << 23, dtype=torch.int32) + 0x3F800000
+    e = torch.arange(0, 255, dtype=torch.int32).repeat_interleave(64) * (1 << 23)
+    e = e + torch.arange(64, dtype=torch.int32).repeat(255) * 131071
+    x = torch.cat([m, e, torch.arange(0, 4096, dtype=torch.int32)]).view(torch.float32)
+    x = torch.cat([x, -x[::7]])
+    parts = [torch.full_like(x, c * 2.0 ** -100) for c in ZERO_SUMS[K]] + [x]
+    live = sum((p != 0).numpy().astype(np.float32) for p in parts)
+    out = iso.iso_merge([torch.zeros_like(x).to(DEV)], [[p.to(DEV)] for p in parts], op="ram", eps_act=0.0, lam=1.0)
+    want = (x.numpy() / live).astype(np.float32)
+    want = np.where(want == 0, np.float32(0), want)
+    assert np.array_equal(out[0].cpu().numpy().view(np.uint32), want.view(np.uint32))
+
+
+@pytest.mark.parametrize("K", [3, 5, 6, 7, 8])
+def test_ties_quotients_are_the_division(K):
+    # K equal experts: the sum of K rounded additions over K, by magnitude and sign
+    m = torch.arange(0, 1 << 20, dtype=torch.int32) * 8 + 0x3F800000 + K
+    x = torch.cat([m.view(torch.float32), -m[::3].view(torch.float32), torch.zeros(64)])
+    out = iso.iso_merge([torch.zeros_like(x).to(DEV)], [[x.to(DEV)]] * K, op="ties", density=1.0, lam=1.0)
+    s = np.zeros(x.numel(), np.float32)
+    for _ in range(K):
+        s = s + x.numpy()
+    want = s / np.float32(K)
+    assert np.array_equal(out[0].cpu().numpy().view(np.uint32), np.where(want == 0, np.float32(0), want).view(np.uint32))
+
+
 @pytest.mark.parametrize("K", [2, 3, 4, 6])
 def test_untrimmed_ties_vector_with_nonfinite_values(K):
     # a TIES vector left untrimmed is read by no counting pass: the call
