@@ -3,10 +3,12 @@
 // Each unit is one block_rows x block_cols tile of a row-major tensor, in
 // row-major tile order; entries inside a tile keep the tensor's own index
 // order, so "lowest index first" among equal |tau| is the tile's row-major
-// order.  One CTA holds a whole unit on chip: it loads the unit's keys into
-// shared memory, finds the k-th largest key by an 11/11/9-bit radix select,
-// and resolves the ties by an ordered block scan.  The result (t, cut) feeds
-// the same streaming apply pass as the other scopes.
+// order.  One CTA holds a whole unit on chip: a full block as task-vector values
+// in registers, 32 consecutive entries a thread, a partial edge block as keys
+// in shared memory.  The k-th largest key comes from a radix select (11 bits a
+// level) and the ties from an ordered block scan.  Where the call is the K = 1
+// TIES update the same kernel writes the unit's outputs; otherwise the result
+// (t, cut) feeds the streaming passes of the other scopes.
 #include "iso_kernels.cuh"
 
 #include <type_traits>

@@ -188,9 +188,7 @@ __global__ void __launch_bounds__(TPB, 2) k_merge_c(Plan P) {
 #pragma unroll
         for (int q = 0; q < KC; ++q) cf[q] = (OPF == OPF_TIES) ? 0.0f : mp.cf[q];
         const int opk = (OPF == OPF_TIES) ? (int)OPK_TIES : mp.opk;
-        const bool iso1d = mp.iso1d;
         compact_tile<KC, BT>(P, cp, K, g, lane, d.base, e0, n, true, ct);
-        uint32_t kmax = 0;
 #pragma unroll 1
         for (int s = 0; s < SPT; ++s) {
             const long long e = e0 + (long long)s * (32 * E) + lane * E;
@@ -209,9 +207,9 @@ __global__ void __launch_bounds__(TPB, 2) k_merge_c(Plan P) {
                 for (int q = 0; q < KC; ++q) tj[q] = tau[q][j];
                 if (exact) {
                     const uint32_t bits = (e + j < n) ? select_bits<KC>(P, d, mp, K, tj, e + j, r, c) : 0u;
-                    o[j] = merged_value<KC>(opk, iso1d, P.lambda, K, th0[j], tj, cf, bits);
+                    o[j] = merged_value<KC>(opk, P.lambda, K, th0[j], tj, cf, bits);
                 } else {
-                    o[j] = merged_fast<KC>(opk, iso1d, P.lambda, K, th0[j], tj, cf, T, kmax);
+                    o[j] = merged_fast<KC>(opk, P.lambda, K, th0[j], tj, cf, T);
                 }
             }
             store_out<BT, E>(d.out, e, n, o);

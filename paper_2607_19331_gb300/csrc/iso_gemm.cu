@@ -198,7 +198,6 @@ __device__ __forceinline__ void gemm_store32(const GemmArgs& g, float* C, long l
 
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 k_gemm_tf32(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, GemmArgs g) {
-    if (g.skip && *reinterpret_cast<const volatile int32_t*>(g.skip)) return;
     extern __shared__ unsigned char gemm_smem_raw[];
     unsigned char* const smem = reinterpret_cast<unsigned char*>(
         (reinterpret_cast<uintptr_t>(gemm_smem_raw) + 1023) & ~(uintptr_t)1023);

@@ -2,7 +2,8 @@
 // optimizer step on the fifth-generation tensor cores: C = A B^T for row-major
 // fp32 operands read as tf32, with tcgen05.mma accumulating in tensor memory.
 //
-// k_gemm_tf32: one product.  One CTA of 128 threads computes one 128 x 128
+// k_gemm_tf32: one product (iso_gemm_tf32 alone; the merge and the step run the
+// kernels after it).  One CTA of 128 threads computes one 128 x 128
 // tile of C:
 //   warp 0, lane 0  loads the operand tiles (TMA, 128 rows x 32 fp32 = 128 B
 //                   per row, 128-byte swizzle) into a GEMM_STAGES-deep ring,
@@ -76,7 +77,7 @@ struct GemmArgs {
     long long ldo;
     int32_t out_dtype;
     int32_t pad;
-    const int32_t* skip;  // optional: the whole grid returns at once while *skip != 0
+    const int32_t* skip;  // k_gemm_x3, optional: the whole grid returns at once while *skip != 0
     int32_t* status;      // header status word for ISO_ERR_TIMEOUT
     AdamwArgs adam;       // GEMM_ADAMW
 };

@@ -210,7 +210,7 @@ __global__ void __launch_bounds__(TPB, 2) k_merge(Plan P) {
                         if (CK) tau[q] = __fsub_rn(tau[q], th0);
                     }
                     const uint32_t bits = select_bits<KC>(P, d, mp, K, tau, e + j, r, cc);
-                    o[j] = merged_value<KC>(opk, mp.iso1d, P.lambda, K, th0, tau, cf, bits);
+                    o[j] = merged_value<KC>(opk, P.lambda, K, th0, tau, cf, bits);
                 }
             });
         } else if (OPF == OPF_TIES) {

@@ -195,20 +195,14 @@ __device__ __forceinline__ uint32_t select_bits(const Plan& P, const TensorDesc&
     return bits;
 }
 
-// the merged output of one entry; every argument is in registers.  RAM never
-// comes here: its tensors are untrimmed (SEL_ALL), so every tile takes the
-// per-tile form below.
+// the merged output of one entry of a trimmed tensor (TIES or ISO 2-D); every
+// argument is in registers.  Untrimmed tensors (SEL_ALL) never come here: every
+// tile of theirs takes a per-tile form.
 template <int KC>
-__device__ __forceinline__ float merged_value(int opk, bool iso1d, float lambda, int K, float th0,
-                                              const float (&tau)[KC], const float (&cf)[KC], uint32_t bits) {
+__device__ __forceinline__ float merged_value(int opk, float lambda, int K, float th0, const float (&tau)[KC],
+                                              const float (&cf)[KC], uint32_t bits) {
     float upd;
-    if (opk == OPK_SUM) {
-        float s = 0.0f;
-#pragma unroll
-        for (int i = 0; i < KC; ++i)
-            if (i < K) s = __fadd_rn(s, tau[i]);
-        upd = iso1d ? __fdiv_rn(s, (float)K) : __fmul_rn(lambda, s);
-    } else if (opk == OPK_TIES) {
+    if (opk == OPK_TIES) {
         // gamma = sign(sum of the trimmed values); the agreeing set holds the
         // non-zero trimmed values of that sign (none when the sum is 0)
         float tt[KC];
@@ -264,33 +258,15 @@ __device__ __forceinline__ bool tile_thresholds(const MergeParams<KC>& mp, int K
     return exact;
 }
 
-// merged output of one entry inside a tile with per-tile thresholds: the
-// selection of expert q is (int)key > T[q] (never for q >= K), unselected
-// terms enter the sums as +0, which leaves every sum and the output as the
-// skipping form gives them
+// merged output of one entry inside a tile with per-tile thresholds (the
+// compact passes; k_merge has merge_pair): the selection of expert q is
+// (int)key > T[q] (never for q >= K), unselected terms enter the sums as +0,
+// which leaves every sum and the output as the skipping form gives them
 template <int KC>
-__device__ __forceinline__ float merged_fast(int opk, bool iso1d, float lambda, int K, float th0,
-                                             const float (&tau)[KC], const float (&cf)[KC], const int (&T)[KC],
-                                             uint32_t& kmax) {
+__device__ __forceinline__ float merged_fast(int opk, float lambda, int K, float th0, const float (&tau)[KC],
+                                             const float (&cf)[KC], const int (&T)[KC]) {
     float upd;
-    if (opk == OPK_RAM) {
-        // RAM (App. F): active experts key > T (|tau| > eps_act; T is past
-        // every key for q >= K); the active values summed in expert order,
-        // divided by their count -- one active value is kept whole (0 + v
-        // and v / 1 are exact), none leaves theta_0
-        float s = 0.0f;
-        int cnt = 0;
-#pragma unroll
-        for (int q = 0; q < KC; ++q) {
-            const uint32_t k = key_of(tau[q]);
-            kmax = (q < K && k > kmax) ? k : kmax;
-            const bool a = (int)k > T[q];
-            s = __fadd_rn(s, a ? tau[q] : 0.0f);
-            cnt += a;
-        }
-        const float m = cnt ? __fdiv_rn(s, (float)cnt) : 0.0f;
-        upd = __fmul_rn(lambda, m);
-    } else if (opk == OPK_TIES) {
+    if (opk == OPK_TIES) {
         // gamma = sign of the trimmed sum; the agreeing set: the non-zero
         // trimmed values of that sign.  u = tt with the sign of the sum
         // cleared is |tt| exactly for the agreeing ones, so their sum in
@@ -327,7 +303,7 @@ __device__ __forceinline__ float merged_fast(int opk, bool iso1d, float lambda, 
 #pragma unroll
         for (int q = 0; q < KC; ++q)
             if (q < K) s = __fadd_rn(s, tau[q]);
-        upd = iso1d ? __fdiv_rn(s, (float)K) : __fmul_rn(lambda, s);
+        upd = __fdiv_rn(s, (float)K);                  // ISO 1-D
     }
     return (upd == 0.0f) ? th0 : __fadd_rn(th0, upd);
 }
