@@ -586,13 +586,22 @@ int run_group(const Call& c, int t0, int t1, char* ws, cudaStream_t s, const iso
         }));
     if (select && c.topk.scope != ISO_SCOPE_BLOCK) {
         ISO_TRY(launch(KD_INIT, s, [&] { pdl_launch(k_init_units, (KU + 255) / 256, 256, 0, s, P, L.global_n); }));
+        long long largest = c.topk.scope == ISO_SCOPE_GLOBAL ? L.global_n : 0;
+        for (int t = t0; c.topk.scope == ISO_SCOPE_TENSOR && t < t1; ++t)
+            if (tensor_trimmed(c, t)) largest = std::max(largest, numel_of(c.x[t]));
+        const bool small = largest <= SAMPLE_SMALL;
         rc = dispatch_src(c.xdt, c.bdt, c.ckpt, [&](auto* xt, auto* bt, auto ck) -> int {
             using XT = std::remove_pointer_t<decltype(xt)>;
             using BT = std::remove_pointer_t<decltype(bt)>;
             constexpr bool CK = decltype(ck)::value;
-            const int smem = (SAMPLE_MAX + SAMPLE_LIST + RADIX_BINS) * 4;
-            ISO_TRY(smem_optin(k_sample<XT, BT, CK>, smem));
-            ISO_TRY(launch(KD_SAMPLE, s, [&] { pdl_launch(k_sample<XT, BT, CK>, KU, SAMPLE_TPB, smem, s, P); }));
+            if (small) {
+                const int smem = (2 * SAMPLE_SMALL + RADIX_BINS) * 4;
+                ISO_TRY(launch(KD_SAMPLE, s, [&] { pdl_launch(k_sample<XT, BT, CK, SMALL_TPB>, KU, SMALL_TPB, smem, s, P); }));
+            } else {
+                const int smem = (SAMPLE_MAX + SAMPLE_LIST + RADIX_BINS) * 4;
+                ISO_TRY(smem_optin(k_sample<XT, BT, CK, SAMPLE_TPB>, smem));
+                ISO_TRY(launch(KD_SAMPLE, s, [&] { pdl_launch(k_sample<XT, BT, CK, SAMPLE_TPB>, KU, SAMPLE_TPB, smem, s, P); }));
+            }
             if (fused)
                 ISO_TRY(launch(KD_SAMPLE, s, [&] { pdl_launch(k_csample<XT, BT, CK>, KU * CS_SPLIT, CS_TPB, 0, s, P); }));
             if (fused) {

@@ -35,6 +35,8 @@ constexpr int SAMPLE_MAX = 24576;           // sampled keys per unit (96 KB of s
 constexpr int SAMPLE_CHUNK = 256;           // contiguous entries per sample chunk
 constexpr int SAMPLE_TPB = 1024;            // one sample block per SM, three chunks per warp
 constexpr int SAMPLE_LIST = 8192;           // sampled keys gathered around the ranks
+constexpr int SAMPLE_SMALL = 2048;          // sets of units of at most this size: SMALL_TPB threads a unit
+constexpr int SMALL_TPB = 256;
 constexpr int SAMPLE_SEL_R = 5;             // ranks selected at once from the sample
 constexpr int CUT_TPB = 1024;
 constexpr int CS_SPLIT = 16;                // count-sample blocks per unit: one round of loads per warp

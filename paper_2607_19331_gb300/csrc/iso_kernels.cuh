@@ -20,7 +20,7 @@ constexpr bool PASS_INTERLEAVE = ISO_PASS_INTERLEAVE != 0;
 // select (TENSOR / GLOBAL scope)
 constexpr int COUNT_BLOCKS_PER_SM = 2;      // k_count: resident blocks of TPB threads per SM
 __global__ void k_init_units(Plan P, long long global_n);
-template <typename XT, typename BT, bool CK> __global__ void k_sample(Plan P);
+template <typename XT, typename BT, bool CK, int T> __global__ void k_sample(Plan P);
 template <typename XT, typename BT, bool CK, bool EMIT> __global__ void k_count(Plan P);
 __global__ void k_decide(Plan P);
 template <typename XT, typename BT, bool CK> __global__ void k_radix_hist(Plan P);

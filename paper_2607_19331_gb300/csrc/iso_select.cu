@@ -101,7 +101,7 @@ __device__ void block_find_from_top(const uint32_t* hist, int nb, long long rank
 }
 
 // The rank[r]-th largest (1-based, 1 <= rank[r] <= n) of n keys in shared
-// memory for R <= SEL_R ranks at once, by the whole block (SAMPLE_TPB
+// memory for R <= SEL_R ranks at once, by the whole block (T
 // threads).  One histogram of the top 11 bits; the keys of the bins that hold
 // the ranks (a few per cent of the sample) are gathered, and 7-bit digits of
 // those settle the rest, one histogram per distinct prefix, each scanned by
@@ -110,26 +110,27 @@ __device__ void block_find_from_top(const uint32_t* hist, int nb, long long rank
 // warp's keys into a handful of counters; on 11 bits a warp's 32 keys meet in
 // a few pairs (with every chunk loaded in one round, k_sample of two 1M-entry
 // binary32 units 36 -> 18 us, of 254 bf16 checkpoint tensors 131 -> 84 us).
-// `hist` holds RADIX_BINS counters, zero on entry; `list` SAMPLE_LIST keys.
+// `hist` holds RADIX_BINS counters, zero on entry; `list` list_cap keys.
 // On return *n_list is the number of gathered keys (all keys equal to a result
 // are among them), or -1.
 constexpr int SEL_R = SAMPLE_SEL_R;
 constexpr int SEL_BITS = 7;
 static_assert(SEL_R << SEL_BITS <= RADIX_BINS, "digit histograms share the counters");
+template <int T>
 __device__ void block_select_ranks(const uint32_t* keys, int n, int R, const long long* rank, uint32_t* hist,
-                                   uint32_t* list, int* n_list, uint32_t* out) {
+                                   uint32_t* list, int list_cap, int* n_list, uint32_t* out) {
     __shared__ uint32_t s_pref[SEL_R];
     __shared__ int s_rem[SEL_R];
     __shared__ uint32_t s_scan[33];
     __shared__ int s_n, s_b0, s_b1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int SH = 31 - RADIX_BITS;                       // shift of the first digit
-    for (int q = threadIdx.x; q < n; q += SAMPLE_TPB) atomicAdd(&hist[keys[q] >> SH], 1u);
+    for (int q = threadIdx.x; q < n; q += T) atomicAdd(&hist[keys[q] >> SH], 1u);
     if (threadIdx.x == 0) { s_n = 0; s_b0 = RADIX_BINS; s_b1 = -1; }
     __syncthreads();
     {
-        // bins from the top, RADIX_BINS / SAMPLE_TPB per thread
-        constexpr int PER = RADIX_BINS / SAMPLE_TPB;
+        // bins from the top, RADIX_BINS / T per thread
+        constexpr int PER = RADIX_BINS / T;
         uint32_t h[PER], sum = 0, tot;
 #pragma unroll
         for (int j = 0; j < PER; ++j) {
@@ -159,8 +160,8 @@ __device__ void block_select_ranks(const uint32_t* keys, int n, int R, const lon
     }
     __syncthreads();
     const uint32_t b0 = (uint32_t)s_b0, b1 = (uint32_t)s_b1;
-    for (int q = threadIdx.x; q < RADIX_BINS; q += SAMPLE_TPB) hist[q] = 0;
-    for (int q0 = 0; q0 < n; q0 += SAMPLE_TPB) {
+    for (int q = threadIdx.x; q < RADIX_BINS; q += T) hist[q] = 0;
+    for (int q0 = 0; q0 < n; q0 += T) {
         const int q = q0 + threadIdx.x;
         const uint32_t v = q < n ? keys[q] : 0;
         const bool in = q < n && (v >> SH) >= b0 && (v >> SH) <= b1;
@@ -168,10 +169,10 @@ __device__ void block_select_ranks(const uint32_t* keys, int n, int R, const lon
         int at = 0;
         if (lane == 0 && m) at = atomicAdd(&s_n, __popc(m));
         at = __shfl_sync(0xFFFFFFFFu, at, 0) + __popc(m & ((1u << lane) - 1u));
-        if (in && at < SAMPLE_LIST) list[at] = v;
+        if (in && at < list_cap) list[at] = v;
     }
     __syncthreads();
-    const bool fits = s_n <= SAMPLE_LIST;
+    const bool fits = s_n <= list_cap;
     const uint32_t* src = fits ? list : keys;
     const int ns = fits ? s_n : n;
     if (threadIdx.x == 0) *n_list = fits ? s_n : -1;
@@ -199,7 +200,7 @@ __device__ void block_select_ranks(const uint32_t* keys, int n, int R, const lon
                 grp[r] = g;
             }
         }
-        for (int q = threadIdx.x; q < ns; q += SAMPLE_TPB) {
+        for (int q = threadIdx.x; q < ns; q += T) {
             const uint32_t v = src[q], top = v >> sh;
             int g = -1;
 #pragma unroll
@@ -259,12 +260,19 @@ __device__ __forceinline__ int tensor_of_upos(const TensorDesc* tens, int n_tens
     return lo;
 }
 
-template <typename XT, typename BT, bool CKPT>
-__global__ void __launch_bounds__(SAMPLE_TPB, 1) k_sample(Plan P) {
+// T threads per unit.  A set whose trimmed tensors all have at most SAMPLE_SMALL
+// entries takes the form of SMALL_TPB threads, whose shared memory holds no
+// more than such units need: several blocks per SM, where one block of
+// SAMPLE_TPB threads spends its time at barriers (six checkpoints of 2000
+// tensors of 1536 entries: 436 us with that, 119 us so).
+template <typename XT, typename BT, bool CKPT, int T>
+__global__ void __launch_bounds__(T, T == SAMPLE_TPB ? 1 : 4) k_sample(Plan P) {
     pdl_enter();
+    constexpr bool SMALL = T != SAMPLE_TPB;
+    constexpr int KEYS = SMALL ? SAMPLE_SMALL : SAMPLE_MAX, LIST = SMALL ? SAMPLE_SMALL : SAMPLE_LIST;
     extern __shared__ __align__(16) uint32_t s_keys[];
-    uint32_t* s_list = s_keys + SAMPLE_MAX;          // SAMPLE_LIST keys
-    uint32_t* s_hist = s_list + SAMPLE_LIST;         // RADIX_BINS counters
+    uint32_t* s_list = s_keys + KEYS;                // LIST keys
+    uint32_t* s_hist = s_list + LIST;                // RADIX_BINS counters
     __shared__ long long s_scan[33];
     __shared__ int s_nl;
 
@@ -280,10 +288,10 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 1) k_sample(Plan P) {
     __shared__ long long s_rk[SEL_R];
     __shared__ uint32_t s_kv[SEL_R];
     __shared__ int s_edge[2];
-    if (S < n) {
+    if (!SMALL && S < n) {
         // the band's sample ranks, by one thread (binary64 is slow on this
         // GPU) while the others load
-        if (threadIdx.x == SAMPLE_TPB - 1) {
+        if (threadIdx.x == T - 1) {
             const double q = (double)U.k / (double)n;
             const double r = (double)U.k * (double)S / (double)n;
             const double delta = SAMPLE_Z * sqrt((double)S * q * (1.0 - q)) + 2.0;
@@ -301,12 +309,12 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 1) k_sample(Plan P) {
         // chunks of 256 contiguous entries at evenly spaced starts: one chunk
         // per warp step, 8 entries per lane, three chunks' loads in flight
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        constexpr int CB = nch / (SAMPLE_TPB / 32);
-        static_assert(CB * (SAMPLE_TPB / 32) == nch, "whole rounds of chunks");
+        constexpr int CB = SMALL ? 1 : nch / (T / 32);
+        static_assert(SMALL || CB * (T / 32) == nch, "whole rounds of chunks");
         float tau[CB][VEC];
 #pragma unroll
         for (int m = 0; m < CB; ++m) {
-            const int c = warp + m * (SAMPLE_TPB / 32);
+            const int c = warp + m * (T / 32);
             // (n - 256) c / 95, rounded down (exact: integer arithmetic)
             long long start = (long long)(((unsigned long long)(n - SAMPLE_CHUNK) * (unsigned long long)c) /
                                           (unsigned long long)(nch - 1));
@@ -333,16 +341,16 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 1) k_sample(Plan P) {
                 }
             }
         }
-        for (int q = threadIdx.x; q < RADIX_BINS; q += SAMPLE_TPB) s_hist[q] = 0;
+        for (int q = threadIdx.x; q < RADIX_BINS; q += T) s_hist[q] = 0;
 #pragma unroll
         for (int m = 0; m < CB; ++m) {
-            const int c = warp + m * (SAMPLE_TPB / 32);
+            const int c = warp + m * (T / 32);
             uint4* d = reinterpret_cast<uint4*>(s_keys + c * SAMPLE_CHUNK + lane * VEC);
             d[0] = make_uint4(key_of(tau[m][0]), key_of(tau[m][1]), key_of(tau[m][2]), key_of(tau[m][3]));
             d[1] = make_uint4(key_of(tau[m][4]), key_of(tau[m][5]), key_of(tau[m][6]), key_of(tau[m][7]));
         }
     } else {
-        for (int q = threadIdx.x; q < S; q += SAMPLE_TPB) {
+        for (int q = threadIdx.x; q < S; q += T) {
             int t = U.tensor;
             long long e = q;
             if (P.scope == ISO_SCOPE_GLOBAL) {
@@ -352,22 +360,22 @@ __global__ void __launch_bounds__(SAMPLE_TPB, 1) k_sample(Plan P) {
             const float tau = TauSrc<XT, BT, CKPT>::load1(P.xptr[i * P.n_tensors + t], P.tens[t].base, e);
             s_keys[q] = key_of(tau);
         }
-        for (int q = threadIdx.x; q < RADIX_BINS; q += SAMPLE_TPB) s_hist[q] = 0;
+        for (int q = threadIdx.x; q < RADIX_BINS; q += T) s_hist[q] = 0;
     }
     __syncthreads();
     uint32_t lo, hi;
     uint32_t that = 0;                       // the estimate of the threshold
-    if (S == n) {
+    if (SMALL || S == n) {
         // the sample is the whole unit: the band is the exact threshold
         if (threadIdx.x == 0) s_rk[0] = U.k;
         __syncthreads();
-        block_select_ranks(s_keys, S, 1, s_rk, s_hist, s_list, &s_nl, s_kv);
+        block_select_ranks<T>(s_keys, S, 1, s_rk, s_hist, s_list, LIST, &s_nl, s_kv);
         hi = lo = that = s_kv[0];
         run_t = true;
     } else {
         // every rank in one selection: the band edges and, for t^, the rank of
         // k and halfway to either edge
-        block_select_ranks(s_keys, S, want_t ? 5 : 2, s_rk, s_hist, s_list, &s_nl, s_kv);
+        block_select_ranks<T>(s_keys, S, want_t ? 5 : 2, s_rk, s_hist, s_list, LIST, &s_nl, s_kv);
         // no two of the five ranks share a key: no run of ties worth setting apart
         const bool distinct = s_kv[0] != s_kv[3] && s_kv[3] != s_kv[2] && s_kv[2] != s_kv[4] && s_kv[4] != s_kv[1];
         hi = s_edge[0] ? s_kv[0] : KEY_MAX;
@@ -1558,7 +1566,8 @@ __global__ void __launch_bounds__(CUT_TPB) k_cut(Plan P) {
 // instantiations
 // ---------------------------------------------------------------------------
 #define ISO_SELECT_INST(XT, BT, CK)                                            \
-    template __global__ void k_sample<XT, BT, CK>(Plan);                      \
+    template __global__ void k_sample<XT, BT, CK, SAMPLE_TPB>(Plan);          \
+    template __global__ void k_sample<XT, BT, CK, SMALL_TPB>(Plan);           \
     template __global__ void k_csample<XT, BT, CK>(Plan);                     \
     template __global__ void k_count<XT, BT, CK, false>(Plan);                \
     template __global__ void k_count<XT, BT, CK, true>(Plan);                 \

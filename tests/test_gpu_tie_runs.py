@@ -59,3 +59,28 @@ def test_a_run_of_infinities_is_reported():
     _, st = iso.iso_topk_mask([tau.to(DEV)], density=0.05, stats=True)
     torch.cuda.synchronize()
     assert int(st.status.item()) == -7
+
+
+@pytest.mark.parametrize("largest", [1, 31, 2047, 2048, 2049])
+@pytest.mark.parametrize("op", ["ties", "iso"])
+@pytest.mark.parametrize("K", [1, 3])
+def test_sets_of_small_units(largest, op, K):
+    # every unit at most 2048 entries, or one entry more (the other sample
+    # form): the masks' figures against the oracle, with runs of ties
+    shapes = [(1, largest)] + [(1, n) for n in (1, 7, 300, 1024, 2000) if n <= largest]
+    th0 = [torch.randn(s, generator=torch.Generator().manual_seed(9 + q)) * 0.02 for q, s in enumerate(shapes)]
+    xs = [[_grid(s[1], 2.0 ** -10, 100 * i + q).reshape(s) for q, s in enumerate(shapes)] for i in range(K)]
+    code = oracle.TIES if op == "ties" else oracle.ISO
+    for density in (0.0, 0.1, 0.55, 1.0):
+        g0, gx = [t.to(DEV) for t in th0], [[t.to(DEV) for t in x] for x in xs]
+        if K == 1:
+            _, st = iso.iso_update(g0, gx[0], op=op, update_is_delta=True, density=density, stats=True)
+            r = oracle.update([t.numpy() for t in th0], [t.numpy() for t in xs[0]], code, update_is_delta=True,
+                              density=density, shapes=shapes, is_1d=[False] * len(shapes))
+        else:
+            _, st = iso.iso_merge(g0, gx, op=op, density=density, stats=True)
+            r = oracle.merge([t.numpy() for t in th0], [[t.numpy() for t in x] for x in xs], code, density=density,
+                             shapes=shapes, is_1d=[False] * len(shapes))
+        torch.cuda.synchronize()
+        assert int(st.status.item()) == 0
+        assert_units_equal(st.units_numpy(), r["units"], f"small {largest} {op} K={K} {density}")
