@@ -1176,7 +1176,17 @@ __global__ void __launch_bounds__(TPB, 4) k_radix_hist(Plan P) {
             // eight loads in flight per lane
             const uint32_t* cs = P.cand + U->cand_off;
             const uint2* tc = P.tcand + (long long)c.i * P.n_tiles + c.g;
-            for (long long q0 = warp * 32; q0 < ntile; q0 += WPB * 32) {
+            // (the fused pass deals its tiles round robin over the warps, so
+            // neighbouring tiles' lists lie apart: one short list per thread.
+            // 300 bf16 tensors of 150K entries: 65 us by ranges, 34 us so)
+            for (long long q = threadIdx.x; P.fused && q < ntile; q += blockDim.x) {
+                const uint2 r = tc[q];
+                for (uint32_t j = r.x; j < r.x + r.y; ++j) {
+                    const uint32_t kk = cs[j], v = kk - base;
+                    if ((v >> pshift) == prefix) add(kk, v);
+                }
+            }
+            for (long long q0 = warp * 32; !P.fused && q0 < ntile; q0 += WPB * 32) {
                 const uint2 r = q0 + lane < ntile ? tc[q0 + lane] : make_uint2(0, 0);
                 const unsigned nz = __ballot_sync(0xFFFFFFFFu, r.y != 0);
                 const unsigned below = nz & ((1u << lane) - 1u);

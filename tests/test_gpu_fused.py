@@ -157,3 +157,14 @@ def test_fused_checkpoint_update_in_place_matches():
     torch.cuda.synchronize()
     for a, b in zip(ref, work):
         assert torch.equal(a.view(torch.int16), b.view(torch.int16))
+
+
+@pytest.mark.parametrize("op", ["iso", "ties"])
+def test_fused_select_over_short_lists(op):
+    # tensors of 74 tiles whose threshold lies inside the band: the radix levels
+    # read the candidates of tiles that different warps counted
+    g = torch.Generator().manual_seed(77)
+    th0 = [(torch.randn(300, 500, generator=g) * 0.02).bfloat16() for _ in range(6)]
+    th1 = [(t.float() * (1 + 2e-2 * torch.randn(300, 500, generator=g))).bfloat16() for t in th0]
+    for density in (0.01, 0.1, 0.4):
+        check_fused(th0, th1, op, density, what=f"short lists {op} {density}")
