@@ -350,6 +350,7 @@ struct OzSrc {
     int32_t* ex;                     // [1 + K][Qp] column exponents
     long long Qp;
     int32_t* peaked;                 // [1 + K][1 + q]: how many columns are left to binary64, and which
+    const double* cd;                // [K][K][q] column dots of the dF (their squared norms on the diagonal)
 };
 // entry e of source z (sg: the column's sign s_ik, for z > 0)
 __device__ __forceinline__ double oz_signed(const OzSrc& a, int z, long long e, double sg) {
@@ -361,8 +362,8 @@ __device__ __forceinline__ double oz_value(const OzSrc& a, int z, long long e, l
 }
 
 // every column's largest magnitude, all sources in one pass (reads each
-// array once: bound by HBM), and its sum of squares in binary32, one partial
-// per row chunk (part[chunk][source][column]; summed in order by
+// array once: bound by HBM), and the first operand's sums of squares in
+// binary32, one partial per row chunk (part[chunk][column]; summed in order by
 // k_oz_columns, so that the same input always gives the same sum)
 template <int SC>
 __global__ void __launch_bounds__(256) k_oz_colmax(OzSrc a, int sources, int row_chunks, float* part) {
@@ -373,29 +374,29 @@ __global__ void __launch_bounds__(256) k_oz_colmax(OzSrc a, int sources, int row
     const long long per = (a.f.d + row_chunks - 1) / row_chunks;
     const long long r0 = (long long)blockIdx.y * per, r1 = k < a.f.q ? min(a.f.d, r0 + per) : r0;
     unsigned long long m[SC];
-    float ss[SC];
+    float ss = 0.0f;
     double sg[SC];
 #pragma unroll
-    for (int z = 0; z < SC; ++z) { m[z] = 0; ss[z] = 0.0f; }
+    for (int z = 0; z < SC; ++z) m[z] = 0;
 #pragma unroll
     for (int i = 0; i + 1 < SC; ++i) sg[i] = i + 1 < sources && k < a.f.q ? sign_of(a.dots, a.f.q, i, k) : 0.0;
-    // the square from the value cut to binary32 by integer arithmetic (20
-    // mantissa bits; below 2^-63 zero, which only ever makes the sum smaller)
-    auto up = [](unsigned long long& x, float& s, double v) {
+    auto up = [](unsigned long long& x, double v) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(v) & 0x7FFFFFFFFFFFFFFFull;
         x = b > x ? b : x;
-        const uint32_t h = (uint32_t)(b >> 32);
-        const float f = __uint_as_float(h < 0x3C000000u ? 0u : (h - 0x38000000u) << 3);
-        s = __fmaf_rn(f, f, s);
+        return (uint32_t)(b >> 32);
     };
 #pragma unroll 4
     for (long long r = r0 + threadIdx.y; r < r1; r += 8) {
         const long long e = r * a.f.q + k;
         const double f0 = a.f.F0[e];
-        up(m[0], ss[0], a.X ? f0 + a.X[e] : f0);
+        const uint32_t h = up(m[0], a.X ? f0 + a.X[e] : f0);
+        // the square of the value cut to binary32 by integer arithmetic (20
+        // mantissa bits; below 2^-63 zero, which only makes the sum smaller)
+        const float c = __uint_as_float(h < 0x3C000000u ? 0u : (h - 0x38000000u) << 3);
+        ss = __fmaf_rn(c, c, ss);
 #pragma unroll
         for (int i = 0; i + 1 < SC; ++i)
-            if (i + 1 < sources) up(m[i + 1], ss[i + 1], fma(sg[i], a.f.F[i][e], -f0));
+            if (i + 1 < sources) up(m[i + 1], fma(sg[i], a.f.F[i][e], -f0));
     }
     // the block's rows first: one atomic per column and block
     __shared__ unsigned long long red[8][33];
@@ -404,17 +405,16 @@ __global__ void __launch_bounds__(256) k_oz_colmax(OzSrc a, int sources, int row
     for (int z = 0; z < SC; ++z) {
         if (z >= sources) break;
         red[threadIdx.y][threadIdx.x] = m[z];
-        reds[threadIdx.y][threadIdx.x] = ss[z];
+        if (z == 0) reds[threadIdx.y][threadIdx.x] = ss;
         __syncthreads();
         if (threadIdx.y == 0 && k < a.f.q) {
             unsigned long long v = m[z];
-            float s = ss[z];
-            for (int y = 1; y < 8; ++y) {
-                v = red[y][threadIdx.x] > v ? red[y][threadIdx.x] : v;
-                s += reds[y][threadIdx.x];
-            }
+            for (int y = 1; y < 8; ++y) v = red[y][threadIdx.x] > v ? red[y][threadIdx.x] : v;
             atomicMax(&a.mx[(long long)z * a.f.q + k], v);
-            part[((long long)blockIdx.y * sources + z) * a.f.q + k] = s;
+            if (z == 0) {
+                for (int y = 1; y < 8; ++y) ss += reds[y][threadIdx.x];
+                part[(long long)blockIdx.y * a.f.q + k] = ss;
+            }
         }
         __syncthreads();
     }
@@ -431,14 +431,15 @@ __device__ __forceinline__ int oz_exponent(unsigned long long bits) {
 // Which columns the slices cannot hold well enough: an entry of the product is
 // off by about sqrt(d) 2^-56.3 2^(e_a + e_b) (the slice pairs left out), a
 // binary64 sum by about 2^-55 |a| |b|, so the slices are the nearer ones while
-// 2^e <= 1.6 d^(-1/4) |x| for both columns.  Dense columns are (random ones
-// from d = 200 on: 2^e is at most 8 |x| / sqrt(d)); a column with an entry that
-// holds much of its norm is not, and its entries come from k_oz_f64.  RMS error
+// 2^e <= 1.6 d^(-1/4) |x| for both columns.  Dense columns are (of random ones,
+// at the least favourable scale, all but 7 % at d = 512, 0.7 % at 1024 and none
+// at 3584); a column with an entry that holds much of its norm is not, and its
+// entries come from k_oz_f64.  RMS error
 // over |a| |b| of the slices and of the binary64 sum, d = 3584: dense 9e-18 and
 // 4e-17; a peak of 0.2 of the norm in each column, on different rows, 4.9e-17
 // and 4.1e-17 (ratio 1.94); of 0.5, 6.6e-16 and 3.2e-17.  Columns outside
-// 2^-55 .. 2^50, where the binary32 sum of squares does not reach, are left to
-// binary64 as well; zero columns are exact, and non-finite ones NaN either way.
+// 2^-55 .. 2^50, where the binary32 sum of the first operand's squares does not
+// reach, are left to binary64 as well; zero columns are exact, and non-finite ones NaN either way.
 __global__ void __launch_bounds__(256) k_oz_columns(OzSrc a, int sources, int row_chunks, const float* part) {
     pdl_enter();
     const long long q = a.f.q, k = (long long)blockIdx.x * 256 + threadIdx.x;
@@ -448,7 +449,8 @@ __global__ void __launch_bounds__(256) k_oz_columns(OzSrc a, int sources, int ro
     const int e = oz_exponent(bits);
     if (bits == 0 || e >= OZ_NONFINITE) return;
     float s = 0.0f;
-    for (int c = 0; c < row_chunks; ++c) s += part[((long long)c * sources + z) * q + k];
+    if (z) s = (float)a.cd[((long long)(z - 1) * (sources - 1) + z - 1) * q + k];
+    else for (int c = 0; c < row_chunks; ++c) s += part[(long long)c * q + k];
     const float lim = 1.6f * 1.6f * rsqrtf((float)a.f.d);            // of (2^e / |x|)^2
     if (e < -55 || e > 50 || !(exp2f((float)(2 * e)) <= lim * s)) {
         int32_t* const list = a.peaked + z * (1 + q);
@@ -1087,7 +1089,7 @@ int exact_product(cudaStream_t s, int sms, const OzSrc& src, int K, double* C, u
     const int rc = (int)std::max(1LL, std::min(256LL, (d + 255) / 256));
     const dim3 mg((unsigned)((q + 31) / 32), rc), mb(32, 8);
     float* const part = reinterpret_cast<float*>(scratch);      // read before the slabs are written
-    if (scratch_bytes / sizeof(float) < (size_t)rc * (K + 1) * q) return ISO_ERR_WORKSPACE;
+    if (scratch_bytes / sizeof(float) < (size_t)rc * q) return ISO_ERR_WORKSPACE;
     if (K == 0) FR_LAUNCH((pdl_launch(k_oz_colmax<1>, mg, mb, 0, s, src, K + 1, rc, part)));
     else if (K <= 2) FR_LAUNCH((pdl_launch(k_oz_colmax<3>, mg, mb, 0, s, src, K + 1, rc, part)));
     else if (K <= 4) FR_LAUNCH((pdl_launch(k_oz_colmax<5>, mg, mb, 0, s, src, K + 1, rc, part)));
@@ -1287,7 +1289,7 @@ int32_t iso_frame_merge(const double* U0, const double* S0, const double* Vt0, c
     // A_i = F_0^T dF_i (binary64), then Sym_i and Kw_i
     for (int sd = 0; sd < 2; ++sd) {
         OzSrc oz{fr[sd], dots, nullptr, reinterpret_cast<unsigned long long*>(ws + L.mx[sd]),
-                 reinterpret_cast<int32_t*>(ws + L.ex), Qp, reinterpret_cast<int32_t*>(ws + L.sym[sd])};
+                 reinterpret_cast<int32_t*>(ws + L.ex), Qp, reinterpret_cast<int32_t*>(ws + L.sym[sd]), D(L.cd[sd])};
         ISO_TRY(exact_product(s, sms, oz, K, D(L.aq[sd]), reinterpret_cast<unsigned char*>(ws + L.tail),
                               L.total - L.tail, &hdr->status));
         FR_LAUNCH((pdl_launch(k_fr_symskew, dim3((unsigned)(Qp / 32), (unsigned)(Qp / 32), K), dim3(32, 8), 0, s, 
@@ -1446,7 +1448,7 @@ int32_t iso_opt_step(double* U, double* V, const double* S0, const iso_tensor* G
     for (int sd = 0; sd < 2; ++sd) {
         const long long Dp = sd == 0 ? L.Mp : L.Np, d = fr[sd].d;
         OzSrc oz{fr[sd], nullptr, D(L.dF[sd]), reinterpret_cast<unsigned long long*>(ws + L.mx[sd]),
-                 reinterpret_cast<int32_t*>(ws + L.ex), Qp, reinterpret_cast<int32_t*>(ws + L.ns_y)};
+                 reinterpret_cast<int32_t*>(ws + L.ex), Qp, reinterpret_cast<int32_t*>(ws + L.ns_y), nullptr};
         ISO_TRY(exact_product(s, sms, oz, 0, D(L.n64), reinterpret_cast<unsigned char*>(ws + L.gw4),
                               L.dF[0] - L.gw4, &hdr->status));
         NsBufs nb{D(L.ns_y), D(L.ns_z), D(L.ns_m), F(L.ns_y4), F(L.ns_z4), F(L.ns_m4), F(L.ns_t1),

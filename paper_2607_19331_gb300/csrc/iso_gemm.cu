@@ -117,7 +117,10 @@ __device__ __forceinline__ bool wait_phase(uint32_t bar, uint32_t parity, volati
     return false;
 }
 // The same for a whole warp, with one answer for all of its lanes: what
-// follows (tensor-memory loads, products, shuffles) takes every lane.
+// follows (tensor-memory loads, products, shuffles) takes every lane.  The
+// answer is a vote, so that the control flow around the products is uniform
+// by construction (their descriptors live in uniform registers); one lane
+// waiting and passing its answer on by a shuffle is not that, and faulted.
 __device__ __forceinline__ bool wait_phase_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
     return __all_sync(0xFFFFFFFFu, wait_phase(bar, parity, abort_flag));
 }
