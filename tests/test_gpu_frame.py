@@ -1,5 +1,6 @@
-"""GPU parity of the frame-space ISO-Merger (App. E) and of its tensor-core
-product, through the C ABI.
+"""GPU parity of the frame-space ISO-Merger (App. E) and of the plain
+tensor-core product, through the C ABI (the products that the merge itself
+runs: test_gpu_split_product.py, test_gpu_exact_product.py).
 
 * iso_gemm_tf32 (tcgen05.mma, operands staged by TMA, accumulator in tensor
   memory): on operands whose products and sums are exact in binary32 (small
@@ -56,7 +57,7 @@ def _cuda():
     (128, 128, 32, 0, 0, 32, 32),            # one tile, one stage
     (256, 384, 1024, 0, 64, 1024, 1088),     # 6 tiles, the six-stage ring wraps five times
     (384, 128, 224, 32, 0, 256, 224),        # offsets, a contraction of seven stages
-    (128, 256, 3072, 1024, 0, 4096, 3072),   # the split layout's segment offsets
+    (128, 256, 3072, 1024, 0, 4096, 3072),   # a long contraction from an offset
 ])
 def test_gemm_tf32_exact(M_, N_, Kc, a_k0, b_k0, lda, ldb):
     g = torch.Generator().manual_seed(M_ * 7 + Kc)
