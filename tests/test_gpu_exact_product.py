@@ -6,12 +6,14 @@ With dF_i = s_i F_i - F_0, A_i = F_0^T dF_i, Sym_i, Kw_i its halves on each side
     Gamma_ij = sum_k s_k^2 [(dF_i^T dF_j)_kk summed over U and V]
                - sum_rc s_c^2 (A_i Sym_j + Sym_i A_j - Sym_i Sym_j)[r, c] (both sides)
                - sum_rc s_r s_c (KwU_i KwV_j + KwU_j KwV_i)[r, c],
-evaluated here in extended precision.  The product's error against the exact
-sum is below that of a binary64 sum: columns rounded to 55 bits below their
+evaluated here in extended precision.  For dense columns the product's error
+against the exact sum is below that of a binary64 sum: columns rounded to 55 bits below their
 largest magnitude and the slice pairs left out below 2^-57 of |F_0|^T |dF_i|'s
 scale per term; the Gram's own binary64 sums add a few roundings.  Bound:
 2^-46 of the magnitudes summed without cancellation (a wrong digit of any but
 the last slice is above it).
+Columns with a dominant entry, where the slices would be the further form, are
+summed in binary64 and have tests of their own below.
 """
 import numpy as np
 import pytest
